@@ -161,37 +161,6 @@ __device__ __forceinline__ uint32_t cell_of(double x, double y, const Dev &s) {
     return (uint32_t)cell_coord(y, s) * (uint32_t)s.nc + (uint32_t)cell_coord(x, s);
 }
 
-// v rounded toward zero to FP32 on the integer pipe (a conversion on this
-// chip's FP64 pipe would occupy it ~64 cycles per warp instruction, whatever
-// the lane mask, with ~60 cycles of dependent latency): relative error below
-// 2^-23, and
-// |v| < 2^-126 gives 0.
-__device__ __forceinline__ float d2f_trunc(double v) {
-    const unsigned long long b = dbits(v);
-    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-    const int e = (int)((b >> 52) & 0x7FFull) - 1023;
-    if (e < -126) return __int_as_float((int)sign);
-    if (e > 127) return __int_as_float((int)(sign | 0x7F800000u));
-    return __int_as_float(
-        (int)(sign | ((unsigned)(e + 127) << 23) | (unsigned)((b >> 29) & 0x7FFFFFull)));
-}
-
-// The stop rule in FP64 as defined (a call of its own, so that the compiler
-// never evaluates its five FP64 instructions -- ~64 cycles of the FP64 unit
-// each on this GPU -- on the path where the FP32 image decides).
-__device__ __noinline__ bool beyond_exact(double a, double d, double eps, int m, double fx,
-                                          unsigned long long cur) {
-    const double thr = __dsub_rn(__dsub_rn(__dmul_rn((double)m, a), fx), d);
-    const double lim = __dadd_rn(__longlong_as_double((long long)cur), eps);
-    return !dneg(thr) && dbits(thr) > dbits(lim);
-}
-
-// The constants of the stop rule, held in registers by the callers' loops.
-struct StopK {
-    float af, df, epsf, stop_e;
-    double a, d, eps;
-};
-
 __device__ __forceinline__ StopK stopk_of(const Dev &s) {
     StopK k;
     k.af = s.af;
@@ -202,21 +171,6 @@ __device__ __forceinline__ StopK stopk_of(const Dev &s) {
     k.d = s.d;
     k.eps = s.eps;
     return k;
-}
-
-// The scan's stop rule: is thr(m) = ((m a) - fx) - d above RN(cur + eps)?
-// Decided on the FP32 image thr_f - lim_f when that lies farther than stop_e
-// from 0 (its error bound is stop_e / 4, so the answer is the exact one),
-// else in FP64 as defined. lim_f = trunc(cur) + eps in FP32.
-__device__ __forceinline__ bool beyond_k(const StopK &k, int m, double fx, float fxf, float lim_f,
-                                         unsigned long long cur) {
-    if (k.stop_e > 0.f) {
-        const float thr_f = __fsub_rn(__fsub_rn(__fmul_rn(__int2float_rn(m), k.af), fxf), k.df);
-        const float diff = __fsub_rn(thr_f, lim_f);
-        if (diff > k.stop_e) return true;
-        if (diff < -k.stop_e) return false;
-    }
-    return beyond_exact(k.a, k.d, k.eps, m, fx, cur);
 }
 
 __device__ __forceinline__ bool beyond(const Dev &s, int m, double fx, float fxf, float lim_f,
@@ -818,15 +772,6 @@ __device__ int commit_step(const Dev &s, int c, ChainReg &r, const StepOut &o, b
     r.D = 0.0;                                          // stalled
     __syncwarp();
     return ST_STALLED;
-}
-
-// A chain blocked by the window's parallel pass (lane 0): counted, listed for
-// the union-find, and counted against its partner.
-__device__ __forceinline__ void note_blocked(const Dev &s, int c, int32_t partner) {
-    atomicAdd(s.lc + LC_BLOCKED, 1ull);
-    const unsigned long long ix = atomicAdd(s.lc + LC_WBLOCKED, 1ull);
-    if (ix < (unsigned long long)s.k) s.blist[ix] = c;
-    if (partner >= 0 && partner < s.k) atomicAdd(s.pcnt + partner, 1);
 }
 
 #include "rowpass.cuh"
@@ -3242,7 +3187,7 @@ static int runner_run(Runner &rn, cudaStream_t st, ecmc_ctx *const *ctxs, int R,
         for (int r = 0; r < R; ++r) gs[r] = ctxs[r]->graph;
         double ms = 0.0;
         const int grc = graph_batch_run(&rn.gscratch, gs.data(), R, max_legs, budgets, st,
-                                        tots.data(), legs_out, &ms, err);
+                                        tots.data(), legs_out, &ms, err, BARRIER_TIMEOUT_NS);
         if (ms_out) *ms_out = ms;
         for (int r = 0; r < R; ++r) {
             ecmc_ctx *c = ctxs[r];
@@ -3447,7 +3392,8 @@ extern "C" int ecmc_run_to_breakpoint(ecmc_ctx *ctx, int32_t n_legs, uint64_t ev
         GraphTotals t;
         std::string err;
         int32_t legs = 0;
-        const int rc = graph_run(ctx->graph, n_legs, event_budget, leg_flags_out, &legs, &t, err);
+        const int rc = graph_run(ctx->graph, n_legs, event_budget, leg_flags_out, &legs, &t, err,
+                                 BARRIER_TIMEOUT_NS);
         if (legs_done) *legs_done = legs;
         ctx->legs_total += t.legs;
         ctx->lifts_total += t.lifts;

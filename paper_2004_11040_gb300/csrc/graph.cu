@@ -11,21 +11,17 @@
 // stored beside it, so the step does no square root.
 //
 // Layout: one 64-byte record per disk (x, local time, owner word, three arrows
-// and their b); y and the claim words in arrays of their own (y never
-// changes along +x; the claims are cleared window by window).
+// and their b, claim word); y in an array of its own (it never changes along
+// +x).
 //
-// Conflicts are claims on disks instead of cells: within a claim window a
-// chain claims (atomicCAS of the disk's claim word from 0 to chain + 1; the
-// words are cleared between windows) every disk a step reads -- its active
-// disk and the arrow targets -- and uses what it read only once the claims
-// stand. A disk is therefore written only by its claimer
-// during a window, a chain that meets another chain's claim stops, and
-// without a meeting each chain follows the path it takes alone, which is the
-// global-time result (Lemma 2). The leg's flag is 1 iff the disks that two
-// chains read, each run alone from the window's start, overlap. Chains that
-// met are rolled back to the earliest time one of them stopped and replayed
-// in global event-time order (Alg. 2), one warp per conflict component, as on
-// the cell path.
+// Conflicts. Every chain first runs alone from the window's start state, which
+// nothing changes meanwhile (g_spec_chain); a chain then publishes its events
+// up to the first one on a disk that another chain's run reaches earlier
+// (g_resolve_chain). The leg's flag is 1 iff the disks that two chains read,
+// each run alone, overlap. Chains that were cut are continued one after
+// another where Eq. 2 allows it, else rolled back to the earliest time one of
+// them stopped and replayed in global event-time order (Alg. 2), one warp per
+// conflict component, as on the cell path.
 //
 // All FP64 arithmetic uses explicit round-to-nearest intrinsics (the file is
 // compiled with -fmad=false) so that results are reproducible bit for bit.
@@ -36,6 +32,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -50,31 +47,49 @@ namespace {
 constexpr int MAX_CHAINS = (int)OWN_CHAIN;
 
 struct __align__(64) GDisk {
-    double x, t;    // position along the motion; local time (leg-relative)
-    uint32_t own;   // owner word (static / active / stalled + chain)
-    uint32_t pad0;
-    uint32_t a[3];  // arrows: centre, upper, lower corridor (NONE: empty)
-    uint32_t pad1;
-    double b[3];    // b_ij = sqrt(d^2 - dy^2) of each arrow
+    double x, t;               // position along the motion; local time (leg-relative)
+    uint32_t own;              // owner word: active / stalled + chain, or static + the leg
+                               // (stamp) in which t was written (t is 0 in any other leg)
+    uint32_t a[3];             // arrows: centre, upper, lower corridor (NONE: empty)
+    unsigned long long claim;  // pass epoch << 32 | chain + 1 holding the disk in that pass
+    double b[3];               // b_ij = sqrt(d^2 - dy^2) of each arrow
 };
 static_assert(sizeof(GDisk) == 64, "one disk record is one 64-byte line");
 
 // One event of a chain: enough to undo it exactly, and the lifting (Eq. 1).
-struct GEv {
+struct __align__(16) GEv {
     uint32_t i, j, seq, pad;  // moved disk, target (NONE: stall), application order
     double x_old;             // x of i before the move
     double ti_old, tj_old;    // local times of i and j before the event
     double t, tau, xi, xj;    // event time (= new t_j), time of flight, x_i at contact, x_j
     double d_after;           // remaining chain length after the event
 };
+static_assert(sizeof(GEv) == 80, "a record is written as five 16-byte words");
+
+// What a chain's run alone in the parallel pass left.
+struct __align__(16) GSpec {
+    int32_t n, touch;     // events; disks touched
+    int32_t end, partner; // SP_*; the chain met
+    double tc, D;
+    uint32_t ci, pad[3];
+};
 
 struct GDev {
     int64_t n;
     int k, cap, windows, nc;
     double L, d, ell;
-    GDisk *g;        // [n]
-    double *y;       // [n]
-    uint32_t *claim; // [n] 0, or chain + 1 holding the disk in this window
+    GDisk *g;   // [n]
+    double *y;  // [n]
+    // parallel pass: per disk the least touch key (time << 32 | chain) of the
+    // chains whose run alone touches it, ~0 untouched; per chain the touched
+    // disks of its run (entry e of chain c at e * k + c)
+    unsigned long long *key;
+    uint32_t *path;        // [(cap + 2) * k]
+    unsigned long long *fl;  // flag words, epoch << 32 | chain + 1: per disk read
+    uint32_t epoch0;       // epoch of the launch's first pass, less one
+    GSpec *sp;             // [k] the run alone of each chain, for the resolve
+    uint32_t stamp0;       // stamp of the launch's first leg, less one
+    uint32_t stamp;        // stamp of the leg (the warp's copy in shared memory)
     // per chain
     uint32_t *ci, *ci0;  // active disk now / at the leg start
     double *D, *tc;
@@ -87,23 +102,28 @@ struct GDev {
     // conflict components (names as the union-find of common.cuh expects)
     double *vt;
     int32_t *uf, *fin, *comp_of, *abort_to, *comp_cnt, *comp_off, *comp_root, *comp_mem, *ctl;
-    int32_t *nabort;  // [2] components that met another chain, by round parity
-    uint64_t *memb;   // (window, round) << 32 | root of the component listing the chain
+    int32_t *blist, *pcnt;
+    uint64_t *memb;   // (pass of the launch, round) << 32 | root of the component listing the chain
     int restart;      // conflicts by restart strategy 2 (Sec. 3.4) instead of local repair
+    int strict;       // the pass claims every disk a step reads, not only those it touches
     double *tstar;    // [1] restart mode: the earliest stop time of a pass
-    unsigned long long *lc;      // [LC_N]
+    unsigned long long *lc;      // [2 LC_N], by leg parity
     unsigned long long *tc_cnt;  // [TC_N]
     ecmc_lift_t *log;
     int64_t log_cap;
     int log_on;
     double *dbg;  // [16] first failed internal check
 };
+
 // Record e of chain c, stored by event index, then chain (the first events of
 // a leg of all chains lie in one dense block).
 __device__ __forceinline__ GEv *grec_at(const GDev &s, int c, int e) {
     return s.rec + (size_t)e * (size_t)s.k + (size_t)c;
 }
 
+__device__ __forceinline__ uint32_t *gpath_at(const GDev &s, int c, int e) {
+    return s.path + (size_t)e * (size_t)s.k + (size_t)c;
+}
 
 __device__ void gdiag(const GDev &s, int kind, double a, double b, double c, double d,
                       double e, double f) {
@@ -119,16 +139,20 @@ __device__ void gdiag(const GDev &s, int kind, double a, double b, double c, dou
     s.dbg[6] = f;
 }
 
-// Requests a disk record into this SM's L1 ahead of its load (no registers
-// held; the load that follows may still go to L2).
-__device__ __forceinline__ void prefetch_l1(const void *p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
 __device__ __forceinline__ double wrap_add(double x, double dx, double L) {
     double r = __dadd_rn(x, dx);
     if (dbits(r) >= dbits(L)) r = __dsub_rn(r, L);  // r >= 0
     return r;
+}
+
+// The owner word says static; the local time of a static disk in this leg.
+__device__ __forceinline__ bool g_static(uint32_t own) { return own < OWN_ACTIVE; }
+__device__ __forceinline__ double g_time(uint32_t own, double t, uint32_t stamp) {
+    return own >= OWN_ACTIVE || own == stamp ? t : 0.0;
+}
+
+__device__ __forceinline__ double shfl_f64(double v, int src) {
+    return __shfl_sync(FULL, v, src);
 }
 
 // ------------------------------------------------------------ graph build
@@ -351,7 +375,6 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
             r.a[q] = bj[q];
             r.b[q] = bj[q] == NONE ? 0.0 : bb[q];
         }
-        r.pad0 = r.pad1 = 0;
     }
 }
 
@@ -361,7 +384,9 @@ __global__ void k_g_init(GDev s) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q < s.n) {
         s.g[q].own = OWN_STATIC;
-        s.claim[q] = 0u;
+        s.g[q].claim = 0ull;
+        s.key[q] = ~0ull;
+        s.fl[q] = 0ull;
     }
 }
 
@@ -377,20 +402,584 @@ __global__ void k_g_init_chains(GDev s, const int32_t *active) {
 }
 
 
-// --------------------------------------------------------------- one step
+// --------------------------------------------------------- parallel pass
 
-// Another chain's active or stalled disk among the arrow targets of disk i
-// (record r, with b): in a run of Alg. 4 it stops chain i (Remark 10) only if
-// i could reach it within its remaining length D; beyond D it matters only
-// through Eq. 2 (t_i + tau > t_j), which must still hold.
-__device__ __forceinline__ bool active_in_reach(const GDisk &r, double b, double xi, double ti,
-                                                double D, double L) {
-    double dx = __dsub_rn(r.x, xi);
-    if (dneg(dx)) dx = __dadd_rn(dx, L);
-    double tau = __dsub_rn(dx, b);
-    if (dneg(tau)) tau = 0.0;
-    if (dbits(tau) < dbits(D)) return true;
-    return !(dbits(__dadd_rn(ti, tau)) > dbits(r.t));
+// How a chain's run alone ended (sp_end; SP_LAP: it may have come round the
+// box, so that a disk can be in its records more than once).
+enum { SP_STALL = 0, SP_PAUSE = 1, SP_NONSTATIC = 2, SP_LIMIT = 3, SP_END = 3, SP_LAP = 4 };
+
+// Two levels of disk records per warp in shared memory: the records that the
+// targets of the active disk's targets may be next (record 3p + q: arrow q of
+// target p), and the level before. They are copied in asynchronously
+// (cp.async): a load into registers shares one of the warp's few scoreboards
+// with the step's arithmetic and shuffles, which then waited for it (~600 of
+// 1400 cycles an event).
+struct GLevels {
+    GDisk r[2][9];
+};
+__device__ __forceinline__ GLevels &g_levels() {
+    __shared__ GLevels lv[8];  // one per warp of the block
+    return lv[threadIdx.x >> 5];
+}
+
+__device__ __forceinline__ void g_copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void g_copy_wait() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+}
+
+// 16 bytes (part 0 .. 3) of disk id's record into dst; nothing for NONE.
+// (A record that stands for no disk in global memory, read by every warp at
+// every step, made its L2 line a hot spot: 3000 cycles an event.)
+__device__ __forceinline__ void g_fetch_part(const GDisk *g, uint32_t id, GDisk *dst, int part) {
+    if (id != NONE)
+        g_copy16(reinterpret_cast<ulonglong2 *>(dst) + part,
+                 reinterpret_cast<const ulonglong2 *>(g + id) + part);
+}
+
+// Requests the records of the nine arrows of targets from[0 .. 2] into to;
+// none: the targets that are no disk (bit p), whose records are not there.
+__device__ __forceinline__ void g_fetch(const GDisk *g, const GDisk *from, unsigned none,
+                                        GDisk *to) {
+    const int lane = threadIdx.x & 31, z = lane >> 2;
+    const int zp = z / 3, zq = z - 3 * zp;
+    g_fetch_part(g, (none >> zp) & 1u ? NONE : from[zp].a[zq], to + z, lane & 3);
+    if (lane < 4) g_fetch_part(g, (none >> 2) & 1u ? NONE : from[2].a[2], to + 8, lane);
+}
+
+// Requests the records of the active disk i's three targets into to[0 .. 2].
+__device__ __forceinline__ void g_fetch_first(const GDisk *g, uint32_t i, GDisk *to) {
+    const int lane = threadIdx.x & 31;
+    if (lane < 12) g_fetch_part(g, g[i].a[lane >> 2], to + (lane >> 2), lane & 3);
+}
+
+// The targets (tid on lanes 0 .. 2) that are no disk, bit p.
+__device__ __forceinline__ unsigned g_none(uint32_t tid) {
+    return __ballot_sync(FULL, tid == NONE) & 7u;
+}
+
+// FP64 fix-ups of the uncommon case, out of line: the compiler then never
+// evaluates them on the common path (an FP64 instruction occupies its unit
+// ~64 cycles on this chip).
+__device__ __noinline__ double g_add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __noinline__ double g_sub(double a, double b) { return __dsub_rn(a, b); }
+
+// The lane (0 .. 2) with the least (tau, j) (tk: tau bits, INF where the lane
+// has no candidate). The high words decide unless two lanes share theirs (or
+// none has a candidate: some lane with INF then).
+__device__ __forceinline__ int g_winner(unsigned long long tk, uint32_t id) {
+    const unsigned hi = (unsigned)(tk >> 32);
+    const unsigned mh = __reduce_min_sync(FULL, hi);
+    const unsigned eq = __ballot_sync(FULL, hi == mh);
+    const int first = __ffs(eq) - 1;
+    if ((eq & (eq - 1u)) == 0u) return first;
+    const unsigned lo = hi == mh ? (unsigned)tk : ~0u;
+    const unsigned ml = __reduce_min_sync(FULL, lo);
+    const bool tie = hi == mh && lo == ml;
+    const unsigned mj = __reduce_min_sync(FULL, tie ? id : ~0u);
+    return (__ffs(__ballot_sync(FULL, tie && id == mj)) - 1) % 3;
+}
+
+// Up to 32 events of a chain, event e on lane e mod 32, as the steps found
+// them: moved disk, its place, time and remaining length before, tau and the
+// target's local time. What else a record holds is the next event's (its
+// disk is this one's target) or one addition for all lanes.
+struct GEvs {
+    uint32_t i;
+    double x, t, D, tau, tj;
+};
+
+// Writes records n0 .. n - 1 of chain c (n - n0 <= 32 events on the lanes;
+// record index nr0 + e, order key seq0 + e). i, xi, ti, D: the state after
+// event n - 1 (lift: that event is a lifting). Returns this lane's event: the
+// moved disk's new place, its event time and target.
+struct GFlush {
+    bool has;
+    double xn, t;
+    uint32_t j;
+};
+__device__ __forceinline__ GFlush g_flush(const GDev &s, int c, int32_t nr0, uint32_t seq0, int n0,
+                                          int n, const GEvs &E, uint32_t i, double xi, double ti,
+                                          double D, bool lift) {
+    const int lane = threadIdx.x & 31;
+    const int e = n0 + ((lane - n0) & 31);  // this lane's event
+    const bool last = e == n - 1;
+    const int nx = (lane + 1) & 31;
+    const uint32_t inx = __shfl_sync(FULL, E.i, nx);
+    const double xnx = shfl_f64(E.x, nx), tnx = shfl_f64(E.t, nx), dnx = shfl_f64(E.D, nx);
+    GFlush f;
+    f.has = e < n;
+    f.j = last ? (lift ? i : NONE) : inx;
+    f.t = last ? ti : tnx;
+    const double xj = last ? (lift ? xi : 0.0) : xnx;
+    const double da = last ? (lift ? D : 0.0) : dnx;
+    f.xn = __dadd_rn(E.x, E.tau);
+    const bool wrap = f.has && dbits(f.xn) >= dbits(s.L);
+    if (__any_sync(FULL, wrap) && wrap) f.xn = g_sub(f.xn, s.L);
+    if (f.has) {
+        ulonglong2 *u = reinterpret_cast<ulonglong2 *>(grec_at(s, c, nr0 + e));
+        u[0] = make_ulonglong2((unsigned long long)E.i | ((unsigned long long)f.j << 32),
+                               (unsigned long long)(seq0 + (uint32_t)e));
+        u[1] = make_ulonglong2(dbits(E.x), dbits(E.t));
+        u[2] = make_ulonglong2(dbits(E.tj), dbits(f.t));
+        u[3] = make_ulonglong2(dbits(E.tau), dbits(f.xn));
+        u[4] = make_ulonglong2(dbits(xj), dbits(da));
+    }
+    return f;
+}
+
+__device__ __forceinline__ unsigned long long g_key(double t, int c) {
+    return ((unsigned long long)(unsigned)__float_as_int(d2f_trunc(t)) << 32) | (unsigned)c;
+}
+
+// Liftings after which a chain's run may come round the box to a disk it
+// moved: n liftings advance by at most n d + (the time gone), and a target
+// behind lies L less that ahead, out of reach while it exceeds what is left
+// of ell.
+__device__ __forceinline__ int g_lap(const GDev &s) {
+    const float f = __fsub_rn(__fdiv_rn(d2f_trunc(__dsub_rn(s.L, s.ell)), d2f_trunc(s.d)), 4.f);
+    return f > 1e9f ? 1000000000 : (int)f;
+}
+
+// Chain c at the start of a leg, on its stalled disk i with D = ell (one warp).
+__device__ __forceinline__ void g_begin_state(const GDev &s, int c, uint32_t i, int lane) {
+    if (lane != 0) return;
+    s.g[i].t = 0.0;
+    s.g[i].own = OWN_ACTIVE | (uint32_t)c;
+    s.ci0[c] = i;
+    s.D[c] = s.ell;
+    s.tc[c] = 0.0;
+    s.status[c] = ST_RUNNING;
+    s.partner[c] = -1;
+    s.nrec[c] = 0;
+    s.nlift[c] = 0;
+}
+
+// Parallel pass of a claim window [tw, tend): one warp runs chain c alone from
+// the window-start state -- the isolated run of the conflict flag -- and
+// writes no disk, so a step waits for one round of loads and for nothing
+// else. While lanes 0 .. 2 compute the times of flight to the active disk's
+// three targets, the records of those targets' nine arrows are already on
+// their way: whichever target wins, the next step's records are there. Events
+// stay on the lanes until 32 are there or the run ends. (One thread per chain
+// with an atomicCAS per disk read took ~4000 cycles an event; a warp that
+// handed records on by shuffles and wrote each event at once 3300; records
+// in registers 1400.)
+//
+// What the run posts, without waiting: its events as records, and the disks
+// it touches (its active disks) in path with a touch key in s.key
+// (g_resolve_chain). The flag's words follow later (g_flag_chain).
+//
+// Another chain's active or stalled disk among the targets ends the run
+// there if it lies in reach nearer than the winner (Remark 10). With claim
+// windows or restarts a chain's disk lies behind its true place at the
+// window's start (lazy frame), so the pass is strict there: such a disk in
+// reach at all, or failing Eq. 2, ends the run, and the read disks are
+// claimed like the touched ones.
+//
+// A step is bound by its instructions (one warp runs alone on its
+// sub-partition, ~10 cycles an instruction), so the loop holds what every
+// step needs; everything else waits for the flush or stands behind any_odd.
+__device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, double tend,
+                                          bool begin) {
+    const int lane = threadIdx.x & 31;
+    // (loads of one round trip: the chain's state, used or not)
+    uint32_t i = s.ci[c];
+    double ti = s.tc[c], D = s.D[c];
+    int32_t nr0 = s.nrec[c];
+    const int32_t st0 = s.status[c];
+    if (begin) {
+        ti = 0.0;
+        D = s.ell;
+        nr0 = 0;
+        g_begin_state(s, c, i, lane);
+    } else if (st0 != ST_RUNNING) {
+        if (lane == 0) s.sp[c].touch = 0;
+        return;
+    }
+    const int l3 = lane % 3;
+    const double L = s.L;
+    const bool strict = s.strict != 0;
+    unsigned long long *const key = s.key;
+    const GDisk *const g = s.g;
+    const uint32_t stamp = s.stamp;
+    const bool bounded = dbits(tend) != INF_BITS;
+    const int room = s.cap - nr0, n_lap = g_lap(s);
+    double xi = g[i].x;
+    const uint32_t own0 = g[i].own;
+    GLevels &lv = g_levels();
+    int cb = 0, sl = 0;  // the active disk's targets: lv.r[cb][sl .. sl + 2]
+    g_fetch_first(g, i, lv.r[0]);
+    uint32_t tid = g[i].a[l3];
+    double tb = g[i].b[l3];
+    unsigned none = g_none(tid);
+    g_copy_wait();
+    if (lane == 0 && (g_static(own0) || (own0 & OWN_CHAIN) != (uint32_t)c))
+        gdiag(s, 6, tw, c, i, own0, 0, 0);
+    if (lane == 31) {
+        *gpath_at(s, c, 0) = i;
+        red_min_u64(key + i, g_key(ti, c));
+    }
+    GEvs E;
+    E.i = NONE;
+    E.x = E.t = E.D = E.tau = E.tj = 0.0;
+    int n = 0, nf = 0, end = SP_PAUSE;  // nf: events written out
+    uint32_t partner = NONE;
+    // events nf .. n - 1 to memory, with the touched disks and their keys
+    auto flush = [&](bool lift) {
+        if (n == nf) return;
+        const GFlush f = g_flush(s, c, nr0, (uint32_t)nr0, nf, n, E, i, xi, ti, D, lift);
+        if (f.has) {
+            if (f.j != NONE) {
+                *gpath_at(s, c, nf + ((lane - nf) & 31) + 1) = f.j;
+                red_min_u64(key + f.j, g_key(f.t, c));
+            }
+            if (strict) {
+#pragma unroll
+                for (int z = 0; z < 3; ++z)
+                    if (g[E.i].a[z] != NONE) red_min_u64(key + g[E.i].a[z], g_key(E.t, c));
+            }
+            if (dbits(f.t) < dbits(tw)) {
+                // a window's events start at its start time (repairs roll back to it)
+                atomicAdd(s.lc + LC_ORDER, 1ull);
+                gdiag(s, 9, tw, c, E.i, f.j, E.t, E.tau);
+            }
+        }
+        E.tj = 0.0;
+        nf = n;
+    };
+    // the next event index at which the loop has to do more than a step
+    int n_stop = min(min(room, 32), max(n_lap + 1, 0));
+    for (;;) {
+        const GDisk *const R = &lv.r[cb][sl];
+        // the records beyond the targets
+        g_fetch(g, R, none, lv.r[cb ^ 1]);
+        const bool ev = lane < 3 && tid != NONE;
+        double rx = R[l3].x, rt = R[l3].t;
+        uint32_t own = R[l3].own;
+        if (n >= n_stop) {
+            if (n - nf == 32) flush(true);
+            if (n > n_lap) {
+                // a target the run itself has moved: its place and time from
+                // the run's latest record of it
+                flush(true);
+                __syncwarp();
+                for (int z = 0; z < 3; ++z) {
+                    const uint32_t id = __shfl_sync(FULL, tid, z);
+                    int best = -1;
+                    for (int e = lane; id != NONE && e < n; e += 32)
+                        if (grec_at(s, c, nr0 + e)->i == id) best = e;
+                    best = __reduce_max_sync(FULL, best);
+                    if (best >= 0 && l3 == z) {
+                        const GEv &u = *grec_at(s, c, nr0 + best);
+                        rx = u.xi;
+                        rt = u.t;
+                        own = stamp;
+                    }
+                }
+                n_stop = n + 1;
+            } else {
+                n_stop = min(nf + 32, n_lap + 1);
+            }
+            n_stop = min(n_stop, max(room, n + (n < room ? 1 : 0)));
+        }
+        // time of flight to each target (Sec. 2.2): forward image in x, b_ij
+        // fixed with the arrow, clamped at 0
+        double dx = __dsub_rn(rx, xi);
+        double tau = __dsub_rn(dx, tb);
+        // (anything but a static disk ahead, not moved in this leg)
+        const bool odd = ev && (own >= OWN_ACTIVE || own == stamp ||
+                                __double_as_longlong(dx) < 0);
+        const bool any_odd = __any_sync(FULL, odd);
+        bool nsc = false, hv = false, lap = false;
+        if (any_odd) {
+            if (odd && __double_as_longlong(dx) < 0) tau = g_sub(g_add(dx, L), tb);
+            if (__double_as_longlong(tau) < 0) tau = 0.0;
+            nsc = ev && own >= OWN_ACTIVE;
+            rt = g_time(own, rt, stamp);
+            if (ev && dbits(rt) != 0ull) {
+                const double sum = g_add(ti, tau);
+                // a target with t_i + tau < t_j became static after the
+                // chain's disk had passed it and is one lap away (lazy
+                // per-chain frame)
+                lap = !nsc && dbits(sum) < dbits(rt);
+                if (lap) tau = g_add(tau, L);
+                hv = nsc && !(dbits(sum) > dbits(rt));
+            }
+        }
+        if (__double_as_longlong(tau) < 0) tau = 0.0;
+        const unsigned long long tk = ev && !nsc ? dbits(tau) : INF_BITS;
+        const int wl = g_winner(tk, tid);
+        const unsigned long long bt = shfl_u64(tk, wl);
+        const uint32_t bj = __shfl_sync(FULL, tid, wl);
+        const double xj = shfl_f64(rx, wl);
+        if (any_odd) {
+            // another chain's disk among the targets
+            const bool stop = nsc && (strict ? hv || dbits(tau) < dbits(D)
+                                             : dbits(tau) <= bt && dbits(tau) < dbits(D));
+            const unsigned sb = __ballot_sync(FULL, stop);
+            if (sb) {
+                partner = __shfl_sync(FULL, own, __ffs(sb) - 1) & OWN_CHAIN;
+                end = SP_NONSTATIC;
+                break;
+            }
+            const double tj = shfl_f64(rt, wl);
+            if (lane == (n & 31)) E.tj = bt < dbits(D) ? tj : 0.0;
+        }
+        const bool lift = bt < dbits(D);
+        const double ts = lift ? __longlong_as_double((long long)bt) : D;
+        const double T = __dadd_rn(ti, ts);
+        if (n >= room) {  // out of records: the repair goes on from here, or reports it
+            end = SP_LIMIT;
+            break;
+        }
+        if (bounded && !(dbits(T) < dbits(tend))) break;  // pauses at the window end
+        if (lane == (n & 31)) {
+            E.i = i;
+            E.x = xi;
+            E.t = ti;
+            E.D = D;
+            E.tau = ts;
+        }
+        ++n;
+        ti = T;
+        if (!lift) {
+            end = SP_STALL;
+            D = 0.0;
+            break;
+        }
+        D = __dsub_rn(D, ts);
+        xi = xj;
+        i = bj;
+        tid = R[wl].a[l3];
+        tb = R[wl].b[l3];
+        none = g_none(tid);
+        g_copy_wait();
+        cb ^= 1;
+        sl = 3 * wl;
+    }
+    g_copy_wait();
+    // (the reads of a step that was evaluated but not taken)
+    if (strict && end != SP_STALL && lane < 3 && tid != NONE) red_min_u64(key + tid, g_key(ti, c));
+    flush(end != SP_STALL);
+    if (lane == 0) {
+        GSpec r;
+        r.n = n;
+        r.touch = end == SP_STALL ? n : n + 1;
+        r.end = end | (n > n_lap ? SP_LAP : 0);
+        r.partner = partner < (uint32_t)s.k ? (int32_t)partner : -1;
+        r.tc = ti;
+        r.D = D;
+        r.ci = i;
+        r.pad[0] = r.pad[1] = r.pad[2] = 0u;
+        s.sp[c] = r;
+    }
+    __syncwarp();
+}
+
+// Touch keys of chain c back to empty (one warp): every disk its last run
+// alone posted a key for.
+__device__ __forceinline__ void g_reset_keys(const GDev &s, int c, int lane) {
+    const int nt = s.sp[c].touch;
+    unsigned long long *const key = s.key;
+    for (int e = lane; e < nt; e += 32) {
+        const uint32_t id = *gpath_at(s, c, e);
+        key[id] = ~0ull;
+        if (s.strict) {
+            const GDisk &r = s.g[id];
+#pragma unroll
+            for (int z = 0; z < 3; ++z)
+                if (r.a[z] != NONE) key[r.a[z]] = ~0ull;
+        }
+    }
+}
+
+// The conflict flag (one warp, after the pass): chain c puts its word (epoch,
+// chain) into s.fl for every disk its run alone read, its start disk and the
+// arrow targets of every disk that was active. Two chains read one disk iff
+// one of them is handed the other's word of this epoch; the epoch makes
+// clearing unnecessary. Nothing waits for the result before the leg's totals,
+// so the warps without a component do this while the others repair.
+__device__ __noinline__ void g_flag_chain(const GDev &s, int c, uint32_t epoch, int lane) {
+    const int nt = s.sp[c].touch;
+    const unsigned long long tag = ((unsigned long long)epoch << 32) | ((unsigned)c + 1u);
+    bool met = false;
+    for (int e = lane; e < nt; e += 32) {
+        const uint32_t id = *gpath_at(s, c, e);
+        const GDisk &r = s.g[id];
+        uint32_t a[4] = {r.a[0], r.a[1], r.a[2], e == 0 ? id : NONE};
+        unsigned long long w[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) w[z] = a[z] != NONE ? atomicExch(s.fl + a[z], tag) : 0ull;
+#pragma unroll
+        for (int z = 0; z < 4; ++z)
+            met |= (uint32_t)(w[z] >> 32) == epoch && (uint32_t)w[z] != (uint32_t)tag;
+    }
+    if (__any_sync(FULL, met) && lane == 0) {
+        atomicAdd(s.lc + LC_WEAK, 1ull);
+        atomicAdd(s.lc + LC_WWEAK, 1ull);
+    }
+}
+
+// After the pass (one warp): the first step of chain c's run that touches a
+// disk another chain holds, the events before it published, the chain's
+// state, the claims of the touched disks.
+//
+// The least key (earliest touch, then lower chain) holds a disk; a chain is
+// cut at its first step that lifts onto a disk it does not hold. Published
+// events are therefore on disks that no other chain's published events
+// touch, and that makes them exact. Take the first event, in global time, at
+// which a published chain A would differ from its run alone. A's disk is
+// where it was in that run. A candidate that nobody touched before is where
+// A read it; one that others touched lies farther ahead (motion is along +x,
+// and no disk passes another within d of it in y) or is active; a disk that
+// was active at the window's start lies no nearer than the winner or beyond
+// reach there, or the run ended (SP_NONSTATIC). The winner itself A holds. So
+// the least time of flight is the one of the run alone: no difference. What
+// a chain only reads needs no claim of its own. (The repair's continuation
+// claims what it reads: there a disk may already lie where another chain
+// moved it at a later time.)
+//
+// With the claims on every disk read (three per event) 508 of 2048 chains on
+// 262144 dense disks were blocked per leg; touched disks alone: about a
+// third of that.
+__device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, uint32_t epoch) {
+    const int lane = threadIdx.x & 31;
+    // the chain's state and the first touched disks in one round of loads
+    const GSpec sp = s.sp[c];
+    const int32_t st0 = s.status[c], nr0 = s.nrec[c];
+    uint32_t pid = lane < s.cap ? *gpath_at(s, c, lane) : NONE;
+    if (st0 != ST_RUNNING) return;
+    const int n = sp.n, nt = sp.touch, end = sp.end & SP_END;
+    const bool serial = (sp.end & SP_LAP) != 0;
+    const unsigned long long tag = ((unsigned long long)epoch << 32) | ((unsigned)c + 1u);
+    int sfail = n;
+    bool lost = false;
+    uint32_t holder = NONE;
+    for (int e0 = 0; e0 < nt && !lost; e0 += 32) {
+        const int e = e0 + lane;
+        // the first step this entry loses: its touch (by the step before), or
+        // (strict) a read of the step it is active in
+        int st = 0x7FFFFFFF;
+        uint32_t h = NONE;
+        if (e < nt) {
+            const uint32_t id = e0 == 0 && lane < s.cap ? pid : *gpath_at(s, c, e);
+            if (s.strict) {
+                const GDisk &r = s.g[id];
+#pragma unroll
+                for (int z = 0; z < 3; ++z)
+                    if (r.a[z] != NONE) {
+                        const uint32_t hz = (uint32_t)__ldcg(s.key + r.a[z]);
+                        if (hz != (uint32_t)c) {
+                            st = e;
+                            h = hz;
+                        }
+                    }
+            }
+            const uint32_t ht = (uint32_t)__ldcg(s.key + id);
+            if (ht != (uint32_t)c) {
+                st = e > 0 ? e - 1 : 0;
+                h = ht;
+            }
+        }
+        const int first = __reduce_min_sync(FULL, st);
+        if (first != 0x7FFFFFFF) {
+            const unsigned hm = __ballot_sync(FULL, st == first);
+            holder = __shfl_sync(FULL, h, __ffs(hm) - 1);
+            lost = true;
+            sfail = first < n ? first : n;
+        }
+    }
+    // publish records 0 .. sfail - 1; the lane of the last one keeps its time
+    // and remaining length for the chain's state
+    int lifts = 0;
+    double lt = 0.0, ld = 0.0;
+    for (int e0 = 0; e0 < sfail; e0 += serial ? 1 : 32) {
+        const int e = e0 + lane;
+        const bool mine = serial ? lane == 0 : e < sfail;
+        uint32_t rj = NONE;
+        if (mine) {
+            const ulonglong2 *u = reinterpret_cast<const ulonglong2 *>(grec_at(s, c, nr0 + e));
+            const ulonglong2 u0 = u[0], u2 = u[2], u3 = u[3], u4 = u[4];
+            rj = (uint32_t)(u0.x >> 32);
+            GDisk &r = s.g[(uint32_t)u0.x];
+            *reinterpret_cast<ulonglong2 *>(&r.x) = make_ulonglong2(u3.y, u2.y);
+            r.own = rj != NONE ? s.stamp : (OWN_STALLED | (uint32_t)c);
+            r.claim = tag;
+            lt = __longlong_as_double((long long)u2.y);
+            ld = __longlong_as_double((long long)u4.y);
+        }
+        lifts += __popc(__ballot_sync(FULL, mine && rj != NONE));
+        if (serial) __syncwarp();
+    }
+    const int ll = serial ? 0 : (sfail + 31) & 31;
+    lt = shfl_f64(lt, ll);
+    ld = shfl_f64(ld, ll);
+    __syncwarp();
+    if (lane == 0) {
+        int st;
+        uint32_t id;
+        double tc, D;
+        int32_t partner = -1;
+        if (sfail < n) {
+            id = *gpath_at(s, c, sfail);
+            tc = sfail > 0 ? lt : s.tc[c];
+            D = sfail > 0 ? ld : s.D[c];
+            st = ST_BLOCKED;
+            partner = (int32_t)holder;
+        } else {
+            id = sp.ci;
+            tc = sp.tc;
+            D = sp.D;
+            st = end == SP_STALL ? ST_STALLED : ST_RUNNING;
+            if (lost) {
+                st = ST_BLOCKED;
+                partner = (int32_t)holder;
+            } else if (end == SP_NONSTATIC || end == SP_LIMIT) {
+                st = ST_BLOCKED;
+                partner = sp.partner;
+            }
+        }
+        if (st != ST_STALLED) {
+            GDisk &r = s.g[id];
+            if (sfail > 0) {
+                r.own = OWN_ACTIVE | (uint32_t)c;
+                r.t = tc;
+            }
+            r.claim = tag;
+        }
+        s.ci[c] = id;
+        s.tc[c] = tc;
+        s.D[c] = D;
+        s.status[c] = st;
+        s.nrec[c] = nr0 + sfail;
+        s.nlift[c] += lifts;
+        s.partner[c] = partner;
+        // events before the blocking time, and all before the window, are exact
+        s.vt[c] = st == ST_BLOCKED ? fmax(tc, tw) : INFINITY;
+        if (st == ST_BLOCKED) note_blocked(s, c, partner);
+        if (lifts) atomicAdd(s.lc + LC_P1LIFTS, (unsigned long long)lifts);
+    }
+    __syncwarp();
+}
+
+// ------------------------------------------------------------ repair steps
+
+// Claims disk id for the pass (tag: epoch << 32 | chain + 1): the word of the
+// chain that holds it in this epoch (chain + 1; that stays), or 0. A word of an
+// earlier epoch is free, so nothing has to be cleared between passes.
+__device__ __forceinline__ uint32_t g_holder(unsigned long long w, unsigned long long tag) {
+    return (uint32_t)(w >> 32) == (uint32_t)(tag >> 32) ? (uint32_t)w : 0u;
+}
+__device__ __forceinline__ uint32_t g_claim(const GDev &s, uint32_t id, unsigned long long tag) {
+    const unsigned long long w = __ldcg(&s.g[id].claim);
+    const uint32_t h = g_holder(w, tag);
+    return h ? h : g_holder(atomicCAS(&s.g[id].claim, w, tag), tag);
 }
 
 // What one step found.
@@ -401,10 +990,6 @@ struct GStep {
     double xj, tj;     // the target's x and local time as read
     int conflict;      // a disk read is held by a chain of the other side
     uint32_t partner;  // that chain
-    int viol;          // a static target fails Eq. 2 (t_i + tau > t_j, strict)
-    int nonstatic;     // a target is another chain's active or stalled disk in reach ...
-    uint32_t ns_owner; // ... of this chain (the first such target)
-    GDisk jr;          // the target's record as read: its arrows serve the next step
 };
 
 // Is chain h, which holds a claim a repair step met, on the repairing side?
@@ -430,29 +1015,25 @@ __device__ __forceinline__ bool holder_ours(const GDev &s, int h, int root, uint
     return hc == root;
 }
 
-// The next event of chain c (Sec. 2.2) along the arrows a[] (with b[]) of
-// its active disk i at x_i, t_i, with remaining length D. Every disk read is
-// claimed for the window (atomicCAS of the disk's claim word from 0 to c + 1,
-// issued together with the loads; what was read is used only once the claims
-// stand): i itself when claim_i, and each arrow target. A claim held by
+// The next event of chain c in a replay (Sec. 2.2) along the arrows a[] (with
+// b[]) of its active disk i at x_i, t_i, with remaining length D. Every disk
+// read -- i and the arrow targets -- is claimed for the pass, together with
+// the loads; what was read is used only once the claims stand. A claim of
 // another chain is a conflict unless that chain is listed in this round's
-// component (memb == tag). adopt (continuation): a holder in no component of
-// this round, whose events are final since the round began, is taken over by
-// the component (it joins it for any later merge) instead of being a conflict;
-// the replay that a failed continuation falls back to does not count such
-// chains as members, so it meets them and merges them next round.
-// Candidates are the static targets (Alg. 2: j not active); a target with
-// t_i + tau < t_j became static after chain c's disk had passed it and is one
-// lap away (lazy per-chain frame); ties go to the lower disk index.
-__device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, const uint32_t a[3],
-                            const double b[3], uint32_t i, double xi, double ti, double D,
-                            bool claim_i, bool adopt = false) {
+// component (memb == tag). Candidates are the static targets (Alg. 2: j not
+// active); a target with t_i + tau < t_j became static after chain c's disk
+// had passed it and is one lap away (lazy per-chain frame); ties go to the
+// lower disk index.
+__device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, uint32_t epoch,
+                            const uint32_t a[3], const double b[3], uint32_t i, double xi,
+                            double ti, double D) {
     const uint32_t mine = (uint32_t)c + 1u;
+    const unsigned long long ct = ((unsigned long long)epoch << 32) | mine;
     uint32_t old[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-        if (a[q] != NONE) old[q] = atomicCAS(s.claim + a[q], 0u, mine);
-    if (claim_i) old[3] = atomicCAS(s.claim + i, 0u, mine);
+        if (a[q] != NONE) old[q] = g_claim(s, a[q], ct);
+    old[3] = g_claim(s, i, ct);
     GDisk r[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q)
@@ -460,9 +1041,6 @@ __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, const 
     GStep o;
     o.conflict = 0;
     o.partner = NONE;
-    o.viol = 0;
-    o.nonstatic = 0;
-    o.ns_owner = NONE;
     // time of flight to each static target (Sec. 2.2): forward image in x,
     // b_ij fixed with the arrow, clamped at 0
     unsigned long long bt = INF_BITS;
@@ -470,23 +1048,13 @@ __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, const 
     uint32_t bjid = NONE;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        if (a[q] == NONE) continue;
-        if (r[q].own != OWN_STATIC) {
-            if (!o.nonstatic && active_in_reach(r[q], b[q], xi, ti, D, s.L)) {
-                o.ns_owner = r[q].own & OWN_CHAIN;
-                o.nonstatic = 1;
-            }
-            continue;
-        }
+        if (a[q] == NONE || !g_static(r[q].own)) continue;
+        const double rt = g_time(r[q].own, r[q].t, s.stamp);
         double dx = __dsub_rn(r[q].x, xi);
         if (dneg(dx)) dx = __dadd_rn(dx, s.L);
         double tau = __dsub_rn(dx, b[q]);
         if (dneg(tau)) tau = 0.0;
-        if (dbits(r[q].t) != 0ull) {
-            const double sum = __dadd_rn(ti, tau);
-            if (!(dbits(sum) > dbits(r[q].t))) o.viol = 1;
-            if (dbits(sum) < dbits(r[q].t)) tau = __dadd_rn(tau, s.L);
-        }
+        if (dbits(rt) != 0ull && dbits(__dadd_rn(ti, tau)) < dbits(rt)) tau = __dadd_rn(tau, s.L);
         const unsigned long long tb = dbits(tau);
         if (bq < 0 || tb < bt || (tb == bt && a[q] < bjid)) {
             bt = tb;
@@ -500,7 +1068,7 @@ __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, const 
         const uint32_t w = old[q];
         if (w == 0u || w == mine) continue;
         const int h = (int)w - 1;
-        if (holder_ours(s, h, root, tag, adopt)) continue;
+        if (holder_ours(s, h, root, tag, false)) continue;
         if (!o.conflict) {
             o.conflict = 1;
             o.partner = (uint32_t)h;
@@ -510,11 +1078,11 @@ __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, const 
         o.lift = 1;
         o.tau = __longlong_as_double((long long)bt);
         o.j = bjid;
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (q == bq) o.jr = r[q];  // a select, not an indexed (local-memory) load
-        o.xj = o.jr.x;
-        o.tj = o.jr.t;
+        // selects, not an indexed (local-memory) load
+        o.xj = bq == 0 ? r[0].x : bq == 1 ? r[1].x : r[2].x;
+        o.tj = bq == 0   ? g_time(r[0].own, r[0].t, s.stamp)
+               : bq == 1 ? g_time(r[1].own, r[1].t, s.stamp)
+                         : g_time(r[2].own, r[2].t, s.stamp);
     } else {
         o.lift = 0;
         o.tau = D;
@@ -545,7 +1113,7 @@ __device__ void graph_apply(const GDev &s, int c, uint32_t i, double xi, double 
         rj.t = tnew;
         ri.t = tnew;
         ri.x = xnew;
-        ri.own = OWN_STATIC;                           // i static
+        ri.own = s.stamp;                              // i static
         u.j = j;
         u.tj_old = tj;
         u.t = tnew;
@@ -572,192 +1140,35 @@ __device__ void graph_apply(const GDev &s, int c, uint32_t i, double xi, double 
 
 // ------------------------------------------------------------------ legs
 
-// Leg start: clear the local times the previous leg wrote (every disk its
-// records name), then start every chain on its stalled disk with D = ell.
-__device__ void g_leg_begin_chain(const GDev &s, int c) {
-    const int32_t nr = s.nrec[c];
-    // in batches: the record loads of a batch are issued before its stores
-    for (int32_t e0 = 0; e0 < nr; e0 += 8) {
-        uint32_t ii[8], jj[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            ii[u] = e0 + u < nr ? grec_at(s, c, e0 + u)->i : NONE;
-            jj[u] = e0 + u < nr ? grec_at(s, c, e0 + u)->j : NONE;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (ii[u] != NONE) s.g[ii[u]].t = 0.0;
-            if (jj[u] != NONE) s.g[jj[u]].t = 0.0;
-        }
-    }
-    const uint32_t i = s.ci[c];
-    s.g[i].own = OWN_ACTIVE | (uint32_t)c;
-    s.ci0[c] = i;
-    s.D[c] = s.ell;
-    s.tc[c] = 0.0;
-    s.status[c] = ST_RUNNING;
-    s.partner[c] = -1;
-    s.nrec[c] = 0;
-    s.nlift[c] = 0;
-}
-
-// Parallel pass of a claim window [tw, tend): one thread runs chain c from
-// its state through its events before tend, until it stalls, pauses at tend
-// or meets another chain: a claim it holds, or its active or stalled disk
-// among the arrow targets within reach (the step is then not taken; cf.
-// Remark 10). Once a
-// step's winner j is known (and the step will be taken unless a claim of it
-// fails), the arrow targets of j are claimed and their records loaded into
-// registers, so that the next step's trips overlap this step's wait and
-// writes (an L1 prefetch measured no better than a plain L2 load). Those
-// disks belong to the chain's run alone, so the claims change no flag.
-__device__ __noinline__ void g_pass1_chain(const GDev &s, int c, double tw, double tend) {
-    if (s.status[c] != ST_RUNNING) return;
-    const uint32_t mine = (uint32_t)c + 1u;
-    uint32_t i = s.ci[c];
-    const GDisk ri = s.g[i];
-    if (ri.own != (OWN_ACTIVE | (uint32_t)c)) gdiag(s, 6, tw, c, i, ri.own, 0, 0);
-    uint32_t a[3] = {ri.a[0], ri.a[1], ri.a[2]};
-    double b[3] = {ri.b[0], ri.b[1], ri.b[2]};
-    double xi = ri.x, ti = s.tc[c], D = s.D[c];
-    int32_t nr = s.nrec[c];
-    bool conflict = false;
-    uint32_t partner = NONE;
-    auto meet = [&](uint32_t h) {
-        if (!conflict) {
-            conflict = true;
-            partner = h;
-        }
-    };
-    // the first step of the window claims the active disk too
-    uint32_t old[3] = {0u, 0u, 0u};
-    {
-        const uint32_t oi = atomicCAS(s.claim + i, 0u, mine);
-        if (oi != 0u && oi != mine) meet(oi - 1u);
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (a[q] != NONE) old[q] = atomicCAS(s.claim + a[q], 0u, mine);
-    }
-    int st = ST_RUNNING;
-    bool blocked = false;
-    uint32_t lifts = 0;
-    GDisk r[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-        if (a[q] != NONE) r[q] = s.g[a[q]];
-    for (;;) {
-        // time of flight and (tau, j) minimum over the static targets (see graph_step)
-        unsigned long long bt = INF_BITS;
-        int bq = -1;
-        uint32_t bjid = NONE, ns_owner = NONE;
-        bool hz = false;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (a[q] == NONE) continue;
-            if (r[q].own != OWN_STATIC) {
-                if (ns_owner == NONE && active_in_reach(r[q], b[q], xi, ti, D, s.L))
-                    ns_owner = r[q].own & OWN_CHAIN;
-                continue;
+// The lifting log of the leg (one warp), in the chain's order.
+__device__ __noinline__ void g_log_chain(const GDev &s, int c, int32_t leg, int lane) {
+    const int32_t nl = s.nlift[c];
+    if (nl > 0) {
+        unsigned long long w = 0ull;
+        if (lane == 0) w = atomicAdd(s.tc_cnt + TC_LOG_N, (unsigned long long)nl);
+        w = shfl_u64(w, 0);
+        const int32_t nr = s.nrec[c];
+        for (int32_t e0 = 0; e0 < nr; e0 += 32) {
+            const int32_t e = e0 + lane;
+            const GEv *u = grec_at(s, c, e < nr ? e : 0);
+            const bool is = e < nr && u->j != NONE;
+            const unsigned m = __ballot_sync(FULL, is);
+            const unsigned long long at = w + __popc(m & ((1u << lane) - 1u));
+            if (is && (int64_t)at < s.log_cap) {
+                ecmc_lift_t Lr;
+                Lr.leg = leg;
+                Lr.c = c;
+                Lr.i = (int32_t)u->i;
+                Lr.j = (int32_t)u->j;
+                Lr.t = u->t;
+                Lr.tau = u->tau;
+                Lr.xi = u->xi;
+                Lr.xj = u->xj;
+                s.log[at] = Lr;
             }
-            double dx = __dsub_rn(r[q].x, xi);
-            if (dneg(dx)) dx = __dadd_rn(dx, s.L);
-            double tau = __dsub_rn(dx, b[q]);
-            if (dneg(tau)) tau = 0.0;
-            if (dbits(r[q].t) != 0ull) {
-                const double sum = __dadd_rn(ti, tau);
-                if (dbits(sum) < dbits(r[q].t)) {
-                    if (dbits(r[q].t) >= dbits(tw)) hz = true;
-                    tau = __dadd_rn(tau, s.L);
-                }
-            }
-            const unsigned long long tb = dbits(tau);
-            if (bq < 0 || tb < bt || (tb == bt && a[q] < bjid)) {
-                bt = tb;
-                bq = q;
-                bjid = a[q];
-            }
-        }
-        const int lift = bq >= 0 && bt < dbits(D);
-        GDisk wr;  // the winner's record, by select (no indexed local-memory access)
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (q == bq) wr = r[q];
-        const double tau = lift ? __longlong_as_double((long long)bt) : D;
-        const double T = __dadd_rn(ti, tau);
-        const bool go = dbits(T) < dbits(tend) && ns_owner == NONE;
-        // the next step's claims and records, requested before this step's
-        // claims are resolved
-        uint32_t oldn[3] = {0u, 0u, 0u};
-        GDisk rn[3];
-        if (lift && go) {
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                if (wr.a[q] != NONE) {
-                    oldn[q] = atomicCAS(s.claim + wr.a[q], 0u, mine);
-                    rn[q] = s.g[wr.a[q]];
-                }
-        }
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (old[q] != 0u && old[q] != mine) meet(old[q] - 1u);
-        if (!conflict && ns_owner != NONE) meet(ns_owner);
-        if (conflict) {
-            blocked = true;
-            break;
-        }
-        // Eq. 2 on the disks of this window: cannot fail while
-        // they are held by a lone chain; an assertion
-        if (hz) atomicAdd(s.lc + LC_HORIZON, 1ull);
-        if (!go) break;  // pauses at the window end
-        if (dbits(T) < dbits(tw)) {
-            atomicAdd(s.lc + LC_ORDER, 1ull);
-            gdiag(s, 9, tw, c, i, lift ? bjid : NONE, ti, tau);
-        }
-        if (nr >= s.cap) {
-            atomicAdd(s.lc + LC_ERR_REC, 1ull);
-            blocked = true;
-            partner = NONE;
-            break;
-        }
-        const uint32_t j = lift ? bjid : NONE;
-        graph_apply(s, c, i, xi, ti, D, lift, j, tau, lift ? wr.x : 0.0, lift ? wr.t : 0.0,
-                    (uint32_t)nr, nr);
-        ++nr;
-        if (!lift) {
-            st = ST_STALLED;
-            xi = wrap_add(xi, D, s.L);
-            ti = T;
-            D = 0.0;
-            break;
-        }
-        ++lifts;
-        xi = wr.x;
-        i = j;
-        ti = T;
-        D = __dsub_rn(D, tau);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            a[q] = wr.a[q];
-            b[q] = wr.b[q];
-            old[q] = oldn[q];
-            r[q] = rn[q];
+            w += __popc(m);
         }
     }
-    if (blocked) st = ST_BLOCKED;
-    // events before the blocking time, and all before the window, are exact
-    s.vt[c] = blocked ? fmax(ti, tw) : INFINITY;
-    s.partner[c] = blocked && partner < (uint32_t)s.k ? (int32_t)partner : -1;
-    s.status[c] = st;
-    s.ci[c] = i;
-    s.tc[c] = ti;
-    s.D[c] = D;
-    s.nrec[c] = nr;
-    s.nlift[c] += (int32_t)lifts;
-    if (blocked) {
-        atomicAdd(s.lc + LC_BLOCKED, 1ull);
-        atomicAdd(s.lc + LC_WBLOCKED, 1ull);
-    }
-    if (lifts) atomicAdd(s.lc + LC_P1LIFTS, (unsigned long long)lifts);
 }
 
 // --------------------------------------------------------------- repairs
@@ -771,8 +1182,9 @@ __device__ void g_undo(const GDev &s, int c, const GEv &u) {
     if (u.j != NONE) {
         GDisk &rj = s.g[u.j];
         rj.t = u.tj_old;
-        rj.own = OWN_STATIC;
+        rj.own = s.stamp;
         s.nlift[c] -= 1;
+        atomicAdd(s.lc + LC_LIFTS, ~0ull);
     }
 }
 
@@ -780,7 +1192,7 @@ __device__ void g_undo(const GDev &s, int c, const GEv &u) {
 // exact): records with event time >= T* are undone, latest first. Records of
 // repair rounds (seq >= REPAIR_SEQ0) may touch one disk from several members
 // and are undone one at a time in descending seq; beneath them, the records
-// of the window's parallel pass touch disks claimed by their own chain only,
+// of the window's parallel pass touch disks held by their own chain only,
 // so each member undoes its own in parallel.
 __device__ void g_rollback(const GDev &s, const int32_t *mem, int m, double Ts) {
     const int lane = threadIdx.x & 31;
@@ -855,12 +1267,12 @@ __device__ void g_resume(const GDev &s, int c) {
 }
 
 // Pending event of member c (one thread), kept with the arrows it read.
-__device__ __noinline__ void g_compute(const GDev &s, int c, int root, uint64_t tag, bool &abort,
-                                       int &met) {
+__device__ __noinline__ void g_compute(const GDev &s, int c, int root, uint64_t tag,
+                                       uint32_t epoch, bool &abort, int &met) {
     const uint32_t i = s.ci[c];
     const GDisk ri = s.g[i];
     const double ti = s.tc[c], D = s.D[c];
-    const GStep o = graph_step(s, c, root, tag, ri.a, ri.b, i, ri.x, ti, D, true);
+    const GStep o = graph_step(s, c, root, tag, epoch, ri.a, ri.b, i, ri.x, ti, D);
     if (o.conflict && !abort) {
         abort = true;
         met = (int)o.partner;
@@ -895,7 +1307,7 @@ __device__ void g_rollback_chain(const GDev &s, int c, double Ts) {
 // infinity, so that a later merge rolls them back to `now` or earlier (their
 // events were applied chain by chain, not in time order).
 __device__ void g_finish(const GDev &s, const int32_t *mem, int m, int root, bool abort,
-                         int met, double now, int round, bool keep_vt = false) {
+                         int met, double now, bool keep_vt = false) {
     const int lane = threadIdx.x & 31;
     if (abort) {
         // events before `now` are exact; the chain met joins next round
@@ -905,7 +1317,7 @@ __device__ void g_finish(const GDev &s, const int32_t *mem, int m, int root, boo
                 s.abort_to[root] = met;
                 atomic_min_time(s.vt + met, now);
             }
-            atomicAdd(s.nabort + (round & 1), 1);
+            atomicAdd(s.ctl + CTL_NABORT, 1);
         }
     } else {
         for (int e = lane; e < m; e += 32) {
@@ -917,211 +1329,303 @@ __device__ void g_finish(const GDev &s, const int32_t *mem, int m, int root, boo
 }
 
 // First repair round of a window: the blocked members continue from where
-// they stopped, one after another (lane 0), over the state the others left.
-// The parallel pass was a run of Alg. 4 in which every chain read only disks
-// it held, every step satisfied the horizon condition and no step was taken
-// towards another chain's active disk. If every continued step satisfies
-// Eq. 2 on each arrow target as well, the whole is a run of Alg. 4 without a
-// horizon violation, which by Lemma 2 ends where Alg. 2 ends: nothing has to
-// be redone. A chain that finds the active disk of another blocked member
-// among its arrow targets waits (Remark 10) while that member continues
-// first. Otherwise the caller rolls the component back to T* and replays it
-// in global order.
+// they stopped, one after another (one warp), over the state the others left.
+// What the pass published is a run of Alg. 4 (g_resolve_chain). If every
+// continued step satisfies Eq. 2 on each arrow target as well, the whole is a
+// run of Alg. 4 without a horizon violation, which by Lemma 2 ends where
+// Alg. 2 ends: nothing has to be redone. A chain that finds the active disk of
+// another blocked member among its arrow targets waits (Remark 10) while that
+// member continues first. Otherwise the caller rolls the component back to T*
+// and replays it in global order. The lanes share a step as in g_spec_chain;
+// a step's claims are asked about one step later, when their round trip is
+// over, and an event is written only once they stand.
 enum { CONT_DONE = 0, CONT_FAIL = 1, CONT_FOREIGN = 2 };
 
 __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m, int root,
-                                       uint64_t tag, int round, double tw, double tend,
-                                       int *met) {
+                                       uint64_t tag, uint32_t epoch, int round, double tw,
+                                       double tend, int *met) {
     const int lane = threadIdx.x & 31;
-    int how = CONT_DONE, who = -1;
-    if (lane == 0) {
-        uint32_t cnt = 0;
-        int switches = 0;
-        int e = 0;
-        int cur = -1;
-        int known = -1;  // a holder already found on this side
-        while (how == CONT_DONE) {
-            if (cur < 0) {  // the next member still blocked
-                while (e < m && s.status[mem[e]] != ST_BLOCKED) ++e;
-                if (e >= m) break;
-                cur = mem[e];
+    const int l3 = lane % 3;
+    const double L = s.L;
+    GLevels &lv = g_levels();
+    GDisk *const g = s.g;
+    const uint32_t stamp = s.stamp;
+    const bool bounded = dbits(tend) != INF_BITS || dbits(tw) != 0ull;
+    const int n_lap = g_lap(s), cap = s.cap;
+    uint32_t cnt = 0;
+    int switches = 0, e = 0, cur = -1;
+    int known = -1;  // a holder already found on this side
+    for (;;) {
+        if (cur < 0) {  // the next member still blocked
+            while (e < m) {
+                const unsigned bm =
+                    __ballot_sync(FULL, e + lane < m && s.status[mem[e + lane]] == ST_BLOCKED);
+                if (bm) {
+                    e += __ffs(bm) - 1;
+                    break;
+                }
+                e += 32;
             }
-            const int c = cur;
-            const uint32_t mine = (uint32_t)c + 1u;
-            uint32_t i = s.ci[c];
-            const GDisk ri = s.g[i];
-            uint32_t a[3] = {ri.a[0], ri.a[1], ri.a[2]};
-            double b[3] = {ri.b[0], ri.b[1], ri.b[2]};
-            double xi = ri.x, ti = s.tc[c], D = s.D[c];
-            int32_t nr = s.nrec[c], nl = 0;
-            int st = ST_RUNNING, next = -1;
-            // claims of the active disk (first step) and of the arrow targets
-            uint32_t oi = atomicCAS(s.claim + i, 0u, mine);
-            uint32_t old[3] = {0u, 0u, 0u};
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                if (a[q] != NONE) old[q] = atomicCAS(s.claim + a[q], 0u, mine);
-            auto ours = [&](uint32_t w) {
-                if (w == 0u || w == mine) return true;
-                const int h = (int)w - 1;
-                if (h == known) return true;
-                if (!holder_ours(s, h, root, tag, true)) {
-                    who = h;
-                    return false;
-                }
-                known = h;
-                return true;
-            };
-            for (;;) {
-                GDisk r[3];
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (a[q] != NONE) r[q] = s.g[a[q]];
-                unsigned long long bt = INF_BITS;
-                int bq = -1;
-                uint32_t bjid = NONE, ns_owner = NONE;
-                bool viol = false;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (a[q] == NONE) continue;
-                    if (r[q].own != OWN_STATIC) {
-                        if (ns_owner == NONE && active_in_reach(r[q], b[q], xi, ti, D, s.L))
-                            ns_owner = r[q].own & OWN_CHAIN;
-                        continue;
-                    }
-                    double dx = __dsub_rn(r[q].x, xi);
-                    if (dneg(dx)) dx = __dadd_rn(dx, s.L);
-                    double tau = __dsub_rn(dx, b[q]);
-                    if (dneg(tau)) tau = 0.0;
-                    // Eq. 2, strict (a lap-away target fails it too)
-                    if (dbits(r[q].t) != 0ull && !(dbits(__dadd_rn(ti, tau)) > dbits(r[q].t)))
-                        viol = true;
-                    const unsigned long long tb = dbits(tau);
-                    if (bq < 0 || tb < bt || (tb == bt && a[q] < bjid)) {
-                        bt = tb;
-                        bq = q;
-                        bjid = a[q];
-                    }
-                }
-                const int lift = bq >= 0 && bt < dbits(D);
-                GDisk wr;
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (q == bq) wr = r[q];
-                const double tau = lift ? __longlong_as_double((long long)bt) : D;
-                const double T = __dadd_rn(ti, tau);
-                const bool go = dbits(T) < dbits(tend) && !viol && ns_owner == NONE;
-                uint32_t oldn[3] = {0u, 0u, 0u};
-                if (lift && go) {
-#pragma unroll
-                    for (int q = 0; q < 3; ++q)
-                        if (wr.a[q] != NONE) {
-                            oldn[q] = atomicCAS(s.claim + wr.a[q], 0u, mine);
-                            prefetch_l1(s.g + wr.a[q]);
-                        }
-                }
-                bool foreign = !ours(oi);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) foreign = foreign || !ours(old[q]);
-                oi = 0u;
-                if (foreign) {
-                    how = CONT_FOREIGN;
-                    break;
-                }
-                if (viol) {
-                    how = CONT_FAIL;
-                    break;
-                }
-                if (ns_owner != NONE) {
-                    const int h = (int)ns_owner;
-                    if (h != c && h >= 0 && h < s.k &&
-                        __ldcg((const unsigned long long *)s.memb + h) == tag &&
-                        s.status[h] == ST_BLOCKED && switches < 4 * m + 4) {
-                        next = h;  // wait for that member (Remark 10)
-                        st = ST_BLOCKED;
-                        ++switches;
-                    } else {
-                        how = CONT_FAIL;
-                    }
-                    break;
-                }
-                if (!(dbits(T) < dbits(tend))) break;  // pauses at the window end
-                if (dbits(T) < dbits(tw) || nr >= s.cap) {
-                    how = CONT_FAIL;
-                    break;
-                }
-                const uint32_t j = lift ? bjid : NONE;
-                graph_apply(s, c, i, xi, ti, D, lift, j, tau, lift ? wr.x : 0.0,
-                            lift ? wr.t : 0.0, ((uint32_t)round << 24) | cnt++, nr);
-                ++nr;
-                if (!lift) {
-                    st = ST_STALLED;
-                    ti = T;
-                    D = 0.0;
-                    break;
-                }
-                ++nl;
-                i = j;
-                xi = wr.x;
-                ti = T;
-                D = __dsub_rn(D, tau);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    a[q] = wr.a[q];
-                    b[q] = wr.b[q];
-                    old[q] = oldn[q];
-                }
-            }
-            // the events so far stand (a failure rolls them back with the rest)
-            s.nrec[c] = nr;
-            s.nlift[c] += nl;
-            if (how != CONT_DONE) break;
-            s.status[c] = st;
-            s.ci[c] = i;
-            s.tc[c] = ti;
-            s.D[c] = D;
-            cur = next;
+            if (e >= m) return CONT_DONE;
+            cur = mem[e];
         }
+        const int c = cur;
+        const uint32_t mine = (uint32_t)c + 1u;
+        const unsigned long long ct = ((unsigned long long)epoch << 32) | mine;
+        uint32_t i = s.ci[c];
+        double ti = s.tc[c], D = s.D[c];
+        const int32_t nr0 = s.nrec[c];
+        const uint32_t seq0 = ((uint32_t)round << 24) | cnt;
+        double xi = g[i].x;
+        int cb = 0, sl = 0;  // the active disk's targets: lv.r[cb][sl .. sl + 2]
+        g_fetch_first(g, i, lv.r[0]);
+        uint32_t tid = g[i].a[l3];
+        double tb = g[i].b[l3];
+        unsigned none = g_none(tid);
+        // the holder of a disk this lane claimed, asked one step later: what the
+        // exchange found (0: free, mine), or the record's own word of this pass
+        unsigned long long cas = 0ull;
+        uint32_t held = 0u;
+        if (lane == 31) held = g_claim(s, i, ct);
+        // false: a disk read in the step before is held by the other side
+        auto claims_stand = [&]() -> bool {
+            const uint32_t h = held ? held : g_holder(cas, ct);
+            const bool ask = h != 0u && h != mine && (int)h - 1 != known;
+            if (!__any_sync(FULL, ask)) return true;
+            const bool ours = !ask || holder_ours(s, (int)h - 1, root, tag, true);
+            const unsigned fb = __ballot_sync(FULL, !ours);
+            if (fb) {
+                *met = (int)__shfl_sync(FULL, h, __ffs(fb) - 1) - 1;
+                return false;
+            }
+            const unsigned ab = __ballot_sync(FULL, ask);
+            known = (int)__shfl_sync(FULL, h, __ffs(ab) - 1) - 1;
+            return true;
+        };
+        g_copy_wait();
+        GEvs E;
+        E.i = NONE;
+        E.x = E.t = E.D = E.tau = E.tj = 0.0;
+        int n = 0, nf = 0, nl = 0, st = ST_RUNNING, next = -1, how = CONT_DONE;
+        // events nf .. n - 1 to memory: records and the moved disks
+        auto flush = [&](bool lift) {
+            if (n == nf) return;
+            const GFlush f = g_flush(s, c, nr0, seq0, nf, n, E, i, xi, ti, D, lift);
+            if (f.has) {
+                *reinterpret_cast<ulonglong2 *>(&g[E.i].x) =
+                    make_ulonglong2(dbits(f.xn), dbits(f.t));
+                g[E.i].own = f.j != NONE ? stamp : (OWN_STALLED | (uint32_t)c);
+            }
+            nf = n;
+        };
+        // back to the state before event n - 1
+        auto drop = [&]() {
+            --n;
+            const int le = n & 31;
+            i = __shfl_sync(FULL, E.i, le);
+            xi = shfl_f64(E.x, le);
+            ti = shfl_f64(E.t, le);
+            D = shfl_f64(E.D, le);
+        };
+        for (;;) {
+            const GDisk *const R = &lv.r[cb][sl];
+            g_fetch(g, R, none, lv.r[cb ^ 1]);
+            const bool ev = lane < 3 && tid != NONE;
+            const double rx = R[l3].x, rt = R[l3].t;
+            const uint32_t own = R[l3].own;
+            const unsigned long long cw = R[l3].claim;
+            double dx = __dsub_rn(rx, xi);
+            double tau = __dsub_rn(dx, tb);
+            // the claims of the step before: if one failed, its event is none
+            // (not written yet) and the component has met another chain
+            if (!claims_stand()) {
+                how = CONT_FOREIGN;
+                if (n > nf) {
+                    drop();
+                    --nl;
+                }
+                break;
+            }
+            // this step's claims: a record whose word is of this pass names its
+            // holder, any other disk is taken
+            held = ev ? g_holder(cw, ct) : 0u;
+            cas = 0ull;
+            if (ev && held == 0u) cas = atomicCAS(&g[tid].claim, cw, ct);
+            // Eq. 2, strict (a lap-away target fails it too), for every target
+            // with a time of this leg; another chain's disk stops the step in
+            // reach or where it fails Eq. 2
+            double sum = __dadd_rn(ti, __double_as_longlong(tau) < 0 ? 0.0 : tau);
+            const bool nsc = ev && own >= OWN_ACTIVE;
+            const bool neg = ev && __double_as_longlong(dx) < 0;
+            bool bad = ev && own == stamp && dbits(rt) != 0ull && !(dbits(sum) > dbits(rt));
+            bool viol = false;
+            uint32_t ns_owner = NONE;
+            const bool any_odd = __any_sync(FULL, nsc || neg || bad);
+            if (any_odd) {
+                if (neg) {
+                    tau = g_sub(g_add(dx, L), tb);
+                    sum = g_add(ti, __double_as_longlong(tau) < 0 ? 0.0 : tau);
+                }
+                bad = ev && (nsc || (own == stamp && dbits(rt) != 0ull)) &&
+                      !(dbits(sum) > dbits(rt));
+                viol = __any_sync(FULL, bad && !nsc);
+                const double tc0 = __double_as_longlong(tau) < 0 ? 0.0 : tau;
+                const unsigned sb = __ballot_sync(FULL, nsc && (bad || dbits(tc0) < dbits(D)));
+                if (sb) ns_owner = __shfl_sync(FULL, own, __ffs(sb) - 1) & OWN_CHAIN;
+            }
+            if (__double_as_longlong(tau) < 0) tau = 0.0;
+            const unsigned long long tk = ev && !nsc ? dbits(tau) : INF_BITS;
+            const int wl = g_winner(tk, tid);
+            const unsigned long long bt = shfl_u64(tk, wl);
+            const bool lift = bt < dbits(D);
+            const double ts = lift ? __longlong_as_double((long long)bt) : D;
+            const double T = lift ? shfl_f64(sum, wl) : g_add(ti, D);
+            const uint32_t bj = __shfl_sync(FULL, tid, wl);
+            const double xj = shfl_f64(rx, wl);
+            const double tj = shfl_f64(own == stamp ? rt : 0.0, wl);
+            if (viol) {
+                how = CONT_FAIL;
+                break;
+            }
+            if (ns_owner != NONE) {
+                const int h = (int)ns_owner;
+                if (h != c && h < s.k && __ldcg((const unsigned long long *)s.memb + h) == tag &&
+                    s.status[h] == ST_BLOCKED && switches < 4 * m + 4) {
+                    next = h;  // wait for that member (Remark 10)
+                    st = ST_BLOCKED;
+                    ++switches;
+                } else {
+                    how = CONT_FAIL;
+                }
+                break;
+            }
+            if (bounded) {
+                if (!(dbits(T) < dbits(tend))) break;  // pauses at the window end
+                if (dbits(T) < dbits(tw)) {
+                    how = CONT_FAIL;
+                    break;
+                }
+            }
+            if (nr0 + n >= cap) {
+                how = CONT_FAIL;
+                break;
+            }
+            if (lane == (n & 31)) {
+                E.i = i;
+                E.x = xi;
+                E.t = ti;
+                E.D = D;
+                E.tau = ts;
+                E.tj = lift ? tj : 0.0;
+            }
+            ++n;
+            ti = T;
+            if (!lift) {
+                st = ST_STALLED;
+                D = 0.0;
+                break;
+            }
+            ++nl;
+            D = __dsub_rn(D, ts);
+            xi = xj;
+            i = bj;
+            tid = R[wl].a[l3];
+            tb = R[wl].b[l3];
+            none = g_none(tid);
+            g_copy_wait();
+            cb ^= 1;
+            sl = 3 * wl;
+            if (n - nf == 32 || n > n_lap) {
+                if (!claims_stand()) {
+                    how = CONT_FOREIGN;
+                    drop();
+                    --nl;
+                    break;
+                }
+                flush(true);
+                if (n > n_lap) {
+                    // the run may come round to a disk it moved: the level
+                    // requested before that write is read again
+                    __threadfence();
+                    __syncwarp();
+                    if (lane < 12) {
+                        const uint32_t id = __shfl_sync(0xFFFu, tid, lane >> 2);
+                        g_fetch_part(g, id, &lv.r[cb][sl + (lane >> 2)], lane & 3);
+                    }
+                    g_copy_wait();
+                }
+            }
+        }
+        g_copy_wait();
+        // the last step's claims: a stall is its event; a pause, a failed Eq. 2
+        // or a wait was decided on what it read
+        if (how != CONT_FOREIGN && !claims_stand()) {
+            how = CONT_FOREIGN;
+            if (st == ST_STALLED) {
+                drop();
+                st = ST_RUNNING;
+            }
+        }
+        flush(st != ST_STALLED);
+        __syncwarp();
+        // the events so far stand (a failure rolls them back with the rest)
+        if (lane == 0) {
+            if (nl > 0 && st != ST_STALLED) {
+                g[i].own = OWN_ACTIVE | (uint32_t)c;
+                g[i].t = ti;
+            }
+            s.nrec[c] = nr0 + n;
+            s.nlift[c] += nl;
+            if (nl) atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
+            if (how == CONT_DONE) {
+                s.status[c] = st;
+                s.ci[c] = i;
+                s.tc[c] = ti;
+                s.D[c] = D;
+            }
+        }
+        __syncwarp();
+        cnt += (uint32_t)n;
+        if (how != CONT_DONE) return how;
+        cur = next;
     }
-    how = __shfl_sync(FULL, how, 0);
-    *met = __shfl_sync(FULL, who, 0);
-    __syncwarp();
-    return how;
 }
 
 // Component q of this round (one warp): roll its members back to T*, then
 // replay them in global event-time order (Alg. 2) up to the window's end.
 // Members are spread over the lanes (member e on lane e mod 32); after each
 // event only the members whose arrows read a disk it changed recompute.
-__device__ __noinline__ void g_repair_component(const GDev &s, int q, int round, uint32_t wr_tag,
-                                                double tw,
-                                   double tend) {
+__device__ __noinline__ void g_repair_component(const GDev &s, int q, int round, uint32_t epoch,
+                                                uint32_t wr_tag, double tw, double tend) {
     const int lane = threadIdx.x & 31;
     const int root = s.comp_root[q];
     const int off = s.comp_off[q], m = s.comp_off[q + 1] - off;
     const int32_t *mem = s.comp_mem + off;
     double Ts = INFINITY;
-    for (int e = lane; e < m; e += 32) Ts = fmin(Ts, s.vt[mem[e]]);
+    // the members listed for this round of this pass (wr_tag names both)
+    const uint64_t tag = ((uint64_t)wr_tag << 32) | (uint32_t)root;
+    for (int e = lane; e < m; e += 32) {
+        const int c = mem[e];
+        Ts = fmin(Ts, s.vt[c]);
+        s.memb[c] = tag;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) Ts = fmin(Ts, __shfl_xor_sync(FULL, Ts, o));
     Ts = fmax(Ts, tw);  // earlier windows are final
     if (lane == 0) atomicAdd(s.lc + LC_REPAIRED, (unsigned long long)m);
-    // the members listed for this round of this window (wr_tag names both)
-    const uint64_t tag = ((uint64_t)wr_tag << 32) | (uint32_t)root;
-    for (int e = lane; e < m; e += 32) s.memb[mem[e]] = tag;
     __syncwarp();
     if (round == 1) {
         int met = -1;
-        const int how = g_continue(s, mem, m, root, tag, round, tw, tend, &met);
+        const int how = g_continue(s, mem, m, root, tag, epoch, round, tw, tend, &met);
         if (how == CONT_DONE) {
             if (lane == 0) atomicAdd(s.lc + LC_CONTINUED, (unsigned long long)m);
-            g_finish(s, mem, m, root, false, -1, Ts, round, true);
+            g_finish(s, mem, m, root, false, -1, Ts, true);
             return;
         }
         if (how == CONT_FOREIGN) {
             // the merged component's replay rolls back to T* (all of this
             // round's events lie after it)
-            g_finish(s, mem, m, root, true, met, Ts, round);
+            g_finish(s, mem, m, root, true, met, Ts);
             return;
         }
     }
@@ -1131,7 +1635,7 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int q, int round,
     bool abort = false;
     int met = -1;
     for (int e = lane; e < m; e += 32)
-        if (s.status[mem[e]] == ST_RUNNING) g_compute(s, mem[e], root, tag, abort, met);
+        if (s.status[mem[e]] == ST_RUNNING) g_compute(s, mem[e], root, tag, epoch, abort, met);
     double now = Ts;
     uint32_t cnt = 0;
     for (;;) {
@@ -1193,7 +1697,10 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int q, int round,
                 graph_apply(s, bc, i, xi, ti, D, o.lift, o.j, o.tau, o.xj, o.tj,
                             ((uint32_t)round << 24) | cnt, nr);
                 s.nrec[bc] = nr + 1;
-                if (o.lift) s.nlift[bc] += 1;
+                if (o.lift) {
+                    s.nlift[bc] += 1;
+                    atomicAdd(s.lc + LC_LIFTS, 1ull);
+                }
                 st = o.lift ? ST_RUNNING : ST_STALLED;
             }
             ib = i;
@@ -1227,38 +1734,11 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int q, int round,
                 const uint32_t v = s.ev_a[3 * (size_t)c + k2];
                 redo |= v != NONE && (v == ib || v == jb);
             }
-            if (redo) g_compute(s, c, root, tag, abort, met);
+            if (redo) g_compute(s, c, root, tag, epoch, abort, met);
         }
         __syncwarp();
     }
-    g_finish(s, mem, m, root, abort, met, now, round);
-}
-
-// Leg end: totals, and the lifting log (chain by chain).
-__device__ void g_leg_end_chain(const GDev &s, int c, int32_t leg) {
-    const int32_t nl = s.nlift[c];
-    atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
-    if (s.log_on && nl > 0) {
-        const unsigned long long base = atomicAdd(s.tc_cnt + TC_LOG_N, (unsigned long long)nl);
-        unsigned long long w = base;
-        for (int32_t e = 0; e < s.nrec[c]; ++e) {
-            const GEv *q = grec_at(s, c, e);
-            if (q->j == NONE) continue;
-            if ((int64_t)w < s.log_cap) {
-                ecmc_lift_t L;
-                L.leg = leg;
-                L.c = c;
-                L.i = (int32_t)q->i;
-                L.j = (int32_t)q->j;
-                L.t = q->t;
-                L.tau = q->tau;
-                L.xi = q->xi;
-                L.xj = q->xj;
-                s.log[w] = L;
-            }
-            ++w;
-        }
-    }
+    g_finish(s, mem, m, root, abort, met, now);
 }
 
 // ------------------------------------------- persistent multi-leg kernel
@@ -1267,25 +1747,29 @@ struct GCtl {
     int64_t budget;  // liftings for this run (0: none)
     int64_t lifts, legs, conflict_legs, repaired, continued, horizon, order_err, p1_lifts,
         repair_lifts, restarts, blocked, cwindows;
+    int64_t leg0;    // legs run before this launch (lifting log)
     uint8_t *flags;  // per-leg conflict flags (device) or null
     int32_t flags_cap;
     int32_t done;    // budget reached or error
     int32_t err;     // LC_ERR_* seen, or too many repair rounds
-    int32_t pad;
-    int64_t leg0;    // batches: legs run before this launch (lifting log)
+    int32_t dbg;     // an internal check recorded in GDev::dbg (set at the end)
 };
 
+enum { GG_WORK = 0, GG_ANY, GG_ERR, GG_REMAIN0, GG_REMAIN1, GG_COUNT, GG_PASSES, GG_N };
 enum { GPH_BEGIN = 0, GPH_PASS1, GPH_REPAIR, GPH_END, GPH_N };
 
-struct GRun {
-    GDev s;
-    GCtl *ctl;
-    unsigned int *bar;               // [2] grid barrier
-    int32_t *err;                    // ECMC_ETIMEOUT from a barrier
-    unsigned long long *phase_ns;    // [GPH_N] device time per phase (block 0 clock)
-    int32_t max_legs;
-    int64_t leg0;                    // legs run before this launch (lifting log)
-    int64_t budget;                  // liftings of this launch after which it stops (0: none)
+// One launch: R systems (their descriptions in device memory), their chains
+// and conflict components flattened by prefix offsets.
+struct GBatchDev {
+    const GDev *reps;              // [R]
+    GCtl *ctl;                     // [R]
+    const int32_t *chain_base;     // [R + 1]
+    int32_t *comp_base;            // [R + 1]
+    unsigned int *bar;             // [1] grid barrier
+    int32_t *g;                    // [GG_N]
+    unsigned long long *phase_ns;  // [GPH_N] device time per phase (block 0 clock)
+    int32_t R, max_legs, windows, pad;
+    unsigned long long wait_ns;    // bound on every grid-barrier wait
 };
 
 __device__ __forceinline__ double g_window_start(const GDev &s, int w) {
@@ -1297,78 +1781,278 @@ __device__ __forceinline__ double g_window_end(const GDev &s, int w) {
                               : __ddiv_rn(__dmul_rn((double)(w + 1), s.ell), (double)s.windows);
 }
 
+// system of flattened item f, with base[r] <= f < base[r + 1]
+__device__ __forceinline__ int g_find_rep(const int32_t *base, int R, int f) {
+    int lo = 0, hi = R;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (base[mid] <= f)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ bool g_rep_on(const GBatchDev &B, int r) { return !B.ctl[r].done; }
+
+// A system with no liftings budget runs every leg of the launch: its next leg
+// is begun by its chains at this leg's end. With a budget, the leg's totals
+// decide first.
+__device__ __forceinline__ bool g_next_at_end(const GBatchDev &B, int r, int leg) {
+    return B.ctl[r].budget == 0 && leg + 1 < B.max_legs;
+}
+
+// The system's description in the warp's slot of shared memory (constant
+// during a launch; a field of the global copy would be re-read from L2 after
+// every store).
+__device__ __forceinline__ const GDev &g_warp_dev(GDev *slot, int *rep, const GDev *reps, int r) {
+    if (*(volatile int *)rep != r) {
+        constexpr int WORDS = (int)(sizeof(GDev) / sizeof(uint32_t));
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(reps + r);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(slot);
+        for (int q = threadIdx.x & 31; q < WORDS; q += 32) dst[q] = src[q];
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) *(volatile int *)rep = r;
+        __syncwarp();
+    }
+    return *slot;
+}
+
+// The leg's stamp in the warp's copy of the description.
+__device__ __forceinline__ void g_set_stamp(GDev *slot, int leg, int lane) {
+    if (lane == 0) slot->stamp = slot->stamp0 + (uint32_t)leg + 1u;
+    __syncwarp();
+}
+
 constexpr int GRUN_THREADS = 256;
-constexpr int GRUN_MIN_BLOCKS = 1;
+constexpr int GRUN_MIN_BLOCKS = 2;
 constexpr int MAX_RESTARTS = 16;  // per leg, then the local repair takes over
 
-// One cooperative launch runs up to max_legs legs. Per leg and claim window:
-// the parallel pass (one thread per chain), then repair rounds (conflict
-// components by one block, their replays by one warp each) until no component
-// met another chain. Phases are separated by grid barriers whose waits are
-// bounded (ECMC_ETIMEOUT).
-__global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GRun R) {
+// One cooperative launch runs up to max_legs legs of every system. Per leg
+// and claim window: the parallel pass (one warp per chain), the resolve, then
+// repair rounds (conflict components by one block per system, their repairs
+// by one warp each from one queue) until no component met another chain; the
+// leg end with each system's totals. Phases are separated by grid barriers
+// whose waits are bounded (ECMC_ETIMEOUT). Restart mode takes one system.
+__global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBatchDev B) {
     extern __shared__ int32_t uf_sm[];  // UF_SMEM_BYTES: the union-find working set
     __shared__ int warp_tot[32];
     __shared__ int tot[2];
     __shared__ int sflag;
-    const GDev &s = R.s;
+    __shared__ double dmin[GRUN_THREADS / 32];
+    __shared__ GDev wdev[GRUN_THREADS / 32];
+    __shared__ int wrep[GRUN_THREADS / 32];
+    if ((threadIdx.x & 31) == 0) wrep[threadIdx.x >> 5] = -1;
+    __syncthreads();
+    GDev *const my_dev = wdev + (threadIdx.x >> 5);
+    int *const my_rep = wrep + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nthreads = gridDim.x * blockDim.x;
-    const int nwarps = nthreads >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    // warps interleaved over the blocks: chains spread over all SMs
     const int gw = blockIdx.x + gridDim.x * (threadIdx.x >> 5);
+    const int R = B.R;
+    const int total_chains = B.chain_base[R];
+    const bool restart = R == 1 && B.reps[0].restart;
+    // one system without claim windows or restarts: a leg has three phases and
+    // three barriers. Its chains begin the next leg at its pass (the stamps
+    // make clearing local times unnecessary, s.lc alternates by leg), the
+    // touch keys go during the repair, and the totals of a leg are taken by
+    // one warp while the next one resolves. Otherwise (several systems, whose
+    // budgets decide which go on) a leg end of its own follows the repair.
+    const bool fast = R == 1 && !B.reps[0].strict;
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long t_prev = timer ? gtimer() : 0ull;
     auto mark = [&](int ph) {
         if (timer) {
             const unsigned long long t = gtimer();
-            R.phase_ns[ph] += t - t_prev;
+            B.phase_ns[ph] += t - t_prev;
             t_prev = t;
         }
     };
-    // The per-leg counters accumulate over the launch: a leg's totals are
-    // differences, and every thread decides alike, after the leg's last
-    // barrier, whether the launch goes on. Without an event budget the next
-    // leg is begun in the same phase as this one ends.
-    unsigned long long prev[LC_N];
-#pragma unroll
-    for (int q = 0; q < LC_N; ++q) prev[q] = 0ull;
-    auto begin_leg = [&]() {
-        for (int c = gt; c < s.k; c += nthreads) g_leg_begin_chain(s, c);
-        for (int64_t q = gt; q < s.n; q += nthreads) s.claim[q] = 0u;
+    auto barrier = [&]() -> bool { return grid_sync(B.bar, B.g + GG_ERR, &sflag, B.wait_ns); };
+    // true in the last block to get here, of all blocks (each comes once per
+    // use; the block barrier, then the master thread's fences, release before
+    // the count and acquire after it, as in the grid barrier)
+    auto last_block = [&]() -> bool {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const int old = atomicAdd(B.g + GG_COUNT, 1);
+            sflag = (old + 1) % (int)gridDim.x == 0;
+            if (sflag) __threadfence();
+        }
+        __syncthreads();
+        const bool last = sflag != 0;
+        __syncthreads();
+        return last;
     };
-    begin_leg();
-    if (gt < LC_N) s.lc[gt] = 0ull;
-    if (gt == 0) s.nabort[0] = s.nabort[1] = 0;
-    if (!grid_sync(R.bar, R.err, &sflag)) return;
-    mark(GPH_BEGIN);
-    __shared__ double dmin[32];
-    for (int leg = 0; leg < R.max_legs; ++leg) {
+    // conflict components of system r (one block)
+    auto uf_system = [&](int r, int round) {
+        if (threadIdx.x < 32) (void)g_warp_dev(wdev, wrep, B.reps, r);
+        __syncthreads();
+        const GDev &s = wdev[0];
+        bool need = false;
+        unsigned long long wbl = 0ull;
+        if (g_rep_on(B, r)) {
+            wbl = __ldcg(s.lc + LC_WBLOCKED);
+            need = round == 1 ? wbl != 0ull : __ldcg(s.ctl + CTL_NABORT) != 0;
+            // the window's flag: the reads of two chains met
+            if (!fast && round == 1 && threadIdx.x == 0 && __ldcg(s.lc + LC_WWEAK) != 0ull)
+                atomicAdd(s.lc + LC_CWINDOWS, 1ull);
+        }
+        if (need && round <= 255) {
+            uf_block(s, round == 1, warp_tot, tot, false, uf_sm, s.blist, s.pcnt,
+                     round == 1 ? (int)min(wbl, (unsigned long long)s.k) : -1);
+        } else if (threadIdx.x == 0) {
+            s.ctl[CTL_NCOMP] = 0;
+            if (need) atomicAdd(s.lc + LC_ERR_CAP, 1ull);  // too many rounds
+        }
+        __syncthreads();
+    };
+    // prefix of component counts over systems (one block)
+    auto comp_prefix = [&]() {
+        const int chunk = (R + blockDim.x - 1) / blockDim.x;
+        const int lo = min(R, (int)threadIdx.x * chunk), hi = min(R, lo + chunk);
+        int sum = 0;
+        for (int r = lo; r < hi; ++r) sum += __ldcg(B.reps[r].ctl + CTL_NCOMP);
+        int off = block_exscan(sum, warp_tot, tot);
+        for (int r = lo; r < hi; ++r) {
+            B.comp_base[r] = off;
+            off += __ldcg(B.reps[r].ctl + CTL_NCOMP);
+            // every block read the abort counts before it counted itself
+            B.reps[r].ctl[CTL_NABORT] = 0;
+        }
+        if (threadIdx.x == 0) {
+            B.comp_base[R] = tot[0];
+            B.g[GG_WORK] = 0;
+            B.g[GG_ANY] = tot[0];
+        }
+    };
+    unsigned long long *const lc0 = B.reps[0].lc;
+    // the totals of leg `leg` of system r from its counters, which go back to
+    // zero (one thread)
+    auto totals = [&](int r, unsigned long long *lcp) -> bool {
+        GCtl *const cp = B.ctl + r;
+        GCtl c = *cp;
+        if (c.done) return true;
+        unsigned long long lc[LC_N];
+#pragma unroll
+        for (int q = 0; q < LC_N; ++q) lc[q] = __ldcg(lcp + q);
+        const int64_t lifts = (int64_t)(lc[LC_P1LIFTS] + lc[LC_LIFTS]);
+        const int flag = lc[LC_WEAK] != 0ull;
+        if (c.flags && c.legs < c.flags_cap) c.flags[c.legs] = (uint8_t)flag;
+        c.lifts += lifts;
+        c.p1_lifts += (int64_t)lc[LC_P1LIFTS];
+        if (flag) c.repair_lifts += lifts;
+        c.legs += 1;
+        c.conflict_legs += flag;
+        c.repaired += (int64_t)lc[LC_REPAIRED];
+        c.continued += (int64_t)lc[LC_CONTINUED];
+        c.restarts += (int64_t)lc[LC_RESTARTS];
+        c.blocked += (int64_t)lc[LC_BLOCKED];
+        c.cwindows += fast ? flag : (int64_t)lc[LC_CWINDOWS];
+        c.horizon += (int64_t)lc[LC_HORIZON];
+        c.order_err += (int64_t)lc[LC_ORDER];
+        if (lc[LC_ERR_REC] != 0ull || lc[LC_ERR_CAP] != 0ull) c.err = 1;
+        if (c.err || (c.budget > 0 && c.lifts >= c.budget)) c.done = 1;
+        *cp = c;
+#pragma unroll
+        for (int q = 0; q < LC_N; ++q) lcp[q] = 0ull;
+        return c.done != 0;
+    };
+    uint32_t pass = 0;  // passes of the launch (the same count in every thread)
+    int leg = 0;
+    for (; leg < B.max_legs; ++leg) {
+        if (fast) {
+            GDev &s = *my_dev;
+            (void)g_warp_dev(my_dev, my_rep, B.reps, 0);
+            if (lane == 0) {
+                s.lc = lc0 + (leg & 1) * LC_N;
+                s.stamp = s.stamp0 + (uint32_t)leg + 1u;
+            }
+            __syncwarp();
+        }
+        // leg start of the systems whose last leg did not begin this one
+        bool begin_here = false;
+        for (int r = 0; r < R && !fast; ++r)
+            if (g_rep_on(B, r) && !(leg > 0 && g_next_at_end(B, r, leg - 1))) begin_here = true;
+        if (begin_here) {
+            for (int f = gw; f < total_chains; f += nwarps) {
+                const int r = g_find_rep(B.chain_base, R, f);
+                if (!g_rep_on(B, r) || (leg > 0 && g_next_at_end(B, r, leg - 1))) continue;
+                const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+                const int c = f - B.chain_base[r];
+                g_begin_state(s, c, s.ci[c], lane);
+            }
+            if (!barrier()) return;
+        }
+        mark(GPH_BEGIN);
         // restart mode (one claim window): a pass that meets a conflict is cut
         // at T*, the earliest time a chain stopped -- every event before it is
         // exact (Remark 6) -- all chains are rolled back to T*, and T* becomes
-        // the next breakpoint of the leg: a new pass from T* with new claims
-        // (Sec. 3.4, second restart strategy). A pass that cannot progress
-        // (T* at its own start), or the last one allowed, is repaired locally.
+        // the next breakpoint of the leg: a new pass from T* (Sec. 3.4, second
+        // restart strategy). A pass that cannot progress (T* at its own
+        // start), or the last one allowed, is repaired locally.
         double tw_r = 0.0;
         int sub = 0;
-        for (int w = 0; w < s.windows; ++w) {
-          for (;;) {
+        for (int w = 0; w < B.windows; ++w) {
             if (w > 0) {
-                // a new claim window: the claims of the last one are void
-                for (int64_t q = gt; q < s.n; q += nthreads) s.claim[q] = 0u;
-                if (!grid_sync(R.bar, R.err, &sflag)) return;
+                // a new claim window: the touch keys of the last one go
+                for (int f = gw; f < total_chains; f += nwarps) {
+                    const int r = g_find_rep(B.chain_base, R, f);
+                    if (!g_rep_on(B, r)) continue;
+                    g_reset_keys(g_warp_dev(my_dev, my_rep, B.reps, r), f - B.chain_base[r], lane);
+                }
+                for (int r = gt; r < R; r += (int)(gridDim.x * blockDim.x)) {
+                    if (!g_rep_on(B, r)) continue;
+                    B.reps[r].lc[LC_WBLOCKED] = 0ull;
+                    B.reps[r].lc[LC_WWEAK] = 0ull;
+                }
+                if (!barrier()) return;
             }
-            const double tw = s.restart ? tw_r : g_window_start(s, w);
-            const double te = g_window_end(s, w);
-            // one chain per warp (lane 0) while they last, warps interleaved over
-            // the blocks so that the chains spread over all SMs
-            for (int c = gw + nwarps * lane; c < s.k; c += nwarps * 32)
-                g_pass1_chain(s, c, tw, te);
-            if (!grid_sync(R.bar, R.err, &sflag)) return;
-            mark(GPH_PASS1);
-            if (s.restart) {
-                if (*(volatile unsigned long long *)(s.lc + LC_WBLOCKED) == 0ull) break;
+            bool uf_early = false;
+            for (;;) {
+                ++pass;
+                for (int f = gw; f < total_chains; f += nwarps) {
+                    const int r = g_find_rep(B.chain_base, R, f);
+                    if (!g_rep_on(B, r)) continue;
+                    const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+                    if (!fast) g_set_stamp(my_dev, leg, lane);
+                    g_spec_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
+                                 g_window_end(s, w), fast);
+                }
+                if (!barrier()) return;
+                if (gt == 0 && w == 0 && sub == 0) B.g[GG_REMAIN0 + ((leg + 1) & 1)] = 0;
+                // (the leg's own counters are the other half of s.lc)
+                if (fast && leg > 0 && gw == nwarps - 1 && lane == 0)
+                    (void)totals(0, lc0 + ((leg - 1) & 1) * LC_N);
+                for (int f = gw; f < total_chains; f += nwarps) {
+                    const int r = g_find_rep(B.chain_base, R, f);
+                    if (!g_rep_on(B, r)) continue;
+                    const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+                    if (!fast) g_set_stamp(my_dev, leg, lane);
+                    g_resolve_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
+                                    s.epoch0 + pass);
+                    if (!fast && sub == 0)
+                        g_flag_chain(s, f - B.chain_base[r], s.epoch0 + pass, lane);
+                }
+                if (R == 1 && !restart) {
+                    // one system: the last block to finish resolving takes the
+                    // first round's union-find and prefix (no barrier between)
+                    if (last_block()) {
+                        uf_system(0, 1);
+                        comp_prefix();
+                    }
+                    uf_early = true;
+                }
+                if (!barrier()) return;
+                mark(GPH_PASS1);
+                if (!restart) break;
+                const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, 0);
+                g_set_stamp(my_dev, leg, lane);
+                if (__ldcg(s.lc + LC_WBLOCKED) == 0ull) break;
                 if (blockIdx.x == 0) {  // T*: the earliest stop of this pass
                     double m = INFINITY;
                     for (int c = threadIdx.x; c < s.k; c += blockDim.x)
@@ -1379,346 +2063,114 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GRu
                     __syncthreads();
                     if (threadIdx.x == 0) {
                         for (int q = 1; q < (int)(blockDim.x >> 5); ++q) m = fmin(m, dmin[q]);
-                        s.tstar[0] = fmax(m, tw);
+                        s.tstar[0] = fmax(m, tw_r);
                     }
                     __syncthreads();
                 }
-                if (!grid_sync(R.bar, R.err, &sflag)) return;
-                const double Ts = *(volatile double *)s.tstar;
-                if (!(dbits(Ts) > dbits(tw)) || sub >= MAX_RESTARTS) {
-                    // no progress: the local repair below
-                } else {
-                    // every thread has read the blocked count: reset for the next pass
-                    if (gt == 0) {
-                        s.lc[LC_WBLOCKED] = 0ull;
-                        s.lc[LC_RESTARTS] += 1ull;
-                        if (sub == 0) s.lc[LC_CWINDOWS] += 1ull;  // the window's flag
-                    }
-                    for (int c = gt; c < s.k; c += nthreads) g_rollback_chain(s, c, Ts);
-                    for (int64_t q = gt; q < s.n; q += nthreads) s.claim[q] = 0u;
-                    if (!grid_sync(R.bar, R.err, &sflag)) return;
-                    tw_r = Ts;
-                    ++sub;
-                    continue;
+                if (!barrier()) return;
+                const double Ts = __ldcg(s.tstar);
+                if (!(dbits(Ts) > dbits(tw_r)) || sub >= MAX_RESTARTS) break;  // local repair
+                // every thread has read the blocked count: reset for the next
+                // pass, with the partner counts of the chains listed
+                const int nbl = (int)min(__ldcg(s.lc + LC_WBLOCKED), (unsigned long long)s.k);
+                for (int f = gw; f < total_chains; f += nwarps) g_reset_keys(s, f, lane);
+                for (int z = gt; z < nbl; z += (int)(gridDim.x * blockDim.x)) {
+                    const int pt = s.partner[s.blist[z]];
+                    if (pt >= 0 && pt < s.k) s.pcnt[pt] = 0;
                 }
+                if (!barrier()) return;
+                if (gt == 0) {
+                    s.lc[LC_WBLOCKED] = 0ull;
+                    s.lc[LC_RESTARTS] += 1ull;
+                }
+                for (int c = gt; c < s.k; c += (int)(gridDim.x * blockDim.x))
+                    g_rollback_chain(s, c, Ts);
+                if (!barrier()) return;
+                tw_r = Ts;
+                ++sub;
             }
-            if (gt == 0) s.nabort[1] = 0;  // the first round's abort count
+            // repair rounds
             for (int round = 1;; ++round) {
-                if (blockIdx.x == 0) {
-                    const bool need = round == 1 ? s.lc[LC_WBLOCKED] != 0ull
-                                                 : s.nabort[(round - 1) & 1] != 0;
-                    __syncthreads();
-                    if (round == 1 && threadIdx.x == 0) {
-                        s.lc[LC_WBLOCKED] = 0ull;
-                        if (need && sub == 0) s.lc[LC_CWINDOWS] += 1ull;
-                    }
-                    if (need && round <= 255) {
-                        uf_block(s, round == 1, warp_tot, tot, false, uf_sm);
-                    } else if (threadIdx.x == 0) {
-                        s.ctl[CTL_NCOMP] = 0;
-                        if (need) atomicAdd(s.lc + LC_ERR_CAP, 1ull);  // too many rounds
-                    }
-                    __syncthreads();
+                if (!(round == 1 && uf_early)) {
+                    for (int r = blockIdx.x; r < R; r += gridDim.x) uf_system(r, round);
+                    // the last block to finish its union-finds takes the prefix
+                    if (last_block()) comp_prefix();
+                    if (!barrier()) return;
                 }
-                if (!grid_sync(R.bar, R.err, &sflag)) return;
-                // every block has read the previous round's abort count
-                if (gt == 0) s.nabort[(round + 1) & 1] = 0;
-                const int ncomp = s.ctl[CTL_NCOMP];
+                const int ncomp = __ldcg(B.g + GG_ANY);
+                if (fast && round == 1)
+                    for (int f = gw; f < total_chains; f += nwarps) {
+                        g_flag_chain(*my_dev, f, my_dev->epoch0 + pass, lane);
+                        g_reset_keys(*my_dev, f, lane);
+                    }
                 if (ncomp == 0) break;
                 for (;;) {
                     int q = 0;
-                    if (lane == 0) q = atomicAdd(s.ctl + CTL_WORK, 1);
-                    q = __shfl_sync(FULL, q, 0);
-                    if (q >= ncomp) break;
-                    g_repair_component(s, q, round,
-                                       ((uint32_t)(leg * s.windows + w) << 8) | (uint32_t)round,
-                                       tw, te);
-                }
-                if (!grid_sync(R.bar, R.err, &sflag)) return;
-                // no component met another chain: the window is repaired
-                if (*(volatile int32_t *)(s.nabort + (round & 1)) == 0) break;
-            }
-            mark(GPH_REPAIR);
-            break;
-          }
-        }
-        // leg end: liftings and the log (and, without a budget, the next leg's
-        // start), then the totals. Every counter but the liftings is final
-        // since the last barrier (the next leg's pass may start as soon as the
-        // coming barrier is passed), so thread 0 takes them now.
-        const volatile unsigned long long *lcv = s.lc;
-        // errors of this leg are final too: all threads read them here, so
-        // that they all take the same decision below
-        const bool err = lcv[LC_ERR_REC] != 0ull || lcv[LC_ERR_CAP] != 0ull;
-        unsigned long long d[LC_N];
-        if (gt == 0) {
-#pragma unroll
-            for (int q = 0; q < LC_N; ++q) {
-                if (q == LC_LIFTS) continue;
-                const unsigned long long v = lcv[q];
-                d[q] = v - prev[q];
-                prev[q] = v;
-            }
-        }
-        const bool more = leg + 1 < R.max_legs && R.budget == 0;
-        for (int c = gt; c < s.k; c += nthreads) {
-            g_leg_end_chain(s, c, (int32_t)(R.leg0 + leg));
-            if (more) g_leg_begin_chain(s, c);
-        }
-        if (more)
-            for (int64_t q = gt; q < s.n; q += nthreads) s.claim[q] = 0u;
-        if (!grid_sync(R.bar, R.err, &sflag)) return;
-        // (read by all threads; with a budget no next leg has begun)
-        const unsigned long long lifts_all = lcv[LC_LIFTS];
-        if (gt == 0) {
-            GCtl &c = *R.ctl;
-            d[LC_LIFTS] = lifts_all - prev[LC_LIFTS];
-            prev[LC_LIFTS] = lifts_all;
-            const int flag = d[LC_BLOCKED] != 0ull;
-            if (c.flags && c.legs < c.flags_cap) c.flags[c.legs] = (uint8_t)flag;
-            c.lifts += (int64_t)d[LC_LIFTS];
-            c.p1_lifts += (int64_t)d[LC_P1LIFTS];
-            if (flag) c.repair_lifts += (int64_t)d[LC_LIFTS];
-            c.legs += 1;
-            c.conflict_legs += flag;
-            c.repaired += (int64_t)d[LC_REPAIRED];
-            c.continued += (int64_t)d[LC_CONTINUED];
-            c.restarts += (int64_t)d[LC_RESTARTS];
-            c.blocked += (int64_t)d[LC_BLOCKED];
-            c.cwindows += (int64_t)d[LC_CWINDOWS];
-            c.horizon += (int64_t)d[LC_HORIZON];
-            c.order_err += (int64_t)d[LC_ORDER];
-            if (err) c.err = 1;
-        }
-        mark(GPH_END);
-        if (err || (R.budget > 0 && (int64_t)lifts_all >= R.budget)) break;
-        if (leg + 1 >= R.max_legs) break;
-        if (!more) {
-            begin_leg();
-            if (!grid_sync(R.bar, R.err, &sflag)) return;
-            mark(GPH_BEGIN);
-        }
-    }
-}
-
-// ------------------------------------- batches of constraint-graph systems
-
-// Launch state of a batch: R systems (descriptors in device memory), their
-// chains and conflict components flattened by prefix offsets.
-struct GBatchDev {
-    const GDev *S;          // [R]
-    GCtl *ctl;              // [R]
-    const int32_t *chain_base;  // [R + 1]
-    int32_t *comp_base;     // [R + 1]
-    int32_t *g;             // [GB_N]
-    unsigned int *bar;      // [1] grid barrier
-    int32_t *err;           // ECMC_ETIMEOUT from a barrier
-    unsigned long long *phase_ns;  // [GPH_N]
-    int32_t R, max_legs, windows;
-    int32_t pad;
-};
-
-enum { GB_WORK = 0, GB_ANY, GB_DONE, GB_REMAIN0, GB_REMAIN1, GB_N };
-
-// replica of flattened item f, with base[r] <= f < base[r + 1]
-__device__ __forceinline__ int g_find_rep(const int32_t *base, int R, int f) {
-    int lo = 0, hi = R - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (base[mid] <= f) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ bool g_rep_on(const GBatchDev &B, int r) {
-    return !B.ctl[r].done;
-}
-
-// k_run_graph over R systems (the local repair; no restart mode): every
-// system's legs exactly as k_run_graph computes them. Per leg and claim
-// window: the parallel pass over all systems' chains (one thread per chain),
-// the union-find of each system's conflict components (one block per
-// system), their repairs from one work queue (one warp per component), the
-// leg end and each system's totals; the launch ends when every system has
-// reached max_legs or its liftings budget.
-__global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph_batch(GBatchDev B) {
-    extern __shared__ int32_t uf_sm[];
-    __shared__ int warp_tot[32];
-    __shared__ int tot[2];
-    __shared__ int sflag;
-    const int lane = threadIdx.x & 31;
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nthreads = gridDim.x * blockDim.x;
-    const int nwarps = nthreads >> 5;
-    const int gw = blockIdx.x + gridDim.x * (threadIdx.x >> 5);
-    const int R = B.R;
-    const int total_chains = B.chain_base[R];
-    const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
-    unsigned long long t_prev = timer ? gtimer() : 0ull;
-    auto mark = [&](int ph) {
-        if (timer) {
-            const unsigned long long t = gtimer();
-            B.phase_ns[ph] += t - t_prev;
-            t_prev = t;
-        }
-    };
-    // true in the last block to get here, of all blocks (each comes once per use)
-    auto last_block = [&]() -> bool {
-        // (as in the grid barrier: the block barrier, then the master
-        // thread's fences, release before the count and acquire after it)
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const int old = atomicAdd(B.g + GB_DONE, 1);
-            sflag = (old + 1) % (int)gridDim.x == 0;
-            if (sflag) __threadfence();
-        }
-        __syncthreads();
-        const bool last = sflag != 0;
-        __syncthreads();
-        return last;
-    };
-    for (int leg = 0; leg < B.max_legs; ++leg) {
-        // leg start of every running system: chains, claims, per-leg counters
-        for (int f = gt; f < total_chains; f += nthreads) {
-            const int r = g_find_rep(B.chain_base, R, f);
-            if (g_rep_on(B, r)) g_leg_begin_chain(B.S[r], f - B.chain_base[r]);
-        }
-        for (int r = 0; r < R; ++r) {
-            if (!g_rep_on(B, r)) continue;
-            const GDev &s = B.S[r];
-            for (int64_t q = gt; q < s.n; q += nthreads) s.claim[q] = 0u;
-            if (gt < LC_N) s.lc[gt] = 0ull;
-            if (gt == 0) s.nabort[0] = s.nabort[1] = 0;
-        }
-        if (!grid_sync(B.bar, B.err, &sflag)) return;
-        if (gt == 0) B.g[GB_REMAIN0 + ((leg + 1) & 1)] = 0;
-        mark(GPH_BEGIN);
-        for (int w = 0; w < B.windows; ++w) {
-            if (w > 0) {
-                for (int r = 0; r < R; ++r) {
-                    if (!g_rep_on(B, r)) continue;
-                    const GDev &s = B.S[r];
-                    for (int64_t q = gt; q < s.n; q += nthreads) s.claim[q] = 0u;
-                }
-                if (!grid_sync(B.bar, B.err, &sflag)) return;
-            }
-            // one chain per thread, warps interleaved over the blocks
-            for (int f = gw + nwarps * lane; f < total_chains; f += nwarps * 32) {
-                const int r = g_find_rep(B.chain_base, R, f);
-                if (!g_rep_on(B, r)) continue;
-                const GDev &s = B.S[r];
-                g_pass1_chain(s, f - B.chain_base[r], g_window_start(s, w), g_window_end(s, w));
-            }
-            if (!grid_sync(B.bar, B.err, &sflag)) return;
-            mark(GPH_PASS1);
-            for (int r = gt; r < R; r += nthreads)
-                if (g_rep_on(B, r)) B.S[r].nabort[1] = 0;  // the first round's abort count
-            for (int round = 1;; ++round) {
-                for (int r = blockIdx.x; r < R; r += gridDim.x) {
-                    const GDev &s = B.S[r];
-                    bool need = false;
-                    if (g_rep_on(B, r))
-                        need = round == 1 ? s.lc[LC_WBLOCKED] != 0ull
-                                          : s.nabort[(round - 1) & 1] != 0;
-                    __syncthreads();
-                    if (round == 1 && threadIdx.x == 0 && g_rep_on(B, r)) {
-                        s.lc[LC_WBLOCKED] = 0ull;
-                        if (need) s.lc[LC_CWINDOWS] += 1ull;
-                    }
-                    if (need && round <= 255) {
-                        uf_block(s, round == 1, warp_tot, tot, false, uf_sm);
-                    } else if (threadIdx.x == 0) {
-                        s.ctl[CTL_NCOMP] = 0;
-                        if (need) atomicAdd(s.lc + LC_ERR_CAP, 1ull);  // too many rounds
-                    }
-                    __syncthreads();
-                }
-                if (last_block()) {
-                    // prefix of component counts over systems
-                    const int chunk = (R + blockDim.x - 1) / blockDim.x;
-                    const int lo = min(R, (int)threadIdx.x * chunk), hi = min(R, lo + chunk);
-                    int sum = 0;
-                    for (int r = lo; r < hi; ++r) sum += B.S[r].ctl[CTL_NCOMP];
-                    int off = block_exscan(sum, warp_tot, tot);
-                    for (int r = lo; r < hi; ++r) {
-                        B.comp_base[r] = off;
-                        off += B.S[r].ctl[CTL_NCOMP];
-                    }
-                    if (threadIdx.x == 0) {
-                        B.comp_base[R] = tot[0];
-                        B.g[GB_WORK] = 0;
-                        B.g[GB_ANY] = tot[0];
-                    }
-                }
-                if (!grid_sync(B.bar, B.err, &sflag)) return;
-                // every block has read the previous round's abort counts
-                for (int r = gt; r < R; r += nthreads)
-                    if (g_rep_on(B, r)) B.S[r].nabort[(round + 1) & 1] = 0;
-                const int ncomp = B.g[GB_ANY];
-                if (ncomp == 0) break;
-                for (;;) {
-                    int q = 0;
-                    if (lane == 0) q = atomicAdd(B.g + GB_WORK, 1);
+                    if (lane == 0) q = atomicAdd(B.g + GG_WORK, 1);
                     q = __shfl_sync(FULL, q, 0);
                     if (q >= ncomp) break;
                     const int r = g_find_rep(B.comp_base, R, q);
-                    const GDev &s = B.S[r];
-                    g_repair_component(s, q - B.comp_base[r], round,
+                    const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+                    if (!fast) g_set_stamp(my_dev, leg, lane);
+                    g_repair_component(s, q - B.comp_base[r], round, s.epoch0 + pass,
                                        ((uint32_t)(leg * B.windows + w) << 8) | (uint32_t)round,
-                                       g_window_start(s, w), g_window_end(s, w));
+                                       restart ? tw_r : g_window_start(s, w), g_window_end(s, w));
                 }
-                if (!grid_sync(B.bar, B.err, &sflag)) return;
+                if (!barrier()) return;
                 // no component met another chain: the window is repaired
                 int aborted = 0;
                 for (int r = threadIdx.x; r < R; r += blockDim.x)
-                    if (g_rep_on(B, r) &&
-                        *(volatile int32_t *)(B.S[r].nabort + (round & 1)) != 0)
-                        aborted = 1;
+                    if (g_rep_on(B, r) && __ldcg(B.reps[r].ctl + CTL_NABORT) != 0) aborted = 1;
                 if (!__syncthreads_or(aborted)) break;
             }
             mark(GPH_REPAIR);
         }
-        // leg end: liftings and the log; the last block takes each system's
-        // totals and budget
-        for (int f = gt; f < total_chains; f += nthreads) {
+        if (fast) {
+            // a leg without components has passed no barrier since its keys went
+            if (__ldcg(B.g + GG_ANY) == 0 && !barrier()) return;
+            const GDev &s = *my_dev;
+            if (s.log_on)
+                for (int f = gw; f < total_chains; f += nwarps)
+                    g_log_chain(s, f, (int32_t)(B.ctl[0].leg0 + leg), lane);
+            mark(GPH_END);
+            // every thread decides alike: the leg's counters are final since
+            // the barrier, the totals before it since the leg's first one
+            const GCtl *const cp = B.ctl;
+            const int64_t lifts = (int64_t)__ldcg((const unsigned long long *)&cp->lifts) +
+                                  (int64_t)(__ldcg(s.lc + LC_P1LIFTS) + __ldcg(s.lc + LC_LIFTS));
+            const bool err = __ldcg(s.lc + LC_ERR_REC) != 0ull || __ldcg(s.lc + LC_ERR_CAP) != 0ull;
+            if (err || (cp->budget > 0 && lifts >= cp->budget)) break;
+            continue;
+        }
+        // leg end: the log and the touch keys of the last window; the last
+        // block takes each system's totals
+        for (int f = gw; f < total_chains; f += nwarps) {
             const int r = g_find_rep(B.chain_base, R, f);
-            if (g_rep_on(B, r))
-                g_leg_end_chain(B.S[r], f - B.chain_base[r],
-                                (int32_t)(B.ctl[r].leg0 + B.ctl[r].legs));
+            if (!g_rep_on(B, r)) continue;
+            const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+            const int c = f - B.chain_base[r];
+            g_reset_keys(s, c, lane);
+            if (s.log_on) g_log_chain(s, c, (int32_t)(B.ctl[r].leg0 + B.ctl[r].legs), lane);
+            if (g_next_at_end(B, r, leg)) g_begin_state(s, c, s.ci[c], lane);
         }
-        if (last_block()) {
-            for (int r = threadIdx.x; r < R; r += blockDim.x) {
-                GCtl *const cp = B.ctl + r;
-                GCtl c = *cp;
-                if (c.done) continue;
-                const unsigned long long *lcp = B.S[r].lc;
-                unsigned long long lc[LC_N];
-#pragma unroll
-                for (int q = 0; q < LC_N; ++q) lc[q] = __ldcg(lcp + q);
-                const int flag = lc[LC_BLOCKED] != 0ull;
-                if (c.flags && c.legs < c.flags_cap) c.flags[c.legs] = (uint8_t)flag;
-                c.lifts += (int64_t)lc[LC_LIFTS];
-                c.p1_lifts += (int64_t)lc[LC_P1LIFTS];
-                if (flag) c.repair_lifts += (int64_t)lc[LC_LIFTS];
-                c.legs += 1;
-                c.conflict_legs += flag;
-                c.repaired += (int64_t)lc[LC_REPAIRED];
-                c.continued += (int64_t)lc[LC_CONTINUED];
-                c.blocked += (int64_t)lc[LC_BLOCKED];
-                c.cwindows += (int64_t)lc[LC_CWINDOWS];
-                c.horizon += (int64_t)lc[LC_HORIZON];
-                c.order_err += (int64_t)lc[LC_ORDER];
-                if (lc[LC_ERR_REC] != 0ull || lc[LC_ERR_CAP] != 0ull) c.err = 1;
-                if (c.err || (c.budget > 0 && c.lifts >= c.budget)) c.done = 1;
-                *cp = c;
-                if (!c.done) atomicAdd(B.g + GB_REMAIN0 + (leg & 1), 1);
-            }
-        }
-        if (!grid_sync(B.bar, B.err, &sflag)) return;
+        if (last_block())
+            for (int r = threadIdx.x; r < R; r += blockDim.x)
+                if (!B.ctl[r].done && !totals(r, B.reps[r].lc))
+                    atomicAdd(B.g + GG_REMAIN0 + (leg & 1), 1);
+        if (!barrier()) return;
         mark(GPH_END);
-        if (B.g[GB_REMAIN0 + (leg & 1)] == 0) break;
+        if (__ldcg(B.g + GG_REMAIN0 + (leg & 1)) == 0) break;
     }
+    // (the last block out: every other thread has decided on these counters)
+    if (fast && last_block() && threadIdx.x == 0) {
+        const int last = leg < B.max_legs ? leg : B.max_legs - 1;
+        (void)totals(0, lc0 + (last & 1) * LC_N);
+    }
+    if (gt == 0) B.g[GG_PASSES] = (int32_t)pass;
+    // the systems whose internal checks recorded a failure (GDev::dbg[0])
+    if (blockIdx.x == 0)
+        for (int r = threadIdx.x; r < R; r += blockDim.x)
+            if (B.reps[r].dbg && __ldcg(B.reps[r].dbg) != 0.0) B.ctl[r].dbg = 1;
 }
 
 // Exports positions (per disk id), local times and active disks.
@@ -1726,7 +2178,7 @@ __global__ void k_g_export(GDev s, double *x, double *t) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= s.n) return;
     if (x) x[q] = s.g[q].x;
-    if (t) t[q] = s.g[q].t;
+    if (t) t[q] = g_time(s.g[q].own, s.g[q].t, s.stamp0);
 }
 
 __global__ void k_g_export_active(GDev s, int32_t *active) {
@@ -1761,15 +2213,10 @@ struct GraphCtx {
     double box = 0.0;
     cudaStream_t st = nullptr;
     std::vector<void *> allocs;
-    GCtl *d_ctl = nullptr;
-    unsigned int *d_bar = nullptr;
-    int32_t *d_err = nullptr;
-    unsigned long long *d_phase = nullptr;
     uint8_t *d_flags = nullptr;
     int32_t flags_cap = 0;
     int64_t log_legs = 0;  // legs logged so far (leg index of the log)
-    int grid = 0;
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    GBatchScratch *launch = nullptr;  // launch tables of graph_run
     void *build_tmp[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     std::vector<std::pair<void **, size_t>> pending;
     int64_t bytes = 0;  // device memory held
@@ -1918,6 +2365,10 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
     };
     chk(galloc(g, &s.g, n, err));
     chk(galloc(g, &s.y, n, err));
+    chk(galloc(g, &s.key, n, err));
+    chk(galloc(g, &s.fl, n, err));
+    chk(galloc(g, &s.path, k * ((size_t)s.cap + 2), err));
+    chk(galloc(g, &s.sp, k, err));
     chk(galloc(g, &s.ci, k, err));
     chk(galloc(g, &s.ci0, k, err));
     chk(galloc(g, &s.D, k, err));
@@ -1926,7 +2377,6 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
     chk(galloc(g, &s.partner, k, err));
     chk(galloc(g, &s.nrec, k, err));
     chk(galloc(g, &s.nlift, k, err));
-    chk(galloc(g, &s.claim, n, err));
     chk(galloc(g, &s.memb, k, err));
     chk(galloc(g, &s.tstar, 1, err));
     s.restart = (p->flags & ECMC_RESTART) ? 1 : 0;
@@ -1947,19 +2397,41 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
     chk(galloc(g, &s.comp_off, k + 1, err));
     chk(galloc(g, &s.comp_root, k, err));
     chk(galloc(g, &s.comp_mem, k, err));
+    chk(galloc(g, &s.blist, k, err));
+    chk(galloc(g, &s.pcnt, k, err));
     chk(galloc(g, &s.ctl, CTL_N, err));
-    chk(galloc(g, &s.nabort, 2, err));
-    chk(galloc(g, &s.lc, LC_N, err));
+    chk(galloc(g, &s.lc, 2 * LC_N, err));
     chk(galloc(g, &s.tc_cnt, TC_N, err));
     chk(galloc(g, &s.dbg, 16, err));
     if (s.log_on) chk(galloc(g, &s.log, (size_t)s.log_cap, err));
-    chk(galloc(g, &g->d_ctl, 1, err));
-    chk(galloc(g, &g->d_bar, 2, err));
-    chk(galloc(g, &g->d_err, 1, err));
-    chk(galloc(g, &g->d_phase, GPH_N, err));
     return rc;
 }
 
+// Blocks of the persistent launch that fit on the current device at once (0:
+// no cooperative launch there): queried once per device.
+static int graph_max_grid() {
+    static std::mutex mu;
+    static int cached[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && cached[dev] > 0) return cached[dev];
+    int n_sm = 1, blocks = 0, coop = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_run_graph, GRUN_THREADS,
+                                                      UF_SMEM_BYTES) != cudaSuccess ||
+        !coop || blocks < 1) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    const int grid = n_sm * std::min(blocks, GRUN_MIN_BLOCKS);
+    if (dev >= 0 && dev < 64) cached[dev] = grid;
+    return grid;
+}
 
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
                  const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err) {
@@ -1986,6 +2458,7 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     s.L = p->box;
     s.d = p->d;
     s.ell = p->ell;
+    s.strict = (s.windows > 1 || (p->flags & ECMC_RESTART)) ? 1 : 0;
     s.log_on = (p->flags & ECMC_LOG_LIFTINGS) ? 1 : 0;
     s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
     const size_t n = (size_t)p->n, k = (size_t)p->n_chains;
@@ -1995,18 +2468,16 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     };
     chk(graph_plan(g, p, err));
     chk(gcommit(g, err));
-    if (!rc && (cudaEventCreate(&g->ev0) != cudaSuccess || cudaEventCreate(&g->ev1) != cudaSuccess)) {
-        err = "event creation";
-        rc = ECMC_ECUDA;
-    }
     if (rc) {
         graph_destroy(g);
         return rc;
     }
     cudaMemcpyAsync(s.y, y, n * 8, cudaMemcpyDeviceToDevice, st);
     cudaMemsetAsync(s.nrec, 0, k * 4, st);
+    cudaMemsetAsync(s.sp, 0, k * sizeof(GSpec), st);
+    cudaMemsetAsync(s.pcnt, 0, k * 4, st);
     cudaMemsetAsync(s.memb, 0xFF, k * 8, st);
-    cudaMemsetAsync(s.lc, 0, LC_N * 8, st);
+    cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
     cudaMemsetAsync(s.tc_cnt, 0, TC_N * 8, st);
     cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
     rc = graph_build(g, x, s.y, err);
@@ -2016,162 +2487,94 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     }
     k_g_init<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s);
     k_g_init_chains<<<(unsigned)((k + 127) / 128), 128, 0, st>>>(s, active);
-    int dev = 0, n_sm = 1, blocks = 0, coop = 0;
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_run_graph, GRUN_THREADS,
-                                                          UF_SMEM_BYTES);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess || !coop || blocks < 1) {
+    if (e != cudaSuccess || graph_max_grid() < 1) {
         (void)cudaGetLastError();
         err = e != cudaSuccess ? std::string("graph create: ") + cudaGetErrorString(e)
                                : std::string("cooperative launch unavailable");
         graph_destroy(g);
         return ECMC_ECUDA;
     }
-    g->grid = n_sm * std::min(blocks, GRUN_MIN_BLOCKS);
     *out = g;
     return 0;
 }
 
-int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
-              int32_t *legs_done, GraphTotals *tot, std::string &err) {
-    memset(tot, 0, sizeof *tot);
-    if (legs_done) *legs_done = 0;
-    if (n_legs <= 0) return 0;
-    if ((int64_t)n_legs * g->s.windows >= ((int64_t)1 << 24)) {
-        err = "too many legs x windows for one call (< 2^24)";
-        return ECMC_EINVAL;
-    }
-    cudaStream_t st = g->st;
-    if (g->flags_cap < n_legs) {
-        dm_free(g->d_flags);
-        g->d_flags = nullptr;
-        g->flags_cap = 0;
-        if (dm_alloc_t(&g->d_flags, (size_t)n_legs) != 0) {
-            err = "flags allocation";
-            return ECMC_ENOMEM;
-        }
-        g->flags_cap = n_legs;
-    }
-    GCtl ctl;
-    memset(&ctl, 0, sizeof ctl);
-    ctl.budget = (int64_t)budget;
-    ctl.flags = g->d_flags;
-    ctl.flags_cap = g->flags_cap;
-    int rc = 0;
-    auto cu = [&](cudaError_t e, const char *what) {
-        if (e != cudaSuccess && !rc) {
-            (void)cudaGetLastError();
-            err = std::string(what) + ": " + cudaGetErrorString(e);
-            rc = ECMC_ECUDA;
-        }
-    };
-    cu(cudaMemcpyAsync(g->d_ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice, st), "ctl");
-    cu(cudaMemsetAsync(g->d_bar, 0, 2 * sizeof(unsigned int), st), "bar");
-    cu(cudaMemsetAsync(g->d_err, 0, sizeof(int32_t), st), "err");
-    cu(cudaMemsetAsync(g->d_phase, 0, GPH_N * sizeof(unsigned long long), st), "phase");
-    // member tags restart with the launch's window count
-    cu(cudaMemsetAsync(g->s.memb, 0xFF, (size_t)g->s.k * 8, st), "memb");
-    if (rc) return rc;
-    GRun R;
-    R.s = g->s;
-    R.ctl = g->d_ctl;
-    R.bar = g->d_bar;
-    R.err = g->d_err;
-    R.phase_ns = g->d_phase;
-    R.max_legs = n_legs;
-    R.leg0 = g->log_legs;
-    R.budget = (int64_t)budget;
-    void *args[] = {&R};
-    cu(cudaEventRecord(g->ev0, st), "event");
-    cu(cudaLaunchCooperativeKernel((void *)k_run_graph, g->grid, GRUN_THREADS, args, UF_SMEM_BYTES,
-                                   st),
-       "launch");
-    cu(cudaEventRecord(g->ev1, st), "event");
-    int32_t gerr = 0;
-    unsigned long long ph[GPH_N];
-    cu(cudaMemcpyAsync(&ctl, g->d_ctl, sizeof ctl, cudaMemcpyDeviceToHost, st), "ctl");
-    cu(cudaMemcpyAsync(&gerr, g->d_err, sizeof gerr, cudaMemcpyDeviceToHost, st), "err");
-    cu(cudaMemcpyAsync(ph, g->d_phase, sizeof ph, cudaMemcpyDeviceToHost, st), "phase");
-    cu(cudaStreamSynchronize(st), "run");
-    if (rc) return rc;
-    float ms = 0.f;
-    cu(cudaEventElapsedTime(&ms, g->ev0, g->ev1), "elapsed");
-    g->log_legs += ctl.legs;
-    tot->legs = ctl.legs;
-    tot->lifts = ctl.lifts;
-    tot->conflict_legs = ctl.conflict_legs;
-    tot->repaired = ctl.repaired;
-    tot->continued = ctl.continued;
-    tot->restarts = ctl.restarts;
-    tot->horizon = ctl.horizon;
-    tot->order_err = ctl.order_err;
-    tot->p1_lifts = ctl.p1_lifts;
-    tot->repair_lifts = ctl.repair_lifts;
-    tot->blocked = ctl.blocked;
-    tot->cwindows = ctl.cwindows;
-    tot->ms = ms;
-    tot->pass1_ms = ph[GPH_PASS1] * 1e-6;
-    tot->repair_ms = ph[GPH_REPAIR] * 1e-6;
-    tot->other_ms = (ph[GPH_BEGIN] + ph[GPH_END]) * 1e-6;
-    if (legs_done) *legs_done = (int32_t)ctl.legs;
-    if (flags_host && ctl.legs > 0) {
-        cu(cudaMemcpy(flags_host, g->d_flags, (size_t)ctl.legs, cudaMemcpyDeviceToHost), "flags");
-        if (rc) return rc;
-    }
-    if (gerr == ECMC_ETIMEOUT) {
-        err = "a grid barrier wait passed its time limit";
-        return ECMC_ETIMEOUT;
-    }
-    if (ctl.err) {
-        err = "undo records or repair rounds overflowed";
-        return ECMC_ECAPACITY;
-    }
-    double dg[7];
-    if (cudaMemcpy(dg, g->s.dbg, sizeof dg, cudaMemcpyDeviceToHost) == cudaSuccess &&
-        dg[0] != 0.0) {
-        char buf[240];
-        snprintf(buf, sizeof buf, "internal check %g failed: %.17g %.17g %.17g %.17g %.17g %.17g",
-                 dg[0], dg[1], dg[2], dg[3], dg[4], dg[5], dg[6]);
-        err = buf;
-        return ECMC_ECUDA;
-    }
-    return 0;
-}
-
+// Launch tables of the persistent kernel: one device block [reps | chain_base
+// | comp_base | ctl | bar | g | phase] (256-byte aligned parts), uploaded
+// whole before a launch and read back from ctl on after it.
 struct GBatchScratch {
     int cap = 0;
-    GDev *d_S = nullptr;
-    GCtl *d_ctl = nullptr;
-    int32_t *d_chain_base = nullptr, *d_comp_base = nullptr, *d_g = nullptr, *d_err = nullptr;
-    unsigned int *d_bar = nullptr;
-    unsigned long long *d_phase = nullptr;
-    int grid = 0;
+    unsigned char *block = nullptr;
+    size_t off_base = 0, off_comp = 0, off_ctl = 0, off_bar = 0, off_g = 0, off_phase = 0,
+           total = 0;
+    std::vector<unsigned char> host;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 };
 
 void graph_batch_free(GBatchScratch *b) {
     if (!b) return;
-    dm_free(b->d_S);
-    dm_free(b->d_ctl);
-    dm_free(b->d_chain_base);
-    dm_free(b->d_comp_base);
-    dm_free(b->d_g);
-    dm_free(b->d_err);
-    dm_free(b->d_bar);
-    dm_free(b->d_phase);
+    dm_free(b->block);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
     delete b;
 }
 
+static int launch_reserve(GBatchScratch **scratch, int n, std::string &err) {
+    GBatchScratch *b = *scratch;
+    if (b && b->cap >= n) return 0;
+    const int cap = std::max(n, b ? 2 * b->cap : 1);
+    graph_batch_free(b);
+    *scratch = nullptr;
+    b = new (std::nothrow) GBatchScratch();
+    if (!b) {
+        err = "host allocation";
+        return ECMC_ENOMEM;
+    }
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 255) & ~(size_t)255;
+        return o;
+    };
+    (void)take((size_t)cap * sizeof(GDev));
+    b->off_base = take((size_t)(cap + 1) * sizeof(int32_t));
+    b->off_comp = take((size_t)(cap + 1) * sizeof(int32_t));
+    b->off_ctl = take((size_t)cap * sizeof(GCtl));
+    b->off_bar = take(sizeof(unsigned int));
+    b->off_g = take(GG_N * sizeof(int32_t));
+    b->off_phase = take(GPH_N * sizeof(unsigned long long));
+    b->total = off;
+    b->host.assign(off, 0);
+    if (dm_alloc_t(&b->block, off) != 0 || cudaEventCreate(&b->ev0) != cudaSuccess ||
+        cudaEventCreate(&b->ev1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        graph_batch_free(b);
+        err = "launch tables";
+        return ECMC_ENOMEM;
+    }
+    b->cap = cap;
+    *scratch = b;
+    return 0;
+}
+
+// Epochs (32-bit pass counts) and stamps (30-bit leg counts) of a context; far
+// before one wraps (a launch makes fewer than 2^29 passes and 2^24 legs) both
+// start again.
+__global__ void k_g_clear_epochs(GDev s) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= s.n) return;
+    GDisk &r = s.g[q];
+    r.claim = 0ull;
+    r.t = g_time(r.own, r.t, s.stamp0);
+    if (g_static(r.own)) r.own = dbits(r.t) != 0ull ? 1u : 0u;
+    s.fl[q] = 0ull;
+}
+
 int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int32_t max_legs,
                     const uint64_t *budgets, cudaStream_t st, GraphTotals *tots,
-                    int32_t *legs_out, double *ms_out, std::string &err) {
+                    int32_t *legs_out, double *ms_out, std::string &err,
+                    unsigned long long wait_ns) {
     if (ms_out) *ms_out = 0.0;
     if (n < 1 || max_legs < 0) {
         err = "bad batch size or leg count";
@@ -2183,7 +2586,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
             err = "all contexts of a batch need the same claim windows";
             return ECMC_EINVAL;
         }
-        if (gs[r]->s.restart) {
+        if (gs[r]->s.restart && (n > 1 || scratch != &gs[r]->launch)) {
             err = "restart-mode contexts run alone (ecmc_run_to_breakpoint)";
             return ECMC_EINVAL;
         }
@@ -2197,54 +2600,9 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         if (legs_out) legs_out[r] = 0;
     }
     if (max_legs == 0) return 0;
+    int rc = launch_reserve(scratch, n, err);
+    if (rc) return rc;
     GBatchScratch *b = *scratch;
-    if (!b) {
-        b = new (std::nothrow) GBatchScratch();
-        if (!b) return ECMC_ENOMEM;
-        *scratch = b;
-    }
-    if (b->cap < n) {
-        const int cap = std::max(n, 2 * b->cap);
-        dm_free(b->d_S);
-        dm_free(b->d_ctl);
-        dm_free(b->d_chain_base);
-        dm_free(b->d_comp_base);
-        b->d_S = nullptr;
-        b->d_ctl = nullptr;
-        b->d_chain_base = b->d_comp_base = nullptr;
-        b->cap = 0;
-        if (dm_alloc_t(&b->d_S, (size_t)cap * sizeof(GDev)) != 0 ||
-            dm_alloc_t(&b->d_ctl, (size_t)cap * sizeof(GCtl)) != 0 ||
-            dm_alloc_t(&b->d_chain_base, (size_t)(cap + 1) * 4) != 0 ||
-            dm_alloc_t(&b->d_comp_base, (size_t)(cap + 1) * 4) != 0) {
-            err = "batch scratch";
-            return ECMC_ENOMEM;
-        }
-        b->cap = cap;
-    }
-    if (!b->d_g) {
-        int dev = 0, n_sm = 1, blocks = 0;
-        if (dm_alloc_t(&b->d_g, GB_N * sizeof(int32_t)) != 0 ||
-            dm_alloc_t(&b->d_err, sizeof(int32_t)) != 0 ||
-            dm_alloc_t(&b->d_bar, 2 * sizeof(unsigned int)) != 0 ||
-            dm_alloc_t(&b->d_phase, GPH_N * sizeof(unsigned long long)) != 0 ||
-            cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess ||
-            cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_run_graph_batch,
-                                                          GRUN_THREADS, UF_SMEM_BYTES) !=
-                cudaSuccess ||
-            blocks < 1) {
-            (void)cudaGetLastError();
-            err = "batch scratch";
-            return ECMC_ENOMEM;
-        }
-        b->grid = n_sm * std::min(blocks, GRUN_MIN_BLOCKS);
-    }
-    std::vector<GDev> S(n);
-    std::vector<GCtl> ctl(n);
-    std::vector<int32_t> base(n + 1, 0);
-    int rc = 0;
     auto cu = [&](cudaError_t e, const char *what) {
         if (e != cudaSuccess && !rc) {
             (void)cudaGetLastError();
@@ -2252,6 +2610,12 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
             rc = ECMC_ECUDA;
         }
     };
+    unsigned char *h = b->host.data();
+    memset(h, 0, b->total);
+    GDev *S = (GDev *)h;
+    int32_t *base = (int32_t *)(h + b->off_base);
+    GCtl *ctl = (GCtl *)(h + b->off_ctl);
+    int64_t chains = 0;
     for (int r = 0; r < n; ++r) {
         GraphCtx *g = gs[r];
         if (g->st != st) cu(cudaStreamSynchronize(g->st), "context stream");
@@ -2265,69 +2629,80 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
             }
             g->flags_cap = max_legs;
         }
+        if (g->s.epoch0 > 0xC0000000u || g->s.stamp0 > 0x3E000000u) {
+            k_g_clear_epochs<<<(unsigned)((g->s.n + 255) / 256), 256, 0, st>>>(g->s);
+            cu(cudaGetLastError(), "epochs");
+            g->s.epoch0 = 0;
+            g->s.stamp0 = 1;  // (the last leg's times, for ecmc_positions)
+        }
         S[r] = g->s;
-        memset(&ctl[r], 0, sizeof(GCtl));
         ctl[r].budget = budgets ? (int64_t)budgets[r] : 0;
         ctl[r].flags = g->d_flags;
         ctl[r].flags_cap = g->flags_cap;
         ctl[r].leg0 = g->log_legs;
-        base[r + 1] = base[r] + g->s.k;
+        base[r] = (int32_t)chains;
+        chains += g->s.k;
         // member tags restart with the launch's window count
         cu(cudaMemsetAsync(g->s.memb, 0xFF, (size_t)g->s.k * 8, st), "memb");
     }
-    if (rc) return rc;
-    cu(cudaMemcpyAsync(b->d_S, S.data(), (size_t)n * sizeof(GDev), cudaMemcpyHostToDevice, st),
-       "descriptors");
-    cu(cudaMemcpyAsync(b->d_ctl, ctl.data(), (size_t)n * sizeof(GCtl), cudaMemcpyHostToDevice, st),
-       "ctl");
-    cu(cudaMemcpyAsync(b->d_chain_base, base.data(), (size_t)(n + 1) * 4, cudaMemcpyHostToDevice,
-                       st),
-       "chain base");
-    cu(cudaMemsetAsync(b->d_g, 0, GB_N * sizeof(int32_t), st), "counters");
-    cu(cudaMemsetAsync(b->d_bar, 0, 2 * sizeof(unsigned int), st), "bar");
-    cu(cudaMemsetAsync(b->d_err, 0, sizeof(int32_t), st), "err");
-    cu(cudaMemsetAsync(b->d_phase, 0, GPH_N * sizeof(unsigned long long), st), "phase");
+    base[n] = (int32_t)chains;
+    if (chains > 0x7FFFFFFF) {
+        err = "too many chains in a batch";
+        return ECMC_EINVAL;
+    }
+    cu(cudaMemcpyAsync(b->block, h, b->total, cudaMemcpyHostToDevice, st), "tables");
     if (rc) return rc;
     GBatchDev B;
-    B.S = b->d_S;
-    B.ctl = b->d_ctl;
-    B.chain_base = b->d_chain_base;
-    B.comp_base = b->d_comp_base;
-    B.g = b->d_g;
-    B.bar = b->d_bar;
-    B.err = b->d_err;
-    B.phase_ns = b->d_phase;
+    B.reps = (const GDev *)b->block;
+    B.ctl = (GCtl *)(b->block + b->off_ctl);
+    B.chain_base = (const int32_t *)(b->block + b->off_base);
+    B.comp_base = (int32_t *)(b->block + b->off_comp);
+    B.bar = (unsigned int *)(b->block + b->off_bar);
+    B.g = (int32_t *)(b->block + b->off_g);
+    B.phase_ns = (unsigned long long *)(b->block + b->off_phase);
     B.R = n;
     B.max_legs = max_legs;
     B.windows = W;
     B.pad = 0;
+    B.wait_ns = wait_ns;
+    const int grid = graph_max_grid();
+    if (grid < 1) {
+        err = "cooperative launch unavailable";
+        return ECMC_ECUDA;
+    }
     void *args[] = {&B};
     cu(cudaEventRecord(b->ev0, st), "event");
-    cu(cudaLaunchCooperativeKernel((void *)k_run_graph_batch, b->grid, GRUN_THREADS, args,
-                                   UF_SMEM_BYTES, st),
+    cu(cudaLaunchCooperativeKernel((void *)k_run_graph, grid, GRUN_THREADS, args, UF_SMEM_BYTES,
+                                   st),
        "launch");
     cu(cudaEventRecord(b->ev1, st), "event");
-    int32_t gerr = 0;
-    unsigned long long ph[GPH_N];
-    cu(cudaMemcpyAsync(ctl.data(), b->d_ctl, (size_t)n * sizeof(GCtl), cudaMemcpyDeviceToHost, st),
-       "ctl");
-    cu(cudaMemcpyAsync(&gerr, b->d_err, sizeof gerr, cudaMemcpyDeviceToHost, st), "err");
-    cu(cudaMemcpyAsync(ph, b->d_phase, sizeof ph, cudaMemcpyDeviceToHost, st), "phase");
+    cu(cudaMemcpyAsync(h + b->off_ctl, b->block + b->off_ctl, b->total - b->off_ctl,
+                       cudaMemcpyDeviceToHost, st),
+       "tables");
     cu(cudaStreamSynchronize(st), "run");
     if (rc) return rc;
+    const int32_t *gg = (const int32_t *)(h + b->off_g);
+    const unsigned long long *ph = (const unsigned long long *)(h + b->off_phase);
     float ms = 0.f;
     cu(cudaEventElapsedTime(&ms, b->ev0, b->ev1), "elapsed");
     if (ms_out) *ms_out = ms;
     bool cap_err = false;
+    // (a launch that gave up on a wait may have made any number of passes)
+    const bool timed_out = gg[GG_ERR] == ECMC_ETIMEOUT;
+    const uint32_t passes =
+        timed_out ? (uint32_t)max_legs * (uint32_t)W * (MAX_RESTARTS + 2u) : (uint32_t)gg[GG_PASSES];
     for (int r = 0; r < n; ++r) {
         const GCtl &c = ctl[r];
         gs[r]->log_legs += c.legs;
+        gs[r]->s.epoch0 += passes;
+        gs[r]->s.stamp0 += timed_out ? (uint32_t)max_legs : (uint32_t)c.legs;
         GraphTotals &t = tots[r];
         t.legs = c.legs;
         t.lifts = c.lifts;
         t.conflict_legs = c.conflict_legs;
         t.repaired = c.repaired;
         t.continued = c.continued;
+        t.restarts = c.restarts;
         t.horizon = c.horizon;
         t.order_err = c.order_err;
         t.p1_lifts = c.p1_lifts;
@@ -2343,7 +2718,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         if (legs_out) legs_out[r] = (int32_t)c.legs;
         if (c.err) cap_err = true;
     }
-    if (gerr == ECMC_ETIMEOUT) {
+    if (timed_out) {
         err = "a grid barrier wait passed its time limit";
         return ECMC_ETIMEOUT;
     }
@@ -2351,7 +2726,42 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         err = "undo records or repair rounds overflowed";
         return ECMC_ECAPACITY;
     }
+    for (int r = 0; r < n; ++r) {
+        double dg[7];
+        if (ctl[r].dbg &&
+            cudaMemcpy(dg, gs[r]->s.dbg, sizeof dg, cudaMemcpyDeviceToHost) == cudaSuccess &&
+            dg[0] != 0.0) {
+            char buf[240];
+            snprintf(buf, sizeof buf,
+                     "internal check %g failed: %.17g %.17g %.17g %.17g %.17g %.17g", dg[0], dg[1],
+                     dg[2], dg[3], dg[4], dg[5], dg[6]);
+            err = buf;
+            return ECMC_ECUDA;
+        }
+    }
     return 0;
+}
+
+int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
+              int32_t *legs_done, GraphTotals *tot, std::string &err,
+              unsigned long long wait_ns) {
+    memset(tot, 0, sizeof *tot);
+    if (legs_done) *legs_done = 0;
+    if (n_legs <= 0) return 0;
+    int32_t legs = 0;
+    const int rc = graph_batch_run(&g->launch, &g, 1, n_legs, &budget, g->st, tot, &legs, nullptr,
+                                   err, wait_ns);
+    if (legs_done) *legs_done = legs;
+    if (flags_host && legs > 0) {
+        const cudaError_t e = cudaMemcpyAsync(flags_host, g->d_flags, (size_t)legs,
+                                              cudaMemcpyDeviceToHost, g->st);
+        if (e != cudaSuccess || cudaStreamSynchronize(g->st) != cudaSuccess) {
+            (void)cudaGetLastError();
+            err = "flags";
+            return rc ? rc : ECMC_ECUDA;
+        }
+    }
+    return rc;
 }
 
 int graph_export(GraphCtx *g, double *x, double *y, double *t, int32_t *active) {
@@ -2439,8 +2849,7 @@ void graph_destroy(GraphCtx *g) {
     for (void *p : g->allocs) dm_free(p);
     for (void *p : g->build_tmp) dm_free(p);
     dm_free(g->d_flags);
-    if (g->ev0) cudaEventDestroy(g->ev0);
-    if (g->ev1) cudaEventDestroy(g->ev1);
+    graph_batch_free(g->launch);
     delete g;
 }
 

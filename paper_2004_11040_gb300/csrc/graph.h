@@ -24,7 +24,8 @@ struct GraphTotals {
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
                  const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err);
 int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
-              int32_t *legs_done, GraphTotals *tot, std::string &err);
+              int32_t *legs_done, GraphTotals *tot, std::string &err,
+              unsigned long long wait_ns);
 // Device outputs (each may be null), filled on the context's stream.
 int graph_export(GraphCtx *g, double *x, double *y, double *t, int32_t *active);
 // Exchanges x and y of every disk (the next legs move along the other axis),
@@ -40,11 +41,13 @@ void graph_destroy(GraphCtx *g);
 // budget (budgets may be null; 0: none), exactly as graph_run would. The
 // scratch (launch tables) is kept by the caller between calls and freed with
 // graph_batch_free. tots[r] and legs_out[r] (may be null) receive each
-// context's totals; *ms_out the launch's device time.
+// context's totals; *ms_out the launch's device time. wait_ns bounds every
+// device wait of the launch.
 struct GBatchScratch;
 int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int32_t max_legs,
                     const uint64_t *budgets, cudaStream_t st, GraphTotals *tots,
-                    int32_t *legs_out, double *ms_out, std::string &err);
+                    int32_t *legs_out, double *ms_out, std::string &err,
+                    unsigned long long wait_ns);
 void graph_batch_free(GBatchScratch *scratch);
 // Device memory held by the context (bytes).
 int64_t graph_device_bytes(const GraphCtx *g);

@@ -522,9 +522,6 @@ __device__ RowStep rp_exact(const Dev &s, const StopK &sk, const RowChain &ch, c
     return r;
 }
 
-__device__ __forceinline__ void red_min_u64(unsigned long long *p, unsigned long long v) {
-    asm volatile("red.relaxed.gpu.global.min.u64 [%0], %1;" ::"l"(p), "l"(v));
-}
 __device__ __forceinline__ void red_min_u32(uint32_t *p, uint32_t v) {
     asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(v));
 }
