@@ -157,17 +157,24 @@ __device__ __forceinline__ double shfl_f64(double v, int src) {
 
 // ------------------------------------------------------------ graph build
 
+// Inputs and scratch of a build: a cell list of the disks (slots fill from
+// the first), their FP32 coordinates per slot relative to the cell's corner (an
+// error of 1e-7 d whatever the box), and one bit per y bin of width d/128 that
+// holds a disk. The disks come by id (x, y, placed by k_gb_cells)
+// or, sx != null, from the slots of a cell-scan context.
 struct GBuild {
     int64_t n;
     int nc, nb;
-    double L, d, d2, a, inv_a, eps, w;  // cells of side a; y bins of width w
-    float Lf, wf, inv_wf, half_f, d_f;     // the same in FP32 (bins only)
-    float dcut_f;        // d + a margin above the FP32 error of |dy| (slot filter)
+    double L, d, d2, a, inv_a;
+    float Lf, df, half_f, af, wf, inv_wf;
+    float del;           // a 2^-20: bound on the FP32 error of a difference of
+                         // coordinates of neighbouring cells
     const double *x, *y;
-    uint32_t *cid;       // [nc*nc*C] disk per slot, EMPTY
-    double *cx, *cy;     // [nc*nc*C]
-    float *cyf;          // [nc*nc*C] y in FP32
-    int32_t *bins;       // [nb + 1]: counts, then their exclusive prefix
+    const double *sx, *sy;
+    const uint32_t *scid;  // [nc*nc*C] disk per slot, EMPTY
+    uint32_t *cid;         // the same, writable (null with sx)
+    float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
+    uint32_t *bits;        // [nb / 32 + 1]
     GDisk *g;
     unsigned long long *err;  // cell overflow count
 };
@@ -179,76 +186,63 @@ __device__ __forceinline__ int cell_coord(double v, double inv_a, int nc) {
     return c;
 }
 
+// A monotone map of y to its bin, the same wherever bins are set or asked for.
+__device__ __forceinline__ int y_bin(const GBuild &b, float y) {
+    const int q = __float2int_rz(__fmul_rn(y, b.inv_wf));
+    return min(max(q, 0), b.nb - 1);
+}
+
+__device__ __forceinline__ void set_bin(const GBuild &b, float y) {
+    const int q = y_bin(b, y);
+    const uint32_t m = 1u << (q & 31);
+    // (most bins are set already: an atomic per disk on a lattice's few bins
+    // took 70 of the 400 us of creation at 2^20 disks)
+    if (!(*(volatile uint32_t *)(b.bits + (q >> 5)) & m)) atomicOr(b.bits + (q >> 5), m);
+}
+
+// Coordinates relative to the corner of cell (row, col); an FP32 x of -0 or a
+// little less (x on the edge) counts as 0, so that only an empty slot is NaN.
+__device__ __forceinline__ float2 in_cell(const GBuild &b, double x, double y, int row, int col) {
+    return make_float2(fmaxf(d2f_trunc(__dsub_rn(x, __dmul_rn((double)col, b.a))), 0.f),
+                       d2f_trunc(__dsub_rn(y, __dmul_rn((double)row, b.a))));
+}
+
 template <int C>
 __global__ void k_gb_cells(GBuild b) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= b.n) return;
     const double x = b.x[q], y = b.y[q];
-    const uint32_t cell = (uint32_t)cell_coord(y, b.inv_a, b.nc) * (uint32_t)b.nc +
-                          (uint32_t)cell_coord(x, b.inv_a, b.nc);
-    // bins only need a monotone map of y, the same as in band_count: FP32
-    int bin = __float2int_rz(__fmul_rn(__double2float_rn(y), b.inv_wf));
-    if (bin >= b.nb) bin = b.nb - 1;
-    if (bin < 0) bin = 0;
-    atomicAdd(b.bins + bin, 1);
+    const int row = cell_coord(y, b.inv_a, b.nc), col = cell_coord(x, b.inv_a, b.nc);
+    const uint32_t cell = (uint32_t)row * (uint32_t)b.nc + (uint32_t)col;
+    const float2 v = in_cell(b, x, y, row, col);
+    set_bin(b, d2f_trunc(y));
     for (int sl = 0; sl < C; ++sl) {
         const uint32_t loc = cell * C + sl;
         if (atomicCAS(b.cid + loc, EMPTY, (uint32_t)q) == EMPTY) {
-            b.cx[loc] = x;
-            b.cy[loc] = y;
-            b.cyf[loc] = __double2float_rn(y);
+            b.cxy[loc] = v;
             return;
         }
     }
     atomicAdd(b.err, 1ull);
 }
 
-// Exclusive prefix of the y-bin counts, in tiles of SCAN_TILE bins (one block
-// of 1024 threads, 4 consecutive bins per thread): k_gb_tile_sums adds each
-// tile, k_gb_scan_tiles scans each tile from the sum of the tiles before it;
-// the last tile also writes the total to bins[nb].
-constexpr int SCAN_TILE = 4096;
-
-__device__ __forceinline__ int tile_bin(const GBuild &b, int64_t q) {
-    return q < b.nb ? b.bins[q] : 0;
-}
-
-__global__ void k_gb_tile_sums(GBuild b, int32_t *part) {
-    __shared__ int warp_tot[32];
-    __shared__ int tot[2];
-    const int64_t q0 = (int64_t)blockIdx.x * SCAN_TILE + 4 * threadIdx.x;
-    const int v = tile_bin(b, q0) + tile_bin(b, q0 + 1) + tile_bin(b, q0 + 2) + tile_bin(b, q0 + 3);
-    block_exscan(v, warp_tot, tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot[0];
-}
-
-__global__ void k_gb_scan_tiles(GBuild b, const int32_t *part) {
-    __shared__ int warp_tot[32];
-    __shared__ int tot[2];
-    __shared__ int base;
-    if (threadIdx.x < 32) {  // sum of the tiles before this one
-        int acc = 0;
-        for (int t = threadIdx.x; t < (int)blockIdx.x; t += 32) acc += part[t];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-        if (threadIdx.x == 0) base = acc;
+// FP32 coordinates and bins from the slots of a cell-scan context.
+template <int C>
+__global__ void k_gb_slots(GBuild b, uint32_t nslot) {
+    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= nslot) return;
+    float2 v = make_float2(__int_as_float(-1), __int_as_float(-1));
+    if (b.scid[q] != EMPTY) {
+        const uint32_t cell = q / C;
+        v = in_cell(b, b.sx[q], b.sy[q], (int)(cell / (uint32_t)b.nc), (int)(cell % (uint32_t)b.nc));
+        set_bin(b, d2f_trunc(b.sy[q]));
     }
-    const int64_t q0 = (int64_t)blockIdx.x * SCAN_TILE + 4 * threadIdx.x;
-    const int v0 = tile_bin(b, q0), v1 = tile_bin(b, q0 + 1), v2 = tile_bin(b, q0 + 2),
-              v3 = tile_bin(b, q0 + 3);
-    const int off = block_exscan(v0 + v1 + v2 + v3, warp_tot, tot) + base;
-    const int o[4] = {off, off + v0, off + v0 + v1, off + v0 + v1 + v2};
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (q0 + u < b.nb) b.bins[q0 + u] = o[u];
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) b.bins[b.nb] = base + tot[0];
+    b.cxy[q] = v;
 }
 
-// Disks whose y falls in a bin that meets [lo, hi) (periodic, hi - lo < L):
-// an upper bound on the disks with y in that range. FP32 is enough: the map
-// to bins is monotone, and the callers' one-bin margin (d/128) is far above
-// the FP32 rounding of y, lo and hi.
-__device__ int band_count(const GBuild &b, float lo, float hi) {
+// Does a bin that meets [lo, hi) (periodic, hi - lo < L) hold a disk? The
+// callers' one-bin margin (d/128) is far above the FP32 rounding of y, lo, hi.
+__device__ bool band_any(const GBuild &b, float lo, float hi) {
     if (lo < 0.f) {
         lo = __fadd_rn(lo, b.Lf);
         hi = __fadd_rn(hi, b.Lf);
@@ -256,151 +250,415 @@ __device__ int band_count(const GBuild &b, float lo, float hi) {
         lo = __fsub_rn(lo, b.Lf);
         hi = __fsub_rn(hi, b.Lf);
     }
-    auto bin = [&](float v) {
-        int q = __float2int_rz(__fmul_rn(v, b.inv_wf));
-        return min(max(q, 0), b.nb - 1);
+    auto any = [&](int q0, int q1) {
+        uint32_t r = 0u;
+        for (int w = q0 >> 5; w <= q1 >> 5; ++w) {
+            uint32_t m = ~0u;
+            if (w == q0 >> 5) m &= ~0u << (q0 & 31);
+            if (w == q1 >> 5) m &= ~0u >> (31 - (q1 & 31));
+            r |= b.bits[w] & m;
+        }
+        return r != 0u;
     };
-    const int b0 = bin(lo);
-    if (hi <= b.Lf) return b.bins[bin(hi) + 1] - b.bins[b0];
-    return (b.bins[b.nb] - b.bins[b0]) + (b.bins[bin(__fsub_rn(hi, b.Lf)) + 1] - b.bins[0]);
+    const int q0 = y_bin(b, lo);
+    if (hi <= b.Lf) return any(q0, y_bin(b, hi));
+    return any(q0, b.nb - 1) || any(0, y_bin(b, __fsub_rn(hi, b.Lf)));
 }
 
-// Arrows of G(3), one thread per disk: the thread scans the columns ahead
-// (rows cy-1..cy+1) and keeps, per corridor, the least (tau, j). Before
-// column m >= 1, if (m a - fx) - d exceeds the worst best tau of the
-// corridors still in play (+ eps), no later column can improve any of them
-// and the scan stops; a corridor that the y bins show empty is not in play,
-// any other one keeps the scan going (once round the box at most).
-// The FP64 pipe costs the same per warp instruction whatever the number of
-// active lanes, so every lane takes a disk of its own, and two tests keep
-// FP64 work off the slots that cannot matter, both exact:
-// - |dy| in FP32 above d plus a margin larger than its rounding error: the
-//   slot lies in no corridor;
-// - RN(dx - d) above the corridor's best: the computed tau = RN(dx - b) with
-//   b = RN(sqrt(d^2 - dy^2)) <= d is at least that (rounding is monotone),
-//   so the candidate can neither win nor tie, and its square root is skipped.
+// One corridor's best so far: the slot, and bounds of its time of flight.
+struct GBest {
+    float lo, hi;
+    uint32_t loc;
+};
+
+// (approximate to 2^-22; the slop below is far above that)
+__device__ __forceinline__ float sqrt_f(float v) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// The corridor of the disk at v (in its cell, rr rows and m columns on) seen
+// from xi, yi (-1: none; 3: FP32 cannot tell) and, for 0 .. 2, bounds of its
+// time of flight.
+__device__ __forceinline__ int corridor_f(const GBuild &b, float xi, float yi, int rr, int m,
+                                          float2 v, float &lo, float &hi) {
+    const float dy = (float)rr * b.af + (v.y - yi);
+    const float ay = fabsf(dy);
+    if (ay > b.df + b.del) return -1;
+    float dx = (float)m * b.af + (v.x - xi);
+    float del = b.del + (float)m * (0.25f * b.del);
+    if (ay > b.df - b.del || fabsf(ay - b.half_f) < b.del || fabsf(dx) < del) return 3;
+    if (dx < 0.f) {  // behind in its own column: nearly a lap ahead
+        dx += b.Lf;
+        del += b.Lf * 0x1p-21f;
+    }
+    const float d2 = b.df * b.df, an = fmaxf(ay - b.del, 0.f), af = ay + b.del;
+    // (2^-19 d covers the roundings of these lines)
+    const float slop = b.df * 0x1p-19f + del;
+    hi = dx - sqrt_f(fmaxf(d2 - af * af - d2 * 0x1p-21f, 0.f)) + slop;
+    lo = dx - sqrt_f(d2 - an * an + d2 * 0x1p-21f) - slop;
+    return ay < b.half_f ? 0 : dy > 0.f ? 1 : 2;
+}
+
+// The candidate of a corridor takes the place of the best or not; true where
+// the bounds cannot tell.
+__device__ __forceinline__ bool take_best(GBest &best, float lo, float hi, uint32_t loc) {
+    if (lo > best.hi) return false;
+    const bool doubt = best.loc != NONE && !(hi < best.lo);
+    if (hi < best.hi) {
+        best.hi = hi;
+        best.loc = loc;
+    }
+    best.lo = doubt ? fminf(best.lo, lo) : lo;
+    return doubt;
+}
+
+__device__ __forceinline__ double gb_x(const GBuild &b, uint32_t loc, uint32_t id) {
+    return b.sx ? b.sx[loc] : b.x[id];
+}
+__device__ __forceinline__ double gb_y(const GBuild &b, uint32_t loc, uint32_t id) {
+    return b.sx ? b.sy[loc] : b.y[id];
+}
+
+// The FP32 coordinates of a cell's slots, all loads at once.
 template <int C>
-__global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
-    const int nc = b.nc;
+struct GCell {
+    float2 v[C];
+};
+template <int C>
+__device__ __forceinline__ GCell<C> load_cell(const GBuild &b, uint32_t c0) {
+    GCell<C> r;
+    const float4 *p = reinterpret_cast<const float4 *>(b.cxy + c0);
+#pragma unroll
+    for (int q = 0; q < C / 2; ++q) {
+        const float4 u = p[q];
+        r.v[2 * q] = make_float2(u.x, u.y);
+        r.v[2 * q + 1] = make_float2(u.z, u.w);
+    }
+    return r;
+}
+
+// The corridors of disk i (slot loc, FP32 place vi) by their definition, in
+// FP64: where FP32 cannot tell. The warp searches 32 columns at a time; the
+// slots of each corridor's arrow (NONE: empty) end in aj on every lane.
+template <int C>
+__device__ __noinline__ void arrows_exact(const GBuild &b, uint32_t i, uint32_t loc, float2 vi,
+                                          double xi, double yi, int cxi, int cyi, bool p1, bool p2,
+                                          uint32_t *aj) {
+    const int nc = b.nc, lane = threadIdx.x & 31;
     const double half = __dmul_rn(0.5, b.d);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < b.n; i += stride) {
-        const double xi = b.x[i], yi = b.y[i];
-        const int cxi = cell_coord(xi, b.inv_a, nc), cyi = cell_coord(yi, b.inv_a, nc);
-        const double fx = __dsub_rn(xi, __dmul_rn((double)cxi, b.a));
-        // corridors that may hold a disk (one bin of margin on each side)
-        bool play[3];
-        const float yf = __double2float_rn(yi);
-        play[0] = band_count(b, yf - b.half_f - b.wf, yf + b.half_f + b.wf) > 1;  // i is there
-        play[1] = band_count(b, yf + b.half_f - b.wf, yf + b.d_f + b.wf) > 0;
-        play[2] = band_count(b, yf - b.d_f - b.wf, yf - b.half_f + b.wf) > 0;
-        unsigned long long bt[3] = {INF_BITS, INF_BITS, INF_BITS};
-        uint32_t bj[3] = {NONE, NONE, NONE};
-        double bb[3] = {0.0, 0.0, 0.0};
-        int rows[3] = {cyi - 1, cyi, cyi + 1};
-        if (rows[0] < 0) rows[0] += nc;
-        if (rows[2] >= nc) rows[2] -= nc;
-        for (int m = 0; m < nc; ++m) {
-            if (m >= 1) {
-                unsigned long long worst = 0ull;
-                bool any = false;
-#pragma unroll
-                for (int kc = 0; kc < 3; ++kc)
-                    if (play[kc]) {
-                        any = true;
-                        if (bt[kc] > worst) worst = bt[kc];
-                    }
-                if (!any) break;
-                if (worst != INF_BITS) {
-                    const double thr =
-                        __dsub_rn(__dsub_rn(__dmul_rn((double)m, b.a), fx), b.d);
-                    const double lim = __dadd_rn(__longlong_as_double((long long)worst), b.eps);
-                    if (!dneg(thr) && dbits(thr) > dbits(lim)) break;
+    unsigned long long bt[3] = {INF_BITS, INF_BITS, INF_BITS};
+    uint32_t bj[3] = {NONE, NONE, NONE}, bl[3] = {NONE, NONE, NONE};
+    for (int m0 = 0; m0 < nc; m0 += 32) {
+        const int m = m0 + lane;
+        int col = cxi + m;
+        if (col >= nc) col -= nc;
+        for (int rr = -1; rr <= 1; ++rr) {
+            int row = cyi + rr;
+            if (row < 0) row += nc;
+            if (row >= nc) row -= nc;
+            for (int sl = 0; sl < C; ++sl) {
+                const uint32_t at = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C + sl;
+                float lo, hi;
+                bool cand = m < nc && at != loc && b.cxy[m < nc ? at : loc].x >= 0.f;
+                cand = cand && corridor_f(b, vi.x, vi.y, rr, m, b.cxy[at], lo, hi) >= 0;
+                if (!__any_sync(FULL, cand)) continue;
+                if (!cand) continue;
+                const uint32_t id = b.scid[at];
+                const double dy = __dsub_rn(gb_y(b, at, id), yi);
+                double ay = fabs(dy);
+                const double la = __dsub_rn(b.L, ay);
+                const bool flip = dbits(la) < dbits(ay);
+                if (flip) ay = la;
+                if (dbits(ay) >= dbits(b.d)) continue;
+                int kc = 0;
+                if (dbits(ay) >= dbits(half)) {
+                    bool up = !dneg(dy) && dbits(dy) != 0ull;
+                    if (flip) up = !up;
+                    kc = up ? 1 : 2;
                 }
-            }
-            int col = cxi + m;
-            if (col >= nc) col -= nc;
+                double dx = __dsub_rn(gb_x(b, at, id), xi);
+                if (dneg(dx)) dx = __dadd_rn(dx, b.L);
+                double tau = __dsub_rn(dx, __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay))));
+                if (dneg(tau)) tau = 0.0;
+                const unsigned long long kt = dbits(tau);
 #pragma unroll
-            for (int rr = 0; rr < 3; ++rr) {
-                const uint32_t cell = (uint32_t)rows[rr] * (uint32_t)nc + (uint32_t)col;
-                for (int sl = 0; sl < C; ++sl) {
-                    const uint32_t loc = cell * C + sl;
-                    const uint32_t id = b.cid[loc];
-                    if (id == EMPTY) break;  // a cell's slots fill from the first
-                    if (id == (uint32_t)i) continue;
-                    const float ayf0 = fabsf(__fsub_rn(b.cyf[loc], yf));
-                    if (fminf(ayf0, __fsub_rn(b.Lf, ayf0)) > b.dcut_f) continue;
-                    const double dy = __dsub_rn(b.cy[loc], yi);
-                    double ay = fabs(dy);
-                    bool flip = false;
-                    const double la = __dsub_rn(b.L, ay);
-                    if (dbits(la) < dbits(ay)) {
-                        ay = la;
-                        flip = true;
+                for (int q = 0; q < 3; ++q)
+                    if (q == kc && (kt < bt[q] || (kt == bt[q] && id < bj[q]))) {
+                        bt[q] = kt;
+                        bj[q] = id;
+                        bl[q] = at;
                     }
-                    if (dbits(ay) >= dbits(b.d)) continue;
-                    int kc = 0;
-                    if (dbits(ay) >= dbits(half)) {
-                        bool up = !dneg(dy) && dbits(dy) != 0ull;
-                        if (flip) up = !up;
-                        kc = up ? 1 : 2;
-                    }
-                    // selects, not indexing, keep the corridor arrays in registers
-                    const bool pk = kc == 0 ? play[0] : kc == 1 ? play[1] : play[2];
-                    if (!pk) continue;
-                    const unsigned long long bk = kc == 0 ? bt[0] : kc == 1 ? bt[1] : bt[2];
-                    double dx = __dsub_rn(b.cx[loc], xi);
-                    if (dneg(dx)) dx = __dadd_rn(dx, b.L);
-                    const double lo = __dsub_rn(dx, b.d);
-                    if (!dneg(lo) && dbits(lo) > bk) continue;
-                    const double bv = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
-                    double tau = __dsub_rn(dx, bv);
-                    if (dneg(tau)) tau = 0.0;
-                    const unsigned long long kt = dbits(tau);
-#pragma unroll
-                    for (int q = 0; q < 3; ++q)
-                        if (q == kc && (kt < bt[q] || (kt == bt[q] && id < bj[q]))) {
-                            bt[q] = kt;
-                            bj[q] = id;
-                            bb[q] = bv;
-                        }
-                }
             }
         }
-        GDisk &r = b.g[i];
-        r.x = xi;
-        r.t = 0.0;
+        float worst = -1.f;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            r.a[q] = bj[q];
-            r.b[q] = bj[q] == NONE ? 0.0 : bb[q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long t2 = shfl_xor_u64(bt[q], o);
+                const uint32_t j2 = __shfl_xor_sync(FULL, bj[q], o);
+                const uint32_t l2 = __shfl_xor_sync(FULL, bl[q], o);
+                if (t2 < bt[q] || (t2 == bt[q] && j2 < bj[q])) {
+                    bt[q] = t2;
+                    bj[q] = j2;
+                    bl[q] = l2;
+                }
+            }
+            if (q == 0 || (q == 1 ? p1 : p2))
+                worst = fmaxf(worst, d2f_trunc(__longlong_as_double((long long)bt[q])));
+        }
+        const int mn = m0 + 32;
+        if ((float)mn * b.af - vi.x - b.df - (float)(mn + 4) * b.del > worst * (1.f + 0x1p-20f))
+            break;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) aj[q] = bl[q];
+}
+
+// Arrows of G(3), and the whole record of every disk (static, time 0): one
+// thread per disk. A block takes BUILD_CELLS cells of consecutive numbers and
+// packs their occupied slots first, so that warps are full and neighbours read
+// the same cells. The search runs in FP32: per corridor, bounds of the time of
+// flight of the best candidate; candidates whose bounds overlap, or whose
+// corridor FP32 cannot tell, send the disk to arrows_exact (a few in 10^5). After NEAR_COLS columns the corridors that still have none -- few
+// disks, but each would hold up its warp for a search of the whole ring -- are
+// searched by the warp together, 32 columns at a time. FP64 is left with one
+// b = sqrt(d^2 - dy^2) per arrow, all lanes at once (an FP64 instruction costs
+// the same whatever its lane mask). Corridors and rows that the y bins show
+// empty are not searched. 65536 dense disks: 31 us along their dense axis, 48 to
+// 88 us along the other (few disks in some corridors), with a thread per disk
+// searching alone in FP64 100 to 550 us; 2^20 lattice disks 107 us (124 us),
+// bound by its instructions and by the scattered reads and records.
+constexpr int BUILD_CELLS = 224;
+constexpr int NEAR_COLS = 8;
+
+template <int C>
+__global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
+    __shared__ uint32_t list[BUILD_CELLS * C];
+    __shared__ int count;
+    const int nc = b.nc, lane = threadIdx.x & 31;
+    const uint32_t ncell = (uint32_t)nc * (uint32_t)nc;
+    const uint32_t cell0 = blockIdx.x * BUILD_CELLS;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    static_assert(BUILD_CELLS * C % 32 == 0, "whole warps pack the slots");
+    for (uint32_t q = threadIdx.x; q < BUILD_CELLS * C; q += blockDim.x) {
+        const bool occ = cell0 + q / C < ncell && b.scid[cell0 * C + q] != EMPTY;
+        const unsigned om = __ballot_sync(FULL, occ);
+        int at = 0;
+        if (lane == 0 && om) at = atomicAdd(&count, __popc(om));
+        at = __shfl_sync(FULL, at, 0) + __popc(om & ((1u << lane) - 1u));
+        if (occ) list[at] = cell0 * C + q;
+    }
+    __syncthreads();
+    const int total = count;
+    for (int e0 = 0; e0 < total; e0 += blockDim.x) {
+        const int e = e0 + (int)threadIdx.x;
+        const bool has = e < total;
+        const uint32_t loc = has ? list[e] : list[0];
+        const uint32_t i = b.scid[loc];
+        const float2 vi = b.cxy[loc];
+        const double xi = gb_x(b, loc, i), yi = gb_y(b, loc, i);
+        const int cyi = (int)((loc / C) / (uint32_t)nc), cxi = (int)((loc / C) % (uint32_t)nc);
+        const float yf = d2f_trunc(yi);
+        // corridors that may hold a disk (one bin of margin on each side; the
+        // centre one holds the disk itself)
+        bool play[3];
+        play[0] = true;
+        play[1] = band_any(b, yf + b.half_f - b.wf, yf + b.df + b.wf);
+        play[2] = band_any(b, yf - b.df - b.wf, yf - b.half_f + b.wf);
+        GBest best[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            best[q].lo = best[q].hi = INFINITY;
+            best[q].loc = NONE;
+        }
+        bool doubt = false;
+        // the rows beside that hold a disk within d (by the bins): on a lattice
+        // neither does
+        const float y0 = d2f_trunc(__dmul_rn((double)cyi, b.a));
+        const bool row_up = band_any(b, y0 + b.af - b.wf, yf + b.df + b.wf);
+        const bool row_dn = band_any(b, yf - b.df - b.wf, y0 + b.wf);
+        // the corridors that column m may still improve: thr(m) within the best
+        auto open_at = [&](int m) {
+            const float thr = (float)m * b.af - vi.x - b.df - (float)(m + 4) * b.del;
+            unsigned o = 0u;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (play[q] && !(thr > best[q].hi)) o |= 1u << q;
+            return o;
+        };
+        auto cell_scan = [&](int row, int col, int rr, int m) {
+            const uint32_t c0 = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C;
+            const GCell<C> cell = load_cell<C>(b, c0);
+#pragma unroll
+            for (int sl = 0; sl < C; ++sl) {
+                const float2 v = cell.v[sl];
+                if (!(v.x >= 0.f)) break;  // a cell's slots fill from the first
+                if (c0 + sl == loc) continue;
+                float lo, hi;
+                const int kc = corridor_f(b, vi.x, vi.y, rr, m, v, lo, hi);
+                if (kc < 0) continue;
+                if (kc == 3) {
+                    doubt = true;
+                    continue;
+                }
+                // (selects, not indexing, keep the corridors in registers)
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (q == kc) doubt |= take_best(best[q], lo, hi, c0 + sl);
+            }
+        };
+        const int rdn = cyi == 0 ? nc - 1 : cyi - 1, rup = cyi == nc - 1 ? 0 : cyi + 1;
+        int m = 0;
+        for (; m < min(NEAR_COLS, nc); ++m) {
+            const unsigned open = open_at(m);
+            if (!open) break;
+            int col = cxi + m;
+            if (col >= nc) col -= nc;
+            if (row_dn && (open & 5u)) cell_scan(rdn, col, -1, m);
+            cell_scan(cyi, col, 0, m);
+            if (row_up && (open & 3u)) cell_scan(rup, col, 1, m);
+        }
+        // the disks that need columns beyond, one by one by the whole warp
+        unsigned todo = __ballot_sync(FULL, has && !doubt && m == NEAR_COLS && m < nc && open_at(m));
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float sx = __shfl_sync(FULL, vi.x, src), sy = __shfl_sync(FULL, vi.y, src);
+            const int scx = __shfl_sync(FULL, cxi, src), scy = __shfl_sync(FULL, cyi, src);
+            const uint32_t sloc = __shfl_sync(FULL, loc, src);
+            GBest w[3];
+            bool sp[3], dbt = false;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                w[q].lo = __shfl_sync(FULL, best[q].lo, src);
+                w[q].hi = __shfl_sync(FULL, best[q].hi, src);
+                w[q].loc = __shfl_sync(FULL, best[q].loc, src);
+                sp[q] = __shfl_sync(FULL, (int)play[q], src) != 0;
+            }
+            for (int m0 = NEAR_COLS; m0 < nc; m0 += 32) {
+                const float thr = (float)m0 * b.af - sx - b.df - (float)(m0 + 4) * b.del;
+                unsigned open = 0u;
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (sp[q] && !(thr > w[q].hi)) open |= 1u << q;
+                if (!open) break;
+                GBest l[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    l[q].lo = l[q].hi = INFINITY;
+                    l[q].loc = NONE;
+                }
+                const int mm = m0 + lane;
+                if (mm < nc) {
+                    int col = scx + mm;
+                    if (col >= nc) col -= nc;
+                    for (int rr = -1; rr <= 1; ++rr) {
+                        if ((rr < 0 && !(open & 5u)) || (rr > 0 && !(open & 3u))) continue;
+                        int row = scy + rr;
+                        if (row < 0) row += nc;
+                        if (row >= nc) row -= nc;
+                        const uint32_t c0 = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C;
+                        const GCell<C> cell = load_cell<C>(b, c0);
+#pragma unroll
+                        for (int sl = 0; sl < C; ++sl) {
+                            const float2 v = cell.v[sl];
+                            if (!(v.x >= 0.f)) break;
+                            if (c0 + sl == sloc) continue;
+                            float lo, hi;
+                            const int kc = corridor_f(b, sx, sy, rr, mm, v, lo, hi);
+                            if (kc == 3) dbt = true;
+#pragma unroll
+                            for (int q = 0; q < 3; ++q)
+                                if (q == kc) dbt |= take_best(l[q], lo, hi, c0 + sl);
+                        }
+                    }
+                }
+                // the lanes' candidates, then the best so far
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    if (!__any_sync(FULL, l[q].loc != NONE)) continue;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const float lo = __shfl_xor_sync(FULL, l[q].lo, o);
+                        const float hi = __shfl_xor_sync(FULL, l[q].hi, o);
+                        const uint32_t lc = __shfl_xor_sync(FULL, l[q].loc, o);
+                        if (lc != NONE) dbt |= take_best(l[q], lo, hi, lc);
+                    }
+                    if (l[q].loc != NONE) dbt |= take_best(w[q], l[q].lo, l[q].hi, l[q].loc);
+                }
+            }
+            dbt = __any_sync(FULL, dbt);
+            if (lane == src) {
+                doubt = dbt;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) best[q] = w[q];
+            }
+        }
+        uint32_t aj[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) aj[q] = best[q].loc;
+        unsigned odd = __ballot_sync(FULL, has && doubt);
+        while (odd) {
+            const int src = __ffs(odd) - 1;
+            odd &= odd - 1;
+            uint32_t ex[3];
+            arrows_exact<C>(b, __shfl_sync(FULL, i, src), __shfl_sync(FULL, loc, src),
+                            make_float2(__shfl_sync(FULL, vi.x, src), __shfl_sync(FULL, vi.y, src)),
+                            __shfl_sync(FULL, xi, src), __shfl_sync(FULL, yi, src),
+                            __shfl_sync(FULL, cxi, src), __shfl_sync(FULL, cyi, src),
+                            __shfl_sync(FULL, (int)play[1], src) != 0,
+                            __shfl_sync(FULL, (int)play[2], src) != 0, ex);
+            if (lane == src) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) aj[q] = ex[q];
+            }
+        }
+        uint32_t id[3];
+        double bv[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            id[q] = NONE;
+            bv[q] = 0.0;
+            if (!__any_sync(FULL, aj[q] != NONE)) continue;
+            const uint32_t l = aj[q] != NONE ? aj[q] : loc;
+            const uint32_t j = b.scid[l];
+            double ay = fabs(__dsub_rn(gb_y(b, l, j), yi));
+            if (__any_sync(FULL, cyi == 0 || cyi == nc - 1 || nc <= 4)) {
+                const double la = __dsub_rn(b.L, ay);
+                if (dbits(la) < dbits(ay)) ay = la;
+            }
+            const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
+            if (aj[q] != NONE) {
+                id[q] = j;
+                bv[q] = v;
+            }
+        }
+        if (has) {
+            ulonglong2 *r = reinterpret_cast<ulonglong2 *>(b.g + i);
+            r[0] = make_ulonglong2(dbits(xi), 0ull);
+            r[1] = make_ulonglong2((unsigned long long)OWN_STATIC | ((unsigned long long)id[0] << 32),
+                                   (unsigned long long)id[1] | ((unsigned long long)id[2] << 32));
+            r[2] = make_ulonglong2(0ull, dbits(bv[0]));
+            r[3] = make_ulonglong2(dbits(bv[1]), dbits(bv[2]));
         }
     }
 }
 
-// Owner words and claims from scratch: every disk static, then the chains'
-// start disks active.
-__global__ void k_g_init(GDev s) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < s.n) {
-        s.g[q].own = OWN_STATIC;
-        s.g[q].claim = 0ull;
-        s.key[q] = ~0ull;
-        s.fl[q] = 0ull;
-    }
-}
-
+// The chains' start disks active (after a build).
 __global__ void k_g_init_chains(GDev s, const int32_t *active) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.k) return;
-    const uint32_t a = (uint32_t)active[c];
+    const uint32_t a = active ? (uint32_t)active[c] : s.ci[c];
     s.ci[c] = a;
     s.ci0[c] = a;
     s.g[a].own = OWN_ACTIVE | (uint32_t)c;
     s.nrec[c] = 0;
     s.status[c] = ST_STALLED;
 }
-
 
 // --------------------------------------------------------- parallel pass
 
@@ -2196,13 +2454,6 @@ __global__ void k_g_swap_xy(GDev s, double *xnew) {
     s.y[q] = xo;
 }
 
-__global__ void k_g_reset_chains(GDev s) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= s.k) return;
-    s.nrec[c] = 0;
-    s.ci0[c] = s.ci[c];
-}
-
 }  // namespace
 
 // ------------------------------------------------------------------ host
@@ -2217,7 +2468,7 @@ struct GraphCtx {
     int32_t flags_cap = 0;
     int64_t log_legs = 0;  // legs logged so far (leg index of the log)
     GBatchScratch *launch = nullptr;  // launch tables of graph_run
-    void *build_tmp[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    void *build_tmp = nullptr;        // scratch of graph_build
     std::vector<std::pair<void **, size_t>> pending;
     int64_t bytes = 0;  // device memory held
 };
@@ -2255,16 +2506,28 @@ int gcommit(GraphCtx *g, std::string &err) {
     return 0;
 }
 
-// Builds the arrows (and x, t = 0) of every disk from positions x, y (device).
-// Bytes of the build's scratch (kept by the context for direction changes).
-static int64_t graph_build_bytes(double L, double d, int nc, int C) {
+// Bytes of a build's scratch (kept by the context for direction changes): the
+// FP32 coordinates, the y bins and the overflow count, and the ids per slot.
+static size_t build_parts(double L, double d, int nc, int C, size_t *off_bits, size_t *off_err,
+                          size_t *off_cid) {
     const size_t nslot = (size_t)nc * nc * C;
     const size_t nb = (size_t)((int)std::ceil(L / (d / 128.0)) + 1);
-    return (int64_t)(nslot * 4 + nslot * 8 + nslot * 8 + (nb + 1) * 4 + 8 + nslot * 4 +
-                     ((nb + SCAN_TILE - 1) / SCAN_TILE) * 4);
+    *off_cid = nslot * sizeof(float2);
+    *off_bits = *off_cid + ((nslot * 4 + 15) & ~(size_t)15);
+    *off_err = *off_bits + ((nb / 32 + 1) * 4 + 15) / 16 * 16;
+    return *off_err + 16;
 }
 
-int graph_build(GraphCtx *g, const double *x, const double *y, std::string &err) {
+static int64_t graph_build_bytes(double L, double d, int nc, int C) {
+    size_t a, b, c;
+    return (int64_t)build_parts(L, d, nc, C, &a, &b, &c);
+}
+
+// Builds the records (x, t = 0, static, arrows) of every disk from positions
+// x, y (device); queued on the context's stream. An overfull cell is counted
+// in *err_dev (device).
+int graph_build(GraphCtx *g, const double *x, const double *y, unsigned long long **err_dev,
+                std::string &err) {
     GDev &s = g->s;
     const int nc = g->nc;
     const double a = g->box / nc;
@@ -2272,6 +2535,7 @@ int graph_build(GraphCtx *g, const double *x, const double *y, std::string &err)
     // with a < sqrt(2) d, at most 6 for a < 1.664 d
     const int C = a < std::sqrt(2.0) * s.d * (1.0 - 1e-9) ? 4 : 8;
     GBuild b;
+    memset(&b, 0, sizeof b);
     b.n = s.n;
     b.nc = nc;
     b.L = s.L;
@@ -2279,69 +2543,67 @@ int graph_build(GraphCtx *g, const double *x, const double *y, std::string &err)
     b.d2 = s.d * s.d;
     b.a = a;
     b.inv_a = (double)nc / s.L;
-    b.eps = std::ldexp(s.L, -30);
-    b.w = s.d / 128.0;
+    const double w = s.d / 128.0;
     b.Lf = (float)s.L;
-    b.wf = (float)b.w;
+    b.af = (float)a;
+    b.wf = (float)w;
     b.inv_wf = 1.0f / b.wf;
     b.half_f = (float)(0.5 * s.d);
-    b.d_f = (float)s.d;
-    // |dy| in FP32 is off by at most 2.5 ulp of L (three roundings of values
-    // below L, one of L itself): L * 1e-6 covers twice that, d * 1e-3 the
-    // rounding of the cut
-    b.dcut_f = (float)(s.d * (1.0 + 1e-3) + s.L * 1e-6);
-    b.nb = (int)std::ceil(s.L / b.w) + 1;
+    b.df = (float)s.d;
+    b.del = (float)std::ldexp(a, -20);
+    b.nb = (int)std::ceil(s.L / w) + 1;
     b.x = x;
     b.y = y;
     b.g = s.g;
     const size_t nslot = (size_t)nc * nc * C;
+    size_t off_bits, off_err, off_cid;
+    const size_t total = build_parts(s.L, s.d, nc, C, &off_bits, &off_err, &off_cid);
     // scratch of the build, kept by the context for the next direction change
-    void **tmp = g->build_tmp;
-    if (!tmp[0]) {
-        if (dm_alloc(&tmp[0], nslot * 4) != 0 || dm_alloc(&tmp[1], nslot * 8) != 0 ||
-            dm_alloc(&tmp[2], nslot * 8) != 0 || dm_alloc(&tmp[3], ((size_t)b.nb + 1) * 4) != 0 ||
-            dm_alloc(&tmp[4], 8) != 0 || dm_alloc(&tmp[5], nslot * 4) != 0 ||
-            dm_alloc(&tmp[6], (((size_t)b.nb + SCAN_TILE - 1) / SCAN_TILE) * 4) != 0) {
-            for (int q = 0; q < 7; ++q) {
-                dm_free(tmp[q]);
-                tmp[q] = nullptr;
-            }
+    if (!g->build_tmp) {
+        if (dm_alloc(&g->build_tmp, total) != 0) {
+            g->build_tmp = nullptr;
             err = "cudaMalloc failed (graph build)";
             return ECMC_ENOMEM;
         }
-        g->bytes += graph_build_bytes(s.L, s.d, nc, C);
+        g->bytes += (int64_t)total;
     }
-    b.cid = (uint32_t *)tmp[0];
-    b.cx = (double *)tmp[1];
-    b.cy = (double *)tmp[2];
-    b.bins = (int32_t *)tmp[3];
-    b.err = (unsigned long long *)tmp[4];
-    b.cyf = (float *)tmp[5];
+    char *tmp = (char *)g->build_tmp;
+    b.cxy = (float2 *)tmp;
+    b.cid = (uint32_t *)(tmp + off_cid);
+    b.scid = b.cid;
+    b.bits = (uint32_t *)(tmp + off_bits);
+    b.err = (unsigned long long *)(tmp + off_err);
+    *err_dev = b.err;
     cudaStream_t st = g->st;
-    cudaMemsetAsync(b.cid, 0xFF, nslot * 4, st);
-    cudaMemsetAsync(b.bins, 0, ((size_t)b.nb + 1) * 4, st);
-    cudaMemsetAsync(b.err, 0, 8, st);
+    // (all ones: NaN coordinates and EMPTY ids)
+    cudaMemsetAsync(tmp, 0xFF, off_bits, st);
+    cudaMemsetAsync(tmp + off_bits, 0, total - off_bits, st);
     const unsigned nblk = (unsigned)((s.n + 255) / 256);
-    if (C == 4)
+    const unsigned ablk = (unsigned)(((size_t)nc * nc + BUILD_CELLS - 1) / BUILD_CELLS);
+    if (C == 4) {
         k_gb_cells<4><<<nblk, 256, 0, st>>>(b);
-    else
-        k_gb_cells<8><<<nblk, 256, 0, st>>>(b);
-    {
-        const unsigned tiles = (unsigned)((b.nb + SCAN_TILE - 1) / SCAN_TILE);
-        int32_t *part = (int32_t *)tmp[6];
-        k_gb_tile_sums<<<tiles, 1024, 0, st>>>(b, part);
-        k_gb_scan_tiles<<<tiles, 1024, 0, st>>>(b, part);
-    }
-    const unsigned ablk = (unsigned)((s.n + 255) / 256);  // one thread per disk
-    if (C == 4)
         k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
-    else
+    } else {
+        k_gb_cells<8><<<nblk, 256, 0, st>>>(b);
         k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
-    unsigned long long overflow = 0;
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&overflow, b.err, 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    }
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
+        err = std::string("graph build: ") + cudaGetErrorString(e);
+        return ECMC_ECUDA;
+    }
+    (void)nslot;
+    return 0;
+}
+
+// Waits for the build and reports an overfull cell.
+static int graph_build_wait(GraphCtx *g, const unsigned long long *err_dev, std::string &err) {
+    unsigned long long overflow = 0;
+    cudaError_t e =
+        cudaMemcpyAsync(&overflow, err_dev, 8, cudaMemcpyDeviceToHost, g->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
         err = std::string("graph build: ") + cudaGetErrorString(e);
         return ECMC_ECUDA;
     }
@@ -2480,21 +2742,21 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
     cudaMemsetAsync(s.tc_cnt, 0, TC_N * 8, st);
     cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
-    rc = graph_build(g, x, s.y, err);
+    cudaMemsetAsync(s.key, 0xFF, n * 8, st);
+    cudaMemsetAsync(s.fl, 0, n * 8, st);
+    unsigned long long *overflow = nullptr;
+    rc = graph_build(g, x, s.y, &overflow, err);
+    if (!rc) {
+        k_g_init_chains<<<(unsigned)((k + 127) / 128), 128, 0, st>>>(s, active);
+        rc = graph_build_wait(g, overflow, err);
+    }
+    if (!rc && graph_max_grid() < 1) {
+        err = "cooperative launch unavailable";
+        rc = ECMC_ECUDA;
+    }
     if (rc) {
         graph_destroy(g);
         return rc;
-    }
-    k_g_init<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s);
-    k_g_init_chains<<<(unsigned)((k + 127) / 128), 128, 0, st>>>(s, active);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess || graph_max_grid() < 1) {
-        (void)cudaGetLastError();
-        err = e != cudaSuccess ? std::string("graph create: ") + cudaGetErrorString(e)
-                               : std::string("cooperative launch unavailable");
-        graph_destroy(g);
-        return ECMC_ECUDA;
     }
     *out = g;
     return 0;
@@ -2800,8 +3062,13 @@ int graph_transpose(GraphCtx *g, std::string &err) {
         return ECMC_ENOMEM;
     }
     k_g_swap_xy<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, xnew);
-    k_g_reset_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, g->st>>>(s);
-    int rc = graph_build(g, xnew, s.y, err);  // x, t = 0 and arrows for the new frame
+    // records (x, t = 0) and arrows for the new frame
+    unsigned long long *overflow = nullptr;
+    int rc = graph_build(g, xnew, s.y, &overflow, err);
+    if (rc == 0) {
+        k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, g->st>>>(s, nullptr);
+        rc = graph_build_wait(g, overflow, err);
+    }
     // (the build's kernels read xnew: done before the block goes back)
     if (cudaStreamSynchronize(g->st) != cudaSuccess && rc == 0) {
         (void)cudaGetLastError();
@@ -2847,7 +3114,7 @@ void graph_destroy(GraphCtx *g) {
     if (!g) return;
     if (cudaStreamSynchronize(g->st) != cudaSuccess) (void)cudaGetLastError();
     for (void *p : g->allocs) dm_free(p);
-    for (void *p : g->build_tmp) dm_free(p);
+    dm_free(g->build_tmp);
     dm_free(g->d_flags);
     graph_batch_free(g->launch);
     delete g;
