@@ -912,13 +912,16 @@ __global__ void __launch_bounds__(ROW_THREADS) k_skip(Dev s, int C) {
     const double lo = __longlong_as_double((long long)lo_up);
     const uint32_t o = blockIdx.x * ROW_THREADS + threadIdx.x;
     if (threadIdx.x == 0) n_occ = 0;
+    bool near = false;
     __syncthreads();
     if (o < nrow) {
         const uint32_t q = (uint32_t)R * nrow + o;
         if (s.cid[q] != EMPTY && nc >= 5)
             occ_q[atomicAdd(&n_occ, 1)] = q;
-        else
+        else {
+            near = s.cid[q] != EMPTY;
             s.cskp[q] = 0;
+        }
     }
     __syncthreads();
     if ((int)threadIdx.x < n_occ) {
@@ -942,7 +945,9 @@ __global__ void __launch_bounds__(ROW_THREADS) k_skip(Dev s, int C) {
             }
         }
         s.cskp[q] = v;
+        near = v != 3;
     }
+    if (__syncthreads_or(near) && threadIdx.x == 0) atomicAdd(s.lc + LC_NEARROW, 1ull);
 }
 
 // Skip bits for the current frame (after the cells are built or transposed).
@@ -2611,6 +2616,18 @@ struct ecmc_ctx {
     bool log_overflow = false;
     int32_t direction = 0;  // 0: +x; 1: +y (the context is stored transposed)
     GraphCtx *graph = nullptr;  // ECMC_GRAPH: the constraint-graph path holds the state
+    // cell scan: a frame in which some disk has a neighbour row in reach (or
+    // the row pass does not apply) is general: its legs run along the arrows of
+    // G(3) (graph.cu) with the flag on cells. The state is then in `arrow` from
+    // the frame's first leg on, and the cells are stale until the next frame.
+    // Such a frame in the cells' own general pass spent ~5000 cycles an event
+    // (a scan's loads, its claims' round trip and ~20 serial FP64
+    // instructions), along the arrows ~1000.
+    GraphCtx *arrow = nullptr;
+    bool general = false;
+    bool in_arrow = false;
+    bool arrow_used = false;
+    uint32_t *loc_of = nullptr;  // [n] scratch of the cell build
 };
 
 static std::string g_create_err;
@@ -2720,6 +2737,38 @@ static int pick_cells(const ecmc_params *p, int *nc_out, int *C_out) {
         return -1;
     *nc_out = nc;
     *C_out = C;
+    return 0;
+}
+
+// The cells as the arrow path takes them over.
+static GraphCells cells_of(const ecmc_ctx *ctx) {
+    const Dev &s = ctx->s;
+    GraphCells c;
+    c.nc = s.nc;
+    c.C = ctx->C;
+    c.a = s.a;
+    c.eps = s.eps;
+    c.af = s.af;
+    c.df = s.df;
+    c.epsf = s.epsf;
+    c.stop_e = s.stop_e;
+    c.colx = s.colx;
+    c.cid = s.cid;
+    c.cx = s.cx;
+    c.cy = s.cy;
+    c.ci = s.ci;
+    c.rec = s.rec;
+    c.log = s.log;
+    c.tc_cnt = s.tc_cnt;
+    return c;
+}
+
+// A general frame's state to the arrow path, before its first leg.
+static int enter_arrow(ecmc_ctx *ctx, std::string &err) {
+    if (ctx->in_arrow) return 0;
+    const int rc = graph_activate(ctx->arrow, cells_of(ctx), !ctx->arrow_used, err);
+    if (rc) return rc;
+    ctx->in_arrow = ctx->arrow_used = true;
     return 0;
 }
 
@@ -2928,6 +2977,12 @@ extern "C" int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes) {
         }
     } else {
         plan_cell_context(ctx, p, nc, C, &arr);
+        graph_bytes = graph_attach_bytes(p, nc, C);
+        if (graph_bytes < 0) {
+            ctx->pending.clear();
+            delete ctx;
+            return ECMC_ENOMEM;
+        }
     }
     // the export scratch of ecmc_positions (allocated by its first call)
     dalloc(ctx, &ctx->exp_x, (size_t)p->n);
@@ -3002,6 +3057,13 @@ extern "C" int ecmc_create(const ecmc_params *p, const double *x, const double *
         ecmc_destroy(ctx);
         return rc;
     }
+    s.colx = arr.colx;
+    s.xbound = arr.xbound;
+    rc = graph_attach(p, cells_of(ctx), ctx->stream, &ctx->arrow, g_create_err);
+    if (rc) {
+        ecmc_destroy(ctx);
+        return rc;
+    }
     double *const dx = arr.dx, *const dy = arr.dy, *const d_colx = arr.colx;
     int32_t *const dact = arr.dact;
     uint32_t *const loc_of = arr.loc_of;
@@ -3037,8 +3099,6 @@ extern "C" int ecmc_create(const ecmc_params *p, const double *x, const double *
         CU(cudaMemcpyAsync(d_colx, colx.data(), colx.size() * 8, cudaMemcpyHostToDevice, st));
         CU(cudaMemcpyAsync(d_xbound, xb.data(), xb.size() * 8, cudaMemcpyHostToDevice, st));
         // (pageable sources: the copies are done when the calls return)
-        s.colx = d_colx;
-        s.xbound = d_xbound;
     }
     // the inputs are checked on the device: the active ids here (loc_of holds
     // the ids seen until k_fill writes the slots into it), the coordinates by
@@ -3074,6 +3134,8 @@ extern "C" int ecmc_create(const ecmc_params *p, const double *x, const double *
         return ECMC_ECAPACITY;
     }
     CU(cudaMemsetAsync(s.lc, 0, LC_N * sizeof(unsigned long long), st));
+    ctx->loc_of = loc_of;
+    ctx->general = !s.rp_ok || h_lc[LC_NEARROW] != 0ull;
     *out = ctx;
     return ECMC_OK;
 }
@@ -3160,6 +3222,88 @@ static int runner_reserve(Runner &rn, int R, std::string &err) {
     return 0;
 }
 
+// Totals of a launch on the constraint-graph path into a context's counters.
+static void fold_graph_totals(ecmc_ctx *c, const GraphTotals &t, bool alone) {
+    c->legs_total += t.legs;
+    c->lifts_total += t.lifts;
+    c->conflict_legs += t.conflict_legs;
+    c->repaired += t.repaired;
+    c->continued += t.continued;
+    c->restarts += t.restarts;
+    c->blocked += t.blocked;
+    c->cwindows += t.cwindows;
+    c->horizon += t.horizon;
+    c->order_err += t.order_err;
+    c->prof.pass1_launches += t.legs;
+    c->prof.other_launches += t.legs;
+    c->prof.repair_launches += t.conflict_legs;
+    c->prof.pass1_liftings += t.p1_lifts;
+    c->prof.repair_liftings += t.repair_lifts;
+    if (alone) {
+        c->device_ms += t.ms;
+        c->prof.pass1_ms += t.pass1_ms;
+        c->prof.repair_ms += t.repair_ms;
+        c->prof.other_ms += t.other_ms;
+    }
+}
+
+// Legs a launch of the arrow path may be asked for (its member tags count
+// 2^24 claim windows); a call for more runs in several launches.
+static int32_t arrow_legs(int windows) { return std::max(1, ((1 << 24) - 1) / windows); }
+
+// The general frames of a batch of cell-scan contexts: the legs of ctxs along
+// their arrows, in one persistent launch (in several beyond arrow_legs).
+static int arrow_batch(Runner &rn, cudaStream_t st, const std::vector<ecmc_ctx *> &ctxs,
+                       int32_t max_legs, const std::vector<uint64_t> &budgets,
+                       std::vector<int64_t> &lifts, std::vector<int32_t> &legs, double *ms_out,
+                       std::string &err) {
+    const int n = (int)ctxs.size();
+    lifts.assign(n, 0);
+    legs.assign(n, 0);
+    std::vector<int> live(n);
+    unsigned long long wait_ns = BARRIER_TIMEOUT_NS;
+    for (int r = 0; r < n; ++r) {
+        live[r] = r;
+        wait_ns = std::min(wait_ns, ctxs[r]->wait_ns);
+        if (ctxs[r]->stream != st && cudaStreamSynchronize(ctxs[r]->stream) != cudaSuccess) {
+            err = "context stream";
+            return ECMC_ECUDA;
+        }
+        const int rc = enter_arrow(ctxs[r], err);
+        if (rc) return rc;
+    }
+    int32_t done = 0;
+    while (done < max_legs && !live.empty()) {
+        const int32_t now = std::min(max_legs - done, arrow_legs(ctxs[0]->s.windows));
+        std::vector<GraphCtx *> gs;
+        std::vector<uint64_t> bud;
+        for (int r : live) {
+            graph_set_leg(ctxs[r]->arrow, ctxs[r]->legs_total);
+            gs.push_back(ctxs[r]->arrow);
+            bud.push_back(budgets[r] ? budgets[r] - (uint64_t)lifts[r] : 0);
+        }
+        std::vector<GraphTotals> tots(live.size());
+        std::vector<int32_t> got(live.size(), 0);
+        double ms = 0.0;
+        const int rc = graph_batch_run(&rn.gscratch, gs.data(), (int)live.size(), now, bud.data(),
+                                       st, tots.data(), got.data(), &ms, err, wait_ns);
+        *ms_out += ms;
+        std::vector<int> next;
+        for (size_t q = 0; q < live.size(); ++q) {
+            const int r = live[q];
+            fold_graph_totals(ctxs[r], tots[q], n == 1);
+            lifts[r] += tots[q].lifts;
+            legs[r] += got[q];
+            if (got[q] == now && !(budgets[r] && (uint64_t)lifts[r] >= budgets[r]))
+                next.push_back(r);
+        }
+        if (rc) return rc;
+        live = next;
+        done += now;
+    }
+    return 0;
+}
+
 // Runs up to max_legs legs of every context in one persistent launch on
 // `st`; per-context totals are folded into each context's host counters.
 static int runner_run(Runner &rn, cudaStream_t st, ecmc_ctx *const *ctxs, int R, int32_t max_legs,
@@ -3190,29 +3334,8 @@ static int runner_run(Runner &rn, cudaStream_t st, ecmc_ctx *const *ctxs, int R,
                                         tots.data(), legs_out, &ms, err, BARRIER_TIMEOUT_NS);
         if (ms_out) *ms_out = ms;
         for (int r = 0; r < R; ++r) {
-            ecmc_ctx *c = ctxs[r];
-            const GraphTotals &t = tots[r];
-            c->legs_total += t.legs;
-            c->lifts_total += t.lifts;
-            c->conflict_legs += t.conflict_legs;
-            c->repaired += t.repaired;
-            c->continued += t.continued;
-            c->blocked += t.blocked;
-            c->cwindows += t.cwindows;
-            c->horizon += t.horizon;
-            c->order_err += t.order_err;
-            c->prof.pass1_launches += t.legs;
-            c->prof.other_launches += t.legs;
-            c->prof.repair_launches += t.conflict_legs;
-            c->prof.pass1_liftings += t.p1_lifts;
-            c->prof.repair_liftings += t.repair_lifts;
-            if (R == 1) {
-                c->device_ms += t.ms;
-                c->prof.pass1_ms += t.pass1_ms;
-                c->prof.repair_ms += t.repair_ms;
-                c->prof.other_ms += t.other_ms;
-            }
-            if (lifts_out) lifts_out[r] = t.lifts;
+            fold_graph_totals(ctxs[r], tots[r], R == 1);
+            if (lifts_out) lifts_out[r] = tots[r].lifts;
         }
         return grc;
     }
@@ -3228,6 +3351,44 @@ static int runner_run(Runner &rn, cudaStream_t st, ecmc_ctx *const *ctxs, int R,
                 err = "a context appears twice in a batch";
                 return ECMC_EINVAL;
             }
+    }
+    // general frames run along their arrows, the others in k_run: a batch of
+    // both kinds is two launches
+    std::vector<ecmc_ctx *> rows, gen;
+    std::vector<int> row_at, gen_at;
+    for (int r = 0; r < R; ++r) {
+        (ctxs[r]->general ? gen : rows).push_back(ctxs[r]);
+        (ctxs[r]->general ? gen_at : row_at).push_back(r);
+    }
+    if (!gen.empty() && max_legs > 0) {
+        std::vector<uint64_t> bud(gen.size(), 0);
+        for (size_t q = 0; q < gen.size(); ++q)
+            if (budgets) bud[q] = budgets[gen_at[q]];
+        std::vector<int64_t> lifts;
+        std::vector<int32_t> legs;
+        double ms = 0.0;
+        int grc = arrow_batch(rn, st, gen, max_legs, bud, lifts, legs, &ms, err);
+        for (size_t q = 0; q < gen.size() && q < lifts.size(); ++q) {
+            if (lifts_out) lifts_out[gen_at[q]] = lifts[q];
+            if (legs_out) legs_out[gen_at[q]] = legs[q];
+        }
+        if (!grc && !rows.empty()) {
+            std::vector<uint64_t> rbud(rows.size(), 0);
+            std::vector<int64_t> rl(rows.size(), 0);
+            std::vector<int32_t> rg(rows.size(), 0);
+            for (size_t q = 0; q < rows.size(); ++q)
+                if (budgets) rbud[q] = budgets[row_at[q]];
+            double rms = 0.0;
+            grc = runner_run(rn, st, rows.data(), (int)rows.size(), max_legs, rbud.data(), rl.data(),
+                             rg.data(), err, &rms);
+            ms += rms;
+            for (size_t q = 0; q < rows.size(); ++q) {
+                if (lifts_out) lifts_out[row_at[q]] = rl[q];
+                if (legs_out) legs_out[row_at[q]] = rg[q];
+            }
+        }
+        if (ms_out) *ms_out = ms;
+        return grc;
     }
     int rc = runner_reserve(rn, R, err);
     if (rc) return rc;
@@ -3395,27 +3556,30 @@ extern "C" int ecmc_run_to_breakpoint(ecmc_ctx *ctx, int32_t n_legs, uint64_t ev
         const int rc = graph_run(ctx->graph, n_legs, event_budget, leg_flags_out, &legs, &t, err,
                                  BARRIER_TIMEOUT_NS);
         if (legs_done) *legs_done = legs;
-        ctx->legs_total += t.legs;
-        ctx->lifts_total += t.lifts;
-        ctx->conflict_legs += t.conflict_legs;
-        ctx->repaired += t.repaired;
-        ctx->continued += t.continued;
-        ctx->restarts += t.restarts;
-        ctx->blocked += t.blocked;
-        ctx->cwindows += t.cwindows;
-        ctx->horizon += t.horizon;
-        ctx->order_err += t.order_err;
-        ctx->device_ms += t.ms;
-        ctx->prof.pass1_launches += t.legs;
-        ctx->prof.other_launches += t.legs;
-        ctx->prof.repair_launches += t.conflict_legs;
-        ctx->prof.pass1_liftings += t.p1_lifts;
-        ctx->prof.repair_liftings += t.repair_lifts;
-        ctx->prof.pass1_ms += t.pass1_ms;
-        ctx->prof.repair_ms += t.repair_ms;
-        ctx->prof.other_ms += t.other_ms;
+        fold_graph_totals(ctx, t, true);
         if (rc) return fail(ctx, rc, err);
         return ECMC_OK;
+    }
+    if (ctx->general) {
+        std::string err;
+        int rc = enter_arrow(ctx, err);
+        int32_t done = 0;
+        uint64_t lifts = 0;
+        while (!rc && done < n_legs) {
+            const int32_t now = std::min(n_legs - done, arrow_legs(ctx->s.windows));
+            GraphTotals t;
+            int32_t legs = 0;
+            graph_set_leg(ctx->arrow, ctx->legs_total);
+            rc = graph_run(ctx->arrow, now, event_budget ? event_budget - lifts : 0,
+                           leg_flags_out ? leg_flags_out + done : nullptr, &legs, &t, err,
+                           ctx->wait_ns);
+            fold_graph_totals(ctx, t, true);
+            done += legs;
+            lifts += (uint64_t)t.lifts;
+            if (legs < now || (event_budget && lifts >= event_budget)) break;
+        }
+        if (legs_done) *legs_done = done;
+        return rc ? fail(ctx, rc, err) : ECMC_OK;
     }
     ecmc_ctx *one[1] = {ctx};
     int32_t legs = 0;
@@ -3471,27 +3635,33 @@ extern "C" void ecmc_batch_destroy(ecmc_batch *b) {
     delete b;
 }
 
+// Device scratch of ecmc_positions (and of a direction change), allocated at
+// the first call and kept by the context.
+static int export_scratch(ecmc_ctx *ctx) {
+    if (ctx->exp_x) return 0;
+    const size_t n = (size_t)ctx->s.n;
+    dalloc(ctx, &ctx->exp_x, n);
+    dalloc(ctx, &ctx->exp_y, n);
+    dalloc(ctx, &ctx->exp_t, n);
+    dalloc(ctx, &ctx->exp_a, (size_t)ctx->s.k);
+    return pool_commit(ctx);
+}
+
 extern "C" int ecmc_positions(ecmc_ctx *ctx, double *x, double *y, double *t, int32_t *active) {
     if (!ctx) return ECMC_EINVAL;
     Dev &s = ctx->s;
     cudaStream_t st = ctx->stream;
     const size_t n = (size_t)s.n;
     const size_t nslot = (size_t)s.nc * s.nc * ctx->C;
-    // device scratch, allocated at the first call and kept by the context
-    if (!ctx->exp_x) {
-        dalloc(ctx, &ctx->exp_x, n);
-        dalloc(ctx, &ctx->exp_y, n);
-        dalloc(ctx, &ctx->exp_t, n);
-        dalloc(ctx, &ctx->exp_a, (size_t)s.k);
-        const int rc = pool_commit(ctx);
-        if (rc) return rc;
-    }
+    const int erc = export_scratch(ctx);
+    if (erc) return erc;
     double *dx = x ? ctx->exp_x : nullptr, *dy = y ? ctx->exp_y : nullptr;
     double *dt = t ? ctx->exp_t : nullptr;
     int32_t *da = active ? ctx->exp_a : nullptr;
-    if (ctx->graph) {
+    GraphCtx *const gr = ctx->graph ? ctx->graph : ctx->in_arrow ? ctx->arrow : nullptr;
+    if (gr) {
         double *ex = ctx->direction ? dy : dx, *ey = ctx->direction ? dx : dy;
-        if (graph_export(ctx->graph, ex, ey, dt, da) != 0)
+        if (graph_export(gr, ex, ey, dt, da) != 0)
             return fail(ctx, ECMC_ECUDA, "positions (graph)");
     } else if (x || y || t) {
         // in a transposed context the stored x is the caller's y
@@ -3501,7 +3671,7 @@ extern "C" int ecmc_positions(ecmc_ctx *ctx, double *x, double *y, double *t, in
         else
             k_export<8><<<(unsigned)((nslot + 255) / 256), 256, 0, st>>>(s, ex, ey, dt);
     }
-    if (active && !ctx->graph)
+    if (active && !gr)
         k_export_active<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, da);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && x) e = cudaMemcpyAsync(x, dx, n * 8, cudaMemcpyDeviceToHost, st);
@@ -3528,7 +3698,20 @@ extern "C" int ecmc_set_direction(ecmc_ctx *ctx, int32_t direction) {
     Dev &s = ctx->s;
     cudaStream_t st = ctx->stream;
     const int64_t ncell = (int64_t)s.nc * s.nc;
-    if (ctx->C == 4) {
+    if (ctx->in_arrow) {
+        // the cells are built again from the arrow path's state
+        const int rc = export_scratch(ctx);
+        if (rc) return rc;
+        const double *ynew = nullptr;
+        const int32_t *act = nullptr;
+        graph_swapped(ctx->arrow, ctx->exp_x, &ynew, &act);
+        cudaMemsetAsync(s.cid, 0xFF, (size_t)ncell * ctx->C * sizeof(uint32_t), st);
+        if (ctx->C == 4)
+            launch_cells<4>(s, ctx->exp_x, ynew, ctx->loc_of, nullptr, st);
+        else
+            launch_cells<8>(s, ctx->exp_x, ynew, ctx->loc_of, nullptr, st);
+        k_init_chains<<<(unsigned)((s.k + 255) / 256), 256, 0, st>>>(s, act, ctx->loc_of);
+    } else if (ctx->C == 4) {
         k_transpose<4><<<(unsigned)((ncell + 255) / 256), 256, 0, st>>>(s);
         k_transpose_chains<4><<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s);
     } else {
@@ -3536,9 +3719,19 @@ extern "C" int ecmc_set_direction(ecmc_ctx *ctx, int32_t direction) {
         k_transpose_chains<8><<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s);
     }
     launch_skip(s, ctx->C, st);  // rows are the old columns
+    unsigned long long near[2] = {0ull, 0ull};  // LC_NEARROW, LC_ERR_CAP
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(near, s.lc + LC_NEARROW, 8, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(near + 1, s.lc + LC_ERR_CAP, 8, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(s.lc, 0, LC_N * sizeof(unsigned long long), st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(ctx, ECMC_ECUDA, std::string("set_direction: ") + cudaGetErrorString(e));
+    ctx->in_arrow = false;
+    ctx->general = !s.rp_ok || near[0] != 0ull;
+    if (near[1]) return fail(ctx, ECMC_ECAPACITY, "set_direction: a cell overflowed");
     ctx->direction = direction;
     return ECMC_OK;
 }
@@ -3561,7 +3754,8 @@ extern "C" int ecmc_stats(ecmc_ctx *ctx, ecmc_stats_t *out) {
     out->row_windows = ctx->row_windows;
     out->blocked_chains = ctx->blocked;
     out->conflict_windows = ctx->cwindows;
-    out->device_bytes = (ctx->graph ? graph_device_bytes(ctx->graph) : 0) + ctx->device_bytes;
+    out->device_bytes = (ctx->graph ? graph_device_bytes(ctx->graph) : 0) +
+                        (ctx->arrow ? graph_device_bytes(ctx->arrow) : 0) + ctx->device_bytes;
     out->horizon_asserts = ctx->horizon;
     out->order_errors = ctx->order_err;
     out->device_ms = ctx->device_ms;
@@ -3617,6 +3811,7 @@ extern "C" void ecmc_destroy(ecmc_ctx *ctx) {
     // returning; this one makes sure before its blocks go to the cache)
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) (void)cudaGetLastError();
     graph_destroy(ctx->graph);
+    graph_destroy(ctx->arrow);
     runner_free(ctx->run);
     dm_free(ctx->d_flags);
     for (void *p : ctx->allocs) dm_free(p);

@@ -71,7 +71,9 @@ struct __align__(16) GSpec {
     int32_t n, touch;     // events; disks touched
     int32_t end, partner; // SP_*; the chain met
     double tc, D;
-    uint32_t ci, pad[3];
+    uint32_t ci;
+    int32_t cut;          // events that may be published (strict: a disk in reach)
+    int32_t pad[2];
 };
 
 struct GDev {
@@ -85,7 +87,19 @@ struct GDev {
     // disks of its run (entry e of chain c at e * k + c)
     unsigned long long *key;
     uint32_t *path;        // [(cap + 2) * k]
-    unsigned long long *fl;  // flag words, epoch << 32 | chain + 1: per disk read
+    unsigned long long *fl;  // flag words, epoch << 32 | chain + 1: per disk read, or
+                             // per cell scanned
+    // a cell-scan context's frame (cells != 0: its flag is on cells): each
+    // disk's cell, the left edges of the columns, the stop rule, and per entry
+    // of path what its step's scan needs -- the active disk's x and the least
+    // of D and its best time of flight, and its cell
+    int cells;
+    double inv_a;
+    uint32_t *ecell;      // [n]
+    const double *colx;   // [nc]
+    StopK sk;
+    double2 *pxt;         // [(cap + 2) * k]
+    uint32_t *pcell;      // [(cap + 2) * k]
     uint32_t epoch0;       // epoch of the launch's first pass, less one
     GSpec *sp;             // [k] the run alone of each chain, for the resolve
     uint32_t stamp0;       // stamp of the launch's first leg, less one
@@ -157,8 +171,8 @@ __device__ __forceinline__ double shfl_f64(double v, int src) {
 
 // ------------------------------------------------------------ graph build
 
-// Inputs and scratch of a build: a cell list of the disks (slots fill from
-// the first), their FP32 coordinates per slot relative to the cell's corner (an
+// Inputs and scratch of a build: a cell list of the disks (in any of a cell's
+// slots), their FP32 coordinates per slot relative to the cell's corner (an
 // error of 1e-7 d whatever the box), and one bit per y bin of width d/128 that
 // holds a disk. The disks come by id (x, y, placed by k_gb_cells)
 // or, sx != null, from the slots of a cell-scan context.
@@ -176,6 +190,8 @@ struct GBuild {
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
     uint32_t *bits;        // [nb / 32 + 1]
     GDisk *g;
+    uint32_t *ecell;          // [n] or null: each disk's cell
+    double *yout;             // [n] or null: each disk's y
     unsigned long long *err;  // cell overflow count
 };
 
@@ -496,8 +512,7 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
 #pragma unroll
             for (int sl = 0; sl < C; ++sl) {
                 const float2 v = cell.v[sl];
-                if (!(v.x >= 0.f)) break;  // a cell's slots fill from the first
-                if (c0 + sl == loc) continue;
+                if (!(v.x >= 0.f) || c0 + sl == loc) continue;
                 float lo, hi;
                 const int kc = corridor_f(b, vi.x, vi.y, rr, m, v, lo, hi);
                 if (kc < 0) continue;
@@ -566,8 +581,7 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
 #pragma unroll
                         for (int sl = 0; sl < C; ++sl) {
                             const float2 v = cell.v[sl];
-                            if (!(v.x >= 0.f)) break;
-                            if (c0 + sl == sloc) continue;
+                            if (!(v.x >= 0.f) || c0 + sl == sloc) continue;
                             float lo, hi;
                             const int kc = corridor_f(b, sx, sy, rr, mm, v, lo, hi);
                             if (kc == 3) dbt = true;
@@ -638,6 +652,8 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
             }
         }
         if (has) {
+            if (b.ecell) b.ecell[i] = loc / C;
+            if (b.yout) b.yout[i] = yi;
             ulonglong2 *r = reinterpret_cast<ulonglong2 *>(b.g + i);
             r[0] = make_ulonglong2(dbits(xi), 0ull);
             r[1] = make_ulonglong2((unsigned long long)OWN_STATIC | ((unsigned long long)id[0] << 32),
@@ -886,16 +902,24 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
     GEvs E;
     E.i = NONE;
     E.x = E.t = E.D = E.tau = E.tj = 0.0;
+    double cur = 0.0;  // the last step, evaluated but not taken: its scan's limit
     int n = 0, nf = 0, end = SP_PAUSE;  // nf: events written out
+    int cut = 0x7FFFFFFF;
     uint32_t partner = NONE;
     // events nf .. n - 1 to memory, with the touched disks and their keys
     auto flush = [&](bool lift) {
         if (n == nf) return;
         const GFlush f = g_flush(s, c, nr0, (uint32_t)nr0, nf, n, E, i, xi, ti, D, lift);
         if (f.has) {
+            const int e = nf + ((lane - nf) & 31);
             if (f.j != NONE) {
-                *gpath_at(s, c, nf + ((lane - nf) & 31) + 1) = f.j;
+                *gpath_at(s, c, e + 1) = f.j;
                 red_min_u64(key + f.j, g_key(f.t, c));
+            }
+            if (s.cells) {
+                const size_t at = (size_t)e * (size_t)s.k + (size_t)c;
+                s.pxt[at] = make_double2(E.x, E.tau);
+                s.pcell[at] = s.ecell[E.i];
             }
             if (strict) {
 #pragma unroll
@@ -981,9 +1005,20 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
             const bool stop = nsc && (strict ? hv || dbits(tau) < dbits(D)
                                              : dbits(tau) <= bt && dbits(tau) < dbits(D));
             const unsigned sb = __ballot_sync(FULL, stop);
-            if (sb) {
+            if (sb && cut == 0x7FFFFFFF) {
                 partner = __shfl_sync(FULL, own, __ffs(sb) - 1) & OWN_CHAIN;
+                // (with the flag on cells a run cut by a disk beyond its winner
+                // goes on for its cells, unpublished from here)
+                cut = n;
+                const bool near = stop && dbits(tau) <= bt && dbits(tau) < dbits(D);
+                if (!s.cells || __any_sync(FULL, near)) {
+                    end = SP_NONSTATIC;
+                    cur = bt < dbits(D) ? __longlong_as_double((long long)bt) : D;
+                    break;
+                }
+            } else if (sb && __any_sync(FULL, stop && dbits(tau) <= bt && dbits(tau) < dbits(D))) {
                 end = SP_NONSTATIC;
+                cur = bt < dbits(D) ? __longlong_as_double((long long)bt) : D;
                 break;
             }
             const double tj = shfl_f64(rt, wl);
@@ -994,9 +1029,13 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         const double T = __dadd_rn(ti, ts);
         if (n >= room) {  // out of records: the repair goes on from here, or reports it
             end = SP_LIMIT;
+            cur = ts;
             break;
         }
-        if (bounded && !(dbits(T) < dbits(tend))) break;  // pauses at the window end
+        if (bounded && !(dbits(T) < dbits(tend))) {  // pauses at the window end
+            cur = ts;
+            break;
+        }
         if (lane == (n & 31)) {
             E.i = i;
             E.x = xi;
@@ -1025,6 +1064,11 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
     // (the reads of a step that was evaluated but not taken)
     if (strict && end != SP_STALL && lane < 3 && tid != NONE) red_min_u64(key + tid, g_key(ti, c));
     flush(end != SP_STALL);
+    if (s.cells && end != SP_STALL && lane == 1) {
+        const size_t at = (size_t)n * (size_t)s.k + (size_t)c;
+        s.pxt[at] = make_double2(xi, cur);
+        s.pcell[at] = s.ecell[i];
+    }
     if (lane == 0) {
         GSpec r;
         r.n = n;
@@ -1034,10 +1078,17 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         r.tc = ti;
         r.D = D;
         r.ci = i;
-        r.pad[0] = r.pad[1] = r.pad[2] = 0u;
+        r.cut = cut;
+        r.pad[0] = r.pad[1] = 0;
         s.sp[c] = r;
     }
     __syncwarp();
+}
+
+// The cell of disk id after a move along x to x: its row stays.
+__device__ __forceinline__ void g_set_cell(const GDev &s, uint32_t id, double x, uint32_t old) {
+    const uint32_t nc = (uint32_t)s.nc;
+    s.ecell[id] = old / nc * nc + (uint32_t)cell_coord(x, s.inv_a, s.nc);
 }
 
 // Touch keys of chain c back to empty (one warp): every disk its last run
@@ -1059,24 +1110,64 @@ __device__ __forceinline__ void g_reset_keys(const GDev &s, int c, int lane) {
 
 // The conflict flag (one warp, after the pass): chain c puts its word (epoch,
 // chain) into s.fl for every disk its run alone read, its start disk and the
-// arrow targets of every disk that was active. Two chains read one disk iff
-// one of them is handed the other's word of this epoch; the epoch makes
-// clearing unnecessary. Nothing waits for the result before the leg's totals,
-// so the warps without a component do this while the others repair.
+// arrow targets of every disk that was active -- or, for a cell-scan context,
+// for every cell its scans covered. Two chains read one disk (scanned one
+// cell) iff one of them is handed the other's word of this epoch; the epoch
+// makes clearing unnecessary. Nothing waits for the result before the leg's
+// totals, so the warps without a component do this while the others repair.
+//
+// The scan of a step covers rows cy - 1 .. cy + 1 and columns cx, cx + 1, ...
+// up to the first m >= 1 whose threshold exceeds min(D, best) + eps. The
+// cell scan forms best column by column; the columns up to the winner's have
+// thresholds within the winner's time of flight (less a rounding far below
+// eps), so the final best gives the same columns.
 __device__ __noinline__ void g_flag_chain(const GDev &s, int c, uint32_t epoch, int lane) {
     const int nt = s.sp[c].touch;
     const unsigned long long tag = ((unsigned long long)epoch << 32) | ((unsigned)c + 1u);
     bool met = false;
+    auto foreign = [&](unsigned long long w) {
+        return (uint32_t)(w >> 32) == epoch && (uint32_t)w != (uint32_t)tag;
+    };
     for (int e = lane; e < nt; e += 32) {
-        const uint32_t id = *gpath_at(s, c, e);
-        const GDisk &r = s.g[id];
-        uint32_t a[4] = {r.a[0], r.a[1], r.a[2], e == 0 ? id : NONE};
-        unsigned long long w[4];
+        const size_t at = (size_t)e * (size_t)s.k + (size_t)c;
+        if (!s.cells) {
+            const uint32_t id = s.path[at];
+            const GDisk &r = s.g[id];
+            uint32_t a[4] = {r.a[0], r.a[1], r.a[2], e == 0 ? id : NONE};
+            unsigned long long w[4];
 #pragma unroll
-        for (int z = 0; z < 4; ++z) w[z] = a[z] != NONE ? atomicExch(s.fl + a[z], tag) : 0ull;
+            for (int z = 0; z < 4; ++z) w[z] = a[z] != NONE ? atomicExch(s.fl + a[z], tag) : 0ull;
 #pragma unroll
-        for (int z = 0; z < 4; ++z)
-            met |= (uint32_t)(w[z] >> 32) == epoch && (uint32_t)w[z] != (uint32_t)tag;
+            for (int z = 0; z < 4; ++z) met |= foreign(w[z]);
+            continue;
+        }
+        const double2 xt = s.pxt[at];
+        const uint32_t cell = s.pcell[at];
+        const int nc = s.nc, cy = (int)(cell / (uint32_t)nc), cx = (int)(cell % (uint32_t)nc);
+        const double fx = __dsub_rn(xt.x, s.colx[cx]);
+        const float fxf = d2f_trunc(fx), lim_f = __fadd_rn(d2f_trunc(xt.y), s.sk.epsf);
+        const int rdn = cy == 0 ? nc - 1 : cy - 1, rup = cy == nc - 1 ? 0 : cy + 1;
+        unsigned long long *const f0 = s.fl + (size_t)rdn * (size_t)nc,
+                                  *const f1 = s.fl + (size_t)cy * (size_t)nc,
+                                  *const f2 = s.fl + (size_t)rup * (size_t)nc;
+        bool more = true;
+        for (int m0 = 0; more && m0 < nc; m0 += 3) {
+            unsigned long long w[9];
+#pragma unroll
+            for (int z = 0; z < 3; ++z) {
+                const int m = m0 + z;
+                if (m >= nc ||
+                    (m > 0 && more && beyond_k(s.sk, m, fx, fxf, lim_f, dbits(xt.y))))
+                    more = false;
+                int col = cx + m;
+                if (col >= nc) col -= nc;
+                w[3 * z] = more ? atomicExch(f0 + col, tag) : 0ull;
+                w[3 * z + 1] = more ? atomicExch(f1 + col, tag) : 0ull;
+                w[3 * z + 2] = more ? atomicExch(f2 + col, tag) : 0ull;
+            }
+#pragma unroll
+            for (int z = 0; z < 9; ++z) met |= foreign(w[z]);
+        }
     }
     if (__any_sync(FULL, met) && lane == 0) {
         atomicAdd(s.lc + LC_WEAK, 1ull);
@@ -1153,6 +1244,11 @@ __device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, ui
             sfail = first < n ? first : n;
         }
     }
+    if (sp.cut <= sfail) {
+        sfail = sp.cut;
+        lost = true;
+        holder = (uint32_t)sp.partner;
+    }
     // publish records 0 .. sfail - 1; the lane of the last one keeps its time
     // and remaining length for the chain's state
     int lifts = 0;
@@ -1169,6 +1265,9 @@ __device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, ui
             *reinterpret_cast<ulonglong2 *>(&r.x) = make_ulonglong2(u3.y, u2.y);
             r.own = rj != NONE ? s.stamp : (OWN_STALLED | (uint32_t)c);
             r.claim = tag;
+            if (s.cells)
+                g_set_cell(s, (uint32_t)u0.x, __longlong_as_double((long long)u3.y),
+                           s.pcell[(size_t)e * (size_t)s.k + (size_t)c]);
             lt = __longlong_as_double((long long)u2.y);
             ld = __longlong_as_double((long long)u4.y);
         }
@@ -1371,6 +1470,7 @@ __device__ void graph_apply(const GDev &s, int c, uint32_t i, double xi, double 
         rj.t = tnew;
         ri.t = tnew;
         ri.x = xnew;
+        if (s.cells) g_set_cell(s, i, xnew, s.ecell[i]);
         ri.own = s.stamp;                              // i static
         u.j = j;
         u.tj_old = tj;
@@ -1383,6 +1483,7 @@ __device__ void graph_apply(const GDev &s, int c, uint32_t i, double xi, double 
         const double tnew = __dadd_rn(ti, D);         // t_i reaches the breakpoint
         const double xnew = wrap_add(xi, D, s.L);     // i moves by D
         ri.x = xnew;
+        if (s.cells) g_set_cell(s, i, xnew, s.ecell[i]);
         ri.t = tnew;
         ri.own = OWN_STALLED | (uint32_t)c;           // stalled
         u.j = NONE;
@@ -1435,6 +1536,7 @@ __device__ __noinline__ void g_log_chain(const GDev &s, int c, int32_t leg, int 
 __device__ void g_undo(const GDev &s, int c, const GEv &u) {
     GDisk &ri = s.g[u.i];
     ri.x = u.x_old;
+    if (s.cells) g_set_cell(s, u.i, u.x_old, s.ecell[u.i]);
     ri.t = u.ti_old;
     ri.own = OWN_ACTIVE | (uint32_t)c;
     if (u.j != NONE) {
@@ -1673,6 +1775,7 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
                 *reinterpret_cast<ulonglong2 *>(&g[E.i].x) =
                     make_ulonglong2(dbits(f.xn), dbits(f.t));
                 g[E.i].own = f.j != NONE ? stamp : (OWN_STALLED | (uint32_t)c);
+                if (s.cells) g_set_cell(s, E.i, f.xn, s.ecell[E.i]);
             }
             nf = n;
         };
@@ -2469,6 +2572,8 @@ struct GraphCtx {
     int64_t log_legs = 0;  // legs logged so far (leg index of the log)
     GBatchScratch *launch = nullptr;  // launch tables of graph_run
     void *build_tmp = nullptr;        // scratch of graph_build
+    float2 *slot_xy = nullptr;        // scratch of graph_activate
+    uint32_t *slot_bits = nullptr;
     std::vector<std::pair<void **, size_t>> pending;
     int64_t bytes = 0;  // device memory held
 };
@@ -2526,36 +2631,41 @@ static int64_t graph_build_bytes(double L, double d, int nc, int C) {
 // Builds the records (x, t = 0, static, arrows) of every disk from positions
 // x, y (device); queued on the context's stream. An overfull cell is counted
 // in *err_dev (device).
-int graph_build(GraphCtx *g, const double *x, const double *y, unsigned long long **err_dev,
-                std::string &err) {
-    GDev &s = g->s;
-    const int nc = g->nc;
-    const double a = g->box / nc;
-    // slots per cell: at most 4 centres at mutual distance >= d fit in a cell
-    // with a < sqrt(2) d, at most 6 for a < 1.664 d
-    const int C = a < std::sqrt(2.0) * s.d * (1.0 - 1e-9) ? 4 : 8;
+// The constants of a build.
+static GBuild build_params(const GraphCtx *g) {
+    const GDev &s = g->s;
     GBuild b;
     memset(&b, 0, sizeof b);
     b.n = s.n;
-    b.nc = nc;
+    b.nc = g->nc;
     b.L = s.L;
     b.d = s.d;
     b.d2 = s.d * s.d;
-    b.a = a;
-    b.inv_a = (double)nc / s.L;
+    b.a = g->box / g->nc;
+    b.inv_a = (double)g->nc / s.L;
     const double w = s.d / 128.0;
     b.Lf = (float)s.L;
-    b.af = (float)a;
+    b.af = (float)b.a;
     b.wf = (float)w;
     b.inv_wf = 1.0f / b.wf;
     b.half_f = (float)(0.5 * s.d);
     b.df = (float)s.d;
-    b.del = (float)std::ldexp(a, -20);
+    b.del = (float)std::ldexp(b.a, -20);
     b.nb = (int)std::ceil(s.L / w) + 1;
+    b.g = s.g;
+    return b;
+}
+
+static int graph_build(GraphCtx *g, const double *x, const double *y, unsigned long long **err_dev,
+                       std::string &err) {
+    GDev &s = g->s;
+    const int nc = g->nc;
+    // slots per cell: at most 4 centres at mutual distance >= d fit in a cell
+    // with a < sqrt(2) d, at most 6 for a < 1.664 d
+    const int C = g->box / nc < std::sqrt(2.0) * s.d * (1.0 - 1e-9) ? 4 : 8;
+    GBuild b = build_params(g);
     b.x = x;
     b.y = y;
-    b.g = s.g;
-    const size_t nslot = (size_t)nc * nc * C;
     size_t off_bits, off_err, off_cid;
     const size_t total = build_parts(s.L, s.d, nc, C, &off_bits, &off_err, &off_cid);
     // scratch of the build, kept by the context for the next direction change
@@ -2592,8 +2702,12 @@ int graph_build(GraphCtx *g, const double *x, const double *y, unsigned long lon
         err = std::string("graph build: ") + cudaGetErrorString(e);
         return ECMC_ECUDA;
     }
-    (void)nslot;
     return 0;
+}
+
+// Flag words of a context: one per disk, or per cell.
+static size_t flag_words(const GDev &s) {
+    return s.cells ? (size_t)s.nc * (size_t)s.nc : (size_t)s.n;
 }
 
 // Waits for the build and reports an overfull cell.
@@ -2618,7 +2732,9 @@ static int graph_build_wait(GraphCtx *g, const unsigned long long *err_dev, std:
 
 // The device arrays of a graph context, requested from the pool (galloc):
 // graph_create commits them, graph_plan_bytes only adds them up.
-static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
+// slots > 0: for a cell-scan context of that many slots (graph_attach), whose
+// records and log are shared; the scratch of its build is planned with it.
+static int graph_plan(GraphCtx *g, const ecmc_params *p, size_t slots, std::string &err) {
     GDev &s = g->s;
     const size_t n = (size_t)p->n, k = (size_t)p->n_chains;
     int rc = 0;
@@ -2628,7 +2744,15 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
     chk(galloc(g, &s.g, n, err));
     chk(galloc(g, &s.y, n, err));
     chk(galloc(g, &s.key, n, err));
-    chk(galloc(g, &s.fl, n, err));
+    s.cells = slots > 0;
+    chk(galloc(g, &s.fl, slots ? (size_t)g->nc * (size_t)g->nc : n, err));
+    if (slots) {
+        chk(galloc(g, &s.ecell, n, err));
+        chk(galloc(g, &s.pxt, k * ((size_t)s.cap + 2), err));
+        chk(galloc(g, &s.pcell, k * ((size_t)s.cap + 2), err));
+        chk(galloc(g, &g->slot_xy, slots, err));
+        chk(galloc(g, &g->slot_bits, (size_t)std::ceil(p->box / (p->d / 128.0)) / 32 + 2, err));
+    }
     chk(galloc(g, &s.path, k * ((size_t)s.cap + 2), err));
     chk(galloc(g, &s.sp, k, err));
     chk(galloc(g, &s.ci, k, err));
@@ -2642,7 +2766,7 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
     chk(galloc(g, &s.memb, k, err));
     chk(galloc(g, &s.tstar, 1, err));
     s.restart = (p->flags & ECMC_RESTART) ? 1 : 0;
-    chk(galloc(g, &s.rec, k * (size_t)s.cap, err));
+    if (!slots) chk(galloc(g, &s.rec, k * (size_t)s.cap, err));
     chk(galloc(g, &s.ev_T, k, err));
     chk(galloc(g, &s.ev_tau, k, err));
     chk(galloc(g, &s.ev_xj, k, err));
@@ -2663,9 +2787,9 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, std::string &err) {
     chk(galloc(g, &s.pcnt, k, err));
     chk(galloc(g, &s.ctl, CTL_N, err));
     chk(galloc(g, &s.lc, 2 * LC_N, err));
-    chk(galloc(g, &s.tc_cnt, TC_N, err));
     chk(galloc(g, &s.dbg, 16, err));
-    if (s.log_on) chk(galloc(g, &s.log, (size_t)s.log_cap, err));
+    if (!slots) chk(galloc(g, &s.tc_cnt, TC_N, err));
+    if (!slots && s.log_on) chk(galloc(g, &s.log, (size_t)s.log_cap, err));
     return rc;
 }
 
@@ -2695,6 +2819,40 @@ static int graph_max_grid() {
     return grid;
 }
 
+// A context's fields that follow from its parameters.
+static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
+    g->nc = nc;
+    g->box = p->box;
+    GDev &s = g->s;
+    memset(&s, 0, sizeof s);
+    s.n = p->n;
+    s.k = p->n_chains;
+    s.nc = nc;
+    s.cap = p->undo_cap > 0 ? p->undo_cap : 1024;
+    s.windows = p->windows > 0 ? p->windows : 1;
+    s.L = p->box;
+    s.d = p->d;
+    s.ell = p->ell;
+    s.inv_a = (double)nc / p->box;
+    s.strict = (s.windows > 1 || (p->flags & ECMC_RESTART)) ? 1 : 0;
+    s.log_on = (p->flags & ECMC_LOG_LIFTINGS) ? 1 : 0;
+    s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
+}
+
+// Counters, run results and touch keys of a new context.
+static void graph_clear(GraphCtx *g) {
+    const GDev &s = g->s;
+    const size_t n = (size_t)s.n, k = (size_t)s.k;
+    cudaStream_t st = g->st;
+    cudaMemsetAsync(s.nrec, 0, k * 4, st);
+    cudaMemsetAsync(s.sp, 0, k * sizeof(GSpec), st);
+    cudaMemsetAsync(s.pcnt, 0, k * 4, st);
+    cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
+    cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
+    cudaMemsetAsync(s.key, 0xFF, n * 8, st);
+    cudaMemsetAsync(s.fl, 0, flag_words(s) * 8, st);
+}
+
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
                  const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err) {
     *out = nullptr;
@@ -2707,47 +2865,27 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
         err = "host allocation";
         return ECMC_ENOMEM;
     }
-    g->nc = nc;
-    g->box = p->box;
     g->st = st;
+    graph_params(g, p, nc);
     GDev &s = g->s;
-    memset(&s, 0, sizeof s);
-    s.n = p->n;
-    s.k = p->n_chains;
-    s.nc = nc;
-    s.cap = p->undo_cap > 0 ? p->undo_cap : 1024;
-    s.windows = p->windows > 0 ? p->windows : 1;
-    s.L = p->box;
-    s.d = p->d;
-    s.ell = p->ell;
-    s.strict = (s.windows > 1 || (p->flags & ECMC_RESTART)) ? 1 : 0;
-    s.log_on = (p->flags & ECMC_LOG_LIFTINGS) ? 1 : 0;
-    s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
-    const size_t n = (size_t)p->n, k = (size_t)p->n_chains;
+    const size_t n = (size_t)p->n;
     int rc = 0;
     auto chk = [&](int r) {
         if (r && !rc) rc = r;
     };
-    chk(graph_plan(g, p, err));
+    chk(graph_plan(g, p, 0, err));
     chk(gcommit(g, err));
     if (rc) {
         graph_destroy(g);
         return rc;
     }
     cudaMemcpyAsync(s.y, y, n * 8, cudaMemcpyDeviceToDevice, st);
-    cudaMemsetAsync(s.nrec, 0, k * 4, st);
-    cudaMemsetAsync(s.sp, 0, k * sizeof(GSpec), st);
-    cudaMemsetAsync(s.pcnt, 0, k * 4, st);
-    cudaMemsetAsync(s.memb, 0xFF, k * 8, st);
-    cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
     cudaMemsetAsync(s.tc_cnt, 0, TC_N * 8, st);
-    cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
-    cudaMemsetAsync(s.key, 0xFF, n * 8, st);
-    cudaMemsetAsync(s.fl, 0, n * 8, st);
+    graph_clear(g);
     unsigned long long *overflow = nullptr;
     rc = graph_build(g, x, s.y, &overflow, err);
     if (!rc) {
-        k_g_init_chains<<<(unsigned)((k + 127) / 128), 128, 0, st>>>(s, active);
+        k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active);
         rc = graph_build_wait(g, overflow, err);
     }
     if (!rc && graph_max_grid() < 1) {
@@ -2760,6 +2898,100 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     }
     *out = g;
     return 0;
+}
+
+int graph_attach(const ecmc_params *p, const GraphCells &c, cudaStream_t st, GraphCtx **out,
+                 std::string &err) {
+    *out = nullptr;
+    GraphCtx *g = new (std::nothrow) GraphCtx();
+    if (!g) {
+        err = "host allocation";
+        return ECMC_ENOMEM;
+    }
+    g->st = st;
+    graph_params(g, p, c.nc);
+    int rc = graph_plan(g, p, (size_t)c.nc * c.nc * c.C, err);
+    if (!rc) rc = gcommit(g, err);
+    if (rc) {
+        graph_destroy(g);
+        return rc;
+    }
+    GDev &s = g->s;
+    s.rec = (GEv *)c.rec;
+    s.log = c.log;
+    s.tc_cnt = c.tc_cnt;
+    s.colx = c.colx;
+    s.sk.af = c.af;
+    s.sk.df = c.df;
+    s.sk.epsf = c.epsf;
+    s.sk.stop_e = c.stop_e;
+    s.sk.a = c.a;
+    s.sk.d = p->d;
+    s.sk.eps = c.eps;
+    *out = g;
+    return 0;
+}
+
+int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &err) {
+    GDev &s = g->s;
+    cudaStream_t st = g->st;
+    if (first) {
+        graph_clear(g);
+        if (graph_max_grid() < 1) {
+            err = "cooperative launch unavailable";
+            return ECMC_ECUDA;
+        }
+    }
+    GBuild b = build_params(g);
+    b.sx = c.cx;
+    b.sy = c.cy;
+    b.scid = c.cid;
+    b.cxy = g->slot_xy;
+    b.bits = g->slot_bits;
+    b.ecell = s.ecell;
+    b.yout = s.y;
+    const uint32_t nslot = (uint32_t)((size_t)c.nc * c.nc * c.C);
+    cudaMemsetAsync(b.bits, 0, ((size_t)b.nb / 32 + 1) * 4, st);
+    const unsigned ablk = (unsigned)(((size_t)c.nc * c.nc + BUILD_CELLS - 1) / BUILD_CELLS);
+    const unsigned sblk = (unsigned)(((size_t)nslot + 255) / 256);
+    if (c.C == 4) {
+        k_gb_slots<4><<<sblk, 256, 0, st>>>(b, nslot);
+        k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
+    } else {
+        k_gb_slots<8><<<sblk, 256, 0, st>>>(b, nslot);
+        k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
+    }
+    k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, (const int32_t *)c.ci);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        err = std::string("graph build: ") + cudaGetErrorString(e);
+        return ECMC_ECUDA;
+    }
+    return 0;
+}
+
+void graph_swapped(GraphCtx *g, double *xnew, const double **ynew, const int32_t **active) {
+    const GDev &s = g->s;
+    k_g_swap_xy<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, xnew);
+    *ynew = s.y;
+    *active = (const int32_t *)s.ci;
+}
+
+void graph_set_leg(GraphCtx *g, int64_t legs) { g->log_legs = legs; }
+
+int64_t graph_attach_bytes(const ecmc_params *p, int nc, int C) {
+    GraphCtx *g = new (std::nothrow) GraphCtx();
+    if (!g) return -1;
+    graph_params(g, p, nc);
+    std::string err;
+    int64_t total = -1;
+    if (graph_plan(g, p, (size_t)nc * nc * C, err) == 0) {
+        total = 0;
+        for (auto &r : g->pending) total += (int64_t)((r.second + 255) & ~(size_t)255);
+    }
+    g->pending.clear();
+    delete g;
+    return total;
 }
 
 // Launch tables of the persistent kernel: one device block [reps | chain_base
@@ -2830,7 +3062,6 @@ __global__ void k_g_clear_epochs(GDev s) {
     r.claim = 0ull;
     r.t = g_time(r.own, r.t, s.stamp0);
     if (g_static(r.own)) r.own = dbits(r.t) != 0ull ? 1u : 0u;
-    s.fl[q] = 0ull;
 }
 
 int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int32_t max_legs,
@@ -2894,6 +3125,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         if (g->s.epoch0 > 0xC0000000u || g->s.stamp0 > 0x3E000000u) {
             k_g_clear_epochs<<<(unsigned)((g->s.n + 255) / 256), 256, 0, st>>>(g->s);
             cu(cudaGetLastError(), "epochs");
+            cu(cudaMemsetAsync(g->s.fl, 0, flag_words(g->s) * 8, st), "epochs");
             g->s.epoch0 = 0;
             g->s.stamp0 = 1;  // (the last leg's times, for ecmc_positions)
         }
@@ -3125,14 +3357,10 @@ int64_t graph_device_bytes(const GraphCtx *g) { return g ? g->bytes : 0; }
 int64_t graph_plan_bytes(const ecmc_params *p, int nc) {
     GraphCtx *g = new (std::nothrow) GraphCtx();
     if (!g) return -1;
-    GDev &s = g->s;
-    memset(&s, 0, sizeof s);
-    s.cap = p->undo_cap > 0 ? p->undo_cap : 1024;
-    s.log_on = (p->flags & ECMC_LOG_LIFTINGS) ? 1 : 0;
-    s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
+    graph_params(g, p, nc);
     std::string err;
     int64_t total = -1;
-    if (graph_plan(g, p, err) == 0) {
+    if (graph_plan(g, p, 0, err) == 0) {
         total = 0;
         for (auto &r : g->pending) total += (int64_t)((r.second + 255) & ~(size_t)255);
         const double a = p->box / nc;
