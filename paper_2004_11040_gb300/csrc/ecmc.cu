@@ -2977,9 +2977,8 @@ extern "C" int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes) {
         }
     } else {
         plan_cell_context(ctx, p, nc, C, &arr);
-        graph_bytes = graph_attach_bytes(p, nc, C);
-        if (graph_bytes < 0) {
-            ctx->pending.clear();
+        ctx->arrow = graph_attach(p, nc, C, nullptr, ctx->pending);
+        if (!ctx->arrow) {
             delete ctx;
             return ECMC_ENOMEM;
         }
@@ -2996,6 +2995,7 @@ extern "C" int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes) {
     ctx->exp_y = nullptr;
     ctx->exp_t = nullptr;
     ctx->exp_a = nullptr;
+    graph_destroy(ctx->arrow);
     delete ctx;
     *bytes = total;
     return ECMC_OK;
@@ -3051,6 +3051,11 @@ extern "C" int ecmc_create(const ecmc_params *p, const double *x, const double *
     const size_t nslot = ncell * C;
     const size_t n = (size_t)p->n, k = (size_t)p->n_chains;
     const bool dev_in = (p->flags & ECMC_INPUT_DEVICE) != 0;
+    ctx->arrow = graph_attach(p, nc, C, ctx->stream, ctx->pending);
+    if (!ctx->arrow) {
+        ctx->pending.clear();
+        chk(fail(ctx, ECMC_ENOMEM, "host allocation"));
+    }
     chk(pool_commit(ctx));
     if (rc) {
         g_create_err = ctx->err;
@@ -3059,11 +3064,6 @@ extern "C" int ecmc_create(const ecmc_params *p, const double *x, const double *
     }
     s.colx = arr.colx;
     s.xbound = arr.xbound;
-    rc = graph_attach(p, cells_of(ctx), ctx->stream, &ctx->arrow, g_create_err);
-    if (rc) {
-        ecmc_destroy(ctx);
-        return rc;
-    }
     double *const dx = arr.dx, *const dy = arr.dy, *const d_colx = arr.colx;
     int32_t *const dact = arr.dact;
     uint32_t *const loc_of = arr.loc_of;

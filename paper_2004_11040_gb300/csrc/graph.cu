@@ -1952,6 +1952,219 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
     }
 }
 
+// Replay of a component with at most 10 members (one warp), rolled back to Ts:
+// lane 3e + p holds target p of member e's active disk -- its record, as the
+// replay has changed it -- so every member's next event is computed at once,
+// and an event costs one round of loads, for the targets of the disk it
+// activated (~1500 cycles; with the pending events in memory, one member per
+// thread and three targets one after another it was ~10700, and the replays
+// were most of a leg on dense boxes). The claims as in graph_step.
+constexpr int SMALL_REPLAY = 10;
+
+__device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, int m, int root,
+                                            uint64_t tag, uint32_t epoch, int round, double Ts,
+                                            double tend) {
+    const int lane = threadIdx.x & 31;
+    const int e = lane / 3, p = lane - 3 * e, base = 3 * e;
+    const bool has = e < m;
+    const double L = s.L;
+    GDisk *const g = s.g;
+    const uint32_t stamp = s.stamp;
+    const bool bounded = dbits(tend) != INF_BITS;
+    const int c = has ? mem[e] : 0x7FFFFFFF;
+    const unsigned long long ct = ((unsigned long long)epoch << 32) | ((unsigned)c + 1u);
+    uint32_t i = NONE, tid = NONE;
+    double xi = 0.0, ti = 0.0, D = 0.0, tb = 0.0;
+    int32_t nrec = 0, nl = 0;
+    bool run = false;
+    if (has) {
+        i = s.ci[c];
+        ti = s.tc[c];
+        D = s.D[c];
+        nrec = s.nrec[c];
+        run = s.status[c] == ST_RUNNING;
+    }
+    if (run) {
+        xi = g[i].x;
+        tid = g[i].a[p];
+        tb = g[i].b[p];
+    }
+    // this lane's target: place, time, owner and its own arrows
+    double rx = 0.0, rt = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0;
+    uint32_t own = 0u, a0 = NONE, a1 = NONE, a2 = NONE;
+    int met = -1;
+    // loads and claims the targets of the lanes with mine (their active disk too
+    // with self); true if one is held by the other side
+    auto take = [&](bool mine, bool self) -> bool {
+        uint32_t h = 0u, h2 = 0u;
+        if (mine && tid != NONE) {
+            h = g_claim(s, tid, ct);
+            const GDisk &r = g[tid];
+            rx = r.x;
+            rt = r.t;
+            own = r.own;
+            a0 = r.a[0];
+            a1 = r.a[1];
+            a2 = r.a[2];
+            b0 = r.b[0];
+            b1 = r.b[1];
+            b2 = r.b[2];
+        }
+        if (mine && self && p == 0) h2 = g_claim(s, i, ct);
+        const uint32_t own_w = (uint32_t)c + 1u;
+        uint32_t bad = 0u;
+        if (h != 0u && h != own_w && !holder_ours(s, (int)h - 1, root, tag, false)) bad = h;
+        if (h2 != 0u && h2 != own_w && !holder_ours(s, (int)h2 - 1, root, tag, false)) bad = h2;
+        const unsigned bm = __ballot_sync(FULL, bad != 0u);
+        if (bm) met = (int)__shfl_sync(FULL, bad, __ffs(bm) - 1) - 1;
+        return bm != 0u;
+    };
+    bool abort = take(run, true);
+    double now = Ts;
+    uint32_t cnt = 0;
+    while (!abort) {
+        // every member's next event (Sec. 2.2): the least (tau, j) of its
+        // static targets, one lap on where the target came after it had passed
+        const bool stc = run && tid != NONE && g_static(own);
+        double dx = __dsub_rn(rx, xi);
+        const bool neg = stc && __double_as_longlong(dx) < 0;
+        if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
+        double tau = __dsub_rn(dx, tb);
+        if (__double_as_longlong(tau) < 0) tau = 0.0;
+        const bool tnz = stc && own == stamp && dbits(rt) != 0ull;
+        if (__any_sync(FULL, tnz)) {
+            if (tnz && dbits(g_add(ti, tau)) < dbits(rt)) tau = g_add(tau, L);
+        }
+        const unsigned long long tk = stc ? dbits(tau) : INF_BITS;
+        const int l0 = min(base, 29);
+        const unsigned long long t0 = shfl_u64(tk, l0), t1 = shfl_u64(tk, l0 + 1),
+                                 t2 = shfl_u64(tk, l0 + 2);
+        const uint32_t j0 = __shfl_sync(FULL, tid, l0), j1 = __shfl_sync(FULL, tid, l0 + 1),
+                       j2 = __shfl_sync(FULL, tid, l0 + 2);
+        unsigned long long bt = t0;
+        uint32_t bj = j0;
+        int w = 0;
+        if (t1 < bt || (t1 == bt && j1 < bj)) {
+            bt = t1;
+            bj = j1;
+            w = 1;
+        }
+        if (t2 < bt || (t2 == bt && j2 < bj)) {
+            bt = t2;
+            bj = j2;
+            w = 2;
+        }
+        const bool lift = bt < dbits(D);
+        const double ts = lift ? __longlong_as_double((long long)bt) : D;
+        const double T = __dadd_rn(ti, ts);
+        // the earliest (T, chain)
+        const unsigned hi = run ? (unsigned)(dbits(T) >> 32) : ~0u;
+        const unsigned mh = __reduce_min_sync(FULL, hi);
+        if (mh == ~0u) break;  // every member has stalled
+        const unsigned lo = hi == mh ? (unsigned)dbits(T) : ~0u;
+        const unsigned ml = __reduce_min_sync(FULL, lo);
+        const bool first = hi == mh && lo == ml;
+        const unsigned mc = __reduce_min_sync(FULL, first ? (unsigned)c : ~0u);
+        const int src = __ffs(__ballot_sync(FULL, first && (unsigned)c == mc)) - 1;
+        const double Tn = shfl_f64(T, src);
+        if (bounded && !(dbits(Tn) < dbits(tend))) break;  // the rest lies in a later window
+        if (dbits(Tn) < dbits(now) && lane == 0) {
+            atomicAdd(s.lc + LC_ORDER, 1ull);
+            gdiag(s, 2, round, mc, Tn, now, Ts, m);
+        }
+        now = Tn;
+        const int ce = (int)mc;
+        const uint32_t ie = __shfl_sync(FULL, i, src);
+        const bool le = __shfl_sync(FULL, (int)lift, src) != 0;
+        const uint32_t je = le ? __shfl_sync(FULL, bj, src) : NONE;
+        const int we = __shfl_sync(FULL, w, src), ls = src / 3 * 3 + we;
+        const int32_t ne = __shfl_sync(FULL, nrec, src);
+        if (ne >= s.cap) {  // out of records: reported by the host
+            if (lane == 0) atomicAdd(s.lc + LC_ERR_REC, 1ull);
+            abort = true;
+            met = -1;
+            break;
+        }
+        const double xe = shfl_f64(xi, src), te = shfl_f64(ti, src), De = shfl_f64(D, src);
+        const double tse = shfl_f64(ts, src), xj = shfl_f64(rx, ls);
+        const double tj = shfl_f64(own == stamp ? rt : 0.0, ls);
+        double xn = __dadd_rn(xe, tse);
+        if (dbits(xn) >= dbits(L)) xn = g_sub(xn, L);
+        const double Dn = __dsub_rn(De, tse);
+        const uint32_t own_i = le ? stamp : (OWN_STALLED | (uint32_t)ce);
+        if (lane < 5) {
+            unsigned long long u0, u1;
+            if (lane == 0) {
+                u0 = (unsigned long long)ie | ((unsigned long long)je << 32);
+                u1 = (unsigned long long)(((uint32_t)round << 24) | cnt);
+            } else if (lane == 1) {
+                u0 = dbits(xe);
+                u1 = dbits(te);
+            } else if (lane == 2) {
+                u0 = le ? dbits(tj) : 0ull;
+                u1 = dbits(Tn);
+            } else if (lane == 3) {
+                u0 = dbits(tse);
+                u1 = dbits(xn);
+            } else {
+                u0 = le ? dbits(xj) : 0ull;
+                u1 = le ? dbits(Dn) : 0ull;
+            }
+            reinterpret_cast<ulonglong2 *>(grec_at(s, ce, ne))[lane] = make_ulonglong2(u0, u1);
+        } else if (lane == 5) {
+            *reinterpret_cast<ulonglong2 *>(&g[ie].x) = make_ulonglong2(dbits(xn), dbits(Tn));
+            g[ie].own = own_i;
+            if (s.cells) g_set_cell(s, ie, xn, s.ecell[ie]);
+        } else if (le && lane == 6) {
+            g[je].own = OWN_ACTIVE | (uint32_t)ce;
+            g[je].t = Tn;
+        }
+        ++cnt;
+        // the copies of the two disks in the other lanes
+        if (tid == ie) {
+            rx = xn;
+            rt = Tn;
+            own = own_i;
+        }
+        if (le && tid == je) {
+            rt = Tn;
+            own = OWN_ACTIVE | (uint32_t)ce;
+        }
+        const uint32_t q0 = __shfl_sync(FULL, a0, ls), q1 = __shfl_sync(FULL, a1, ls),
+                       q2 = __shfl_sync(FULL, a2, ls);
+        const double d0 = shfl_f64(b0, ls), d1 = shfl_f64(b1, ls), d2 = shfl_f64(b2, ls);
+        __syncwarp();
+        const bool acts = has && c == ce;
+        if (acts) {
+            ++nrec;
+            ti = Tn;
+            if (le) {
+                ++nl;
+                i = je;
+                xi = xj;
+                D = Dn;
+                tid = p == 0 ? q0 : p == 1 ? q1 : q2;
+                tb = p == 0 ? d0 : p == 1 ? d1 : d2;
+            } else {
+                D = 0.0;
+                run = false;
+            }
+        }
+        if (le && take(acts, false)) abort = true;
+    }
+    if (has && p == 0) {
+        s.status[c] = run ? ST_RUNNING : ST_STALLED;
+        s.ci[c] = i;
+        s.tc[c] = ti;
+        s.D[c] = D;
+        s.nrec[c] = nrec;
+        s.nlift[c] += nl;
+        if (nl) atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
+    }
+    __syncwarp();
+    g_finish(s, mem, m, root, abort, met, now);
+}
+
 // Component q of this round (one warp): roll its members back to T*, then
 // replay them in global event-time order (Alg. 2) up to the window's end.
 // Members are spread over the lanes (member e on lane e mod 32); after each
@@ -1993,6 +2206,10 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int q, int round,
     g_rollback(s, mem, m, Ts);
     for (int e = lane; e < m; e += 32) g_resume(s, mem[e]);
     __syncwarp();
+    if (m <= SMALL_REPLAY) {
+        g_replay_small(s, mem, m, root, tag, epoch, round, Ts, tend);
+        return;
+    }
     bool abort = false;
     int met = -1;
     for (int e = lane; e < m; e += 32)
@@ -2900,22 +3117,20 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     return 0;
 }
 
-int graph_attach(const ecmc_params *p, const GraphCells &c, cudaStream_t st, GraphCtx **out,
-                 std::string &err) {
-    *out = nullptr;
+GraphCtx *graph_attach(const ecmc_params *p, int nc, int C, cudaStream_t st,
+                       std::vector<std::pair<void **, size_t>> &pending) {
     GraphCtx *g = new (std::nothrow) GraphCtx();
-    if (!g) {
-        err = "host allocation";
-        return ECMC_ENOMEM;
-    }
+    if (!g) return nullptr;
     g->st = st;
-    graph_params(g, p, c.nc);
-    int rc = graph_plan(g, p, (size_t)c.nc * c.nc * c.C, err);
-    if (!rc) rc = gcommit(g, err);
-    if (rc) {
-        graph_destroy(g);
-        return rc;
-    }
+    graph_params(g, p, nc);
+    std::string err;
+    (void)graph_plan(g, p, (size_t)nc * nc * C, err);
+    pending.insert(pending.end(), g->pending.begin(), g->pending.end());
+    g->pending.clear();
+    return g;
+}
+
+static void graph_bind(GraphCtx *g, const GraphCells &c) {
     GDev &s = g->s;
     s.rec = (GEv *)c.rec;
     s.log = c.log;
@@ -2926,16 +3141,15 @@ int graph_attach(const ecmc_params *p, const GraphCells &c, cudaStream_t st, Gra
     s.sk.epsf = c.epsf;
     s.sk.stop_e = c.stop_e;
     s.sk.a = c.a;
-    s.sk.d = p->d;
+    s.sk.d = s.d;
     s.sk.eps = c.eps;
-    *out = g;
-    return 0;
 }
 
 int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &err) {
     GDev &s = g->s;
     cudaStream_t st = g->st;
     if (first) {
+        graph_bind(g, c);
         graph_clear(g);
         if (graph_max_grid() < 1) {
             err = "cooperative launch unavailable";
@@ -2978,21 +3192,6 @@ void graph_swapped(GraphCtx *g, double *xnew, const double **ynew, const int32_t
 }
 
 void graph_set_leg(GraphCtx *g, int64_t legs) { g->log_legs = legs; }
-
-int64_t graph_attach_bytes(const ecmc_params *p, int nc, int C) {
-    GraphCtx *g = new (std::nothrow) GraphCtx();
-    if (!g) return -1;
-    graph_params(g, p, nc);
-    std::string err;
-    int64_t total = -1;
-    if (graph_plan(g, p, (size_t)nc * nc * C, err) == 0) {
-        total = 0;
-        for (auto &r : g->pending) total += (int64_t)((r.second + 255) & ~(size_t)255);
-    }
-    g->pending.clear();
-    delete g;
-    return total;
-}
 
 // Launch tables of the persistent kernel: one device block [reps | chain_base
 // | comp_base | ctl | bar | g | phase] (256-byte aligned parts), uploaded
@@ -3344,7 +3543,10 @@ int graph_liftings(GraphCtx *g, ecmc_lift_t *buf, int64_t cap, int64_t *n_out,
 
 void graph_destroy(GraphCtx *g) {
     if (!g) return;
-    if (cudaStreamSynchronize(g->st) != cudaSuccess) (void)cudaGetLastError();
+    // (a context of the cells' path holds no block of its own: ecmc_destroy has
+    // waited for its work)
+    if (!g->allocs.empty() && cudaStreamSynchronize(g->st) != cudaSuccess)
+        (void)cudaGetLastError();
     for (void *p : g->allocs) dm_free(p);
     dm_free(g->build_tmp);
     dm_free(g->d_flags);

@@ -6,6 +6,8 @@
 
 #include <cstdint>
 #include <string>
+#include <utility>
+#include <vector>
 
 #include "ecmc.h"
 
@@ -50,9 +52,9 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
                     unsigned long long wait_ns);
 void graph_batch_free(GBatchScratch *scratch);
 // A cell-scan context's general frames (rows within reach of each other) run
-// on this path too, with the conflict flag on cells. graph_attach makes the
-// context's arrays beside the cells (its records and log are the cells'
-// own); graph_activate builds the records and arrows from the cells as they
+// on this path too, with the conflict flag on cells. graph_attach adds the
+// path's arrays to the context's requests (records and log are the cells'
+// own; null: host allocation); graph_activate builds the records and arrows from the cells as they
 // stand at a breakpoint (queued on the stream; first: the first time of the
 // context), after which the state is here: graph_swapped gives x and y
 // exchanged (x into xnew) and the active disks, to build cells from again.
@@ -68,14 +70,12 @@ struct GraphCells {
     ecmc_lift_t *log;
     unsigned long long *tc_cnt;
 };
-int graph_attach(const ecmc_params *p, const GraphCells &c, cudaStream_t st, GraphCtx **out,
-                 std::string &err);
+GraphCtx *graph_attach(const ecmc_params *p, int nc, int C, cudaStream_t st,
+                       std::vector<std::pair<void **, size_t>> &pending);
 int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &err);
 void graph_swapped(GraphCtx *g, double *xnew, const double **ynew, const int32_t **active);
 // Legs run before (leg index of the lifting log).
 void graph_set_leg(GraphCtx *g, int64_t legs);
-// What graph_attach would hold.
-int64_t graph_attach_bytes(const ecmc_params *p, int nc, int C);
 // Device memory held by the context (bytes).
 int64_t graph_device_bytes(const GraphCtx *g);
 // What graph_create(p, nc, ...) would hold, without allocating (-1: error).
