@@ -89,13 +89,12 @@ struct GDev {
     uint32_t *path;        // [(cap + 2) * k]
     unsigned long long *fl;  // flag words, epoch << 32 | chain + 1: per disk read, or
                              // per cell scanned
-    // a cell-scan context's frame (cells != 0: its flag is on cells): each
-    // disk's cell, the left edges of the columns, the stop rule, and per entry
-    // of path what its step's scan needs -- the active disk's x and the least
-    // of D and its best time of flight, and its cell
+    // a cell-scan context's frame (cells != 0: its flag is on cells): the left
+    // edges of the columns, the stop rule, and per entry of path what its
+    // step's scan needs -- the active disk's x and the least of D and its best
+    // time of flight, and its cell
     int cells;
     double inv_a;
-    uint32_t *ecell;      // [n]
     const double *colx;   // [nc]
     StopK sk;
     double2 *pxt;         // [(cap + 2) * k]
@@ -153,6 +152,19 @@ __device__ void gdiag(const GDev &s, int kind, double a, double b, double c, dou
     s.dbg[6] = f;
 }
 
+__device__ __forceinline__ int cell_coord(double v, double inv_a, int nc) {
+    int c = __double2int_rz(__dmul_rn(v, inv_a));
+    if (c >= nc) c = nc - 1;
+    if (c < 0) c = 0;
+    return c;
+}
+
+// A disk's cell, as the cell scan keeps it.
+__device__ __forceinline__ uint32_t cell_of(const GDev &s, double x, double y) {
+    return (uint32_t)cell_coord(y, s.inv_a, s.nc) * (uint32_t)s.nc +
+           (uint32_t)cell_coord(x, s.inv_a, s.nc);
+}
+
 __device__ __forceinline__ double wrap_add(double x, double dx, double L) {
     double r = __dadd_rn(x, dx);
     if (dbits(r) >= dbits(L)) r = __dsub_rn(r, L);  // r >= 0
@@ -190,17 +202,9 @@ struct GBuild {
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
     uint32_t *bits;        // [nb / 32 + 1]
     GDisk *g;
-    uint32_t *ecell;          // [n] or null: each disk's cell
     double *yout;             // [n] or null: each disk's y
     unsigned long long *err;  // cell overflow count
 };
-
-__device__ __forceinline__ int cell_coord(double v, double inv_a, int nc) {
-    int c = __double2int_rz(__dmul_rn(v, inv_a));
-    if (c >= nc) c = nc - 1;
-    if (c < 0) c = 0;
-    return c;
-}
 
 // A monotone map of y to its bin, the same wherever bins are set or asked for.
 __device__ __forceinline__ int y_bin(const GBuild &b, float y) {
@@ -652,7 +656,6 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
             }
         }
         if (has) {
-            if (b.ecell) b.ecell[i] = loc / C;
             if (b.yout) b.yout[i] = yi;
             ulonglong2 *r = reinterpret_cast<ulonglong2 *>(b.g + i);
             r[0] = make_ulonglong2(dbits(xi), 0ull);
@@ -919,7 +922,7 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
             if (s.cells) {
                 const size_t at = (size_t)e * (size_t)s.k + (size_t)c;
                 s.pxt[at] = make_double2(E.x, E.tau);
-                s.pcell[at] = s.ecell[E.i];
+                s.pcell[at] = cell_of(s, E.x, s.y[E.i]);
             }
             if (strict) {
 #pragma unroll
@@ -1067,7 +1070,7 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
     if (s.cells && end != SP_STALL && lane == 1) {
         const size_t at = (size_t)n * (size_t)s.k + (size_t)c;
         s.pxt[at] = make_double2(xi, cur);
-        s.pcell[at] = s.ecell[i];
+        s.pcell[at] = cell_of(s, xi, s.y[i]);
     }
     if (lane == 0) {
         GSpec r;
@@ -1083,12 +1086,6 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         s.sp[c] = r;
     }
     __syncwarp();
-}
-
-// The cell of disk id after a move along x to x: its row stays.
-__device__ __forceinline__ void g_set_cell(const GDev &s, uint32_t id, double x, uint32_t old) {
-    const uint32_t nc = (uint32_t)s.nc;
-    s.ecell[id] = old / nc * nc + (uint32_t)cell_coord(x, s.inv_a, s.nc);
 }
 
 // Touch keys of chain c back to empty (one warp): every disk its last run
@@ -1265,9 +1262,6 @@ __device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, ui
             *reinterpret_cast<ulonglong2 *>(&r.x) = make_ulonglong2(u3.y, u2.y);
             r.own = rj != NONE ? s.stamp : (OWN_STALLED | (uint32_t)c);
             r.claim = tag;
-            if (s.cells)
-                g_set_cell(s, (uint32_t)u0.x, __longlong_as_double((long long)u3.y),
-                           s.pcell[(size_t)e * (size_t)s.k + (size_t)c]);
             lt = __longlong_as_double((long long)u2.y);
             ld = __longlong_as_double((long long)u4.y);
         }
@@ -1470,7 +1464,6 @@ __device__ void graph_apply(const GDev &s, int c, uint32_t i, double xi, double 
         rj.t = tnew;
         ri.t = tnew;
         ri.x = xnew;
-        if (s.cells) g_set_cell(s, i, xnew, s.ecell[i]);
         ri.own = s.stamp;                              // i static
         u.j = j;
         u.tj_old = tj;
@@ -1483,7 +1476,6 @@ __device__ void graph_apply(const GDev &s, int c, uint32_t i, double xi, double 
         const double tnew = __dadd_rn(ti, D);         // t_i reaches the breakpoint
         const double xnew = wrap_add(xi, D, s.L);     // i moves by D
         ri.x = xnew;
-        if (s.cells) g_set_cell(s, i, xnew, s.ecell[i]);
         ri.t = tnew;
         ri.own = OWN_STALLED | (uint32_t)c;           // stalled
         u.j = NONE;
@@ -1536,7 +1528,6 @@ __device__ __noinline__ void g_log_chain(const GDev &s, int c, int32_t leg, int 
 __device__ void g_undo(const GDev &s, int c, const GEv &u) {
     GDisk &ri = s.g[u.i];
     ri.x = u.x_old;
-    if (s.cells) g_set_cell(s, u.i, u.x_old, s.ecell[u.i]);
     ri.t = u.ti_old;
     ri.own = OWN_ACTIVE | (uint32_t)c;
     if (u.j != NONE) {
@@ -1554,39 +1545,69 @@ __device__ void g_undo(const GDev &s, int c, const GEv &u) {
 // and are undone one at a time in descending seq; beneath them, the records
 // of the window's parallel pass touch disks held by their own chain only,
 // so each member undoes its own in parallel.
-__device__ void g_rollback(const GDev &s, const int32_t *mem, int m, double Ts) {
+__device__ __noinline__ void g_rollback(const GDev &s, const int32_t *mem, int m, double Ts) {
     const int lane = threadIdx.x & 31;
-    for (;;) {
-        uint32_t bseq = 0;
-        int bmem = -1;
-        for (int e = lane; e < m; e += 32) {
-            const int c = mem[e];
-            const int32_t nr = s.nrec[c];
-            if (nr == 0) continue;
-            const GEv &u = *grec_at(s, c, nr - 1);
-            if (!(u.t >= Ts) || u.seq < REPAIR_SEQ0) continue;
-            if (bmem < 0 || u.seq > bseq || (u.seq == bseq && e < bmem)) {
-                bseq = u.seq;
-                bmem = e;
+    if (m <= 32) {
+        // a member per lane, its last record in registers: an undo waits for
+        // the member's next record at most
+        const int c = lane < m ? mem[lane] : 0;
+        int32_t nr = lane < m ? s.nrec[c] : 0;
+        GEv u;
+        bool top = false;  // u is a repair record to undo
+        auto load = [&]() {
+            top = false;
+            if (nr > 0) {
+                u = *grec_at(s, c, nr - 1);
+                top = u.t >= Ts && u.seq >= REPAIR_SEQ0;
             }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const uint32_t s2 = __shfl_xor_sync(FULL, bseq, o);
-            const int m2 = __shfl_xor_sync(FULL, bmem, o);
-            if (m2 >= 0 && (bmem < 0 || s2 > bseq || (s2 == bseq && m2 < bmem))) {
-                bseq = s2;
-                bmem = m2;
+        };
+        load();
+        for (;;) {
+            const unsigned best = __reduce_max_sync(FULL, top ? u.seq : 0u);
+            if (best == 0u) break;
+            const unsigned bm = __ballot_sync(FULL, top && u.seq == best);
+            if (lane == __ffs(bm) - 1) {
+                g_undo(s, c, u);
+                --nr;
+                load();
             }
+            __syncwarp();
         }
-        if (bmem < 0) break;
-        if (lane == 0) {
-            const int c = mem[bmem];
-            const int32_t nr = s.nrec[c];
-            g_undo(s, c, *grec_at(s, c, nr - 1));
-            s.nrec[c] = nr - 1;
-        }
+        if (lane < m) s.nrec[c] = nr;
         __syncwarp();
+    } else {
+        for (;;) {
+            uint32_t bseq = 0;
+            int bmem = -1;
+            for (int e = lane; e < m; e += 32) {
+                const int c = mem[e];
+                const int32_t nr = s.nrec[c];
+                if (nr == 0) continue;
+                const GEv &u = *grec_at(s, c, nr - 1);
+                if (!(u.t >= Ts) || u.seq < REPAIR_SEQ0) continue;
+                if (bmem < 0 || u.seq > bseq || (u.seq == bseq && e < bmem)) {
+                    bseq = u.seq;
+                    bmem = e;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const uint32_t s2 = __shfl_xor_sync(FULL, bseq, o);
+                const int m2 = __shfl_xor_sync(FULL, bmem, o);
+                if (m2 >= 0 && (bmem < 0 || s2 > bseq || (s2 == bseq && m2 < bmem))) {
+                    bseq = s2;
+                    bmem = m2;
+                }
+            }
+            if (bmem < 0) break;
+            if (lane == 0) {
+                const int c = mem[bmem];
+                const int32_t nr = s.nrec[c];
+                g_undo(s, c, *grec_at(s, c, nr - 1));
+                s.nrec[c] = nr - 1;
+            }
+            __syncwarp();
+        }
     }
     for (int e = lane; e < m; e += 32) {
         const int c = mem[e];
@@ -1775,7 +1796,6 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
                 *reinterpret_cast<ulonglong2 *>(&g[E.i].x) =
                     make_ulonglong2(dbits(f.xn), dbits(f.t));
                 g[E.i].own = f.j != NONE ? stamp : (OWN_STALLED | (uint32_t)c);
-                if (s.cells) g_set_cell(s, E.i, f.xn, s.ecell[E.i]);
             }
             nf = n;
         };
@@ -1956,9 +1976,10 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
 // lane 3e + p holds target p of member e's active disk -- its record, as the
 // replay has changed it -- so every member's next event is computed at once,
 // and an event costs one round of loads, for the targets of the disk it
-// activated (~1500 cycles; with the pending events in memory, one member per
-// thread and three targets one after another it was ~10700, and the replays
-// were most of a leg on dense boxes). The claims as in graph_step.
+// activated (with the pending events in memory, one member per thread and
+// three targets one after another it took ~10700 cycles, and the replays were
+// most of a leg on dense boxes). The claims are those of graph_step, checked
+// one event later.
 constexpr int SMALL_REPLAY = 10;
 
 __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, int m, int root,
@@ -1993,35 +2014,55 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
     double rx = 0.0, rt = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0;
     uint32_t own = 0u, a0 = NONE, a1 = NONE, a2 = NONE;
     int met = -1;
-    // loads and claims the targets of the lanes with mine (their active disk too
-    // with self); true if one is held by the other side
-    auto take = [&](bool mine, bool self) -> bool {
-        uint32_t h = 0u, h2 = 0u;
+    // The claims asked for and not checked yet: the holder that a record's word
+    // of this pass names, or what the exchange for a free disk found.
+    uint32_t held = 0u, held_i = 0u;
+    unsigned long long cas = 0ull;
+    auto take = [&](bool mine) {
+        held = 0u;
+        cas = 0ull;
         if (mine && tid != NONE) {
-            h = g_claim(s, tid, ct);
-            const GDisk &r = g[tid];
-            rx = r.x;
-            rt = r.t;
-            own = r.own;
-            a0 = r.a[0];
-            a1 = r.a[1];
-            a2 = r.a[2];
-            b0 = r.b[0];
-            b1 = r.b[1];
-            b2 = r.b[2];
+            const ulonglong2 *r = reinterpret_cast<const ulonglong2 *>(g + tid);
+            const ulonglong2 u0 = __ldcg(r), u1 = __ldcg(r + 1), u2 = __ldcg(r + 2),
+                             u3 = __ldcg(r + 3);
+            rx = __longlong_as_double((long long)u0.x);
+            rt = __longlong_as_double((long long)u0.y);
+            own = (uint32_t)u1.x;
+            a0 = (uint32_t)(u1.x >> 32);
+            a1 = (uint32_t)u1.y;
+            a2 = (uint32_t)(u1.y >> 32);
+            b0 = __longlong_as_double((long long)u2.y);
+            b1 = __longlong_as_double((long long)u3.x);
+            b2 = __longlong_as_double((long long)u3.y);
+            held = g_holder(u2.x, ct);
+            if (held == 0u) cas = atomicCAS(&g[tid].claim, u2.x, ct);
         }
-        if (mine && self && p == 0) h2 = g_claim(s, i, ct);
-        const uint32_t own_w = (uint32_t)c + 1u;
-        uint32_t bad = 0u;
-        if (h != 0u && h != own_w && !holder_ours(s, (int)h - 1, root, tag, false)) bad = h;
-        if (h2 != 0u && h2 != own_w && !holder_ours(s, (int)h2 - 1, root, tag, false)) bad = h2;
-        const unsigned bm = __ballot_sync(FULL, bad != 0u);
-        if (bm) met = (int)__shfl_sync(FULL, bad, __ffs(bm) - 1) - 1;
+    };
+    // true if a disk taken is held by a chain that is no member
+    auto conflict = [&]() -> bool {
+        const uint32_t h = held ? held : g_holder(cas, ct);
+        const uint32_t me = (uint32_t)c + 1u;
+        bool ask = h != 0u && h != me, ask_i = held_i != 0u && held_i != me;
+        if (!__any_sync(FULL, ask || ask_i)) return false;
+        for (int z = 0; z < m; ++z) {
+            const uint32_t cz = (uint32_t)__shfl_sync(FULL, c, 3 * z) + 1u;
+            ask = ask && h != cz;
+            ask_i = ask_i && held_i != cz;
+        }
+        const unsigned bm = __ballot_sync(FULL, ask || ask_i);
+        if (bm) met = (int)__shfl_sync(FULL, ask ? h : held_i, __ffs(bm) - 1) - 1;
         return bm != 0u;
     };
-    bool abort = take(run, true);
+    if (run && p == 0) held_i = g_claim(s, i, ct);
+    take(run);
+    bool abort = false;
+    double taken = Ts;  // time of the event after which the claims were asked for,
+    int taker = -1;     // and the chain that asked
     double now = Ts;
     uint32_t cnt = 0;
+    if (conflict()) abort = true;
+    held = held_i = 0u;
+    cas = 0ull;
     while (!abort) {
         // every member's next event (Sec. 2.2): the least (tau, j) of its
         // static targets, one lap on where the target came after it had passed
@@ -2085,6 +2126,18 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
             met = -1;
             break;
         }
+        // a disk is written only once the claims on it stand: those asked for
+        // after the last event are checked here if they are this member's, else
+        // below, when this event has overlapped their round trip
+        if (ce == taker) {
+            if (conflict()) {
+                abort = true;
+                now = taken;
+                break;
+            }
+            held = 0u;
+            cas = 0ull;
+        }
         const double xe = shfl_f64(xi, src), te = shfl_f64(ti, src), De = shfl_f64(D, src);
         const double tse = shfl_f64(ts, src), xj = shfl_f64(rx, ls);
         const double tj = shfl_f64(own == stamp ? rt : 0.0, ls);
@@ -2114,7 +2167,6 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
         } else if (lane == 5) {
             *reinterpret_cast<ulonglong2 *>(&g[ie].x) = make_ulonglong2(dbits(xn), dbits(Tn));
             g[ie].own = own_i;
-            if (s.cells) g_set_cell(s, ie, xn, s.ecell[ie]);
         } else if (le && lane == 6) {
             g[je].own = OWN_ACTIVE | (uint32_t)ce;
             g[je].t = Tn;
@@ -2133,8 +2185,14 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
         const uint32_t q0 = __shfl_sync(FULL, a0, ls), q1 = __shfl_sync(FULL, a1, ls),
                        q2 = __shfl_sync(FULL, a2, ls);
         const double d0 = shfl_f64(b0, ls), d1 = shfl_f64(b1, ls), d2 = shfl_f64(b2, ls);
-        __syncwarp();
         const bool acts = has && c == ce;
+        __syncwarp();
+        // (if one failed, what was read then is no basis for anything from the
+        // time of that event on)
+        if (conflict()) {
+            abort = true;
+            now = taken;
+        }
         if (acts) {
             ++nrec;
             ti = Tn;
@@ -2150,7 +2208,13 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
                 run = false;
             }
         }
-        if (le && take(acts, false)) abort = true;
+        take(le && !abort && acts);
+        taken = Tn;
+        taker = ce;
+    }
+    if (!abort && conflict()) {
+        abort = true;
+        now = taken;
     }
     if (has && p == 0) {
         s.status[c] = run ? ST_RUNNING : ST_STALLED;
@@ -2964,7 +3028,6 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, size_t slots, std::stri
     s.cells = slots > 0;
     chk(galloc(g, &s.fl, slots ? (size_t)g->nc * (size_t)g->nc : n, err));
     if (slots) {
-        chk(galloc(g, &s.ecell, n, err));
         chk(galloc(g, &s.pxt, k * ((size_t)s.cap + 2), err));
         chk(galloc(g, &s.pcell, k * ((size_t)s.cap + 2), err));
         chk(galloc(g, &g->slot_xy, slots, err));
@@ -3162,7 +3225,6 @@ int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &er
     b.scid = c.cid;
     b.cxy = g->slot_xy;
     b.bits = g->slot_bits;
-    b.ecell = s.ecell;
     b.yout = s.y;
     const uint32_t nslot = (uint32_t)((size_t)c.nc * c.nc * c.C);
     cudaMemsetAsync(b.bits, 0, ((size_t)b.nb / 32 + 1) * 4, st);
