@@ -35,7 +35,8 @@ enum { LC_BLOCKED = 0, LC_LIFTS, LC_HORIZON, LC_ERR_CAP, LC_ERR_REC, LC_ORDER, L
        LC_ROWWIN,  // claim windows run by the row pass (cell scan)
        LC_WWEAK,   // chains whose claim sets met on a weak claim, this window
        LC_BADXY, LC_BADID,  // inputs out of range (creation only)
-       LC_NEARROW,  // blocks with a disk whose neighbour rows are in reach (k_skip)
+       LC_NEARROW,  // rows that are no rings, at least (k_skip)
+       LC_RINGLAP,  // chains whose run came round its ring (a frame of rings)
        LC_N };
 enum { CTL_NCOMP = 0, CTL_WORK, CTL_NABORT, CTL_NMEMB, CTL_N };
 // cumulative counters

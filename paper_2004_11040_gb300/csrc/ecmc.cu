@@ -891,6 +891,8 @@ __global__ void __launch_bounds__(ROW_THREADS) k_bands(Dev s, int C) {
     }
 }
 
+constexpr double RING_SPREAD = 0.86;  // of d (graph.cu, frames of rings)
+
 // In the edge rows (R = 0 below, R = nc - 1 above) the neighbour row lies
 // across the box edge, and the scan takes the periodic image: for j in row
 // nc - 1 seen from row 0 its |dy| is RN(L - RN(y_j - y)), which only grows as
@@ -908,6 +910,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_skip(Dev s, int C) {
     const uint32_t nrow = (uint32_t)nc * (uint32_t)C;
     const int Rdn = R == 0 ? nc - 1 : R - 1, Rup = R == nc - 1 ? 0 : R + 1;
     const unsigned long long lo_dn = s.rband[Rdn], lo_up = s.rband[Rup];
+    const unsigned long long lo_r = s.rband[R];
     const double hi_dn = __longlong_as_double((long long)s.rband[nc + Rdn]);
     const double lo = __longlong_as_double((long long)lo_up);
     const uint32_t o = blockIdx.x * ROW_THREADS + threadIdx.x;
@@ -947,6 +950,11 @@ __global__ void __launch_bounds__(ROW_THREADS) k_skip(Dev s, int C) {
         s.cskp[q] = v;
         near = v != 3;
     }
+    // (a ring's disks lie within RING_SPREAD d in y)
+    if (threadIdx.x == 0 && blockIdx.x == 0 && lo_r != INF_BITS)
+        near = near || !(__dsub_rn(__longlong_as_double((long long)s.rband[nc + R]),
+                                   __longlong_as_double((long long)lo_r)) <
+                         __dmul_rn(RING_SPREAD, s.d));
     if (__syncthreads_or(near) && threadIdx.x == 0) atomicAdd(s.lc + LC_NEARROW, 1ull);
 }
 
@@ -2616,15 +2624,14 @@ struct ecmc_ctx {
     bool log_overflow = false;
     int32_t direction = 0;  // 0: +x; 1: +y (the context is stored transposed)
     GraphCtx *graph = nullptr;  // ECMC_GRAPH: the constraint-graph path holds the state
-    // cell scan: a frame in which some disk has a neighbour row in reach (or
-    // the row pass does not apply) is general: its legs run along the arrows of
-    // G(3) (graph.cu) with the flag on cells. The state is then in `arrow` from
-    // the frame's first leg on, and the cells are stale until the next frame.
-    // Such a frame in the cells' own general pass spent ~5000 cycles an event
-    // (a scan's loads, its claims' round trip and ~20 serial FP64
-    // instructions), along the arrows ~1000.
+    // cell scan: the legs run in graph.cu with the flag on cells, from records
+    // built from the cells at the frame's first leg; the cells are stale until
+    // the next frame. A frame whose rows all are rings runs along them (a leg of
+    // 1024 chains on 2^20 lattice disks 65 us against ~79 along the arrows), any
+    // other along the arrows of G(3).
     GraphCtx *arrow = nullptr;
     bool general = false;
+    bool ring = false;  // the frame's rows are rings (graph.cu)
     bool in_arrow = false;
     bool arrow_used = false;
     uint32_t *loc_of = nullptr;  // [n] scratch of the cell build
@@ -2766,7 +2773,7 @@ static GraphCells cells_of(const ecmc_ctx *ctx) {
 // A general frame's state to the arrow path, before its first leg.
 static int enter_arrow(ecmc_ctx *ctx, std::string &err) {
     if (ctx->in_arrow) return 0;
-    const int rc = graph_activate(ctx->arrow, cells_of(ctx), !ctx->arrow_used, err);
+    const int rc = graph_activate(ctx->arrow, cells_of(ctx), !ctx->arrow_used, ctx->ring, err);
     if (rc) return rc;
     ctx->in_arrow = ctx->arrow_used = true;
     return 0;
@@ -3135,7 +3142,8 @@ extern "C" int ecmc_create(const ecmc_params *p, const double *x, const double *
     }
     CU(cudaMemsetAsync(s.lc, 0, LC_N * sizeof(unsigned long long), st));
     ctx->loc_of = loc_of;
-    ctx->general = !s.rp_ok || h_lc[LC_NEARROW] != 0ull;
+    ctx->ring = s.rp_ok && h_lc[LC_NEARROW] == 0ull;
+    ctx->general = true;
     *out = ctx;
     return ECMC_OK;
 }
@@ -3232,6 +3240,7 @@ static void fold_graph_totals(ecmc_ctx *c, const GraphTotals &t, bool alone) {
     c->restarts += t.restarts;
     c->blocked += t.blocked;
     c->cwindows += t.cwindows;
+    c->row_windows += t.row_windows;
     c->horizon += t.horizon;
     c->order_err += t.order_err;
     c->prof.pass1_launches += t.legs;
@@ -3730,7 +3739,8 @@ extern "C" int ecmc_set_direction(ecmc_ctx *ctx, int32_t direction) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(ctx, ECMC_ECUDA, std::string("set_direction: ") + cudaGetErrorString(e));
     ctx->in_arrow = false;
-    ctx->general = !s.rp_ok || near[0] != 0ull;
+    ctx->ring = s.rp_ok && near[0] == 0ull;
+    ctx->general = true;
     if (near[1]) return fail(ctx, ECMC_ECAPACITY, "set_direction: a cell overflowed");
     ctx->direction = direction;
     return ECMC_OK;

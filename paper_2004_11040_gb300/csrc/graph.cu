@@ -99,6 +99,10 @@ struct GDev {
     StopK sk;
     double2 *pxt;         // [(cap + 2) * k]
     uint32_t *pcell;      // [(cap + 2) * k]
+    // a frame of rings (ring != 0): the disks ring after ring, each in the order
+    // of x, and every disk's place there
+    int ring;
+    uint32_t *rid, *posof;  // [n]
     uint32_t epoch0;       // epoch of the launch's first pass, less one
     GSpec *sp;             // [k] the run alone of each chain, for the resolve
     uint32_t stamp0;       // stamp of the launch's first leg, less one
@@ -667,6 +671,115 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
     }
 }
 
+// ---------------------------------------------------------- frames of rings
+//
+// A cell row whose disks lie within RING_SPREAD d of each other in y, d or
+// more from every disk of the rows beside, is a ring: a chain there never
+// leaves it, its disks keep their cyclic order in x (all pairs are within d in
+// y), and a disk's target is always the next one (every b lies in 0.51 d .. d,
+// so the disk after the next is reached 0.02 d later at least). In a frame
+// whose rows all are rings -- a lattice start on cells aligned with it -- a
+// chain's run is a stretch of consecutive places (g_leap_chain) instead of a
+// walk from record to record. The cells' row bands decide (k_skip).
+
+// What a record of a ring frame holds in b[1] and b[2] (a[1] and a[2] are
+// NONE): its ring's first place and length, and its row of cells.
+__device__ __forceinline__ double two_words(uint32_t lo, uint32_t hi) {
+    return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
+}
+
+// Disks per cell row (one block per row).
+__global__ void __launch_bounds__(256) k_ring_count(GBuild b, int C, uint32_t *row_off) {
+    const uint32_t nrow = (uint32_t)b.nc * (uint32_t)C, q0 = blockIdx.x * nrow;
+    int n = 0;
+    for (uint32_t o0 = 0; o0 < nrow; o0 += blockDim.x) {
+        const uint32_t o = o0 + threadIdx.x;
+        n += __syncthreads_count(o < nrow && b.scid[q0 + o] != EMPTY);
+    }
+    if (threadIdx.x == 0) row_off[blockIdx.x] = (uint32_t)n;
+}
+
+// Counts to first places (one block).
+__global__ void k_ring_offsets(int nc, uint32_t *row_off) {
+    __shared__ int warp_tot[32];
+    __shared__ int tot[2];
+    const int chunk = (nc + blockDim.x - 1) / blockDim.x;
+    const int lo = min(nc, (int)threadIdx.x * chunk), hi = min(nc, lo + chunk);
+    int sum = 0;
+    for (int q = lo; q < hi; ++q) sum += (int)row_off[q];
+    int off = block_exscan(sum, warp_tot, tot);
+    for (int q = lo; q < hi; ++q) {
+        const int n = (int)row_off[q];
+        row_off[q] = (uint32_t)off;
+        off += n;
+    }
+    if (threadIdx.x == 0) row_off[nc] = (uint32_t)tot[0];
+}
+
+// The places and records of a frame of rings (one block per row): a cell's
+// disks, in the order of x, follow those of the cells before; then every disk
+// gets its record, its successor the only arrow. Bound by the records' 64
+// bytes per disk.
+template <int C>
+__global__ void __launch_bounds__(256) k_ring_place(GBuild b, const uint32_t *row_off, GDev s) {
+    __shared__ int warp_tot[32];
+    __shared__ int tot[2];
+    const uint32_t nc = (uint32_t)b.nc, first = row_off[blockIdx.x];
+    const uint32_t len = row_off[blockIdx.x + 1] - first;
+    uint32_t at0 = first;
+    for (uint32_t c0 = 0; c0 < nc; c0 += blockDim.x) {
+        const uint32_t col = c0 + threadIdx.x;
+        uint32_t id[C];
+        double x[C], y[C];
+        int n = 0;
+        if (col < nc) {
+            const uint32_t loc = (blockIdx.x * nc + col) * C;
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                id[q] = b.scid[loc + q];
+                x[q] = INFINITY;
+                y[q] = 0.0;
+                if (id[q] != EMPTY) {
+                    x[q] = b.sx[loc + q];
+                    y[q] = b.sy[loc + q];
+                    ++n;
+                }
+            }
+        }
+        const uint32_t at = at0 + (uint32_t)block_exscan(n, warp_tot, tot);
+        if (n > 0) {
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                if (id[q] == EMPTY) continue;
+                int rank = 0;  // x >= 0: ordered by bits
+#pragma unroll
+                for (int z = 0; z < C; ++z)
+                    rank += dbits(x[z]) < dbits(x[q]) || (z < q && dbits(x[z]) == dbits(x[q]));
+                const uint32_t p = at + (uint32_t)rank;
+                s.rid[p] = id[q];
+                s.posof[id[q]] = p;
+                s.y[id[q]] = y[q];
+                s.g[id[q]].x = x[q];
+            }
+        }
+        at0 += (uint32_t)tot[0];
+        __syncthreads();
+    }
+    for (uint32_t o = threadIdx.x; o < len; o += blockDim.x) {
+        const uint32_t i = s.rid[first + o], j = s.rid[first + (o + 1 < len ? o + 1 : 0)];
+        const double ay = fabs(__dsub_rn(s.y[j], s.y[i]));
+        const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
+        const bool has = len > 1;
+        ulonglong2 *g = reinterpret_cast<ulonglong2 *>(s.g + i);
+        s.g[i].t = 0.0;
+        g[1] = make_ulonglong2((unsigned long long)OWN_STATIC |
+                                   ((unsigned long long)(has ? j : NONE) << 32),
+                               ~0ull);
+        g[2] = make_ulonglong2(0ull, has ? dbits(v) : 0ull);
+        g[3] = make_ulonglong2(dbits(two_words(first, len)), dbits(two_words(blockIdx.x, 0u)));
+    }
+}
+
 // The chains' start disks active (after a build).
 __global__ void k_g_init_chains(GDev s, const int32_t *active) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1077,6 +1190,8 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         r.n = n;
         r.touch = end == SP_STALL ? n : n + 1;
         r.end = end | (n > n_lap ? SP_LAP : 0);
+        if (s.ring && strict && n > 0 && (uint32_t)n >= (uint32_t)(dbits(g[i].b[1]) >> 32))
+            atomicAdd(s.lc + LC_RINGLAP, 1ull);
         r.partner = partner < (uint32_t)s.k ? (int32_t)partner : -1;
         r.tc = ti;
         r.D = D;
@@ -1086,6 +1201,149 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         s.sp[c] = r;
     }
     __syncwarp();
+}
+
+// The same pass in a frame of rings, of a leg from its start (not strict): the
+// run's disks are consecutive places, so lane e holds the e-th from the active
+// disk on and finds its gap to the next; only the sums of Eq. 1 -- the time and
+// the remaining length before each event -- are a chain of additions, each
+// rounded as the steps round it, on half the lanes each, one FP64 instruction
+// an event. A stretch covers 31 events; most legs end within the first.
+// What the run leaves is g_spec_chain's, word by word. A run that comes round
+// its ring, or out of records, is left to g_spec_chain (false).
+//
+// Bound by that chain (~100 cycles an event against ~1000 of a step) and the
+// four dependent loads before it. 1024 chains on 2^20 disks: a leg 82 us with
+// the scan of row bands this replaces, 65 with it; 16384 chains: 890 -> 605.
+__device__ __noinline__ bool g_leap_chain(const GDev &s, int c, bool begin) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t i0 = s.ci[c];
+    if (begin) g_begin_state(s, c, i0, lane);
+    const GDisk *const g = s.g;
+    const double L = s.L;
+    const uint32_t p0 = s.posof[i0];
+    const unsigned long long info = dbits(g[i0].b[1]);
+    const uint32_t row = (uint32_t)dbits(g[i0].b[2]);
+    const uint32_t first = (uint32_t)info, len = (uint32_t)(info >> 32);
+    uint32_t id = 0u;
+    double t = 0.0, D = s.ell;  // before the event on lane 0
+    int n0 = 0, end = SP_STALL, n = 0;
+    uint32_t partner = NONE, iend = i0;
+    if (lane == 31) {
+        *gpath_at(s, c, 0) = i0;
+        red_min_u64(s.key + i0, g_key(0.0, c));
+    }
+    for (;; n0 += 31) {
+        uint32_t q = p0 - first + (uint32_t)(n0 + lane);
+        if (q >= len) q %= len;
+        id = s.rid[first + q];
+        const double x = g[id].x, bb = g[id].b[0];
+        const uint32_t own = g[id].own;
+        const double xn = shfl_f64(x, (lane + 1) & 31);
+        const uint32_t idn = __shfl_sync(FULL, id, (lane + 1) & 31);
+        const uint32_t ownn = __shfl_sync(FULL, own, (lane + 1) & 31);
+        // targets: the last but one of the ring is the last the run has not moved
+        const bool in = lane < 31 && (uint32_t)(n0 + lane) + 1u < len;
+        const bool nsc = in && ownn >= OWN_ACTIVE;
+        double dx = __dsub_rn(xn, x);
+        const bool neg = __double_as_longlong(dx) < 0;
+        if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
+        double tau = __dsub_rn(dx, bb);
+        if (__double_as_longlong(tau) < 0) tau = 0.0;
+        // the sums: time on the lower lanes, remaining length on the upper;
+        // before event e they go to lane e of the half (e < 16), or to a second
+        // register of lane e - 16
+        const int half = lane & 15;
+        const unsigned long long flip = lane < 16 ? 0ull : 1ull << 63;
+        const unsigned stops = __ballot_sync(FULL, lane < 31 && (nsc || !in));
+        const int bound = stops ? __ffs(stops) - 1 : 31;  // no event after this one
+        double v = lane < 16 ? t : D, v0 = v, v1 = v;
+        for (int e0 = 0; e0 <= bound; e0 += 8) {
+#pragma unroll
+            for (int z = 0; z < 8; ++z) {
+                const int e = e0 + z;
+                if (half == (e & 15)) {
+                    if (e0 < 16)
+                        v0 = v;
+                    else
+                        v1 = v;
+                }
+                const unsigned long long dt = shfl_u64(dbits(tau), e) ^ flip;
+                v = __dadd_rn(v, __longlong_as_double((long long)dt));
+            }
+            if (__any_sync(FULL, lane >= 16 && __double_as_longlong(v) < 0)) break;
+        }
+        {
+            const double ta = shfl_f64(v0, half), tb = shfl_f64(v1, half);
+            const double da = shfl_f64(v0, half + 16), db = shfl_f64(v1, half + 16);
+            t = lane < 16 ? ta : tb;
+            D = lane < 16 ? da : db;
+        }
+        const bool lift = dbits(tau) < dbits(D);
+        const unsigned fin = __ballot_sync(FULL, lane < 31 && (!in || nsc || !lift));
+        const int f = fin ? __ffs(fin) - 1 : 31;  // the event that ends the run, or none
+        const bool round = fin && !__shfl_sync(FULL, (int)in, f);
+        const bool met = fin && !round && __shfl_sync(FULL, (int)lift, f);  // lift onto an active disk
+        n = n0 + f + (fin && !met ? 1 : 0);
+        if ((round && len > 1) || n >= s.cap) {
+            if (lane == 0 && round) atomicAdd(s.lc + LC_RINGLAP, 1ull);
+            return false;
+        }
+        // events n0 .. n - 1
+        const int e = n0 + lane;
+        const bool has = e < n, stall = has && lane == f;
+        const double ts = stall ? D : tau;
+        const double tn_lift = shfl_f64(t, (lane + 1) & 31), dn_lift = shfl_f64(D, (lane + 1) & 31);
+        const double tn_stall = __dadd_rn(t, D);
+        double xe = __dadd_rn(x, ts);
+        const bool wrap = has && dbits(xe) >= dbits(L);
+        if (__any_sync(FULL, wrap) && wrap) xe = g_sub(xe, L);
+        const double tn = stall ? tn_stall : tn_lift;
+        if (has || (met && lane == f)) {
+            const size_t at = (size_t)e * (size_t)s.k + (size_t)c;
+            s.pxt[at] = make_double2(x, has ? ts : D);
+            s.pcell[at] = row * (uint32_t)s.nc + (uint32_t)cell_coord(x, s.inv_a, s.nc);
+        }
+        if (has) {
+            ulonglong2 *u = reinterpret_cast<ulonglong2 *>(grec_at(s, c, e));
+            u[0] = make_ulonglong2((unsigned long long)id |
+                                       ((unsigned long long)(stall ? NONE : idn) << 32),
+                                   (unsigned long long)(uint32_t)e);
+            u[1] = make_ulonglong2(dbits(x), dbits(t));
+            u[2] = make_ulonglong2(0ull, dbits(tn));
+            u[3] = make_ulonglong2(dbits(ts), dbits(xe));
+            u[4] = make_ulonglong2(stall ? 0ull : dbits(xn), stall ? 0ull : dbits(dn_lift));
+            if (!stall) {
+                *gpath_at(s, c, e + 1) = idn;
+                red_min_u64(s.key + idn, g_key(tn, c));
+            }
+        }
+        if (fin) {
+            end = met ? SP_NONSTATIC : SP_STALL;
+            if (met) partner = __shfl_sync(FULL, ownn, f) & OWN_CHAIN;
+            iend = __shfl_sync(FULL, id, f);
+            t = shfl_f64(met ? t : tn, f);
+            D = met ? shfl_f64(D, f) : 0.0;
+            break;
+        }
+        t = shfl_f64(t, 31);
+        D = shfl_f64(D, 31);
+    }
+    if (lane == 0) {
+        GSpec r;
+        r.n = n;
+        r.touch = end == SP_STALL ? n : n + 1;
+        r.end = end;
+        r.partner = partner < (uint32_t)s.k ? (int32_t)partner : -1;
+        r.tc = t;
+        r.D = D;
+        r.ci = iend;
+        r.cut = end == SP_STALL ? 0x7FFFFFFF : n;
+        r.pad[0] = r.pad[1] = 0;
+        s.sp[c] = r;
+    }
+    __syncwarp();
+    return true;
 }
 
 // Touch keys of chain c back to empty (one warp): every disk its last run
@@ -2388,7 +2646,7 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int q, int round,
 struct GCtl {
     int64_t budget;  // liftings for this run (0: none)
     int64_t lifts, legs, conflict_legs, repaired, continued, horizon, order_err, p1_lifts,
-        repair_lifts, restarts, blocked, cwindows;
+        repair_lifts, restarts, blocked, cwindows, row_windows;
     int64_t leg0;    // legs run before this launch (lifting log)
     uint8_t *flags;  // per-leg conflict flags (device) or null
     int32_t flags_cap;
@@ -2595,6 +2853,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         c.restarts += (int64_t)lc[LC_RESTARTS];
         c.blocked += (int64_t)lc[LC_BLOCKED];
         c.cwindows += fast ? flag : (int64_t)lc[LC_CWINDOWS];
+        if (B.reps[r].ring && lc[LC_RINGLAP] == 0ull) c.row_windows += B.windows;
         c.horizon += (int64_t)lc[LC_HORIZON];
         c.order_err += (int64_t)lc[LC_ORDER];
         if (lc[LC_ERR_REC] != 0ull || lc[LC_ERR_CAP] != 0ull) c.err = 1;
@@ -2662,6 +2921,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     if (!g_rep_on(B, r)) continue;
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
                     if (!fast) g_set_stamp(my_dev, leg, lane);
+                    if (s.ring && !s.strict && g_leap_chain(s, f - B.chain_base[r], fast)) continue;
                     g_spec_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
                                  g_window_end(s, w), fast);
                 }
@@ -2855,6 +3115,7 @@ struct GraphCtx {
     void *build_tmp = nullptr;        // scratch of graph_build
     float2 *slot_xy = nullptr;        // scratch of graph_activate
     uint32_t *slot_bits = nullptr;
+    uint32_t *row_off = nullptr;      // [nc + 1]
     std::vector<std::pair<void **, size_t>> pending;
     int64_t bytes = 0;  // device memory held
 };
@@ -3031,6 +3292,7 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, size_t slots, std::stri
         chk(galloc(g, &s.pxt, k * ((size_t)s.cap + 2), err));
         chk(galloc(g, &s.pcell, k * ((size_t)s.cap + 2), err));
         chk(galloc(g, &g->slot_xy, slots, err));
+        chk(galloc(g, &g->row_off, (size_t)g->nc + 1, err));
         chk(galloc(g, &g->slot_bits, (size_t)std::ceil(p->box / (p->d / 128.0)) / 32 + 2, err));
     }
     chk(galloc(g, &s.path, k * ((size_t)s.cap + 2), err));
@@ -3208,7 +3470,7 @@ static void graph_bind(GraphCtx *g, const GraphCells &c) {
     s.sk.eps = c.eps;
 }
 
-int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &err) {
+int graph_activate(GraphCtx *g, const GraphCells &c, bool first, bool ring, std::string &err) {
     GDev &s = g->s;
     cudaStream_t st = g->st;
     if (first) {
@@ -3226,16 +3488,29 @@ int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &er
     b.cxy = g->slot_xy;
     b.bits = g->slot_bits;
     b.yout = s.y;
-    const uint32_t nslot = (uint32_t)((size_t)c.nc * c.nc * c.C);
-    cudaMemsetAsync(b.bits, 0, ((size_t)b.nb / 32 + 1) * 4, st);
-    const unsigned ablk = (unsigned)(((size_t)c.nc * c.nc + BUILD_CELLS - 1) / BUILD_CELLS);
-    const unsigned sblk = (unsigned)(((size_t)nslot + 255) / 256);
-    if (c.C == 4) {
-        k_gb_slots<4><<<sblk, 256, 0, st>>>(b, nslot);
-        k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
+    s.ring = ring;
+    if (ring) {
+        // (places in the scratch of the other kind of frame: 8 bytes a slot)
+        s.rid = (uint32_t *)g->slot_xy;
+        s.posof = s.rid + s.n;
+        k_ring_count<<<(unsigned)c.nc, 256, 0, st>>>(b, c.C, g->row_off);
+        k_ring_offsets<<<1, 1024, 0, st>>>(c.nc, g->row_off);
+        if (c.C == 4)
+            k_ring_place<4><<<(unsigned)c.nc, 256, 0, st>>>(b, g->row_off, s);
+        else
+            k_ring_place<8><<<(unsigned)c.nc, 256, 0, st>>>(b, g->row_off, s);
     } else {
-        k_gb_slots<8><<<sblk, 256, 0, st>>>(b, nslot);
-        k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
+        const uint32_t nslot = (uint32_t)((size_t)c.nc * c.nc * c.C);
+        const unsigned ablk = (unsigned)(((size_t)c.nc * c.nc + BUILD_CELLS - 1) / BUILD_CELLS);
+        const unsigned sblk = (unsigned)(((size_t)nslot + 255) / 256);
+        cudaMemsetAsync(b.bits, 0, ((size_t)b.nb / 32 + 1) * 4, st);
+        if (c.C == 4) {
+            k_gb_slots<4><<<sblk, 256, 0, st>>>(b, nslot);
+            k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
+        } else {
+            k_gb_slots<8><<<sblk, 256, 0, st>>>(b, nslot);
+            k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
+        }
     }
     k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, (const int32_t *)c.ci);
     const cudaError_t e = cudaGetLastError();
@@ -3464,6 +3739,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         t.repair_lifts = c.repair_lifts;
         t.blocked = c.blocked;
         t.cwindows = c.cwindows;
+        t.row_windows = c.row_windows;
         if (n == 1) {
             t.ms = ms;
             t.pass1_ms = ph[GPH_PASS1] * 1e-6;

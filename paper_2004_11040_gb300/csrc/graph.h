@@ -16,7 +16,7 @@ struct GraphCtx;
 // Totals of one graph_run call.
 struct GraphTotals {
     int64_t legs, lifts, conflict_legs, repaired, continued, horizon, order_err, p1_lifts,
-        repair_lifts, restarts, blocked, cwindows;
+        repair_lifts, restarts, blocked, cwindows, row_windows;
     double ms, pass1_ms, repair_ms, other_ms;
 };
 
@@ -56,7 +56,7 @@ void graph_batch_free(GBatchScratch *scratch);
 // path's arrays to the context's requests (records and log are the cells'
 // own; null: host allocation); graph_activate builds the records and arrows from the cells as they
 // stand at a breakpoint (queued on the stream; first: the first time of the
-// context), after which the state is here: graph_swapped gives x and y
+// context; ring: every row is a ring), after which the state is here: graph_swapped gives x and y
 // exchanged (x into xnew) and the active disks, to build cells from again.
 struct GraphCells {
     int nc, C;
@@ -72,7 +72,7 @@ struct GraphCells {
 };
 GraphCtx *graph_attach(const ecmc_params *p, int nc, int C, cudaStream_t st,
                        std::vector<std::pair<void **, size_t>> &pending);
-int graph_activate(GraphCtx *g, const GraphCells &c, bool first, std::string &err);
+int graph_activate(GraphCtx *g, const GraphCells &c, bool first, bool ring, std::string &err);
 void graph_swapped(GraphCtx *g, double *xnew, const double **ynew, const int32_t **active);
 // Legs run before (leg index of the lifting log).
 void graph_set_leg(GraphCtx *g, int64_t legs);
