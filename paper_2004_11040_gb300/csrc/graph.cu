@@ -119,7 +119,9 @@ struct GDev {
     // conflict components (names as the union-find of common.cuh expects)
     double *vt;
     int32_t *uf, *fin, *comp_of, *abort_to, *comp_cnt, *comp_off, *comp_root, *comp_mem, *ctl;
-    int32_t *blist, *pcnt;
+    // the trees of the union-find while the pass builds them: a root's last
+    // hooked child, the child hooked before it, and the pass that took the root
+    int32_t *child, *sib, *taken;
     uint64_t *memb;   // (pass of the launch, round) << 32 | root of the component listing the chain
     int restart;      // conflicts by restart strategy 2 (Sec. 3.4) instead of local repair
     int strict;       // the pass claims every disk a step reads, not only those it touches
@@ -1452,7 +1454,70 @@ __device__ __noinline__ void g_flag_chain(const GDev &s, int c, uint32_t epoch, 
 // With the claims on every disk read (three per event) 508 of 2048 chains on
 // 262144 dense disks were blocked per leg; touched disks alone: about a
 // third of that.
-__device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, uint32_t epoch) {
+// Blocked chains of a pass, over all systems: chain f (numbered over the
+// systems) is entry *cnt - base of list.
+struct GBlocked {
+    unsigned *cnt;
+    int32_t *list;
+    unsigned base;
+};
+
+// A pass's components start as single chains with final events (one warp).
+__device__ __forceinline__ void g_begin_pass(const GDev &s, int c, int lane) {
+    if (lane < 6) {
+        int32_t *const a[6] = {s.uf, s.comp_of, s.fin, s.abort_to, s.child, s.ctl};
+        const int32_t v[6] = {c, c, 1, -1, -1, 0};
+        int32_t *p = a[0];
+        int32_t w = v[0];
+#pragma unroll
+        for (int z = 1; z < 6; ++z) {
+            p = lane == z ? a[z] : p;
+            w = lane == z ? v[z] : w;
+        }
+        if (lane < 5) p[c] = w;
+        if (lane == 5 && c == 0) {
+            p[CTL_NABORT] = 0;
+            p[CTL_NMEMB] = 0;
+        }
+    }
+}
+
+// The root of chain c's tree (no path is shortened: the trees stay as hooked).
+__device__ __forceinline__ int g_root(const GDev &s, int c) {
+    for (;;) {
+        const int p = ((volatile int32_t *)s.uf)[c];
+        if (p == c) return c;
+        c = p;
+    }
+}
+
+// A chain blocked by the pass (one thread): counted, listed for the repair,
+// and in one component with its partner from here on. The component's members
+// are its root's tree: a hooked root goes on its new root's list of children.
+__device__ void g_note_blocked(const GDev &s, int c, int32_t partner, int f, const GBlocked &bl) {
+    const unsigned ix = atomicAdd(bl.cnt, 1u) - bl.base;
+    atomicAdd(s.lc + LC_BLOCKED, 1ull);
+    atomicAdd(s.lc + LC_WBLOCKED, 1ull);
+    s.fin[c] = 0;
+    if (partner >= 0 && partner < s.k) {
+        s.fin[partner] = 0;
+        int a = c, b = partner;
+        for (;;) {
+            a = g_root(s, a);
+            b = g_root(s, b);
+            if (a == b) break;
+            const int lo = min(a, b), hi = max(a, b);
+            if (atomicCAS(s.uf + hi, hi, lo) == hi) {
+                s.sib[hi] = atomicExch(s.child + lo, hi);
+                break;
+            }
+        }
+    }
+    bl.list[ix] = f;
+}
+
+__device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, uint32_t epoch, int f,
+                                             const GBlocked &bl) {
     const int lane = threadIdx.x & 31;
     // the chain's state and the first touched disks in one round of loads
     const GSpec sp = s.sp[c];
@@ -1571,7 +1636,7 @@ __device__ __noinline__ void g_resolve_chain(const GDev &s, int c, double tw, ui
         s.partner[c] = partner;
         // events before the blocking time, and all before the window, are exact
         s.vt[c] = st == ST_BLOCKED ? fmax(tc, tw) : INFINITY;
-        if (st == ST_BLOCKED) note_blocked(s, c, partner);
+        if (st == ST_BLOCKED) g_note_blocked(s, c, partner, f, bl);
         if (lifts) atomicAdd(s.lc + LC_P1LIFTS, (unsigned long long)lifts);
     }
     __syncwarp();
@@ -1605,7 +1670,8 @@ struct GStep {
 // Yes if this round's component lists it (memb == tag); with adopt, also if
 // it was, or now is, taken over: a chain in no component of this round whose
 // events are final since the round began joins the component (and any later
-// merge that reaches the component takes it along).
+// merge that reaches the component takes it along: the next round's union-find
+// adds it from comp_of).
 __device__ __forceinline__ bool holder_ours(const GDev &s, int h, int root, uint64_t tag,
                                             bool adopt) {
     if (h < 0 || h >= s.k) return false;
@@ -1614,12 +1680,7 @@ __device__ __forceinline__ bool holder_ours(const GDev &s, int h, int root, uint
     int hc = __ldcg(s.comp_of + h);
     if (hc == h && h != root && __ldcg(s.fin + h) == 1) {
         const int prev = atomicCAS(s.comp_of + h, h, root);
-        if (prev == h) {
-            uf_union(s.uf, h, root);
-            hc = root;
-        } else {
-            hc = prev;
-        }
+        hc = prev == h ? root : prev;
     }
     return hc == root;
 }
@@ -2487,16 +2548,70 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
     g_finish(s, mem, m, root, abort, met, now);
 }
 
-// Component q of this round (one warp): roll its members back to T*, then
+// The members of the component of blocked chain a (one warp): the root's tree,
+// 16 members at a time. The list grows from the warp's buffer into parts of
+// comp_mem (each twice the last: 4 k words hold all of them). False if another
+// blocked chain's warp has taken the component for this pass.
+//
+// So a pass's components need no phase of their own. (One block made them in
+// shared memory or, beyond 2048 chains, in global memory, between the resolve
+// and the repair: 8 us of a leg at 1024 chains, ~300 of 605 us at 16384.)
+constexpr int MEMBER_BUF = 64;
+__device__ __noinline__ bool g_members(const GDev &s, int a, uint32_t epoch, int *root_out,
+                                       const int32_t **mem_out, int *m_out) {
+    __shared__ int32_t buf[8][MEMBER_BUF];
+    const int lane = threadIdx.x & 31;
+    int32_t *mem = buf[threadIdx.x >> 5];
+    const int root = g_root(s, a);
+    // (asked now, answered while the members are gathered)
+    int prev = 0;
+    if (lane == 0) prev = atomicExch(s.taken + root, (int32_t)epoch);
+    int cap = MEMBER_BUF, n = 1, done = 0;
+    __syncwarp();
+    if (lane == 0) mem[0] = root;
+    __syncwarp();
+    while (done < n) {
+        if (n + 32 > cap) {
+            // (only the component's one owner takes parts of comp_mem)
+            if (__shfl_sync(FULL, prev, 0) == (int32_t)epoch) return false;
+            int off = 0;
+            if (lane == 0) off = atomicAdd(s.ctl + CTL_NMEMB, 2 * cap);
+            off = __shfl_sync(FULL, off, 0);
+            int32_t *const to = s.comp_mem + off;
+            for (int e = lane; e < n; e += 32) to[e] = mem[e];
+            mem = to;
+            cap *= 2;
+            __syncwarp();
+        }
+        const int e = done + lane, end = min(n, done + 16);
+        int ch = -1, sb = -1;
+        if (e < end) {
+            const int c = mem[e];
+            ch = ((volatile int32_t *)s.child)[c];
+            if (e > 0) sb = ((volatile int32_t *)s.sib)[c];
+        }
+        const unsigned mc = __ballot_sync(FULL, ch >= 0), ms = __ballot_sync(FULL, sb >= 0);
+        const unsigned below = (1u << lane) - 1u;
+        if (ch >= 0) mem[n + __popc(mc & below)] = ch;
+        if (sb >= 0) mem[n + __popc(mc) + __popc(ms & below)] = sb;
+        n += __popc(mc) + __popc(ms);
+        done = end;
+        __syncwarp();
+    }
+    *root_out = root;
+    *mem_out = mem;
+    *m_out = n;
+    return __shfl_sync(FULL, prev, 0) != (int32_t)epoch;
+}
+
+// A component of this round (one warp): roll its members back to T*, then
 // replay them in global event-time order (Alg. 2) up to the window's end.
 // Members are spread over the lanes (member e on lane e mod 32); after each
 // event only the members whose arrows read a disk it changed recompute.
-__device__ __noinline__ void g_repair_component(const GDev &s, int q, int round, uint32_t epoch,
-                                                uint32_t wr_tag, double tw, double tend) {
+__device__ __noinline__ void g_repair_component(const GDev &s, const int32_t *mem, int m, int root,
+                                                int round, uint32_t epoch, uint32_t wr_tag,
+                                                double tw, double tend) {
     const int lane = threadIdx.x & 31;
-    const int root = s.comp_root[q];
-    const int off = s.comp_off[q], m = s.comp_off[q + 1] - off;
-    const int32_t *mem = s.comp_mem + off;
     double Ts = INFINITY;
     // the members listed for this round of this pass (wr_tag names both)
     const uint64_t tag = ((uint64_t)wr_tag << 32) | (uint32_t)root;
@@ -2655,7 +2770,8 @@ struct GCtl {
     int32_t dbg;     // an internal check recorded in GDev::dbg (set at the end)
 };
 
-enum { GG_WORK = 0, GG_ANY, GG_ERR, GG_REMAIN0, GG_REMAIN1, GG_COUNT, GG_PASSES, GG_N };
+enum { GG_WORK = 0, GG_ANY, GG_ERR, GG_REMAIN0, GG_REMAIN1, GG_COUNT, GG_PASSES,
+       GG_NBLK, GG_N };
 enum { GPH_BEGIN = 0, GPH_PASS1, GPH_REPAIR, GPH_END, GPH_N };
 
 // One launch: R systems (their descriptions in device memory), their chains
@@ -2667,6 +2783,7 @@ struct GBatchDev {
     int32_t *comp_base;            // [R + 1]
     unsigned int *bar;             // [1] grid barrier
     int32_t *g;                    // [GG_N]
+    int32_t *blocked;              // [chain_base[R]] blocked chains of a pass
     unsigned long long *phase_ns;  // [GPH_N] device time per phase (block 0 clock)
     int32_t R, max_legs, windows, pad;
     unsigned long long wait_ns;    // bound on every grid-barrier wait
@@ -2788,23 +2905,20 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         __syncthreads();
         return last;
     };
-    // conflict components of system r (one block)
+    // conflict components of system r after round 1 (one block)
     auto uf_system = [&](int r, int round) {
         if (threadIdx.x < 32) (void)g_warp_dev(wdev, wrep, B.reps, r);
         __syncthreads();
         const GDev &s = wdev[0];
-        bool need = false;
-        unsigned long long wbl = 0ull;
-        if (g_rep_on(B, r)) {
-            wbl = __ldcg(s.lc + LC_WBLOCKED);
-            need = round == 1 ? wbl != 0ull : __ldcg(s.ctl + CTL_NABORT) != 0;
-            // the window's flag: the reads of two chains met
-            if (!fast && round == 1 && threadIdx.x == 0 && __ldcg(s.lc + LC_WWEAK) != 0ull)
-                atomicAdd(s.lc + LC_CWINDOWS, 1ull);
-        }
+        const bool need = g_rep_on(B, r) && __ldcg(s.ctl + CTL_NABORT) != 0;
         if (need && round <= 255) {
-            uf_block(s, round == 1, warp_tot, tot, false, uf_sm, s.blist, s.pcnt,
-                     round == 1 ? (int)min(wbl, (unsigned long long)s.k) : -1);
+            // the chains taken over in the last round
+            for (int c = threadIdx.x; c < s.k; c += blockDim.x) {
+                const int to = s.comp_of[c];
+                if (to != c) uf_union(s.uf, c, to);
+            }
+            __syncthreads();
+            uf_block(s, 0, warp_tot, tot, false, uf_sm);
         } else if (threadIdx.x == 0) {
             s.ctl[CTL_NCOMP] = 0;
             if (need) atomicAdd(s.lc + LC_ERR_CAP, 1ull);  // too many rounds
@@ -2864,6 +2978,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         return c.done != 0;
     };
     uint32_t pass = 0;  // passes of the launch (the same count in every thread)
+    GBlocked bl = {(unsigned *)(B.g + GG_NBLK), B.blocked, 0u};
     int leg = 0;
     for (; leg < B.max_legs; ++leg) {
         if (fast) {
@@ -2898,6 +3013,14 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         // start), or the last one allowed, is repaired locally.
         double tw_r = 0.0;
         int sub = 0;
+        bool any = false;  // (fast) the leg had something to repair
+        auto flags = [&]() {
+            for (int f = gw; f < total_chains; f += nwarps) {
+                const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, 0);
+                g_flag_chain(s, f, s.epoch0 + pass, lane);
+                g_reset_keys(s, f, lane);
+            }
+        };
         for (int w = 0; w < B.windows; ++w) {
             if (w > 0) {
                 // a new claim window: the touch keys of the last one go
@@ -2913,14 +3036,16 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 }
                 if (!barrier()) return;
             }
-            bool uf_early = false;
+            int nblk = 0;  // blocked chains of the pass, of all systems
             for (;;) {
                 ++pass;
+                if (gt == 0) B.g[GG_WORK] = 0;
                 for (int f = gw; f < total_chains; f += nwarps) {
                     const int r = g_find_rep(B.chain_base, R, f);
                     if (!g_rep_on(B, r)) continue;
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
                     if (!fast) g_set_stamp(my_dev, leg, lane);
+                    g_begin_pass(s, f - B.chain_base[r], lane);
                     if (s.ring && !s.strict && g_leap_chain(s, f - B.chain_base[r], fast)) continue;
                     g_spec_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
                                  g_window_end(s, w), fast);
@@ -2936,21 +3061,17 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
                     if (!fast) g_set_stamp(my_dev, leg, lane);
                     g_resolve_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
-                                    s.epoch0 + pass);
+                                    s.epoch0 + pass, f, bl);
                     if (!fast && sub == 0)
                         g_flag_chain(s, f - B.chain_base[r], s.epoch0 + pass, lane);
                 }
-                if (R == 1 && !restart) {
-                    // one system: the last block to finish resolving takes the
-                    // first round's union-find and prefix (no barrier between)
-                    if (last_block()) {
-                        uf_system(0, 1);
-                        comp_prefix();
-                    }
-                    uf_early = true;
-                }
                 if (!barrier()) return;
                 mark(GPH_PASS1);
+                {
+                    const unsigned now = (unsigned)__ldcg(B.g + GG_NBLK);
+                    nblk = (int)(now - bl.base);
+                    bl.base = now;
+                }
                 if (!restart) break;
                 const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, 0);
                 g_set_stamp(my_dev, leg, lane);
@@ -2972,15 +3093,9 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 if (!barrier()) return;
                 const double Ts = __ldcg(s.tstar);
                 if (!(dbits(Ts) > dbits(tw_r)) || sub >= MAX_RESTARTS) break;  // local repair
-                // every thread has read the blocked count: reset for the next
-                // pass, with the partner counts of the chains listed
-                const int nbl = (int)min(__ldcg(s.lc + LC_WBLOCKED), (unsigned long long)s.k);
                 for (int f = gw; f < total_chains; f += nwarps) g_reset_keys(s, f, lane);
-                for (int z = gt; z < nbl; z += (int)(gridDim.x * blockDim.x)) {
-                    const int pt = s.partner[s.blist[z]];
-                    if (pt >= 0 && pt < s.k) s.pcnt[pt] = 0;
-                }
                 if (!barrier()) return;
+                // (every thread has read the blocked count: back to 0)
                 if (gt == 0) {
                     s.lc[LC_WBLOCKED] = 0ull;
                     s.lc[LC_RESTARTS] += 1ull;
@@ -2991,33 +3106,55 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 tw_r = Ts;
                 ++sub;
             }
+            // the window's flag: the reads of two chains met
+            for (int r = gt; r < R && !fast; r += (int)(gridDim.x * blockDim.x))
+                if (g_rep_on(B, r) && __ldcg(B.reps[r].lc + LC_WWEAK) != 0ull)
+                    atomicAdd(B.reps[r].lc + LC_CWINDOWS, 1ull);
             // repair rounds
-            for (int round = 1;; ++round) {
-                if (!(round == 1 && uf_early)) {
+            for (int round = 1; nblk > 0; ++round) {
+                int ncomp = nblk;
+                if (round > 1) {
                     for (int r = blockIdx.x; r < R; r += gridDim.x) uf_system(r, round);
                     // the last block to finish its union-finds takes the prefix
                     if (last_block()) comp_prefix();
                     if (!barrier()) return;
+                    ncomp = __ldcg(B.g + GG_ANY);
+                    if (ncomp == 0) break;
                 }
-                const int ncomp = __ldcg(B.g + GG_ANY);
-                if (fast && round == 1)
-                    for (int f = gw; f < total_chains; f += nwarps) {
-                        g_flag_chain(*my_dev, f, my_dev->epoch0 + pass, lane);
-                        g_reset_keys(*my_dev, f, lane);
+                // round 1: an entry per blocked chain, the first ones to the last
+                // warps (of few chains, those without one of their own); the
+                // others, and later rounds, from a queue
+                for (int z = round == 1 ? nwarps - 1 - gw : -1;;) {
+                    if (z < 0) {
+                        if (lane == 0) z = atomicAdd(B.g + GG_WORK, 1);
+                        z = __shfl_sync(FULL, z, 0) + (round == 1 ? nwarps : 0);
                     }
-                if (ncomp == 0) break;
-                for (;;) {
-                    int q = 0;
-                    if (lane == 0) q = atomicAdd(B.g + GG_WORK, 1);
-                    q = __shfl_sync(FULL, q, 0);
-                    if (q >= ncomp) break;
-                    const int r = g_find_rep(B.comp_base, R, q);
+                    if (z >= ncomp) break;
+                    const int f = round == 1 ? __ldcg(B.blocked + z) : z;
+                    const int32_t *const base = round == 1 ? B.chain_base : B.comp_base;
+                    const int r = g_find_rep(base, R, f), q = f - base[r];
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
                     if (!fast) g_set_stamp(my_dev, leg, lane);
-                    g_repair_component(s, q - B.comp_base[r], round, s.epoch0 + pass,
-                                       ((uint32_t)(leg * B.windows + w) << 8) | (uint32_t)round,
-                                       restart ? tw_r : g_window_start(s, w), g_window_end(s, w));
+                    int root, m;
+                    const int32_t *mem;
+                    bool mine = true;
+                    if (round == 1) {
+                        mine = g_members(s, q, s.epoch0 + pass, &root, &mem, &m);
+                    } else {
+                        root = s.comp_root[q];
+                        const int off = s.comp_off[q];
+                        m = s.comp_off[q + 1] - off;
+                        mem = s.comp_mem + off;
+                    }
+                    if (mine)
+                        g_repair_component(s, mem, m, root, round, s.epoch0 + pass,
+                                           ((uint32_t)(leg * B.windows + w) << 8) | (uint32_t)round,
+                                           restart ? tw_r : g_window_start(s, w),
+                                           g_window_end(s, w));
+                    if (round == 1 && ncomp <= nwarps) break;
+                    z = -1;
                 }
+                if (fast && round == 1) flags();
                 if (!barrier()) return;
                 // no component met another chain: the window is repaired
                 int aborted = 0;
@@ -3025,11 +3162,13 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     if (g_rep_on(B, r) && __ldcg(B.reps[r].ctl + CTL_NABORT) != 0) aborted = 1;
                 if (!__syncthreads_or(aborted)) break;
             }
+            if (fast && nblk == 0) flags();
+            any = nblk > 0;
             mark(GPH_REPAIR);
         }
         if (fast) {
             // a leg without components has passed no barrier since its keys went
-            if (__ldcg(B.g + GG_ANY) == 0 && !barrier()) return;
+            if (!any && !barrier()) return;
             const GDev &s = *my_dev;
             if (s.log_on)
                 for (int f = gw; f < total_chains; f += nwarps)
@@ -3324,9 +3463,10 @@ static int graph_plan(GraphCtx *g, const ecmc_params *p, size_t slots, std::stri
     chk(galloc(g, &s.comp_cnt, k, err));
     chk(galloc(g, &s.comp_off, k + 1, err));
     chk(galloc(g, &s.comp_root, k, err));
-    chk(galloc(g, &s.comp_mem, k, err));
-    chk(galloc(g, &s.blist, k, err));
-    chk(galloc(g, &s.pcnt, k, err));
+    chk(galloc(g, &s.comp_mem, 4 * k, err));  // (g_members)
+    chk(galloc(g, &s.child, k, err));
+    chk(galloc(g, &s.sib, k, err));
+    chk(galloc(g, &s.taken, k, err));
     chk(galloc(g, &s.ctl, CTL_N, err));
     chk(galloc(g, &s.lc, 2 * LC_N, err));
     chk(galloc(g, &s.dbg, 16, err));
@@ -3388,7 +3528,7 @@ static void graph_clear(GraphCtx *g) {
     cudaStream_t st = g->st;
     cudaMemsetAsync(s.nrec, 0, k * 4, st);
     cudaMemsetAsync(s.sp, 0, k * sizeof(GSpec), st);
-    cudaMemsetAsync(s.pcnt, 0, k * 4, st);
+    cudaMemsetAsync(s.taken, 0, k * 4, st);
     cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
     cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
     cudaMemsetAsync(s.key, 0xFF, n * 8, st);
@@ -3535,9 +3675,10 @@ void graph_set_leg(GraphCtx *g, int64_t legs) { g->log_legs = legs; }
 // whole before a launch and read back from ctl on after it.
 struct GBatchScratch {
     int cap = 0;
+    int64_t chains = 0;
     unsigned char *block = nullptr;
     size_t off_base = 0, off_comp = 0, off_ctl = 0, off_bar = 0, off_g = 0, off_phase = 0,
-           total = 0;
+           off_list = 0, total = 0;
     std::vector<unsigned char> host;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 };
@@ -3550,10 +3691,11 @@ void graph_batch_free(GBatchScratch *b) {
     delete b;
 }
 
-static int launch_reserve(GBatchScratch **scratch, int n, std::string &err) {
+static int launch_reserve(GBatchScratch **scratch, int n, int64_t chains, std::string &err) {
     GBatchScratch *b = *scratch;
-    if (b && b->cap >= n) return 0;
-    const int cap = std::max(n, b ? 2 * b->cap : 1);
+    if (b && b->cap >= n && b->chains >= chains) return 0;
+    const int cap = b && b->cap >= n ? b->cap : std::max(n, b ? 2 * b->cap : 1);
+    chains = std::max(chains, b ? b->chains : 0);
     graph_batch_free(b);
     *scratch = nullptr;
     b = new (std::nothrow) GBatchScratch();
@@ -3576,6 +3718,7 @@ static int launch_reserve(GBatchScratch **scratch, int n, std::string &err) {
     b->off_phase = take(GPH_N * sizeof(unsigned long long));
     b->total = off;
     b->host.assign(off, 0);
+    b->off_list = take((size_t)chains * sizeof(int32_t));  // (device only)
     if (dm_alloc_t(&b->block, off) != 0 || cudaEventCreate(&b->ev0) != cudaSuccess ||
         cudaEventCreate(&b->ev1) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -3584,6 +3727,7 @@ static int launch_reserve(GBatchScratch **scratch, int n, std::string &err) {
         return ECMC_ENOMEM;
     }
     b->cap = cap;
+    b->chains = chains;
     *scratch = b;
     return 0;
 }
@@ -3629,7 +3773,13 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         if (legs_out) legs_out[r] = 0;
     }
     if (max_legs == 0) return 0;
-    int rc = launch_reserve(scratch, n, err);
+    int64_t chains = 0;
+    for (int r = 0; r < n; ++r) chains += gs[r]->s.k;
+    if (chains > 0x7FFFFFFF) {
+        err = "too many chains in a batch";
+        return ECMC_EINVAL;
+    }
+    int rc = launch_reserve(scratch, n, chains, err);
     if (rc) return rc;
     GBatchScratch *b = *scratch;
     auto cu = [&](cudaError_t e, const char *what) {
@@ -3644,7 +3794,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
     GDev *S = (GDev *)h;
     int32_t *base = (int32_t *)(h + b->off_base);
     GCtl *ctl = (GCtl *)(h + b->off_ctl);
-    int64_t chains = 0;
+    chains = 0;
     for (int r = 0; r < n; ++r) {
         GraphCtx *g = gs[r];
         if (g->st != st) cu(cudaStreamSynchronize(g->st), "context stream");
@@ -3662,6 +3812,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
             k_g_clear_epochs<<<(unsigned)((g->s.n + 255) / 256), 256, 0, st>>>(g->s);
             cu(cudaGetLastError(), "epochs");
             cu(cudaMemsetAsync(g->s.fl, 0, flag_words(g->s) * 8, st), "epochs");
+            cu(cudaMemsetAsync(g->s.taken, 0, (size_t)g->s.k * 4, st), "epochs");
             g->s.epoch0 = 0;
             g->s.stamp0 = 1;  // (the last leg's times, for ecmc_positions)
         }
@@ -3676,10 +3827,6 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         cu(cudaMemsetAsync(g->s.memb, 0xFF, (size_t)g->s.k * 8, st), "memb");
     }
     base[n] = (int32_t)chains;
-    if (chains > 0x7FFFFFFF) {
-        err = "too many chains in a batch";
-        return ECMC_EINVAL;
-    }
     cu(cudaMemcpyAsync(b->block, h, b->total, cudaMemcpyHostToDevice, st), "tables");
     if (rc) return rc;
     GBatchDev B;
@@ -3690,6 +3837,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
     B.bar = (unsigned int *)(b->block + b->off_bar);
     B.g = (int32_t *)(b->block + b->off_g);
     B.phase_ns = (unsigned long long *)(b->block + b->off_phase);
+    B.blocked = (int32_t *)(b->block + b->off_list);
     B.R = n;
     B.max_legs = max_legs;
     B.windows = W;
