@@ -1205,12 +1205,41 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
     __syncwarp();
 }
 
+// The sums of a stretch of events, tau of event e on lane e: t and D before
+// event 0 (the same on every lane) become those before this lane's event, each
+// addition rounded as the steps round it, for the events up to `bound` as long
+// as D is not negative. Time is summed on the lower lanes and remaining length
+// on the upper, in one FP64 instruction an event; before event e they go to
+// lane e of each half (e < 16), or to a second register of lane e - 16.
+__device__ __forceinline__ void g_sums(double tau, int bound, double &t, double &D) {
+    const int lane = threadIdx.x & 31, half = lane & 15;
+    const unsigned long long flip = lane < 16 ? 0ull : 1ull << 63;
+    double v = lane < 16 ? t : D, v0 = v, v1 = v;
+    for (int e0 = 0; e0 <= bound; e0 += 8) {
+#pragma unroll
+        for (int z = 0; z < 8; ++z) {
+            const int e = e0 + z;
+            if (half == (e & 15)) {
+                if (e0 < 16)
+                    v0 = v;
+                else
+                    v1 = v;
+            }
+            v = __dadd_rn(v, __longlong_as_double((long long)(shfl_u64(dbits(tau), e) ^ flip)));
+        }
+        if (__any_sync(FULL, lane >= 16 && __double_as_longlong(v) < 0)) break;
+    }
+    const double ta = shfl_f64(v0, half), tb = shfl_f64(v1, half);
+    const double da = shfl_f64(v0, half + 16), db = shfl_f64(v1, half + 16);
+    t = lane < 16 ? ta : tb;
+    D = lane < 16 ? da : db;
+}
+
 // The same pass in a frame of rings, of a leg from its start (not strict): the
 // run's disks are consecutive places, so lane e holds the e-th from the active
 // disk on and finds its gap to the next; only the sums of Eq. 1 -- the time and
 // the remaining length before each event -- are a chain of additions, each
-// rounded as the steps round it, on half the lanes each, one FP64 instruction
-// an event. A stretch covers 31 events; most legs end within the first.
+// rounded as the steps round it (g_sums). A stretch covers 31 events; most legs end within the first.
 // What the run leaves is g_spec_chain's, word by word. A run that comes round
 // its ring, or out of records, is left to g_spec_chain (false).
 //
@@ -1252,35 +1281,8 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c, bool begin) {
         if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
         double tau = __dsub_rn(dx, bb);
         if (__double_as_longlong(tau) < 0) tau = 0.0;
-        // the sums: time on the lower lanes, remaining length on the upper;
-        // before event e they go to lane e of the half (e < 16), or to a second
-        // register of lane e - 16
-        const int half = lane & 15;
-        const unsigned long long flip = lane < 16 ? 0ull : 1ull << 63;
         const unsigned stops = __ballot_sync(FULL, lane < 31 && (nsc || !in));
-        const int bound = stops ? __ffs(stops) - 1 : 31;  // no event after this one
-        double v = lane < 16 ? t : D, v0 = v, v1 = v;
-        for (int e0 = 0; e0 <= bound; e0 += 8) {
-#pragma unroll
-            for (int z = 0; z < 8; ++z) {
-                const int e = e0 + z;
-                if (half == (e & 15)) {
-                    if (e0 < 16)
-                        v0 = v;
-                    else
-                        v1 = v;
-                }
-                const unsigned long long dt = shfl_u64(dbits(tau), e) ^ flip;
-                v = __dadd_rn(v, __longlong_as_double((long long)dt));
-            }
-            if (__any_sync(FULL, lane >= 16 && __double_as_longlong(v) < 0)) break;
-        }
-        {
-            const double ta = shfl_f64(v0, half), tb = shfl_f64(v1, half);
-            const double da = shfl_f64(v0, half + 16), db = shfl_f64(v1, half + 16);
-            t = lane < 16 ? ta : tb;
-            D = lane < 16 ? da : db;
-        }
+        g_sums(tau, stops ? __ffs(stops) - 1 : 31, t, D);
         const bool lift = dbits(tau) < dbits(D);
         const unsigned fin = __ballot_sync(FULL, lane < 31 && (!in || nsc || !lift));
         const int f = fin ? __ffs(fin) - 1 : 31;  // the event that ends the run, or none
@@ -2291,6 +2293,165 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
     }
 }
 
+// The same in a frame of rings: a member goes on along its ring by stretches of
+// 31 events as in g_leap_chain, with Eq. 2 asked of every target and every disk
+// read claimed before anything is written. The words are exchanged after the
+// records were read, so a word that was free stands for a record nobody has
+// written since. (Claims beyond one that fails stay; the component they belong
+// to is repaired again.) A run that comes round its ring is left to the replay.
+// 1024 chains on 2^20 disks: the repair phase of a leg 33 us with a step per
+// event, 21 by stretches.
+__device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, int m, int root,
+                                            uint64_t tag, uint32_t epoch, int round, int *met) {
+    const int lane = threadIdx.x & 31, up = (lane + 1) & 31;
+    GDisk *const g = s.g;
+    const double L = s.L;
+    const uint32_t stamp = s.stamp;
+    uint32_t cnt = 0;
+    int switches = 0, e = 0, cur = -1;
+    for (;;) {
+        if (cur < 0) {  // the next member still blocked
+            while (e < m) {
+                const unsigned bm =
+                    __ballot_sync(FULL, e + lane < m && s.status[mem[e + lane]] == ST_BLOCKED);
+                if (bm) {
+                    e += __ffs(bm) - 1;
+                    break;
+                }
+                e += 32;
+            }
+            if (e >= m) return CONT_DONE;
+            cur = mem[e];
+        }
+        const int c = cur;
+        const uint32_t mine = (uint32_t)c + 1u;
+        const unsigned long long ct = ((unsigned long long)epoch << 32) | mine;
+        uint32_t i = s.ci[c];
+        double t = s.tc[c], D = s.D[c];
+        const int32_t nr0 = s.nrec[c];
+        const uint32_t seq0 = ((uint32_t)round << 24) | cnt;
+        const uint32_t p0 = s.posof[i];
+        const unsigned long long info = dbits(g[i].b[1]);
+        const uint32_t first = (uint32_t)info, len = (uint32_t)(info >> 32);
+        int nl = 0, n = 0, st = ST_RUNNING, next = -1, how = CONT_DONE;
+        for (bool more = true; more;) {
+            uint32_t q = p0 - first + (uint32_t)(n + lane);
+            if (q >= len) q %= len;
+            const uint32_t id = s.rid[first + q];
+            const ulonglong2 *const r = reinterpret_cast<const ulonglong2 *>(g + id);
+            const ulonglong2 r0 = __ldcg(r), r1 = __ldcg(r + 1), r2 = __ldcg(r + 2);
+            const double x = __longlong_as_double((long long)r0.x);
+            const double xn = shfl_f64(x, up);
+            const double rt = __longlong_as_double((long long)shfl_u64(r0.y, up));
+            const uint32_t ownn = __shfl_sync(FULL, (uint32_t)r1.x, up);
+            const uint32_t idn = __shfl_sync(FULL, id, up);
+            const bool in = lane < 31 && (uint32_t)(n + lane) + 1u < len;
+            const bool nsc = in && ownn >= OWN_ACTIVE;
+            double dx = __dsub_rn(xn, x);
+            const bool neg = __double_as_longlong(dx) < 0;
+            if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
+            double tau = __dsub_rn(dx, __longlong_as_double((long long)r2.y));
+            if (__double_as_longlong(tau) < 0) tau = 0.0;
+            const unsigned stops = __ballot_sync(FULL, lane < 31 && (nsc || !in));
+            g_sums(tau, stops ? __ffs(stops) - 1 : 31, t, D);
+            const double sum = __dadd_rn(t, tau);
+            const bool timed = ownn == stamp && dbits(rt) != 0ull;
+            const bool bad = (nsc || timed) && !(dbits(sum) > dbits(rt));
+            const bool lift = !nsc && dbits(tau) < dbits(D);
+            const bool ends = !in || (bad && !nsc) || !lift;
+            const unsigned fin = __ballot_sync(FULL, lane < 31 && ends);
+            const int f = fin ? __ffs(fin) - 1 : 31;
+            // what event f is, if it ends the run
+            enum { STALLS = 0, FAILS = 1, WAITS = 2 };
+            const int kind = __shfl_sync(FULL, !in || (bad && !nsc)                     ? FAILS
+                                               : nsc && (bad || dbits(tau) < dbits(D)) ? WAITS
+                                                                                       : STALLS,
+                                         f);
+            // the disks read, the active one and the targets of the events up to f
+            uint32_t h = 0u;
+            if (lane <= (fin ? f + 1 : 31)) {
+                h = g_holder(r2.x, ct);
+                if (h == 0u) h = g_holder(atomicCAS(&g[id].claim, r2.x, ct), ct);
+            }
+            const bool ask = h != 0u && h != mine;
+            unsigned fb = 0u;
+            if (__any_sync(FULL, ask)) {
+                const bool ours = !ask || holder_ours(s, (int)h - 1, root, tag, true);
+                fb = __ballot_sync(FULL, !ours);
+            }
+            const int nev = f + (fin && kind == STALLS ? 1 : 0);  // events of this stretch
+            if (fb || nr0 + n + nev > s.cap) {  // none of them is written
+                if (fb) *met = (int)__shfl_sync(FULL, h, __ffs(fb) - 1) - 1;
+                how = fb ? CONT_FOREIGN : CONT_FAIL;
+                i = __shfl_sync(FULL, id, 0);
+                t = shfl_f64(t, 0);
+                break;
+            }
+            const bool has = lane < nev, stall = has && lane == f;
+            const double ts = stall ? D : tau, tn = stall ? g_add(t, D) : sum;
+            const double dn = shfl_f64(D, up);
+            double xe = __dadd_rn(x, ts);
+            const bool wrap = has && dbits(xe) >= dbits(L);
+            if (__any_sync(FULL, wrap) && wrap) xe = g_sub(xe, L);
+            if (has) {
+                ulonglong2 *u = reinterpret_cast<ulonglong2 *>(grec_at(s, c, nr0 + n + lane));
+                u[0] = make_ulonglong2((unsigned long long)id |
+                                           ((unsigned long long)(stall ? NONE : idn) << 32),
+                                       (unsigned long long)(seq0 + (uint32_t)(n + lane)));
+                u[1] = make_ulonglong2(dbits(x), dbits(t));
+                u[2] = make_ulonglong2(!stall && ownn == stamp ? dbits(rt) : 0ull, dbits(tn));
+                u[3] = make_ulonglong2(dbits(ts), dbits(xe));
+                u[4] = make_ulonglong2(stall ? 0ull : dbits(xn), stall ? 0ull : dbits(dn));
+                *reinterpret_cast<ulonglong2 *>(&g[id].x) = make_ulonglong2(dbits(xe), dbits(tn));
+                g[id].own = stall ? (OWN_STALLED | (uint32_t)c) : stamp;
+            }
+            n += nev;
+            nl += f;
+            // the state before event f, or after the stall
+            i = __shfl_sync(FULL, id, f);
+            t = shfl_f64(stall ? tn : t, f);
+            D = shfl_f64(stall ? 0.0 : D, f);
+            more = fin == 0u;
+            if (more) continue;
+            if (kind == STALLS) st = ST_STALLED;
+            if (kind == FAILS) how = CONT_FAIL;
+            if (kind == WAITS) {
+                const int hc = (int)(__shfl_sync(FULL, ownn, f) & OWN_CHAIN);
+                if (hc != c && hc < s.k &&
+                    __ldcg((const unsigned long long *)s.memb + hc) == tag &&
+                    s.status[hc] == ST_BLOCKED && switches < 4 * m + 4) {
+                    next = hc;  // wait for that member (Remark 10)
+                    st = ST_BLOCKED;
+                    ++switches;
+                } else {
+                    how = CONT_FAIL;
+                }
+            }
+        }
+        __syncwarp();
+        // the events so far stand (a failure rolls them back with the rest)
+        if (lane == 0) {
+            if (nl > 0 && st != ST_STALLED) {
+                g[i].own = OWN_ACTIVE | (uint32_t)c;
+                g[i].t = t;
+            }
+            s.nrec[c] = nr0 + n;
+            s.nlift[c] += nl;
+            if (nl) atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
+            if (how == CONT_DONE) {
+                s.status[c] = st;
+                s.ci[c] = i;
+                s.tc[c] = t;
+                s.D[c] = D;
+            }
+        }
+        __syncwarp();
+        cnt += (uint32_t)n;
+        if (how != CONT_DONE) return how;
+        cur = next;
+    }
+}
+
 // Replay of a component with at most 10 members (one warp), rolled back to Ts:
 // lane 3e + p holds target p of member e's active disk -- its record, as the
 // replay has changed it -- so every member's next event is computed at once,
@@ -2627,7 +2788,9 @@ __device__ __noinline__ void g_repair_component(const GDev &s, const int32_t *me
     __syncwarp();
     if (round == 1) {
         int met = -1;
-        const int how = g_continue(s, mem, m, root, tag, epoch, round, tw, tend, &met);
+        const int how = s.ring && !s.strict
+                            ? g_continue_ring(s, mem, m, root, tag, epoch, round, &met)
+                            : g_continue(s, mem, m, root, tag, epoch, round, tw, tend, &met);
         if (how == CONT_DONE) {
             if (lane == 0) atomicAdd(s.lc + LC_CONTINUED, (unsigned long long)m);
             g_finish(s, mem, m, root, false, -1, Ts, true);
