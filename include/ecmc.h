@@ -46,9 +46,9 @@ extern "C" {
                                   instead of the cell scan; see "Constraint-graph mode" */
 #define ECMC_RESTART 0x8u      /* with ECMC_GRAPH and windows <= 1: conflicts handled by
                                   restart strategy 2 (Sec. 3.4); see "Restart mode" */
-#define ECMC_NO_ROWPASS 0x10u  /* cell scan: always use the general parallel pass, also in
-                                  windows where the row pass applies (see "Row pass");
-                                  results are the same either way */
+#define ECMC_NO_ROWPASS 0x10u  /* always run along the arrows of G(3), also in frames whose
+                                  rows are rings (see "Row pass"); results are the same
+                                  either way */
 
 typedef struct ecmc_ctx ecmc_ctx;
 
@@ -83,13 +83,14 @@ typedef struct {
                                  the blocked chains (Lemma 2), nothing redone */
     int64_t restarts;         /* ECMC_RESTART: passes begun again at an earlier stop time
                                  T* taken as a breakpoint (Sec. 3.4, strategy 2) */
-    int64_t row_windows;      /* claim windows whose parallel pass was the row pass */
+    int64_t row_windows;      /* cell scan: claim windows run along rings (see "Row pass")
+                                 by chains none of which came round its ring in the leg */
     int64_t device_bytes;     /* device memory the context holds (its pooled state) */
-    int64_t blocked_chains;   /* chains whose parallel pass stopped at a strong claim of
-                                 another chain, summed over windows and legs: the chains
-                                 that met another one (Sec. 3.4) */
+    int64_t blocked_chains;   /* chains whose parallel pass was cut where another chain's
+                                 run comes first, summed over windows and legs: the
+                                 chains that met another one (Sec. 3.4) */
     int64_t conflict_windows; /* claim windows (legs x W in all) whose conflict flag is 1:
-                                 the claim sets of two chains met in the window */
+                                 the reads of two chains met in the window */
 } ecmc_stats_t;
 
 /* One lifting i -> j (Eq. 1): chain c, leg index, time t (= new t_j),
@@ -117,9 +118,9 @@ int ecmc_create(const ecmc_params *p, const double *x, const double *y,
 
 /*
  * ecmc_context_bytes -- the device memory a context created with *p would
- * hold, without allocating anything: its arrays (cells, chain table, event
- * records, claims; with ECMC_GRAPH the disk records, arrows and the graph
- * build's scratch instead of the cells) and the scratch of ecmc_positions,
+ * hold, without allocating anything: its arrays (disk records with their
+ * arrows, chain table, event records, flag words, the build's scratch) and the
+ * scratch of ecmc_positions,
  * i.e. the device_bytes that ecmc_stats reports once positions have been
  * read. (The persistent launch's scratch, a few kilobytes per system, is not
  * included.) A scheduler admits systems by it. The paper has no counterpart.
@@ -136,21 +137,26 @@ int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes);
  * closer than d in y cannot pass one another, so the arrows stay valid over
  * any number of legs, and a step reads only the (at most three) arrow targets
  * of the active disk. Results (positions, local times, liftings) are those of
- * the cell scan, i.e. of Alg. 2. Claims are taken on the disks a step reads
- * (the active disk and its arrow targets) instead of cells, so a leg's flag
- * is 1 iff in some window the disks that two chains read, each run alone,
- * overlap. Limits: n_chains <= 2^20 - 2. Such contexts are batched with
- * each other only (their own persistent kernel; same claim windows, no
- * ECMC_RESTART). cells_per_side only sets the cell scan that builds the
- * graph.
+ * the cell scan, i.e. of Alg. 2. The flag is on the disks a step reads (the
+ * active disk and its arrow targets) instead of cells, so a leg's flag is 1
+ * iff in some window the disks that two chains read, each run alone, overlap.
+ * Limits: n_chains <= 2^20 - 2. Such contexts are batched with each other only
+ * (same claim windows, no ECMC_RESTART). cells_per_side only sets the cells
+ * that the graph is built from. (A context without ECMC_GRAPH finds its
+ * liftings through G(3) too; what its flag says is what a scan of cells
+ * would.)
  *
- * Conflicts. Within a claim window every chain claims, with atomicCAS, each
- * cell it scans; two chains that want one cell "meet". A leg's flag is 1 iff
- * in some window the cells that two chains would scan, each run alone from the
- * window's start, overlap. A cell whose row holds no disk within d in y of the
- * scanning chain's active disk is claimed weakly: it counts for the flag but
- * stops no chain. Chains that met over a cell they read are rolled back and
- * redone in global time order, so results are always those of Alg. 2.
+ * Conflicts. A leg's flag is 1 iff in some window the cells that two chains
+ * would scan (ECMC_GRAPH: the disks they would read), each run alone from the
+ * window's start, overlap. Chains whose runs reach the same disk are cut
+ * there, all but the one that reaches it first; they go on where Eq. 2 allows
+ * it or are rolled back and redone in global time order, so results are always
+ * those of Alg. 2.
+ *
+ * Row pass. A row of cells whose disks are within reach of each other in y and
+ * of no disk of the rows beside is a ring: its disks keep their order, and a
+ * chain there moves along consecutive disks. Frames whose rows all are rings
+ * (lattice starts on cells aligned with the lattice) run along them.
  *
  * ecmc_run_to_breakpoint -- runs n_legs legs of length ell (Alg. 2 semantics:
  * each leg ends at the breakpoint h' with all chains stalled, Remark on
@@ -160,8 +166,8 @@ int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes);
  *   leg_flags_out host, n_legs bytes or NULL: the leg's conflict flag (see
  *                 above); entries past *legs_done are untouched.
  *   legs_done     host or NULL: number of legs completed.
- * All legs run in one persistent cooperative launch; returns when they are
- * done (the stream is synchronised).
+ * All legs run in one persistent cooperative launch (2^24 / windows of them
+ * at a time); returns when they are done (the stream is synchronised).
  * Errors: EINVAL, ECUDA, ECAPACITY (undo log), ETIMEOUT (a grid barrier wait
  * passed its 60 s limit).
  */
@@ -188,8 +194,8 @@ int ecmc_positions(ecmc_ctx *ctx, double *x, double *y, double *t, int32_t *acti
  * Alg. 2 with v along that direction).
  *   direction  0: +x (the state after ecmc_create); 1: +y.
  * Call between runs (the state is always at a breakpoint then). The context
- * keeps motion along +x of its own frame and is transposed in place (x and y
- * swapped, cells (r, c) <-> (c, r)); ecmc_positions returns x and y in the
+ * keeps motion along +x of its own frame and is built again with x and y
+ * swapped; ecmc_positions returns x and y in the
  * caller's frame; the xi, xj of ecmc_liftings are along the direction of
  * motion. Local times are reset to 0 (they are leg-relative), and the lifting
  * log is kept. Synchronises the context's stream.
@@ -198,8 +204,8 @@ int ecmc_positions(ecmc_ctx *ctx, double *x, double *y, double *t, int32_t *acti
 int ecmc_set_direction(ecmc_ctx *ctx, int32_t direction);
 
 /*
- * ecmc_set_wait_limit -- bound on every wait of the persistent kernels of the
- * cell-scan path (their grid barriers), in nanoseconds of the device clock;
+ * ecmc_set_wait_limit -- bound on every wait of the persistent kernel's grid
+ * barriers for a context without ECMC_GRAPH, in nanoseconds of the device clock;
  * the default, and the largest value, is 60 s. A wait that runs out makes the
  * launch return ECMC_ETIMEOUT (every block stops at its next barrier or
  * gives up waiting for the blocks that stopped), and the context is then in
@@ -244,9 +250,9 @@ int ecmc_graph_arrows(ecmc_ctx *ctx, int32_t *a, double *b);
  * ecmc_profile -- device time per phase of the persistent kernel, read from
  * the device clock at the phase boundaries of every ecmc_run_to_breakpoint:
  *   pass1   the parallel pass (one warp per chain, each a task of Alg. 5/6);
- *   repair  component rollback and global-time redo (Alg. 2), with its
- *           union-find rounds;
- *   other   leg start (claims, chain table) and leg end (totals, log).
+ *   repair  continuation of the chains cut, rollback and global-time redo
+ *           (Alg. 2), with their rounds; the flag;
+ *   other   leg start (chain table) and leg end (totals, log).
  * *_launches count legs (pass1, other) and legs with a repair (repair);
  * pass1_liftings counts liftings of the parallel pass (redone ones included),
  * repair_liftings the liftings of legs that needed a repair.
@@ -333,8 +339,8 @@ const char *ecmc_last_error(const ecmc_ctx *ctx);
  *
  * It allocates nothing (no cudaMalloc, cudaFree or allocating library call, on
  * the device or the host). Its working memory is one file-scope device array
- * of ECMC_NOALLOC_SCRATCH_MIB MiB that the library holds on every GPU that
- * loads it, until the process exits. The first call on a device looks up the
+ * of 52 MiB that the library holds on every GPU that loads it, until the
+ * process exits. The first call on a device looks up the
  * array's address (cudaGetSymbolAddress) with that device current; make that
  * first call before any stream capture. Every call shares the array and
  * clears what it needs, so calls that overlap on the GPU (other streams or
@@ -349,9 +355,9 @@ const char *ecmc_last_error(const ecmc_ctx *ctx);
  *   stream   cudaStream_t (NULL = default stream); synchronised on return
  *   flag_out host, 1 byte (NULL to skip): 1 if two chains' cells met
  *   lifts_out host (NULL to skip): liftings made in the leg
- * Sizes whose arrays (cells, per-disk and per-chain state, ECMC_NOALLOC_RECORDS
- * event records per chain) do not fit the array return ECMC_EINVAL before any
- * device work; so do bad scalars, coordinates outside [0, L) and repeated or
+ * Sizes that count for more than ECMC_NOALLOC_SCRATCH_MIB MiB (33 bytes a cell
+ * slot, 4 a disk, 24.7 KB a chain for ECMC_NOALLOC_RECORDS events) return
+ * ECMC_EINVAL before any device work; so do bad scalars, coordinates outside [0, L) and repeated or
  * out-of-range active ids. ECMC_ECAPACITY: a chain made more than
  * ECMC_NOALLOC_RECORDS events in the leg, or a cell overflowed. ECMC_ECUDA: a
  * CUDA call failed. Example limits: N = 65536 disks with 256 chains fit.

@@ -1,7 +1,7 @@
 """Builds libecmc.so in-tree with nvcc for sm_103a (GB300).
 
-Two translation units -- the cell-scan path with the C ABI (ecmc.cu) and the
-constraint-graph path (graph.cu) -- are compiled in parallel, then linked.
+Two translation units -- the C ABI (ecmc.cu) and the legs (graph.cu) -- are
+compiled in parallel, then linked.
 """
 from __future__ import annotations
 

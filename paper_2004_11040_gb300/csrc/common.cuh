@@ -1,7 +1,7 @@
-// common.cuh -- device pieces shared by the cell-scan path (ecmc.cu) and the
-// constraint-graph path (graph.cu) of libecmc: owner-word encoding, chain
-// states, counters, bit-level FP64 order, union-find of conflict components,
-// block scans and the bounded grid barrier of the persistent kernels.
+// common.cuh -- device pieces of libecmc: owner-word encoding, chain states,
+// counters, bit-level FP64 order, the stop rule of a cell scan, union-find of
+// conflict components, block scans and the bounded grid barrier of the
+// persistent kernel.
 // Everything lives in an unnamed namespace: each translation unit keeps its
 // own copy.
 #pragma once
@@ -29,19 +29,14 @@ constexpr unsigned long long INF_BITS = 0x7FF0000000000000ull;  // +inf
 constexpr int ST_RUNNING = 0, ST_STALLED = 1, ST_BLOCKED = 2;
 
 // per-leg counters (reset at every leg start)
-enum { LC_BLOCKED = 0, LC_LIFTS, LC_HORIZON, LC_ERR_CAP, LC_ERR_REC, LC_ORDER, LC_OWNER_FAIL,
-       LC_CONTINUED,
+enum { LC_BLOCKED = 0, LC_LIFTS, LC_HORIZON, LC_ERR_CAP, LC_ERR_REC, LC_ORDER, LC_CONTINUED,
        LC_P1LIFTS, LC_REPAIRED, LC_WBLOCKED, LC_CWINDOWS, LC_RESTARTS, LC_WEAK,
-       LC_ROWWIN,  // claim windows run by the row pass (cell scan)
-       LC_WWEAK,   // chains whose claim sets met on a weak claim, this window
-       LC_BADXY, LC_BADID,  // inputs out of range (creation only)
-       LC_NEARROW,  // rows that are no rings, at least (k_skip)
+       LC_WWEAK,    // chains whose reads met another's, this window
        LC_RINGLAP,  // chains whose run came round its ring (a frame of rings)
        LC_N };
-enum { CTL_NCOMP = 0, CTL_WORK, CTL_NABORT, CTL_NMEMB, CTL_N };
+enum { CTL_NCOMP = 0, CTL_NABORT, CTL_NMEMB, CTL_N };
 // cumulative counters
-enum { TC_LIFTS = 0, TC_LEGS, TC_CONFLICT_LEGS, TC_REPAIRED, TC_HORIZON, TC_ORDER,
-       TC_LOG_N, TC_N };
+enum { TC_LOG_N = 0, TC_N };
 
 // Event records of repair rounds carry seq = round << 24 | count; those of a
 // window's parallel pass have seq < 2^24.
@@ -129,16 +124,6 @@ __device__ __forceinline__ void red_min_u64(unsigned long long *p, unsigned long
     asm volatile("red.relaxed.gpu.global.min.u64 [%0], %1;" ::"l"(p), "l"(v));
 }
 
-// A chain blocked by the window's parallel pass (one thread): counted, listed
-// for the union-find, and counted against its partner.
-template <class S>
-__device__ __forceinline__ void note_blocked(const S &s, int c, int32_t partner) {
-    atomicAdd(s.lc + LC_BLOCKED, 1ull);
-    const unsigned long long ix = atomicAdd(s.lc + LC_WBLOCKED, 1ull);
-    if (ix < (unsigned long long)s.k) s.blist[ix] = c;
-    if (partner >= 0 && partner < s.k) atomicAdd(s.pcnt + partner, 1);
-}
-
 __device__ int uf_find(int32_t *p, int x) {
     for (;;) {
         const int px = ((volatile int32_t *)p)[x];
@@ -198,130 +183,30 @@ __device__ int block_exscan(int v, int *warp_tot, int *total) {
 constexpr int UF_SMEM_CAP = 2048;
 constexpr size_t UF_SMEM_BYTES = 4 * UF_SMEM_CAP * sizeof(int32_t);
 
-// Conflict components (one block). first: edges from the parallel pass
-// (blocked chain -> holder of the claim it met); later rounds: edges from
-// components that met another chain. Components holding a chain whose events
-// are not final ("dirty") are listed for the repair with their members.
-// reset_abort: clear the abort count here (the persistent kernels clear it
-// elsewhere, after every block has read it).
-// sm (UF_SMEM_BYTES of shared memory, or null): with k <= UF_SMEM_CAP the
-// parents, counts, roots and flags live there during the phases (each phase
-// then waits on shared instead of global memory) and are written back to
-// s.uf, s.comp_of and s.fin at the end.
-// Round 1 when every blocked chain makes a pair with its partner alone (the
-// common case): blist[0 .. nblk) are the window's blocked chains, pcnt[c]
-// the blocked chains naming c as partner. A pair {a, p} is a component when
-// nobody names a (pcnt[a] = 0), only a names p (pcnt[p] = 1) and p is not
-// blocked; a chain without a partner is a component alone. Then the result
-// is the dense union-find's, written directly: identity for every chain in
-// no component, the root (the smaller index) for the members, components in
-// increasing root order, the blocked member first. Returns false (nothing
-// written) otherwise. Either way pcnt is back to 0 for the chains listed.
+// Conflict components after the first repair round (one block): the trees in
+// s.uf, with an edge from each component that met another chain (abort_to of
+// its root, cleared here). Components holding a chain whose events are not
+// final ("dirty") are listed for the repair with their members.
+// sm (UF_SMEM_BYTES of shared memory): with k <= UF_SMEM_CAP the parents,
+// counts, roots and flags live there during the phases (each phase then waits
+// on shared instead of global memory) and are written back to s.uf, s.comp_of
+// and s.fin at the end.
 template <class S>
-__device__ bool uf_pairs(const S &s, const int32_t *blist, int32_t *pcnt, int nblk,
-                         bool reset_abort, int32_t *sm) {
+__device__ void uf_block(const S &s, int *warp_tot, int *tot, int32_t *sm) {
     const int k = s.k, tid = threadIdx.x, nt = blockDim.x;
-    int a = -1, p = -1;
-    bool simple = true;
-    if (tid < nblk) {
-        a = blist[tid];
-        p = s.partner[a];
-        if (p < 0 || p >= k) p = -1;
-        const int pa = pcnt[a];
-        const int pp = p >= 0 ? pcnt[p] : 1;
-        const int sp = p >= 0 ? s.status[p] : ST_STALLED;
-        simple = pa == 0 && (p < 0 || (pp == 1 && sp != ST_BLOCKED));
-    }
-    const bool ok = __syncthreads_and(simple) != 0;
-    if (tid < nblk && p >= 0) pcnt[p] = 0;
-    if (!ok) return false;
-    for (int c = tid; c < k; c += nt) {
-        s.uf[c] = c;
-        s.comp_of[c] = c;
-        s.fin[c] = 1;
-        s.abort_to[c] = -1;
-    }
-    // the pairs by root: rank and offset among them
-    int32_t *root_sm = sm, *size_sm = sm + 64;
-    const int root = p >= 0 ? min(a, p) : a;
-    if (tid < nblk) {
-        root_sm[tid] = root;
-        size_sm[tid] = p >= 0 ? 2 : 1;
-    }
-    __syncthreads();
-    if (tid < nblk) {
-        int rank = 0, off = 0, total = 0;
-        for (int j = 0; j < nblk; ++j) {
-            total += size_sm[j];
-            if (root_sm[j] < root) {
-                ++rank;
-                off += size_sm[j];
-            }
-        }
-        s.uf[a] = root;
-        s.comp_of[a] = root;
-        s.fin[a] = 0;
-        s.comp_root[rank] = root;
-        s.comp_off[rank] = off;
-        s.comp_mem[off] = a;
-        if (p >= 0) {
-            s.uf[p] = root;
-            s.comp_of[p] = root;
-            s.fin[p] = 0;
-            s.comp_mem[off + 1] = p;
-        }
-        if (rank == 0) {
-            s.comp_off[nblk] = total;
-            s.ctl[CTL_NCOMP] = nblk;
-            s.ctl[CTL_NMEMB] = total;
-            s.ctl[CTL_WORK] = 0;
-            if (reset_abort) s.ctl[CTL_NABORT] = 0;
-        }
-    }
-    __syncthreads();
-    return true;
-}
-
-template <class S>
-__device__ void uf_block(const S &s, int first, int *warp_tot, int *tot, bool reset_abort,
-                         int32_t *sm = nullptr, const int32_t *blist = nullptr,
-                         int32_t *pcnt = nullptr, int nblk = -1) {
-    const int k = s.k, tid = threadIdx.x, nt = blockDim.x;
-    if (first && blist && sm && nblk >= 1 && nblk <= 64 && nblk <= nt) {
-        if (uf_pairs(s, blist, pcnt, nblk, reset_abort, sm)) return;
-        __syncthreads();
-    } else if (first && blist && pcnt) {
-        // (the dense pass does not read the partner counts: back to 0)
-        for (int q = tid; q < nblk && q < k; q += nt) {
-            const int p = s.partner[blist[q]];
-            if (p >= 0 && p < k) pcnt[p] = 0;
-        }
-    }
-    const bool local = sm != nullptr && k <= UF_SMEM_CAP;
+    const bool local = k <= UF_SMEM_CAP;
     int32_t *uf = local ? sm : s.uf;
     int32_t *cnt = local ? sm + UF_SMEM_CAP : s.comp_cnt;
     int32_t *cof = local ? sm + 2 * UF_SMEM_CAP : s.comp_of;
     int32_t *fin = local ? sm + 3 * UF_SMEM_CAP : s.fin;
-    for (int c = tid; c < k; c += nt) {
-        if (first) {
-            uf[c] = c;
-            fin[c] = s.status[c] != ST_BLOCKED;
-            s.abort_to[c] = -1;
-        } else if (local) {
-            // (adoptions in the last round may have joined trees in s.uf)
-            uf[c] = s.uf[c];
-            fin[c] = s.fin[c];
-        }
+    for (int c = tid; c < k && local; c += nt) {
+        uf[c] = s.uf[c];
+        fin[c] = s.fin[c];
     }
     __syncthreads();
     for (int c = tid; c < k; c += nt) {
-        int other = -1;
-        if (first) {
-            if (s.status[c] == ST_BLOCKED) other = s.partner[c];
-        } else {
-            other = s.abort_to[c];
-            s.abort_to[c] = -1;
-        }
+        const int other = s.abort_to[c];
+        s.abort_to[c] = -1;
         if (other >= 0 && other < k) uf_union(uf, c, other);
     }
     __syncthreads();
@@ -376,8 +261,6 @@ __device__ void uf_block(const S &s, int first, int *warp_tot, int *tot, bool re
         s.comp_off[tot[1]] = tot[0];
         s.ctl[CTL_NCOMP] = tot[1];
         s.ctl[CTL_NMEMB] = tot[0];
-        s.ctl[CTL_WORK] = 0;
-        if (reset_abort) s.ctl[CTL_NABORT] = 0;
     }
     __syncthreads();
 }

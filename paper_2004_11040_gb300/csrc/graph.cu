@@ -1,6 +1,7 @@
-// graph.cu -- libecmc's constraint-graph path (ECMC_GRAPH): the liftings of
-// a chain are found through the arrows of the constraint graph G(3) of
-// Sec. 3.1 instead of a scan of the cells ahead.
+// graph.cu -- the legs of libecmc. The liftings of a chain are found through the
+// arrows of the constraint graph G(3) of Sec. 3.1; contexts differ in the
+// conflict flag, which is on the disks a chain reads (ECMC_GRAPH) or on the
+// cells that the scans of a cell search would cover.
 //
 // For v = (1, 0) the arrows of disk i are, in each of three corridors of
 // dy = y_j - y_i (minimum image) -- centre |dy| < d/2, upper d/2 <= dy < d,
@@ -21,7 +22,11 @@
 // each run alone, overlap. Chains that were cut are continued one after
 // another where Eq. 2 allows it, else rolled back to the earliest time one of
 // them stopped and replayed in global event-time order (Alg. 2), one warp per
-// conflict component, as on the cell path.
+// conflict component.
+//
+// A frame whose cell rows are out of reach of each other (a lattice start on
+// cells aligned with it) is a set of rings, on which runs and continuations
+// are stretches of consecutive disks (frames of rings, below).
 //
 // All FP64 arithmetic uses explicit round-to-nearest intrinsics (the file is
 // compiled with -fmad=false) so that results are reproducible bit for bit.
@@ -35,6 +40,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -89,20 +95,19 @@ struct GDev {
     uint32_t *path;        // [(cap + 2) * k]
     unsigned long long *fl;  // flag words, epoch << 32 | chain + 1: per disk read, or
                              // per cell scanned
-    // a cell-scan context's frame (cells != 0: its flag is on cells): the left
-    // edges of the columns, the stop rule, and per entry of path what its
-    // step's scan needs -- the active disk's x and the least of D and its best
-    // time of flight, and its cell
+    // a cell-scan context (cells != 0: its flag is on cells): the stop rule of
+    // the scan, and per entry of path what its step's scan needs -- the active
+    // disk's x and the least of D and its best time of flight, and its cell
     int cells;
     double inv_a;
-    const double *colx;   // [nc]
     StopK sk;
     double2 *pxt;         // [(cap + 2) * k]
     uint32_t *pcell;      // [(cap + 2) * k]
     // a frame of rings (ring != 0): the disks ring after ring, each in the order
-    // of x, and every disk's place there
+    // of x; every disk's place there, its ring's first place and length, its row
     int ring;
-    uint32_t *rid, *posof;  // [n]
+    uint32_t *rid;  // [n]
+    uint4 *pos;     // [n]
     uint32_t epoch0;       // epoch of the launch's first pass, less one
     GSpec *sp;             // [k] the run alone of each chain, for the resolve
     uint32_t stamp0;       // stamp of the launch's first leg, less one
@@ -192,8 +197,7 @@ __device__ __forceinline__ double shfl_f64(double v, int src) {
 // Inputs and scratch of a build: a cell list of the disks (in any of a cell's
 // slots), their FP32 coordinates per slot relative to the cell's corner (an
 // error of 1e-7 d whatever the box), and one bit per y bin of width d/128 that
-// holds a disk. The disks come by id (x, y, placed by k_gb_cells)
-// or, sx != null, from the slots of a cell-scan context.
+// holds a disk.
 struct GBuild {
     int64_t n;
     int nc, nb;
@@ -202,7 +206,6 @@ struct GBuild {
     float del;           // a 2^-20: bound on the FP32 error of a difference of
                          // coordinates of neighbouring cells
     const double *x, *y;
-    const double *sx, *sy;
     const uint32_t *scid;  // [nc*nc*C] disk per slot, EMPTY
     uint32_t *cid;         // the same, writable (null with sx)
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
@@ -250,20 +253,6 @@ __global__ void k_gb_cells(GBuild b) {
         }
     }
     atomicAdd(b.err, 1ull);
-}
-
-// FP32 coordinates and bins from the slots of a cell-scan context.
-template <int C>
-__global__ void k_gb_slots(GBuild b, uint32_t nslot) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nslot) return;
-    float2 v = make_float2(__int_as_float(-1), __int_as_float(-1));
-    if (b.scid[q] != EMPTY) {
-        const uint32_t cell = q / C;
-        v = in_cell(b, b.sx[q], b.sy[q], (int)(cell / (uint32_t)b.nc), (int)(cell % (uint32_t)b.nc));
-        set_bin(b, d2f_trunc(b.sy[q]));
-    }
-    b.cxy[q] = v;
 }
 
 // Does a bin that meets [lo, hi) (periodic, hi - lo < L) hold a disk? The
@@ -341,10 +330,10 @@ __device__ __forceinline__ bool take_best(GBest &best, float lo, float hi, uint3
 }
 
 __device__ __forceinline__ double gb_x(const GBuild &b, uint32_t loc, uint32_t id) {
-    return b.sx ? b.sx[loc] : b.x[id];
+    return b.x[id];
 }
 __device__ __forceinline__ double gb_y(const GBuild &b, uint32_t loc, uint32_t id) {
-    return b.sx ? b.sy[loc] : b.y[id];
+    return b.y[id];
 }
 
 // The FP32 coordinates of a cell's slots, all loads at once.
@@ -684,102 +673,166 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
 // chain's run is a stretch of consecutive places (g_leap_chain) instead of a
 // walk from record to record. The cells' row bands decide (k_skip).
 
-// What a record of a ring frame holds in b[1] and b[2] (a[1] and a[2] are
-// NONE): its ring's first place and length, and its row of cells.
-__device__ __forceinline__ double two_words(uint32_t lo, uint32_t hi) {
-    return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
-}
+constexpr double RING_SPREAD = 0.86;
+constexpr int RING_CHUNK = 256;  // columns of a row per block of the kernels below
 
-// Disks per cell row (one block per row).
-__global__ void __launch_bounds__(256) k_ring_count(GBuild b, int C, uint32_t *row_off) {
-    const uint32_t nrow = (uint32_t)b.nc * (uint32_t)C, q0 = blockIdx.x * nrow;
+struct GRing {
+    uint32_t *off;             // [nc * chunks + 1] disks per chunk, then first places
+    unsigned long long *band;  // [2 nc] least and largest y (bits) per row
+};
+
+static int ring_chunks(int nc) { return (nc + RING_CHUNK - 1) / RING_CHUNK; }
+
+// Disks per chunk, and the rows' bands (least: all ones; largest: 0 before).
+template <int C>
+__global__ void __launch_bounds__(RING_CHUNK) k_ring_count(GBuild b, GRing r) {
+    __shared__ unsigned long long wlo[RING_CHUNK / 32], whi[RING_CHUNK / 32];
+    __shared__ int wn[RING_CHUNK / 32];
+    const uint32_t nc = (uint32_t)b.nc, row = blockIdx.y;
+    const uint32_t col = blockIdx.x * RING_CHUNK + threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned long long lo = INF_BITS, hi = 0ull;
     int n = 0;
-    for (uint32_t o0 = 0; o0 < nrow; o0 += blockDim.x) {
-        const uint32_t o = o0 + threadIdx.x;
-        n += __syncthreads_count(o < nrow && b.scid[q0 + o] != EMPTY);
+    if (col < nc) {
+        uint32_t id[C];
+        const uint4 *q = reinterpret_cast<const uint4 *>(b.scid + ((size_t)row * nc + col) * C);
+#pragma unroll
+        for (int z = 0; z < C / 4; ++z) {
+            const uint4 v = q[z];
+            id[4 * z] = v.x;
+            id[4 * z + 1] = v.y;
+            id[4 * z + 2] = v.z;
+            id[4 * z + 3] = v.w;
+        }
+#pragma unroll
+        for (int z = 0; z < C; ++z) {
+            if (id[z] == EMPTY) continue;
+            const unsigned long long y = dbits(b.y[id[z]]);  // y >= 0: ordered by bits
+            lo = y < lo ? y : lo;
+            hi = y > hi ? y : hi;
+            ++n;
+        }
     }
-    if (threadIdx.x == 0) row_off[blockIdx.x] = (uint32_t)n;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long l2 = shfl_xor_u64(lo, o), h2 = shfl_xor_u64(hi, o);
+        lo = l2 < lo ? l2 : lo;
+        hi = h2 > hi ? h2 : hi;
+        n += __shfl_xor_sync(FULL, n, o);
+    }
+    if (lane == 0) {
+        wlo[w] = lo;
+        whi[w] = hi;
+        wn[w] = n;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < RING_CHUNK / 32; ++q) {
+            lo = wlo[q] < lo ? wlo[q] : lo;
+            hi = whi[q] > hi ? whi[q] : hi;
+            n += wn[q];
+        }
+        if (n) {
+            atomicMin(r.band + row, lo);
+            atomicMax(r.band + nc + row, hi);
+        }
+        r.off[row * gridDim.x + blockIdx.x] = (uint32_t)n;
+    }
 }
 
-// Counts to first places (one block).
-__global__ void k_ring_offsets(int nc, uint32_t *row_off) {
+// The rows that are no rings (added to *bad), and the chunks' first places
+// (one block). Two neighbour rows lie d apart when RN(ylo(above) - yhi(below))
+// >= d: rounding is monotone, so |RN(dy)| >= d for every pair; across the box
+// edge RN(L - RN(yhi(nc - 1) - ylo(0))) bounds every pair's periodic image.
+__global__ void k_ring_rows(GBuild b, GRing r, int chunks, unsigned long long *bad) {
     __shared__ int warp_tot[32];
     __shared__ int tot[2];
-    const int chunk = (nc + blockDim.x - 1) / blockDim.x;
-    const int lo = min(nc, (int)threadIdx.x * chunk), hi = min(nc, lo + chunk);
+    const int nc = b.nc;
+    bool no = nc < 5;
+    for (int q = threadIdx.x; q < nc; q += blockDim.x) {
+        const unsigned long long l = r.band[q];
+        if (l == ~0ull) continue;
+        const double yl = __longlong_as_double((long long)l),
+                     yh = __longlong_as_double((long long)r.band[nc + q]);
+        no = no || !(__dsub_rn(yh, yl) < __dmul_rn(RING_SPREAD, b.d));
+        const int up = q == nc - 1 ? 0 : q + 1;
+        const unsigned long long u = r.band[up];
+        if (u != ~0ull) {
+            const double yu = __longlong_as_double((long long)u);
+            no = no || !((up ? __dsub_rn(yu, yh) : __dsub_rn(b.L, __dsub_rn(yh, yu))) >= b.d);
+        }
+    }
+    const int any = __syncthreads_or(no);
+    const int n = nc * chunks, per = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int lo = min(n, (int)threadIdx.x * per), hi = min(n, lo + per);
     int sum = 0;
-    for (int q = lo; q < hi; ++q) sum += (int)row_off[q];
+    for (int q = lo; q < hi; ++q) sum += (int)r.off[q];
     int off = block_exscan(sum, warp_tot, tot);
     for (int q = lo; q < hi; ++q) {
-        const int n = (int)row_off[q];
-        row_off[q] = (uint32_t)off;
-        off += n;
+        const int c = (int)r.off[q];
+        r.off[q] = (uint32_t)off;
+        off += c;
     }
-    if (threadIdx.x == 0) row_off[nc] = (uint32_t)tot[0];
+    if (threadIdx.x == 0) {
+        r.off[n] = (uint32_t)tot[0];
+        if (any) *bad = 1ull;
+    }
 }
 
-// The places and records of a frame of rings (one block per row): a cell's
-// disks, in the order of x, follow those of the cells before; then every disk
-// gets its record, its successor the only arrow. Bound by the records' 64
-// bytes per disk.
+// Places: a cell's disks, in the order of x, follow those of the cells before.
 template <int C>
-__global__ void __launch_bounds__(256) k_ring_place(GBuild b, const uint32_t *row_off, GDev s) {
+__global__ void __launch_bounds__(RING_CHUNK) k_ring_place(GBuild b, GRing r, GDev s) {
     __shared__ int warp_tot[32];
     __shared__ int tot[2];
-    const uint32_t nc = (uint32_t)b.nc, first = row_off[blockIdx.x];
-    const uint32_t len = row_off[blockIdx.x + 1] - first;
-    uint32_t at0 = first;
-    for (uint32_t c0 = 0; c0 < nc; c0 += blockDim.x) {
-        const uint32_t col = c0 + threadIdx.x;
-        uint32_t id[C];
-        double x[C], y[C];
-        int n = 0;
-        if (col < nc) {
-            const uint32_t loc = (blockIdx.x * nc + col) * C;
+    const uint32_t nc = (uint32_t)b.nc, row = blockIdx.y, ch = gridDim.x;
+    const uint32_t col = blockIdx.x * RING_CHUNK + threadIdx.x;
+    const uint32_t first = r.off[row * ch], len = r.off[(row + 1) * ch] - first;
+    uint32_t id[C];
+    double x[C];
+    int n = 0;
+    if (col < nc) {
 #pragma unroll
-            for (int q = 0; q < C; ++q) {
-                id[q] = b.scid[loc + q];
-                x[q] = INFINITY;
-                y[q] = 0.0;
-                if (id[q] != EMPTY) {
-                    x[q] = b.sx[loc + q];
-                    y[q] = b.sy[loc + q];
-                    ++n;
-                }
-            }
+        for (int q = 0; q < C; ++q) id[q] = b.scid[((size_t)row * nc + col) * C + q];
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            x[q] = id[q] != EMPTY ? b.x[id[q]] : INFINITY;
+            n += id[q] != EMPTY;
         }
-        const uint32_t at = at0 + (uint32_t)block_exscan(n, warp_tot, tot);
-        if (n > 0) {
-#pragma unroll
-            for (int q = 0; q < C; ++q) {
-                if (id[q] == EMPTY) continue;
-                int rank = 0;  // x >= 0: ordered by bits
-#pragma unroll
-                for (int z = 0; z < C; ++z)
-                    rank += dbits(x[z]) < dbits(x[q]) || (z < q && dbits(x[z]) == dbits(x[q]));
-                const uint32_t p = at + (uint32_t)rank;
-                s.rid[p] = id[q];
-                s.posof[id[q]] = p;
-                s.y[id[q]] = y[q];
-                s.g[id[q]].x = x[q];
-            }
-        }
-        at0 += (uint32_t)tot[0];
-        __syncthreads();
     }
-    for (uint32_t o = threadIdx.x; o < len; o += blockDim.x) {
-        const uint32_t i = s.rid[first + o], j = s.rid[first + (o + 1 < len ? o + 1 : 0)];
-        const double ay = fabs(__dsub_rn(s.y[j], s.y[i]));
-        const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
-        const bool has = len > 1;
-        ulonglong2 *g = reinterpret_cast<ulonglong2 *>(s.g + i);
-        s.g[i].t = 0.0;
-        g[1] = make_ulonglong2((unsigned long long)OWN_STATIC |
-                                   ((unsigned long long)(has ? j : NONE) << 32),
-                               ~0ull);
-        g[2] = make_ulonglong2(0ull, has ? dbits(v) : 0ull);
-        g[3] = make_ulonglong2(dbits(two_words(first, len)), dbits(two_words(blockIdx.x, 0u)));
+    const uint32_t at = r.off[row * ch + blockIdx.x] + (uint32_t)block_exscan(n, warp_tot, tot);
+    if (n == 0) return;
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+        if (id[q] == EMPTY) continue;
+        int rank = 0;  // x >= 0: ordered by bits
+#pragma unroll
+        for (int z = 0; z < C; ++z)
+            rank += dbits(x[z]) < dbits(x[q]) || (z < q && dbits(x[z]) == dbits(x[q]));
+        s.rid[at + rank] = id[q];
+        s.pos[id[q]] = make_uint4(at + (uint32_t)rank, first, len, row);
     }
+}
+
+// The records of a frame of rings, each disk's successor its only arrow (a
+// cell-scan context; one with graph arrows has them from k_gb_arrows). Bound
+// by the 64 bytes a record takes.
+__global__ void k_ring_records(GBuild b, GDev s) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= s.n) return;
+    const uint32_t i = s.rid[p];
+    const uint4 at = s.pos[i];
+    const uint32_t j = s.rid[(uint32_t)p + 1u < at.y + at.z ? (uint32_t)p + 1u : at.y];
+    const double yi = b.y[i], ay = fabs(__dsub_rn(b.y[j], yi));
+    const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
+    const bool has = at.z > 1u;
+    ulonglong2 *g = reinterpret_cast<ulonglong2 *>(s.g + i);
+    g[0] = make_ulonglong2(dbits(b.x[i]), 0ull);
+    g[1] = make_ulonglong2((unsigned long long)OWN_STATIC |
+                               ((unsigned long long)(has ? j : NONE) << 32),
+                           ~0ull);
+    g[2] = make_ulonglong2(0ull, has ? dbits(v) : 0ull);
+    g[3] = make_ulonglong2(0ull, 0ull);
+    s.y[i] = yi;
 }
 
 // The chains' start disks active (after a build).
@@ -1192,7 +1245,7 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         r.n = n;
         r.touch = end == SP_STALL ? n : n + 1;
         r.end = end | (n > n_lap ? SP_LAP : 0);
-        if (s.ring && strict && n > 0 && (uint32_t)n >= (uint32_t)(dbits(g[i].b[1]) >> 32))
+        if (s.ring && strict && n > 0 && (uint32_t)n >= s.pos[i].z)
             atomicAdd(s.lc + LC_RINGLAP, 1ull);
         r.partner = partner < (uint32_t)s.k ? (int32_t)partner : -1;
         r.tc = ti;
@@ -1235,6 +1288,34 @@ __device__ __forceinline__ void g_sums(double tau, int bound, double &t, double 
     D = lane < 16 ? da : db;
 }
 
+// A disk of a ring as a stretch needs it: the record in three loads, four where
+// it has more than one arrow.
+struct GRingDisk {
+    double x, t;
+    uint32_t own, a0, a1, a2;
+    unsigned long long claim;
+    double b0, b1, b2;
+    __device__ __forceinline__ explicit GRingDisk(const GDisk *g) {
+        const ulonglong2 *const r = reinterpret_cast<const ulonglong2 *>(g);
+        const ulonglong2 r0 = __ldcg(r), r1 = __ldcg(r + 1), r2 = __ldcg(r + 2), r3 = __ldcg(r + 3);
+        x = __longlong_as_double((long long)r0.x);
+        t = __longlong_as_double((long long)r0.y);
+        own = (uint32_t)r1.x;
+        a0 = (uint32_t)(r1.x >> 32);
+        a1 = (uint32_t)r1.y;
+        a2 = (uint32_t)(r1.y >> 32);
+        claim = r2.x;
+        b0 = __longlong_as_double((long long)r2.y);
+        b1 = __longlong_as_double((long long)r3.x);
+        b2 = __longlong_as_double((long long)r3.y);
+    }
+    // b towards disk j; false if no arrow leads there
+    __device__ __forceinline__ bool towards(uint32_t j, double &b) const {
+        b = a0 == j ? b0 : a1 == j ? b1 : b2;
+        return a0 == j || a1 == j || a2 == j;
+    }
+};
+
 // The same pass in a frame of rings, of a leg from its start (not strict): the
 // run's disks are consecutive places, so lane e holds the e-th from the active
 // disk on and finds its gap to the next; only the sums of Eq. 1 -- the time and
@@ -1252,10 +1333,8 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c, bool begin) {
     if (begin) g_begin_state(s, c, i0, lane);
     const GDisk *const g = s.g;
     const double L = s.L;
-    const uint32_t p0 = s.posof[i0];
-    const unsigned long long info = dbits(g[i0].b[1]);
-    const uint32_t row = (uint32_t)dbits(g[i0].b[2]);
-    const uint32_t first = (uint32_t)info, len = (uint32_t)(info >> 32);
+    const uint4 at0 = s.pos[i0];
+    const uint32_t p0 = at0.x, first = at0.y, len = at0.z, row = at0.w;
     uint32_t id = 0u;
     double t = 0.0, D = s.ell;  // before the event on lane 0
     int n0 = 0, end = SP_STALL, n = 0;
@@ -1268,13 +1347,15 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c, bool begin) {
         uint32_t q = p0 - first + (uint32_t)(n0 + lane);
         if (q >= len) q %= len;
         id = s.rid[first + q];
-        const double x = g[id].x, bb = g[id].b[0];
-        const uint32_t own = g[id].own;
+        const GRingDisk k(g + id);
+        const double x = k.x;
+        const uint32_t own = k.own;
         const double xn = shfl_f64(x, (lane + 1) & 31);
         const uint32_t idn = __shfl_sync(FULL, id, (lane + 1) & 31);
         const uint32_t ownn = __shfl_sync(FULL, own, (lane + 1) & 31);
+        double bb;
         // targets: the last but one of the ring is the last the run has not moved
-        const bool in = lane < 31 && (uint32_t)(n0 + lane) + 1u < len;
+        const bool in = lane < 31 && (uint32_t)(n0 + lane) + 1u < len && k.towards(idn, bb);
         const bool nsc = in && ownn >= OWN_ACTIVE;
         double dx = __dsub_rn(xn, x);
         const bool neg = __double_as_longlong(dx) < 0;
@@ -1303,7 +1384,7 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c, bool begin) {
         const bool wrap = has && dbits(xe) >= dbits(L);
         if (__any_sync(FULL, wrap) && wrap) xe = g_sub(xe, L);
         const double tn = stall ? tn_stall : tn_lift;
-        if (has || (met && lane == f)) {
+        if (s.cells && (has || (met && lane == f))) {
             const size_t at = (size_t)e * (size_t)s.k + (size_t)c;
             s.pxt[at] = make_double2(x, has ? ts : D);
             s.pcell[at] = row * (uint32_t)s.nc + (uint32_t)cell_coord(x, s.inv_a, s.nc);
@@ -1403,7 +1484,7 @@ __device__ __noinline__ void g_flag_chain(const GDev &s, int c, uint32_t epoch, 
         const double2 xt = s.pxt[at];
         const uint32_t cell = s.pcell[at];
         const int nc = s.nc, cy = (int)(cell / (uint32_t)nc), cx = (int)(cell % (uint32_t)nc);
-        const double fx = __dsub_rn(xt.x, s.colx[cx]);
+        const double fx = __dsub_rn(xt.x, __dmul_rn((double)cx, s.sk.a));
         const float fxf = d2f_trunc(fx), lim_f = __fadd_rn(d2f_trunc(xt.y), s.sk.epsf);
         const int rdn = cy == 0 ? nc - 1 : cy - 1, rup = cy == nc - 1 ? 0 : cy + 1;
         unsigned long long *const f0 = s.fl + (size_t)rdn * (size_t)nc,
@@ -2330,27 +2411,24 @@ __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, i
         double t = s.tc[c], D = s.D[c];
         const int32_t nr0 = s.nrec[c];
         const uint32_t seq0 = ((uint32_t)round << 24) | cnt;
-        const uint32_t p0 = s.posof[i];
-        const unsigned long long info = dbits(g[i].b[1]);
-        const uint32_t first = (uint32_t)info, len = (uint32_t)(info >> 32);
+        const uint4 at0 = s.pos[i];
+        const uint32_t p0 = at0.x, first = at0.y, len = at0.z;
         int nl = 0, n = 0, st = ST_RUNNING, next = -1, how = CONT_DONE;
         for (bool more = true; more;) {
             uint32_t q = p0 - first + (uint32_t)(n + lane);
             if (q >= len) q %= len;
             const uint32_t id = s.rid[first + q];
-            const ulonglong2 *const r = reinterpret_cast<const ulonglong2 *>(g + id);
-            const ulonglong2 r0 = __ldcg(r), r1 = __ldcg(r + 1), r2 = __ldcg(r + 2);
-            const double x = __longlong_as_double((long long)r0.x);
-            const double xn = shfl_f64(x, up);
-            const double rt = __longlong_as_double((long long)shfl_u64(r0.y, up));
-            const uint32_t ownn = __shfl_sync(FULL, (uint32_t)r1.x, up);
+            const GRingDisk k(g + id);
+            const double x = k.x, xn = shfl_f64(x, up), rt = shfl_f64(k.t, up);
+            const uint32_t ownn = __shfl_sync(FULL, k.own, up);
             const uint32_t idn = __shfl_sync(FULL, id, up);
-            const bool in = lane < 31 && (uint32_t)(n + lane) + 1u < len;
+            double bb;
+            const bool in = lane < 31 && (uint32_t)(n + lane) + 1u < len && k.towards(idn, bb);
             const bool nsc = in && ownn >= OWN_ACTIVE;
             double dx = __dsub_rn(xn, x);
             const bool neg = __double_as_longlong(dx) < 0;
             if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
-            double tau = __dsub_rn(dx, __longlong_as_double((long long)r2.y));
+            double tau = __dsub_rn(dx, bb);
             if (__double_as_longlong(tau) < 0) tau = 0.0;
             const unsigned stops = __ballot_sync(FULL, lane < 31 && (nsc || !in));
             g_sums(tau, stops ? __ffs(stops) - 1 : 31, t, D);
@@ -2370,8 +2448,8 @@ __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, i
             // the disks read, the active one and the targets of the events up to f
             uint32_t h = 0u;
             if (lane <= (fin ? f + 1 : 31)) {
-                h = g_holder(r2.x, ct);
-                if (h == 0u) h = g_holder(atomicCAS(&g[id].claim, r2.x, ct), ct);
+                h = g_holder(k.claim, ct);
+                if (h == 0u) h = g_holder(atomicCAS(&g[id].claim, k.claim, ct), ct);
             }
             const bool ask = h != 0u && h != mine;
             unsigned fb = 0u;
@@ -2930,6 +3008,7 @@ struct GCtl {
     int32_t flags_cap;
     int32_t done;    // budget reached or error
     int32_t err;     // LC_ERR_* seen, or too many repair rounds
+    int32_t failed;  // 1 until a leg is done without one
     int32_t dbg;     // an internal check recorded in GDev::dbg (set at the end)
 };
 
@@ -3081,7 +3160,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 if (to != c) uf_union(s.uf, c, to);
             }
             __syncthreads();
-            uf_block(s, 0, warp_tot, tot, false, uf_sm);
+            uf_block(s, warp_tot, tot, uf_sm);
         } else if (threadIdx.x == 0) {
             s.ctl[CTL_NCOMP] = 0;
             if (need) atomicAdd(s.lc + LC_ERR_CAP, 1ull);  // too many rounds
@@ -3130,10 +3209,11 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         c.restarts += (int64_t)lc[LC_RESTARTS];
         c.blocked += (int64_t)lc[LC_BLOCKED];
         c.cwindows += fast ? flag : (int64_t)lc[LC_CWINDOWS];
-        if (B.reps[r].ring && lc[LC_RINGLAP] == 0ull) c.row_windows += B.windows;
+        if (B.reps[r].ring && B.reps[r].cells && lc[LC_RINGLAP] == 0ull) c.row_windows += B.windows;
         c.horizon += (int64_t)lc[LC_HORIZON];
         c.order_err += (int64_t)lc[LC_ORDER];
         if (lc[LC_ERR_REC] != 0ull || lc[LC_ERR_CAP] != 0ull) c.err = 1;
+        c.failed = c.err;
         if (c.err || (c.budget > 0 && c.lifts >= c.budget)) c.done = 1;
         *cp = c;
 #pragma unroll
@@ -3378,16 +3458,17 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
 }
 
 // Exports positions (per disk id), local times and active disks.
-__global__ void k_g_export(GDev s, double *x, double *t) {
+// failed: a word that is not 0 if nothing is to be written (or null).
+__global__ void k_g_export(GDev s, double *x, double *t, const int32_t *failed) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= s.n) return;
+    if (q >= s.n || (failed && *failed)) return;
     if (x) x[q] = s.g[q].x;
     if (t) t[q] = g_time(s.g[q].own, s.g[q].t, s.stamp0);
 }
 
-__global__ void k_g_export_active(GDev s, int32_t *active) {
+__global__ void k_g_export_active(GDev s, int32_t *active, const int32_t *failed) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < s.k) active[c] = (int32_t)s.ci[c];
+    if (c < s.k && !(failed && *failed)) active[c] = (int32_t)s.ci[c];
 }
 
 // Direction change: the disks' x and y are exchanged (x from y_old, y from
@@ -3415,9 +3496,10 @@ struct GraphCtx {
     int64_t log_legs = 0;  // legs logged so far (leg index of the log)
     GBatchScratch *launch = nullptr;  // launch tables of graph_run
     void *build_tmp = nullptr;        // scratch of graph_build
-    float2 *slot_xy = nullptr;        // scratch of graph_activate
-    uint32_t *slot_bits = nullptr;
-    uint32_t *row_off = nullptr;      // [nc + 1]
+    GRing ring = {};
+    int C = 4;                          // slots per cell of a build
+    bool try_ring[2] = {false, false};  // per axis: its last frame was of rings, or none was
+    int axis = 0;
     std::vector<std::pair<void **, size_t>> pending;
     int64_t bytes = 0;  // device memory held
 };
@@ -3427,10 +3509,9 @@ namespace {
 // Device arrays of a context: requested one by one, then placed in a single
 // allocation (each on a 256-byte boundary) by gcommit.
 template <typename T>
-int galloc(GraphCtx *g, T **ptr, size_t count, std::string &) {
+void galloc(GraphCtx *g, T **ptr, size_t count) {
     *ptr = nullptr;
     g->pending.emplace_back((void **)ptr, std::max<size_t>(count, 1) * sizeof(T));
-    return 0;
 }
 
 int gcommit(GraphCtx *g, std::string &err) {
@@ -3472,9 +3553,13 @@ static int64_t graph_build_bytes(double L, double d, int nc, int C) {
     return (int64_t)build_parts(L, d, nc, C, &a, &b, &c);
 }
 
-// Builds the records (x, t = 0, static, arrows) of every disk from positions
-// x, y (device); queued on the context's stream. An overfull cell is counted
-// in *err_dev (device).
+static int launched(const char *what, std::string &err) {
+    const cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) return 0;
+    err = std::string(what) + ": " + cudaGetErrorString(e);
+    return ECMC_ECUDA;
+}
+
 // The constants of a build.
 static GBuild build_params(const GraphCtx *g) {
     const GDev &s = g->s;
@@ -3500,18 +3585,20 @@ static GBuild build_params(const GraphCtx *g) {
     return b;
 }
 
-static int graph_build(GraphCtx *g, const double *x, const double *y, unsigned long long **err_dev,
+// The first half of a frame's build, queued on the context's stream: every
+// disk in a cell, and whether the rows are rings (asked again on an axis only
+// while they were: rows that motion across them has mixed stay mixed).
+// b.err[0] counts overfull cells, b.err[1] rows that are no rings.
+static int graph_place(GraphCtx *g, const double *x, const double *y, GBuild *out,
                        std::string &err) {
     GDev &s = g->s;
     const int nc = g->nc;
-    // slots per cell: at most 4 centres at mutual distance >= d fit in a cell
-    // with a < sqrt(2) d, at most 6 for a < 1.664 d
-    const int C = g->box / nc < std::sqrt(2.0) * s.d * (1.0 - 1e-9) ? 4 : 8;
     GBuild b = build_params(g);
     b.x = x;
     b.y = y;
+    b.yout = s.y;
     size_t off_bits, off_err, off_cid;
-    const size_t total = build_parts(s.L, s.d, nc, C, &off_bits, &off_err, &off_cid);
+    const size_t total = build_parts(s.L, s.d, nc, g->C, &off_bits, &off_err, &off_cid);
     // scratch of the build, kept by the context for the next direction change
     if (!g->build_tmp) {
         if (dm_alloc(&g->build_tmp, total) != 0) {
@@ -3527,26 +3614,83 @@ static int graph_build(GraphCtx *g, const double *x, const double *y, unsigned l
     b.scid = b.cid;
     b.bits = (uint32_t *)(tmp + off_bits);
     b.err = (unsigned long long *)(tmp + off_err);
-    *err_dev = b.err;
     cudaStream_t st = g->st;
     // (all ones: NaN coordinates and EMPTY ids)
     cudaMemsetAsync(tmp, 0xFF, off_bits, st);
     cudaMemsetAsync(tmp + off_bits, 0, total - off_bits, st);
     const unsigned nblk = (unsigned)((s.n + 255) / 256);
-    const unsigned ablk = (unsigned)(((size_t)nc * nc + BUILD_CELLS - 1) / BUILD_CELLS);
-    if (C == 4) {
+    if (g->C == 4)
         k_gb_cells<4><<<nblk, 256, 0, st>>>(b);
-        k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
-    } else {
+    else
         k_gb_cells<8><<<nblk, 256, 0, st>>>(b);
-        k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
+    if (g->try_ring[g->axis]) {
+        const int chunks = ring_chunks(nc);
+        cudaMemsetAsync(g->ring.band, 0xFF, (size_t)nc * 8, st);
+        cudaMemsetAsync(g->ring.band + nc, 0, (size_t)nc * 8, st);
+        const dim3 grid((unsigned)chunks, (unsigned)nc);
+        if (g->C == 4)
+            k_ring_count<4><<<grid, RING_CHUNK, 0, st>>>(b, g->ring);
+        else
+            k_ring_count<8><<<grid, RING_CHUNK, 0, st>>>(b, g->ring);
+        k_ring_rows<<<1, 1024, 0, st>>>(b, g->ring, chunks, b.err + 1);
     }
-    const cudaError_t e = cudaGetLastError();
+    *out = b;
+    return launched("graph build", err);
+}
+
+// The second half: the records, along the rings (rings) or with the arrows of
+// G(3), and the chains on their start disks (null: where they are).
+static int graph_records(GraphCtx *g, const GBuild &b, bool rings, const int32_t *active,
+                         std::string &err) {
+    GDev &s = g->s;
+    cudaStream_t st = g->st;
+    s.ring = rings && g->try_ring[g->axis];
+    g->try_ring[g->axis] = s.ring != 0;
+    if (s.ring) {
+        const dim3 grid((unsigned)ring_chunks(g->nc), (unsigned)g->nc);
+        if (g->C == 4)
+            k_ring_place<4><<<grid, RING_CHUNK, 0, st>>>(b, g->ring, s);
+        else
+            k_ring_place<8><<<grid, RING_CHUNK, 0, st>>>(b, g->ring, s);
+    }
+    const unsigned ablk = (unsigned)(((size_t)g->nc * g->nc + BUILD_CELLS - 1) / BUILD_CELLS);
+    if (s.ring && s.cells)
+        k_ring_records<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(b, s);
+    else if (g->C == 4)
+        k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
+    else
+        k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
+    k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active);
+    return launched("graph build", err);
+}
+
+// A frame from positions x, y and active disks (device): both halves, with a
+// wait for the first one's result between. bad: the two counters of a check of
+// the inputs queued before (null: they are known to be good).
+static int graph_build(GraphCtx *g, const double *x, const double *y, const int32_t *active,
+                       const unsigned long long *bad, std::string &err) {
+    GBuild b;
+    int rc = graph_place(g, x, y, &b, err);
+    if (rc) return rc;
+    unsigned long long h[2] = {0ull, 0ull}, hb[2] = {0ull, 0ull};
+    cudaError_t e = cudaMemcpyAsync(h, b.err, sizeof h, cudaMemcpyDeviceToHost, g->st);
+    if (e == cudaSuccess && bad)
+        e = cudaMemcpyAsync(hb, bad, sizeof hb, cudaMemcpyDeviceToHost, g->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);
     if (e != cudaSuccess) {
+        (void)cudaGetLastError();
         err = std::string("graph build: ") + cudaGetErrorString(e);
         return ECMC_ECUDA;
     }
-    return 0;
+    if (hb[0] || hb[1]) {
+        err = hb[0] ? "coordinate outside [0, L)" : "active ids must be distinct and in [0, n)";
+        return ECMC_EINVAL;
+    }
+    if (h[0]) {
+        err = "more disks in a cell than it has slots (overlapping input?)";
+        return ECMC_ECAPACITY;
+    }
+    return graph_records(g, b, h[1] == 0ull, active, err);
 }
 
 // Flag words of a context: one per disk, or per cell.
@@ -3554,88 +3698,68 @@ static size_t flag_words(const GDev &s) {
     return s.cells ? (size_t)s.nc * (size_t)s.nc : (size_t)s.n;
 }
 
-// Waits for the build and reports an overfull cell.
-static int graph_build_wait(GraphCtx *g, const unsigned long long *err_dev, std::string &err) {
-    unsigned long long overflow = 0;
-    cudaError_t e =
-        cudaMemcpyAsync(&overflow, err_dev, 8, cudaMemcpyDeviceToHost, g->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        err = std::string("graph build: ") + cudaGetErrorString(e);
-        return ECMC_ECUDA;
-    }
-    if (overflow) {
-        err = "more disks in a cell than it has slots (overlapping input?)";
-        return ECMC_ECAPACITY;
-    }
-    return 0;
-}
-
 }  // namespace
 
-// The device arrays of a graph context, requested from the pool (galloc):
-// graph_create commits them, graph_plan_bytes only adds them up.
-// slots > 0: for a cell-scan context of that many slots (graph_attach), whose
-// records and log are shared; the scratch of its build is planned with it.
-static int graph_plan(GraphCtx *g, const ecmc_params *p, size_t slots, std::string &err) {
+// The device arrays of a context: take(pointer, count) for each.
+template <class Take>
+static void graph_arrays(GraphCtx *g, Take take) {
     GDev &s = g->s;
-    const size_t n = (size_t)p->n, k = (size_t)p->n_chains;
-    int rc = 0;
-    auto chk = [&](int r) {
-        if (r && !rc) rc = r;
-    };
-    chk(galloc(g, &s.g, n, err));
-    chk(galloc(g, &s.y, n, err));
-    chk(galloc(g, &s.key, n, err));
-    s.cells = slots > 0;
-    chk(galloc(g, &s.fl, slots ? (size_t)g->nc * (size_t)g->nc : n, err));
-    if (slots) {
-        chk(galloc(g, &s.pxt, k * ((size_t)s.cap + 2), err));
-        chk(galloc(g, &s.pcell, k * ((size_t)s.cap + 2), err));
-        chk(galloc(g, &g->slot_xy, slots, err));
-        chk(galloc(g, &g->row_off, (size_t)g->nc + 1, err));
-        chk(galloc(g, &g->slot_bits, (size_t)std::ceil(p->box / (p->d / 128.0)) / 32 + 2, err));
+    const size_t n = (size_t)s.n, k = (size_t)s.k;
+    const size_t path = k * ((size_t)s.cap + 2);
+    take(&s.g, n);
+    take(&s.y, n);
+    take(&s.key, n);
+    take(&s.fl, flag_words(s));
+    take(&s.rid, n);
+    take(&s.pos, n);
+    take(&g->ring.off, (size_t)g->nc * ring_chunks(g->nc) + 1);
+    take(&g->ring.band, 2 * (size_t)g->nc);
+    if (s.cells) {
+        take(&s.pxt, path);
+        take(&s.pcell, path);
     }
-    chk(galloc(g, &s.path, k * ((size_t)s.cap + 2), err));
-    chk(galloc(g, &s.sp, k, err));
-    chk(galloc(g, &s.ci, k, err));
-    chk(galloc(g, &s.ci0, k, err));
-    chk(galloc(g, &s.D, k, err));
-    chk(galloc(g, &s.tc, k, err));
-    chk(galloc(g, &s.status, k, err));
-    chk(galloc(g, &s.partner, k, err));
-    chk(galloc(g, &s.nrec, k, err));
-    chk(galloc(g, &s.nlift, k, err));
-    chk(galloc(g, &s.memb, k, err));
-    chk(galloc(g, &s.tstar, 1, err));
-    s.restart = (p->flags & ECMC_RESTART) ? 1 : 0;
-    if (!slots) chk(galloc(g, &s.rec, k * (size_t)s.cap, err));
-    chk(galloc(g, &s.ev_T, k, err));
-    chk(galloc(g, &s.ev_tau, k, err));
-    chk(galloc(g, &s.ev_xj, k, err));
-    chk(galloc(g, &s.ev_tj, k, err));
-    chk(galloc(g, &s.ev_j, k, err));
-    chk(galloc(g, &s.ev_a, 3 * k, err));
-    chk(galloc(g, &s.ev_lift, k, err));
-    chk(galloc(g, &s.vt, k, err));
-    chk(galloc(g, &s.uf, k, err));
-    chk(galloc(g, &s.fin, k, err));
-    chk(galloc(g, &s.comp_of, k, err));
-    chk(galloc(g, &s.abort_to, k, err));
-    chk(galloc(g, &s.comp_cnt, k, err));
-    chk(galloc(g, &s.comp_off, k + 1, err));
-    chk(galloc(g, &s.comp_root, k, err));
-    chk(galloc(g, &s.comp_mem, 4 * k, err));  // (g_members)
-    chk(galloc(g, &s.child, k, err));
-    chk(galloc(g, &s.sib, k, err));
-    chk(galloc(g, &s.taken, k, err));
-    chk(galloc(g, &s.ctl, CTL_N, err));
-    chk(galloc(g, &s.lc, 2 * LC_N, err));
-    chk(galloc(g, &s.dbg, 16, err));
-    if (!slots) chk(galloc(g, &s.tc_cnt, TC_N, err));
-    if (!slots && s.log_on) chk(galloc(g, &s.log, (size_t)s.log_cap, err));
-    return rc;
+    take(&s.path, path);
+    take(&s.sp, k);
+    take(&s.ci, k);
+    take(&s.ci0, k);
+    take(&s.D, k);
+    take(&s.tc, k);
+    take(&s.status, k);
+    take(&s.partner, k);
+    take(&s.nrec, k);
+    take(&s.nlift, k);
+    take(&s.memb, k);
+    take(&s.tstar, 1);
+    take(&s.rec, k * (size_t)s.cap);
+    take(&s.ev_T, k);
+    take(&s.ev_tau, k);
+    take(&s.ev_xj, k);
+    take(&s.ev_tj, k);
+    take(&s.ev_j, k);
+    take(&s.ev_a, 3 * k);
+    take(&s.ev_lift, k);
+    take(&s.vt, k);
+    take(&s.uf, k);
+    take(&s.fin, k);
+    take(&s.comp_of, k);
+    take(&s.abort_to, k);
+    take(&s.comp_cnt, k);
+    take(&s.comp_off, k + 1);
+    take(&s.comp_root, k);
+    take(&s.comp_mem, 4 * k);  // (g_members)
+    take(&s.child, k);
+    take(&s.sib, k);
+    take(&s.taken, k);
+    take(&s.ctl, CTL_N);
+    take(&s.lc, 2 * LC_N);
+    take(&s.dbg, 16);
+    take(&s.tc_cnt, TC_N);
+    if (s.log_on) take(&s.log, (size_t)s.log_cap);
+}
+
+// Requests for all of them (galloc; gcommit allocates, graph_plan_bytes adds up).
+static void graph_plan(GraphCtx *g) {
+    graph_arrays(g, [&](auto **p, size_t count) { galloc(g, p, count); });
 }
 
 // Blocks of the persistent launch that fit on the current device at once (0:
@@ -3680,6 +3804,32 @@ static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
     s.ell = p->ell;
     s.inv_a = (double)nc / p->box;
     s.strict = (s.windows > 1 || (p->flags & ECMC_RESTART)) ? 1 : 0;
+    s.restart = (p->flags & ECMC_RESTART) ? 1 : 0;
+    s.cells = (p->flags & ECMC_GRAPH) ? 0 : 1;
+    const double a = p->box / nc;
+    // slots per cell: at most 4 centres at mutual distance >= d fit in a cell
+    // with a < sqrt(2) d, at most 6 for a < 1.664 d
+    g->C = a < std::sqrt(2.0) * p->d * (1.0 - 1e-9) ? 4 : 8;
+    // rings need four stretches' worth of columns and a leg that cannot come
+    // round the box; a context may go without
+    g->try_ring[0] = g->try_ring[1] = !(p->flags & ECMC_NO_ROWPASS) && nc >= 4 * (32 / g->C) &&
+                                      p->ell < p->box - 3.0 * a;
+    // FP32 image of the scan's stop rule thr(m) = ((m a) - fx) - d > RN(cur +
+    // eps): thr_f = ((m af - fxf) - df) and lim_f = trunc(cur) + epsf, with af,
+    // df, epsf the FP32 roundings, fxf = trunc(fx). Each of the four FP32
+    // roundings and the two truncations errs by at most 2^-23 of a term of
+    // magnitude at most m a + a + d + cur + eps <= L + a + d + ell + eps (m < nc,
+    // |fx| <= a, cur <= ell), so |(thr_f - lim_f) - (thr - lim)| < 2^-22 (L + a +
+    // d + ell + eps) (the FP64 roundings are 2^29 times smaller). stop_e is 4
+    // times that.
+    const double eps = std::ldexp(p->box, -30);
+    s.sk.a = a;
+    s.sk.d = p->d;
+    s.sk.eps = eps;
+    s.sk.af = (float)a;
+    s.sk.df = (float)p->d;
+    s.sk.epsf = (float)eps;
+    s.sk.stop_e = (float)std::ldexp(p->box + a + p->d + p->ell + eps + 1.0, -20);
     s.log_on = (p->flags & ECMC_LOG_LIFTINGS) ? 1 : 0;
     s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
 }
@@ -3694,12 +3844,14 @@ static void graph_clear(GraphCtx *g) {
     cudaMemsetAsync(s.taken, 0, k * 4, st);
     cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
     cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
+    cudaMemsetAsync(s.tc_cnt, 0, TC_N * 8, st);
     cudaMemsetAsync(s.key, 0xFF, n * 8, st);
     cudaMemsetAsync(s.fl, 0, flag_words(s) * 8, st);
 }
 
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
-                 const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err) {
+                 const int32_t *active, const unsigned long long *bad, cudaStream_t st,
+                 GraphCtx **out, std::string &err) {
     *out = nullptr;
     if (p->n_chains > MAX_CHAINS) {
         err = "too many chains";
@@ -3712,27 +3864,14 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     }
     g->st = st;
     graph_params(g, p, nc);
-    GDev &s = g->s;
-    const size_t n = (size_t)p->n;
-    int rc = 0;
-    auto chk = [&](int r) {
-        if (r && !rc) rc = r;
-    };
-    chk(graph_plan(g, p, 0, err));
-    chk(gcommit(g, err));
+    graph_plan(g);
+    int rc = gcommit(g, err);
     if (rc) {
         graph_destroy(g);
         return rc;
     }
-    cudaMemcpyAsync(s.y, y, n * 8, cudaMemcpyDeviceToDevice, st);
-    cudaMemsetAsync(s.tc_cnt, 0, TC_N * 8, st);
     graph_clear(g);
-    unsigned long long *overflow = nullptr;
-    rc = graph_build(g, x, s.y, &overflow, err);
-    if (!rc) {
-        k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active);
-        rc = graph_build_wait(g, overflow, err);
-    }
+    rc = graph_build(g, x, y, active, bad, err);
     if (!rc && graph_max_grid() < 1) {
         err = "cooperative launch unavailable";
         rc = ECMC_ECUDA;
@@ -3744,94 +3883,6 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
     *out = g;
     return 0;
 }
-
-GraphCtx *graph_attach(const ecmc_params *p, int nc, int C, cudaStream_t st,
-                       std::vector<std::pair<void **, size_t>> &pending) {
-    GraphCtx *g = new (std::nothrow) GraphCtx();
-    if (!g) return nullptr;
-    g->st = st;
-    graph_params(g, p, nc);
-    std::string err;
-    (void)graph_plan(g, p, (size_t)nc * nc * C, err);
-    pending.insert(pending.end(), g->pending.begin(), g->pending.end());
-    g->pending.clear();
-    return g;
-}
-
-static void graph_bind(GraphCtx *g, const GraphCells &c) {
-    GDev &s = g->s;
-    s.rec = (GEv *)c.rec;
-    s.log = c.log;
-    s.tc_cnt = c.tc_cnt;
-    s.colx = c.colx;
-    s.sk.af = c.af;
-    s.sk.df = c.df;
-    s.sk.epsf = c.epsf;
-    s.sk.stop_e = c.stop_e;
-    s.sk.a = c.a;
-    s.sk.d = s.d;
-    s.sk.eps = c.eps;
-}
-
-int graph_activate(GraphCtx *g, const GraphCells &c, bool first, bool ring, std::string &err) {
-    GDev &s = g->s;
-    cudaStream_t st = g->st;
-    if (first) {
-        graph_bind(g, c);
-        graph_clear(g);
-        if (graph_max_grid() < 1) {
-            err = "cooperative launch unavailable";
-            return ECMC_ECUDA;
-        }
-    }
-    GBuild b = build_params(g);
-    b.sx = c.cx;
-    b.sy = c.cy;
-    b.scid = c.cid;
-    b.cxy = g->slot_xy;
-    b.bits = g->slot_bits;
-    b.yout = s.y;
-    s.ring = ring;
-    if (ring) {
-        // (places in the scratch of the other kind of frame: 8 bytes a slot)
-        s.rid = (uint32_t *)g->slot_xy;
-        s.posof = s.rid + s.n;
-        k_ring_count<<<(unsigned)c.nc, 256, 0, st>>>(b, c.C, g->row_off);
-        k_ring_offsets<<<1, 1024, 0, st>>>(c.nc, g->row_off);
-        if (c.C == 4)
-            k_ring_place<4><<<(unsigned)c.nc, 256, 0, st>>>(b, g->row_off, s);
-        else
-            k_ring_place<8><<<(unsigned)c.nc, 256, 0, st>>>(b, g->row_off, s);
-    } else {
-        const uint32_t nslot = (uint32_t)((size_t)c.nc * c.nc * c.C);
-        const unsigned ablk = (unsigned)(((size_t)c.nc * c.nc + BUILD_CELLS - 1) / BUILD_CELLS);
-        const unsigned sblk = (unsigned)(((size_t)nslot + 255) / 256);
-        cudaMemsetAsync(b.bits, 0, ((size_t)b.nb / 32 + 1) * 4, st);
-        if (c.C == 4) {
-            k_gb_slots<4><<<sblk, 256, 0, st>>>(b, nslot);
-            k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
-        } else {
-            k_gb_slots<8><<<sblk, 256, 0, st>>>(b, nslot);
-            k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
-        }
-    }
-    k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, (const int32_t *)c.ci);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        err = std::string("graph build: ") + cudaGetErrorString(e);
-        return ECMC_ECUDA;
-    }
-    return 0;
-}
-
-void graph_swapped(GraphCtx *g, double *xnew, const double **ynew, const int32_t **active) {
-    const GDev &s = g->s;
-    k_g_swap_xy<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, xnew);
-    *ynew = s.y;
-    *active = (const int32_t *)s.ci;
-}
-
-void graph_set_leg(GraphCtx *g, int64_t legs) { g->log_legs = legs; }
 
 // Launch tables of the persistent kernel: one device block [reps | chain_base
 // | comp_base | ctl | bar | g | phase] (256-byte aligned parts), uploaded
@@ -4109,9 +4160,10 @@ int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
 int graph_export(GraphCtx *g, double *x, double *y, double *t, int32_t *active) {
     const GDev &s = g->s;
     cudaStream_t st = g->st;
-    if (x || t) k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t);
+    if (x || t) k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t, nullptr);
     if (y) cudaMemcpyAsync(y, s.y, (size_t)s.n * 8, cudaMemcpyDeviceToDevice, st);
-    if (active) k_g_export_active<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active);
+    if (active)
+        k_g_export_active<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active, nullptr);
     return cudaGetLastError() == cudaSuccess ? 0 : ECMC_ECUDA;
 }
 
@@ -4143,12 +4195,8 @@ int graph_transpose(GraphCtx *g, std::string &err) {
     }
     k_g_swap_xy<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, xnew);
     // records (x, t = 0) and arrows for the new frame
-    unsigned long long *overflow = nullptr;
-    int rc = graph_build(g, xnew, s.y, &overflow, err);
-    if (rc == 0) {
-        k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, g->st>>>(s, nullptr);
-        rc = graph_build_wait(g, overflow, err);
-    }
+    g->axis ^= 1;
+    int rc = graph_build(g, xnew, s.y, nullptr, nullptr, err);
     // (the build's kernels read xnew: done before the block goes back)
     if (cudaStreamSynchronize(g->st) != cudaSuccess && rc == 0) {
         (void)cudaGetLastError();
@@ -4192,10 +4240,7 @@ int graph_liftings(GraphCtx *g, ecmc_lift_t *buf, int64_t cap, int64_t *n_out,
 
 void graph_destroy(GraphCtx *g) {
     if (!g) return;
-    // (a context of the cells' path holds no block of its own: ecmc_destroy has
-    // waited for its work)
-    if (!g->allocs.empty() && cudaStreamSynchronize(g->st) != cudaSuccess)
-        (void)cudaGetLastError();
+    if (cudaStreamSynchronize(g->st) != cudaSuccess) (void)cudaGetLastError();
     for (void *p : g->allocs) dm_free(p);
     dm_free(g->build_tmp);
     dm_free(g->d_flags);
@@ -4209,16 +4254,140 @@ int64_t graph_plan_bytes(const ecmc_params *p, int nc) {
     GraphCtx *g = new (std::nothrow) GraphCtx();
     if (!g) return -1;
     graph_params(g, p, nc);
-    std::string err;
-    int64_t total = -1;
-    if (graph_plan(g, p, 0, err) == 0) {
-        total = 0;
-        for (auto &r : g->pending) total += (int64_t)((r.second + 255) & ~(size_t)255);
-        const double a = p->box / nc;
-        const int C = a < std::sqrt(2.0) * p->d * (1.0 - 1e-9) ? 4 : 8;
-        total += graph_build_bytes(p->box, p->d, nc, C);
-    }
+    graph_plan(g);
+    int64_t total = graph_build_bytes(p->box, p->d, nc, g->C);
+    for (auto &r : g->pending) total += (int64_t)((r.second + 255) & ~(size_t)255);
     g->pending.clear();
     delete g;
     return total;
+}
+
+// -------------------------------------------- one leg on given memory
+
+namespace {
+
+// Tables of a launch of one system, as they lie on the device.
+struct LegTables {
+    GDev dev;
+    int32_t chain_base[2], comp_base[2];
+    GCtl ctl;
+    unsigned bar;
+    int32_t g[GG_N];
+    unsigned long long phase[GPH_N];
+};
+
+// Places the arrays of a leg in [base, ...) on 256-byte boundaries (base null:
+// only counts). seen: the ids seen by the input check.
+struct LegArrays {
+    LegTables *tables;
+    int32_t *blocked;
+    uint32_t *seen;
+    unsigned long long *bad;  // [2]
+};
+
+size_t leg_arrays(GraphCtx *g, unsigned char *base, LegArrays *out) {
+    size_t off = 0;
+    auto take = [&](auto **p, size_t count) {
+        off = (off + 255) & ~(size_t)255;
+        *p = base ? reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + off) : nullptr;
+        off += std::max<size_t>(count, 1) * sizeof(**p);
+    };
+    graph_arrays(g, take);
+    take(&out->tables, 1);
+    take(&out->blocked, (size_t)g->s.k);
+    out->seen = g->s.rid;  // (written again by the build)
+    take(&out->bad, 2);
+    char *tmp;
+    take(&tmp, (size_t)graph_build_bytes(g->s.L, g->s.d, g->nc, g->C));
+    g->build_tmp = tmp;
+    return off;
+}
+
+}  // namespace
+
+size_t graph_leg_bytes(const ecmc_params *p, int nc) {
+    GraphCtx g;
+    graph_params(&g, p, nc);
+    LegArrays a;
+    return leg_arrays(&g, nullptr, &a);
+}
+
+int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, const double *y,
+              int32_t *active, double *t_out, cudaStream_t st, uint8_t *flag, int64_t *lifts,
+              std::string &err) {
+    GraphCtx g;
+    g.st = st;
+    graph_params(&g, p, nc);
+    LegArrays a;
+    (void)leg_arrays(&g, base, &a);
+    GDev &s = g.s;
+    int rc = 0;
+    auto cu = [&](cudaError_t e) {
+        if (e != cudaSuccess && !rc) {
+            (void)cudaGetLastError();
+            rc = ECMC_ECUDA;
+        }
+    };
+    const int grid = graph_max_grid();
+    if (grid < 1) return ECMC_ECUDA;
+    // the first half of the build reads any coordinates; ids are used after
+    // the check's result
+    cu(cudaMemsetAsync(a.seen, 0, (size_t)s.n * 4, st));
+    cu(cudaMemsetAsync(a.bad, 0, 16, st));
+    graph_check_inputs(x, y, active, s.n, s.k, s.L, a.seen, a.bad, a.bad + 1, st);
+    graph_clear(&g);
+    cu(cudaMemsetAsync(s.memb, 0xFF, (size_t)s.k * 8, st));
+    GBuild b;
+    if (!rc) rc = graph_place(&g, x, y, &b, err);
+    unsigned long long bad[2], built[2];
+    if (!rc) {
+        cu(cudaMemcpyAsync(bad, a.bad, sizeof bad, cudaMemcpyDeviceToHost, st));
+        cu(cudaMemcpyAsync(built, b.err, sizeof built, cudaMemcpyDeviceToHost, st));
+        cu(cudaStreamSynchronize(st));
+    }
+    if (rc) return rc;
+    if (bad[0] || bad[1]) return ECMC_EINVAL;
+    if (built[0]) return ECMC_ECAPACITY;
+    rc = graph_records(&g, b, built[1] == 0ull, active, err);
+    if (rc) return rc;
+    LegTables t;
+    memset(&t, 0, sizeof t);
+    t.dev = s;
+    t.chain_base[1] = s.k;
+    t.ctl.failed = 1;
+    GBatchDev B;
+    B.reps = &a.tables->dev;
+    B.ctl = &a.tables->ctl;
+    B.chain_base = a.tables->chain_base;
+    B.comp_base = a.tables->comp_base;
+    B.bar = &a.tables->bar;
+    B.g = a.tables->g;
+    B.blocked = a.blocked;
+    B.phase_ns = a.tables->phase;
+    B.R = 1;
+    B.max_legs = 1;
+    B.windows = 1;
+    B.pad = 0;
+    B.wait_ns = BARRIER_TIMEOUT_NS;
+    cu(cudaMemcpyAsync(a.tables, &t, sizeof t, cudaMemcpyHostToDevice, st));
+    void *args[] = {&B};
+    cu(cudaLaunchCooperativeKernel((void *)k_run_graph, grid, GRUN_THREADS, args, UF_SMEM_BYTES,
+                                   st));
+    s.stamp0 = 1;  // (the leg's times)
+    if (!rc) {
+        // (a leg out of records leaves the inputs as they are; one that gave up
+        // on a wait never counted itself)
+        const int32_t *const failed = &a.tables->ctl.failed;
+        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t_out, failed);
+        k_g_export_active<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active, failed);
+        cu(cudaGetLastError());
+    }
+    cu(cudaMemcpyAsync(&t, a.tables, sizeof t, cudaMemcpyDeviceToHost, st));
+    cu(cudaStreamSynchronize(st));
+    if (rc) return rc;
+    if (t.ctl.err) return ECMC_ECAPACITY;
+    if (t.g[GG_ERR] || t.ctl.dbg) return ECMC_ECUDA;
+    if (flag) *flag = t.ctl.conflict_legs != 0;
+    if (lifts) *lifts = t.ctl.lifts;
+    return 0;
 }

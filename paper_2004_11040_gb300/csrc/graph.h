@@ -20,11 +20,13 @@ struct GraphTotals {
     double ms, pass1_ms, repair_ms, other_ms;
 };
 
-// A context on device inputs x, y (n each) and active (k), all device
-// pointers valid until the call returns; nc cells per side are used only to
-// build the graph.
+// A context on device inputs x, y (n each) and active (k), which the work it
+// queues on the stream reads; bad: the counters of graph_check_inputs on them,
+// queued before. nc cells per side. With ECMC_GRAPH the conflict flag is on the
+// disks read, otherwise on the cells scanned.
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
-                 const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err);
+                 const int32_t *active, const unsigned long long *bad, cudaStream_t st,
+                 GraphCtx **out, std::string &err);
 int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
               int32_t *legs_done, GraphTotals *tot, std::string &err,
               unsigned long long wait_ns);
@@ -51,32 +53,18 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
                     int32_t *legs_out, double *ms_out, std::string &err,
                     unsigned long long wait_ns);
 void graph_batch_free(GBatchScratch *scratch);
-// A cell-scan context's general frames (rows within reach of each other) run
-// on this path too, with the conflict flag on cells. graph_attach adds the
-// path's arrays to the context's requests (records and log are the cells'
-// own; null: host allocation); graph_activate builds the records and arrows from the cells as they
-// stand at a breakpoint (queued on the stream; first: the first time of the
-// context; ring: every row is a ring), after which the state is here: graph_swapped gives x and y
-// exchanged (x into xnew) and the active disks, to build cells from again.
-struct GraphCells {
-    int nc, C;
-    double a, eps;
-    float af, df, epsf, stop_e;
-    const double *colx;
-    const uint32_t *cid;
-    const double *cx, *cy;
-    const uint32_t *ci;
-    void *rec;  // [k * cap] of at least 80 bytes each
-    ecmc_lift_t *log;
-    unsigned long long *tc_cnt;
-};
-GraphCtx *graph_attach(const ecmc_params *p, int nc, int C, cudaStream_t st,
-                       std::vector<std::pair<void **, size_t>> &pending);
-int graph_activate(GraphCtx *g, const GraphCells &c, bool first, bool ring, std::string &err);
-void graph_swapped(GraphCtx *g, double *xnew, const double **ynew, const int32_t **active);
-// Legs run before (leg index of the lifting log).
-void graph_set_leg(GraphCtx *g, int64_t legs);
 // Device memory held by the context (bytes).
 int64_t graph_device_bytes(const GraphCtx *g);
 // What graph_create(p, nc, ...) would hold, without allocating (-1: error).
 int64_t graph_plan_bytes(const ecmc_params *p, int nc);
+// One leg of a cell-scan system in given device memory (graph_leg_bytes of it,
+// 256-byte aligned), nothing allocated; inputs as in ecmc_leg_noalloc.
+size_t graph_leg_bytes(const ecmc_params *p, int nc);
+int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, const double *y,
+              int32_t *active, double *t_out, cudaStream_t st, uint8_t *flag, int64_t *lifts,
+              std::string &err);
+// Counts coordinates outside [0, L) in *bad_xy and active ids that repeat or
+// lie outside [0, n) in *bad_id (seen: n words of zero).
+void graph_check_inputs(const double *x, const double *y, const int32_t *active, int64_t n, int k,
+                        double L, uint32_t *seen, unsigned long long *bad_xy,
+                        unsigned long long *bad_id, cudaStream_t st);

@@ -60,6 +60,16 @@ def test_rings_equal_oracle(nc, a, spread, lengths, k, ell, windows, seed):
         assert g[5]["row_windows"] == 4 * windows
 
 
+@pytest.mark.parametrize("k,ell,windows,seed", [
+    (60, 1.0, 1, 3), (300, 3.0, 1, 4), (200, 2.0, 3, 7),
+])
+def test_rings_of_a_graph_context(k, ell, windows, seed):
+    """With the arrows of G(3) a ring's successor may be any of the three."""
+    s = rings(40, 1.35, 0.3, EDGES, k, seed)
+    g = run(s, ell, 4, windows, graph=True, nc=40)
+    same(g, oracle(s, ell, 4, windows, search=2, nc=40))
+
+
 def test_a_wide_row_is_no_ring():
     s = rings(40, 1.6, 0.3, [10, 20, 3], 60, 8, wide_row=True)
     g = run(s, 1.0, 4, nc=40)
