@@ -2126,11 +2126,18 @@ __device__ void g_finish(const GDev &s, const int32_t *mem, int m, int root, boo
 // and replays it in global order. The lanes share a step as in g_spec_chain;
 // a step's claims are asked about one step later, when their round trip is
 // over, and an event is written only once they stand.
+//
+// The disks that the continuation moves it holds, and one that another
+// component holds ends it. A disk that it only reads need not be held (as in
+// g_resolve_chain; strict: it is): nobody has touched it in this leg, and
+// whatever moves it, at whatever time, moves it farther ahead of a disk whose
+// target it was not. With every disk read held 30% more continuations met
+// another component.
 enum { CONT_DONE = 0, CONT_FAIL = 1, CONT_FOREIGN = 2 };
 
 __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m, int root,
                                        uint64_t tag, uint32_t epoch, int round, double tw,
-                                       double tend, int *met) {
+                                       double tend, int *met, uint32_t *cnt_out) {
     const int lane = threadIdx.x & 31;
     const int l3 = lane % 3;
     const double L = s.L;
@@ -2138,6 +2145,7 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
     GDisk *const g = s.g;
     const uint32_t stamp = s.stamp;
     const bool bounded = dbits(tend) != INF_BITS || dbits(tw) != 0ull;
+    const bool strict = s.strict != 0;
     const int n_lap = g_lap(s), cap = s.cap;
     uint32_t cnt = 0;
     int switches = 0, e = 0, cur = -1;
@@ -2153,7 +2161,10 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
                 }
                 e += 32;
             }
-            if (e >= m) return CONT_DONE;
+            if (e >= m) {
+                *cnt_out = cnt;
+                return CONT_DONE;
+            }
             cur = mem[e];
         }
         const int c = cur;
@@ -2234,10 +2245,12 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
                 break;
             }
             // this step's claims: a record whose word is of this pass names its
-            // holder, any other disk is taken
+            // holder; of the others the winner is taken, once it is known
+            // (strict: all), and the words of the rest are read again -- one that
+            // is still free stands for a record that was not written
             held = ev ? g_holder(cw, ct) : 0u;
             cas = 0ull;
-            if (ev && held == 0u) cas = atomicCAS(&g[tid].claim, cw, ct);
+            if (strict && ev && held == 0u) cas = atomicCAS(&g[tid].claim, cw, ct);
             // Eq. 2, strict (a lap-away target fails it too), for every target
             // with a time of this leg; another chain's disk stops the step in
             // reach or where it fails Eq. 2
@@ -2270,6 +2283,9 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
             const uint32_t bj = __shfl_sync(FULL, tid, wl);
             const double xj = shfl_f64(rx, wl);
             const double tj = shfl_f64(own == stamp ? rt : 0.0, wl);
+            if (!strict && ev && held == 0u)
+                cas = lift && lane == wl ? atomicCAS(&g[tid].claim, cw, ct)
+                                         : __ldcg(&g[tid].claim);
             if (viol) {
                 how = CONT_FAIL;
                 break;
@@ -2364,16 +2380,17 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
             s.nrec[c] = nr0 + n;
             s.nlift[c] += nl;
             if (nl) atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
-            if (how != CONT_FAIL) {
-                s.status[c] = how == CONT_FOREIGN ? ST_BLOCKED : st;
-                s.ci[c] = i;
-                s.tc[c] = ti;
-                s.D[c] = D;
-            }
+            s.status[c] = how != CONT_DONE ? ST_BLOCKED : st;
+            s.ci[c] = i;
+            s.tc[c] = ti;
+            s.D[c] = D;
         }
         __syncwarp();
         cnt += (uint32_t)n;
-        if (how != CONT_DONE) return how;
+        if (how != CONT_DONE) {
+            *cnt_out = cnt;
+            return how;
+        }
         cur = next;
     }
 }
@@ -2387,7 +2404,8 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
 // 1024 chains on 2^20 disks: the repair phase of a leg 33 us with a step per
 // event, 21 by stretches.
 __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, int m, int root,
-                                            uint64_t tag, uint32_t epoch, int round, int *met) {
+                                            uint64_t tag, uint32_t epoch, int round, int *met,
+                                            uint32_t *cnt_out) {
     const int lane = threadIdx.x & 31, up = (lane + 1) & 31;
     GDisk *const g = s.g;
     const double L = s.L;
@@ -2405,7 +2423,10 @@ __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, i
                 }
                 e += 32;
             }
-            if (e >= m) return CONT_DONE;
+            if (e >= m) {
+                *cnt_out = cnt;
+                return CONT_DONE;
+            }
             cur = mem[e];
         }
         const int c = cur;
@@ -2520,16 +2541,17 @@ __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, i
             s.nrec[c] = nr0 + n;
             s.nlift[c] += nl;
             if (nl) atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
-            if (how != CONT_FAIL) {
-                s.status[c] = how == CONT_FOREIGN ? ST_BLOCKED : st;
-                s.ci[c] = i;
-                s.tc[c] = t;
-                s.D[c] = D;
-            }
+            s.status[c] = how != CONT_DONE ? ST_BLOCKED : st;
+            s.ci[c] = i;
+            s.tc[c] = t;
+            s.D[c] = D;
         }
         __syncwarp();
         cnt += (uint32_t)n;
-        if (how != CONT_DONE) return how;
+        if (how != CONT_DONE) {
+            *cnt_out = cnt;
+            return how;
+        }
         cur = next;
     }
 }
@@ -2544,9 +2566,9 @@ __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, i
 // one event later.
 constexpr int SMALL_REPLAY = 10;
 
-__device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, int m, int root,
-                                            uint64_t tag, uint32_t epoch, int round, double Ts,
-                                            double tend) {
+__device__ __noinline__ bool g_replay_small(const GDev &s, const int32_t *mem, int m,
+                                            uint32_t epoch, int round, double Ts, double tend,
+                                            int *met_out, double *now_out, uint32_t *seq) {
     const int lane = threadIdx.x & 31;
     const int e = lane / 3, p = lane - 3 * e, base = 3 * e;
     const bool has = e < m;
@@ -2621,7 +2643,7 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
     double taken = Ts;  // time of the event after which the claims were asked for,
     int taker = -1;     // and the chain that asked
     double now = Ts;
-    uint32_t cnt = 0;
+    uint32_t cnt = *seq;
     if (conflict()) abort = true;
     held = held_i = 0u;
     cas = 0ull;
@@ -2788,7 +2810,10 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
         if (nl) atomicAdd(s.lc + LC_LIFTS, (unsigned long long)nl);
     }
     __syncwarp();
-    g_finish(s, mem, m, root, abort, met, now);
+    *met_out = met;
+    *now_out = now;
+    *seq = cnt;
+    return abort;
 }
 
 // The members of the component of blocked chain a (one warp): the root's tree,
@@ -2801,7 +2826,7 @@ __device__ __noinline__ void g_replay_small(const GDev &s, const int32_t *mem, i
 // and the repair: 8 us of a leg at 1024 chains, ~300 of 605 us at 16384.)
 constexpr int MEMBER_BUF = 64;
 __device__ __noinline__ bool g_members(const GDev &s, int a, uint32_t epoch, int *root_out,
-                                       const int32_t **mem_out, int *m_out) {
+                                       int32_t **mem_out, int *m_out, int *cap_out) {
     __shared__ int32_t buf[8][MEMBER_BUF];
     const int lane = threadIdx.x & 31;
     int32_t *mem = buf[threadIdx.x >> 5];
@@ -2844,68 +2869,24 @@ __device__ __noinline__ bool g_members(const GDev &s, int a, uint32_t epoch, int
     *root_out = root;
     *mem_out = mem;
     *m_out = n;
+    *cap_out = cap;
     return __shfl_sync(FULL, prev, 0) != (int32_t)epoch;
 }
 
-// A component of this round (one warp): roll its members back to T*, then
-// replay them in global event-time order (Alg. 2) up to the window's end.
-// Members are spread over the lanes (member e on lane e mod 32); after each
-// event only the members whose arrows read a disk it changed recompute.
-__device__ __noinline__ void g_repair_component(const GDev &s, const int32_t *mem, int m, int root,
-                                                int round, uint32_t epoch, uint32_t wr_tag,
-                                                double tw, double tend) {
+// Replay of a larger component: its members spread over the lanes (member e on
+// lane e mod 32); after each event only the members whose arrows read a disk it
+// changed recompute.
+__device__ __noinline__ bool g_replay_large(const GDev &s, const int32_t *mem, int m, int root,
+                                            uint64_t tag, uint32_t epoch, int round, double Ts,
+                                            double tend, int *met_out, double *now_out,
+                                            uint32_t *seq) {
     const int lane = threadIdx.x & 31;
-    double Ts = INFINITY;
-    // the members listed for this round of this pass (wr_tag names both)
-    const uint64_t tag = ((uint64_t)wr_tag << 32) | (uint32_t)root;
-    for (int e = lane; e < m; e += 32) {
-        const int c = mem[e];
-        Ts = fmin(Ts, s.vt[c]);
-        s.memb[c] = tag;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) Ts = fmin(Ts, __shfl_xor_sync(FULL, Ts, o));
-    Ts = fmax(Ts, tw);  // earlier windows are final
-    if (lane == 0) atomicAdd(s.lc + LC_REPAIRED, (unsigned long long)m);
-    __syncwarp();
-    // (a later round of a leg without claim windows: chains that a repair which
-    // met another component left unfinished)
-    const bool whole = dbits(tend) == INF_BITS && dbits(tw) == 0ull;
-    if (round > 1 && whole) {
-        for (int e = lane; e < m; e += 32)
-            if (s.status[mem[e]] == ST_RUNNING) s.status[mem[e]] = ST_BLOCKED;
-        __syncwarp();
-    }
-    if (round == 1 || whole) {
-        int met = -1;
-        const int how = s.ring && !s.strict
-                            ? g_continue_ring(s, mem, m, root, tag, epoch, round, &met)
-                            : g_continue(s, mem, m, root, tag, epoch, round, tw, tend, &met);
-        if (how == CONT_DONE) {
-            if (lane == 0) atomicAdd(s.lc + LC_CONTINUED, (unsigned long long)m);
-            g_finish(s, mem, m, root, false, -1, Ts, true);
-            return;
-        }
-        if (how == CONT_FOREIGN) {
-            // its events so far stand for the merged component to go on from (or
-            // to roll back to T*: all of this round's events lie after it)
-            g_finish(s, mem, m, root, true, met, Ts);
-            return;
-        }
-    }
-    g_rollback(s, mem, m, Ts);
-    for (int e = lane; e < m; e += 32) g_resume(s, mem[e]);
-    __syncwarp();
-    if (m <= SMALL_REPLAY) {
-        g_replay_small(s, mem, m, root, tag, epoch, round, Ts, tend);
-        return;
-    }
     bool abort = false;
     int met = -1;
     for (int e = lane; e < m; e += 32)
         if (s.status[mem[e]] == ST_RUNNING) g_compute(s, mem[e], root, tag, epoch, abort, met);
     double now = Ts;
-    uint32_t cnt = 0;
+    uint32_t cnt = *seq;
     for (;;) {
         {
             const unsigned ab = __ballot_sync(FULL, abort);
@@ -3006,7 +2987,105 @@ __device__ __noinline__ void g_repair_component(const GDev &s, const int32_t *me
         }
         __syncwarp();
     }
-    g_finish(s, mem, m, root, abort, met, now);
+    *met_out = met;
+    *now_out = now;
+    *seq = cnt;
+    return abort;
+}
+
+// A component of this round (one warp; room for cap members in mem): continue
+// its blocked chains, or else roll its members back to T* and replay them in
+// global event-time order (Alg. 2) up to the window's end. A replay of the
+// first round that needs a disk of a chain in no component takes that chain
+// in and starts again: left to the next round, it made one of 70 us on nearly
+// every leg of 2048 chains on 262144 dense disks.
+__device__ __noinline__ void g_repair_component(const GDev &s, int32_t *mem, int m, int cap,
+                                                int root, int round, uint32_t epoch,
+                                                uint32_t wr_tag, double tw, double tend) {
+    const int lane = threadIdx.x & 31;
+    double Ts = INFINITY;
+    // the members listed for this round of this pass (wr_tag names both)
+    const uint64_t tag = ((uint64_t)wr_tag << 32) | (uint32_t)root;
+    for (int e = lane; e < m; e += 32) {
+        const int c = mem[e];
+        Ts = fmin(Ts, s.vt[c]);
+        s.memb[c] = tag;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) Ts = fmin(Ts, __shfl_xor_sync(FULL, Ts, o));
+    Ts = fmax(Ts, tw);  // earlier windows are final
+    if (lane == 0) atomicAdd(s.lc + LC_REPAIRED, (unsigned long long)m);
+    __syncwarp();
+    uint32_t seq = 0;  // events of this repair so far: what is kept of one attempt
+                       // comes before the next one's in order
+    // (a later round of a leg without claim windows: chains that a repair which
+    // met another component left unfinished)
+    const bool whole = dbits(tend) == INF_BITS && dbits(tw) == 0ull;
+    if (round > 1 && whole) {
+        for (int e = lane; e < m; e += 32)
+            if (s.status[mem[e]] == ST_RUNNING) s.status[mem[e]] = ST_BLOCKED;
+        __syncwarp();
+    }
+    if (round == 1 || whole) {
+        int met = -1;
+        const int how = s.ring && !s.strict
+                            ? g_continue_ring(s, mem, m, root, tag, epoch, round, &met, &seq)
+                            : g_continue(s, mem, m, root, tag, epoch, round, tw, tend, &met,
+                                         &seq);
+        if (how == CONT_DONE) {
+            if (lane == 0) atomicAdd(s.lc + LC_CONTINUED, (unsigned long long)m);
+            g_finish(s, mem, m, root, false, -1, Ts, true);
+            return;
+        }
+        if (how == CONT_FOREIGN) {
+            // its events so far stand for the merged component to go on from (or
+            // to roll back to T*: all of this round's events lie after it)
+            g_finish(s, mem, m, root, true, met, Ts);
+            return;
+        }
+        // What was done is a run of Alg. 4 without a violation, so every event
+        // before the earliest time an unfinished chain stands at is exact
+        // (Remark 6): the replay starts there, not where the pass was cut.
+        if (whole) {
+            Ts = INFINITY;
+            for (int e = lane; e < m; e += 32)
+                if (s.status[mem[e]] == ST_BLOCKED) Ts = fmin(Ts, s.tc[mem[e]]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) Ts = fmin(Ts, __shfl_xor_sync(FULL, Ts, o));
+        }
+    }
+    for (;;) {
+        g_rollback(s, mem, m, Ts);
+        for (int e = lane; e < m; e += 32) g_resume(s, mem[e]);
+        __syncwarp();
+        int met = -1;
+        double now = Ts;
+        const bool abort =
+            m <= SMALL_REPLAY
+                ? g_replay_small(s, mem, m, epoch, round, Ts, tend, &met, &now, &seq)
+                : g_replay_large(s, mem, m, root, tag, epoch, round, Ts, tend, &met, &now,
+                                 &seq);
+        int more = 0;
+        if (abort && whole && round == 1 && m < cap && met >= 0 && met < s.k && lane == 0) {
+            // a chain of no component: it joins this one at once
+            int h = __ldcg(s.comp_of + met);
+            if (h == met && met != root && __ldcg(s.fin + met) == 1)
+                h = atomicCAS(s.comp_of + met, met, root) == met ? root : -1;
+            if (h == root) {
+                mem[m] = met;
+                s.memb[met] = tag;
+                atomicAdd(s.lc + LC_REPAIRED, 1ull);
+                more = 1;
+            }
+        }
+        if (!__shfl_sync(FULL, more, 0)) {
+            g_finish(s, mem, m, root, abort, met, now);
+            return;
+        }
+        ++m;
+        Ts = now;  // (the events before are exact)
+        __syncwarp();
+    }
 }
 
 // ------------------------------------------- persistent multi-leg kernel
@@ -3391,10 +3470,11 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
                     if (!fast) g_set_stamp(my_dev, leg, lane);
                     int root, m;
-                    const int32_t *mem;
+                    int32_t *mem;
+                    int cap = 0;
                     bool mine = true;
                     if (round == 1) {
-                        mine = g_members(s, q, s.epoch0 + pass, &root, &mem, &m);
+                        mine = g_members(s, q, s.epoch0 + pass, &root, &mem, &m, &cap);
                     } else {
                         root = s.comp_root[q];
                         const int off = s.comp_off[q];
@@ -3402,7 +3482,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                         mem = s.comp_mem + off;
                     }
                     if (mine)
-                        g_repair_component(s, mem, m, root, round, s.epoch0 + pass,
+                        g_repair_component(s, mem, m, cap, root, round, s.epoch0 + pass,
                                            ((uint32_t)(leg * B.windows + w) << 8) | (uint32_t)round,
                                            restart ? tw_r : g_window_start(s, w),
                                            g_window_end(s, w));
