@@ -161,8 +161,7 @@ struct ecmc_ctx {
     // scratch of ecmc_positions, one block
     char *exp = nullptr;
     int64_t exp_bytes = 0;
-    double *exp_x = nullptr, *exp_y = nullptr, *exp_t = nullptr;
-    int32_t *exp_a = nullptr;
+    double *exp_x = nullptr, *exp_t = nullptr;
 };
 
 static std::string g_create_err;
@@ -206,16 +205,14 @@ static int pick_cells(const ecmc_params *p, int *nc_out, int *C_out) {
     return 0;
 }
 
-// Parts of the scratch of ecmc_positions (each on a 256-byte boundary).
-static int64_t export_layout(int64_t n, int32_t k, ecmc_ctx *ctx) {
+// Parts of the scratch of ecmc_positions (x and t, each on a 256-byte boundary).
+static int64_t export_layout(int64_t n, ecmc_ctx *ctx) {
     const int64_t n8 = (n * 8 + 255) & ~(int64_t)255;
     if (ctx) {
         ctx->exp_x = (double *)ctx->exp;
-        ctx->exp_y = (double *)(ctx->exp + n8);
-        ctx->exp_t = (double *)(ctx->exp + 2 * n8);
-        ctx->exp_a = (int32_t *)(ctx->exp + 3 * n8);
+        ctx->exp_t = (double *)(ctx->exp + n8);
     }
-    return 3 * n8 + (((int64_t)k * 4 + 255) & ~(int64_t)255);
+    return 2 * n8;
 }
 
 // The system of a new context. With host inputs they are uploaded first; the
@@ -253,7 +250,8 @@ static int create_graph(ecmc_ctx *ctx, int nc, const double *x, const double *y,
         sa = da;
     }
     if (e == cudaSuccess) {
-        graph_check_inputs(sx, sy, sa, (int64_t)n, (int)k, p->box, seen, bad, bad + 1, ctx->stream);
+        graph_check_inputs(nullptr, nullptr, sa, (int64_t)n, (int)k, p->box, seen, bad, bad + 1,
+                           ctx->stream);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
@@ -289,7 +287,7 @@ extern "C" int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes) {
     const int64_t graph_bytes = graph_plan_bytes(p, nc);
     if (graph_bytes < 0) return ECMC_EINVAL;
     // (with the scratch of ecmc_positions, allocated by its first call)
-    *bytes = graph_bytes + export_layout(p->n, p->n_chains, nullptr);
+    *bytes = graph_bytes + export_layout(p->n, nullptr);
     return ECMC_OK;
 }
 
@@ -502,27 +500,27 @@ extern "C" int ecmc_positions(ecmc_ctx *ctx, double *x, double *y, double *t, in
     cudaStream_t st = ctx->stream;
     const size_t n = (size_t)ctx->p.n, k = (size_t)ctx->p.n_chains;
     if (!ctx->exp) {  // device scratch, allocated at the first call and kept
-        const int64_t total = export_layout(ctx->p.n, ctx->p.n_chains, nullptr);
+        const int64_t total = export_layout(ctx->p.n, nullptr);
         const int e = dm_alloc_t(&ctx->exp, (size_t)total);
         if (e != 0) {
             ctx->exp = nullptr;
             return fail(ctx, ECMC_ENOMEM,
                         std::string("cudaMalloc: ") + cudaGetErrorString((cudaError_t)e));
         }
-        ctx->exp_bytes = export_layout(ctx->p.n, ctx->p.n_chains, ctx);
+        ctx->exp_bytes = export_layout(ctx->p.n, ctx);
     }
-    double *dx = x ? ctx->exp_x : nullptr, *dy = y ? ctx->exp_y : nullptr;
-    double *dt = t ? ctx->exp_t : nullptr;
-    int32_t *da = active ? ctx->exp_a : nullptr;
-    // in a transposed context the stored x is the caller's y
-    if (graph_export(ctx->graph, ctx->direction ? dy : dx, ctx->direction ? dx : dy, dt, da) != 0)
+    // (in a transposed context the stored x is the caller's y)
+    double *const ox = ctx->direction ? y : x, *const oy = ctx->direction ? x : y;
+    const double *sy = nullptr;
+    const int32_t *sa = nullptr;
+    if (graph_export(ctx->graph, ox ? ctx->exp_x : nullptr, t ? ctx->exp_t : nullptr, &sy, &sa) != 0)
         return fail(ctx, ECMC_ECUDA, "positions (graph)");
     cudaError_t e = cudaSuccess;
-    if (x) e = cudaMemcpyAsync(x, dx, n * 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && y) e = cudaMemcpyAsync(y, dy, n * 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && t) e = cudaMemcpyAsync(t, dt, n * 8, cudaMemcpyDeviceToHost, st);
+    if (ox) e = cudaMemcpyAsync(ox, ctx->exp_x, n * 8, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && oy) e = cudaMemcpyAsync(oy, sy, n * 8, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && t) e = cudaMemcpyAsync(t, ctx->exp_t, n * 8, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess && active)
-        e = cudaMemcpyAsync(active, da, k * 4, cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(active, sa, k * 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess)
         return fail(ctx, ECMC_ECUDA, std::string("positions: ") + cudaGetErrorString(e));

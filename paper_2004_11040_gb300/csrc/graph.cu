@@ -206,6 +206,7 @@ struct GBuild {
     float del;           // a 2^-20: bound on the FP32 error of a difference of
                          // coordinates of neighbouring cells
     const double *x, *y;
+    unsigned long long *bad_xy;  // counts coordinates outside [0, L) (or null)
     const uint32_t *scid;  // [nc*nc*C] disk per slot, EMPTY
     uint32_t *cid;         // the same, writable (null with sx)
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
@@ -241,6 +242,7 @@ __global__ void k_gb_cells(GBuild b) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= b.n) return;
     const double x = b.x[q], y = b.y[q];
+    if (b.bad_xy && !(x >= 0.0 && x < b.L && y >= 0.0 && y < b.L)) atomicAdd(b.bad_xy, 1ull);
     const int row = cell_coord(y, b.inv_a, b.nc), col = cell_coord(x, b.inv_a, b.nc);
     const uint32_t cell = (uint32_t)row * (uint32_t)b.nc + (uint32_t)col;
     const float2 v = in_cell(b, x, y, row, col);
@@ -815,24 +817,38 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_place(GBuild b, GRing r, GD
 
 // The records of a frame of rings, each disk's successor its only arrow (a
 // cell-scan context; one with graph arrows has them from k_gb_arrows). Bound
-// by the 64 bytes a record takes.
-__global__ void k_ring_records(GBuild b, GDev s) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= s.n) return;
-    const uint32_t i = s.rid[p];
-    const uint4 at = s.pos[i];
-    const uint32_t j = s.rid[(uint32_t)p + 1u < at.y + at.z ? (uint32_t)p + 1u : at.y];
-    const double yi = b.y[i], ay = fabs(__dsub_rn(b.y[j], yi));
-    const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
-    const bool has = at.z > 1u;
-    ulonglong2 *g = reinterpret_cast<ulonglong2 *>(s.g + i);
-    g[0] = make_ulonglong2(dbits(b.x[i]), 0ull);
-    g[1] = make_ulonglong2((unsigned long long)OWN_STATIC |
-                               ((unsigned long long)(has ? j : NONE) << 32),
-                           ~0ull);
-    g[2] = make_ulonglong2(0ull, has ? dbits(v) : 0ull);
-    g[3] = make_ulonglong2(0ull, 0ull);
-    s.y[i] = yi;
+// by the 64 bytes a record takes: a thread per disk finds its fields, then four
+// lanes write a record, so that a store covers eight whole ones. 2^20 disks:
+// 59 us with a thread per record, 22 so.
+__global__ void __launch_bounds__(256) k_ring_records(GBuild b, GDev s) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i0 = i - lane;
+    unsigned long long xb = 0ull, vb = 0ull;
+    uint32_t a0 = NONE;
+    if (i < s.n) {
+        const uint4 at = s.pos[i];
+        const double yi = b.y[i];
+        xb = dbits(b.x[i]);
+        s.y[i] = yi;
+        if (at.z > 1u) {
+            a0 = s.rid[at.x + 1u < at.y + at.z ? at.x + 1u : at.y];
+            const double ay = fabs(__dsub_rn(b.y[a0], yi));
+            vb = dbits(__dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay))));
+        }
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+        const int src = 8 * z + (lane >> 2), part = lane & 3;
+        const unsigned long long x2 = shfl_u64(xb, src), v2 = shfl_u64(vb, src);
+        const uint32_t a2 = __shfl_sync(FULL, a0, src);
+        ulonglong2 w = make_ulonglong2(0ull, 0ull);
+        if (part == 0) w.x = x2;
+        if (part == 1)
+            w = make_ulonglong2((unsigned long long)OWN_STATIC | ((unsigned long long)a2 << 32),
+                                ~0ull);
+        if (part == 2) w.y = v2;
+        if (i0 + src < s.n) reinterpret_cast<ulonglong2 *>(s.g + i0 + src)[part] = w;
+    }
 }
 
 // The chains' start disks active (after a build).
@@ -3680,15 +3696,17 @@ static GBuild build_params(const GraphCtx *g) {
 // The first half of a frame's build, queued on the context's stream: every
 // disk in a cell, and whether the rows are rings (asked again on an axis only
 // while they were: rows that motion across them has mixed stay mixed).
-// b.err[0] counts overfull cells, b.err[1] rows that are no rings.
-static int graph_place(GraphCtx *g, const double *x, const double *y, GBuild *out,
-                       std::string &err) {
+// b.err[0] counts overfull cells, b.err[1] rows that are no rings, *bad_xy (if
+// not null) coordinates outside [0, L), which count as the nearest cell's.
+static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned long long *bad_xy,
+                       GBuild *out, std::string &err) {
     GDev &s = g->s;
     const int nc = g->nc;
     GBuild b = build_params(g);
     b.x = x;
     b.y = y;
     b.yout = s.y;
+    b.bad_xy = bad_xy;
     size_t off_bits, off_err, off_cid;
     const size_t total = build_parts(s.L, s.d, nc, g->C, &off_bits, &off_err, &off_cid);
     // scratch of the build, kept by the context for the next direction change
@@ -3757,12 +3775,13 @@ static int graph_records(GraphCtx *g, const GBuild &b, bool rings, const int32_t
 }
 
 // A frame from positions x, y and active disks (device): both halves, with a
-// wait for the first one's result between. bad: the two counters of a check of
-// the inputs queued before (null: they are known to be good).
+// wait for the first one's result between. bad: two counters, of coordinates
+// outside [0, L), counted here, and of bad ids, counted by a check queued before
+// (null: the inputs are known to be good).
 static int graph_build(GraphCtx *g, const double *x, const double *y, const int32_t *active,
-                       const unsigned long long *bad, std::string &err) {
+                       unsigned long long *bad, std::string &err) {
     GBuild b;
-    int rc = graph_place(g, x, y, &b, err);
+    int rc = graph_place(g, x, y, bad, &b, err);
     if (rc) return rc;
     unsigned long long h[2] = {0ull, 0ull}, hb[2] = {0ull, 0ull};
     cudaError_t e = cudaMemcpyAsync(h, b.err, sizeof h, cudaMemcpyDeviceToHost, g->st);
@@ -3942,7 +3961,7 @@ static void graph_clear(GraphCtx *g) {
 }
 
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
-                 const int32_t *active, const unsigned long long *bad, cudaStream_t st,
+                 const int32_t *active, unsigned long long *bad, cudaStream_t st,
                  GraphCtx **out, std::string &err) {
     *out = nullptr;
     if (p->n_chains > MAX_CHAINS) {
@@ -3983,7 +4002,8 @@ struct GBatchScratch {
     int cap = 0;
     int64_t chains = 0;
     unsigned char *block = nullptr;
-    size_t off_base = 0, off_comp = 0, off_ctl = 0, off_bar = 0, off_g = 0, off_phase = 0,
+    // (and the flags of a run of one system, up to FLAG_TABLE legs)
+    size_t off_flags = 0, off_base = 0, off_comp = 0, off_ctl = 0, off_bar = 0, off_g = 0, off_phase = 0,
            off_list = 0, total = 0;
     std::vector<unsigned char> host;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -3996,6 +4016,8 @@ void graph_batch_free(GBatchScratch *b) {
     if (b->ev1) cudaEventDestroy(b->ev1);
     delete b;
 }
+
+constexpr int32_t FLAG_TABLE = 1024;
 
 static int launch_reserve(GBatchScratch **scratch, int n, int64_t chains, std::string &err) {
     GBatchScratch *b = *scratch;
@@ -4022,6 +4044,7 @@ static int launch_reserve(GBatchScratch **scratch, int n, int64_t chains, std::s
     b->off_bar = take(sizeof(unsigned int));
     b->off_g = take(GG_N * sizeof(int32_t));
     b->off_phase = take(GPH_N * sizeof(unsigned long long));
+    b->off_flags = take(FLAG_TABLE);
     b->total = off;
     b->host.assign(off, 0);
     b->off_list = take((size_t)chains * sizeof(int32_t));  // (device only)
@@ -4104,7 +4127,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
     for (int r = 0; r < n; ++r) {
         GraphCtx *g = gs[r];
         if (g->st != st) cu(cudaStreamSynchronize(g->st), "context stream");
-        if (g->flags_cap < max_legs) {
+        if (max_legs > FLAG_TABLE && g->flags_cap < max_legs) {
             dm_free(g->d_flags);
             g->d_flags = nullptr;
             g->flags_cap = 0;
@@ -4124,8 +4147,11 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         }
         S[r] = g->s;
         ctl[r].budget = budgets ? (int64_t)budgets[r] : 0;
-        ctl[r].flags = g->d_flags;
-        ctl[r].flags_cap = g->flags_cap;
+        // (only a run of one system reports its flags)
+        ctl[r].flags = n > 1                    ? nullptr
+                       : max_legs <= FLAG_TABLE ? (uint8_t *)(b->block + b->off_flags)
+                                                : g->d_flags;
+        ctl[r].flags_cap = max_legs;
         ctl[r].leg0 = g->log_legs;
         base[r] = (int32_t)chains;
         chains += g->s.k;
@@ -4237,7 +4263,9 @@ int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
     const int rc = graph_batch_run(&g->launch, &g, 1, n_legs, &budget, g->st, tot, &legs, nullptr,
                                    err, wait_ns);
     if (legs_done) *legs_done = legs;
-    if (flags_host && legs > 0) {
+    if (flags_host && legs > 0 && n_legs <= FLAG_TABLE) {
+        memcpy(flags_host, g->launch->host.data() + g->launch->off_flags, (size_t)legs);
+    } else if (flags_host && legs > 0) {
         const cudaError_t e = cudaMemcpyAsync(flags_host, g->d_flags, (size_t)legs,
                                               cudaMemcpyDeviceToHost, g->st);
         if (e != cudaSuccess || cudaStreamSynchronize(g->st) != cudaSuccess) {
@@ -4249,13 +4277,12 @@ int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
     return rc;
 }
 
-int graph_export(GraphCtx *g, double *x, double *y, double *t, int32_t *active) {
+int graph_export(GraphCtx *g, double *x, double *t, const double **y, const int32_t **active) {
     const GDev &s = g->s;
-    cudaStream_t st = g->st;
-    if (x || t) k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t, nullptr);
-    if (y) cudaMemcpyAsync(y, s.y, (size_t)s.n * 8, cudaMemcpyDeviceToDevice, st);
-    if (active)
-        k_g_export_active<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active, nullptr);
+    *y = s.y;
+    *active = (const int32_t *)s.ci;
+    if (x || t)
+        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, x, t, nullptr);
     return cudaGetLastError() == cudaSuccess ? 0 : ECMC_ECUDA;
 }
 
@@ -4426,11 +4453,11 @@ int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, cons
     // the check's result
     cu(cudaMemsetAsync(a.seen, 0, (size_t)s.n * 4, st));
     cu(cudaMemsetAsync(a.bad, 0, 16, st));
-    graph_check_inputs(x, y, active, s.n, s.k, s.L, a.seen, a.bad, a.bad + 1, st);
+    graph_check_inputs(nullptr, nullptr, active, s.n, s.k, s.L, a.seen, a.bad, a.bad + 1, st);
     graph_clear(&g);
     cu(cudaMemsetAsync(s.memb, 0xFF, (size_t)s.k * 8, st));
     GBuild b;
-    if (!rc) rc = graph_place(&g, x, y, &b, err);
+    if (!rc) rc = graph_place(&g, x, y, a.bad, &b, err);
     unsigned long long bad[2], built[2];
     if (!rc) {
         cu(cudaMemcpyAsync(bad, a.bad, sizeof bad, cudaMemcpyDeviceToHost, st));

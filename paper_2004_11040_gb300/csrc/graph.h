@@ -21,17 +21,18 @@ struct GraphTotals {
 };
 
 // A context on device inputs x, y (n each) and active (k), which the work it
-// queues on the stream reads; bad: the counters of graph_check_inputs on them,
-// queued before. nc cells per side. With ECMC_GRAPH the conflict flag is on the
+// queues on the stream reads; bad: two counters, the second that of
+// graph_check_inputs on active, queued before. nc cells per side. With ECMC_GRAPH the conflict flag is on the
 // disks read, otherwise on the cells scanned.
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
-                 const int32_t *active, const unsigned long long *bad, cudaStream_t st,
+                 const int32_t *active, unsigned long long *bad, cudaStream_t st,
                  GraphCtx **out, std::string &err);
 int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
               int32_t *legs_done, GraphTotals *tot, std::string &err,
               unsigned long long wait_ns);
-// Device outputs (each may be null), filled on the context's stream.
-int graph_export(GraphCtx *g, double *x, double *y, double *t, int32_t *active);
+// x and t (device, each may be null) filled on the context's stream; *y and
+// *active point to the context's own arrays.
+int graph_export(GraphCtx *g, double *x, double *t, const double **y, const int32_t **active);
 // Exchanges x and y of every disk (the next legs move along the other axis),
 // clears the local times and rebuilds the graph.
 int graph_transpose(GraphCtx *g, std::string &err);
