@@ -1343,10 +1343,10 @@ struct GRingDisk {
 // Bound by that chain (~100 cycles an event against ~1000 of a step) and the
 // four dependent loads before it. 1024 chains on 2^20 disks: a leg 82 us with
 // the scan of row bands this replaces, 65 with it; 16384 chains: 890 -> 605.
-__device__ __noinline__ bool g_leap_chain(const GDev &s, int c, bool begin) {
+__device__ __noinline__ bool g_leap_chain(const GDev &s, int c) {
     const int lane = threadIdx.x & 31;
     const uint32_t i0 = s.ci[c];
-    if (begin) g_begin_state(s, c, i0, lane);
+    g_begin_state(s, c, i0, lane);
     const GDisk *const g = s.g;
     const double L = s.L;
     const uint4 at0 = s.pos[i0];
@@ -3221,13 +3221,15 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
     const int R = B.R;
     const int total_chains = B.chain_base[R];
     const bool restart = R == 1 && B.reps[0].restart;
-    // one system without claim windows or restarts: a leg has three phases and
-    // three barriers. Its chains begin the next leg at its pass (the stamps
-    // make clearing local times unnecessary, s.lc alternates by leg), the
-    // touch keys go during the repair, and the totals of a leg are taken by
-    // one warp while the next one resolves. Otherwise (several systems, whose
-    // budgets decide which go on) a leg end of its own follows the repair.
-    const bool fast = R == 1 && !B.reps[0].strict;
+    // Without claim windows or restarts a leg has one pass. Its chains begin the
+    // leg there (the stamps make clearing local times unnecessary), and the flag
+    // is found and the touch keys go during the repair. (In a phase of their own
+    // before the pass, and with the resolve and the leg end: a batch of 128 21.3
+    // ms, 20.0 so, 12 served requests 25.4 and 23.7.) One such system also needs no leg end: s.lc
+    // alternates by leg, and the totals of a leg are taken by one warp while the
+    // next one resolves. Of several systems the budgets decide which go on.
+    const bool simple = !B.reps[0].strict;
+    const bool fast = R == 1 && simple;
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long t_prev = timer ? gtimer() : 0ull;
     auto mark = [&](int ph) {
@@ -3315,7 +3317,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         c.continued += (int64_t)lc[LC_CONTINUED];
         c.restarts += (int64_t)lc[LC_RESTARTS];
         c.blocked += (int64_t)lc[LC_BLOCKED];
-        c.cwindows += fast ? flag : (int64_t)lc[LC_CWINDOWS];
+        c.cwindows += simple ? flag : (int64_t)lc[LC_CWINDOWS];
         if (B.reps[r].ring && B.reps[r].cells && lc[LC_RINGLAP] == 0ull) c.row_windows += B.windows;
         c.horizon += (int64_t)lc[LC_HORIZON];
         c.order_err += (int64_t)lc[LC_ORDER];
@@ -3342,7 +3344,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         }
         // leg start of the systems whose last leg did not begin this one
         bool begin_here = false;
-        for (int r = 0; r < R && !fast; ++r)
+        for (int r = 0; r < R && !simple; ++r)
             if (g_rep_on(B, r) && !(leg > 0 && g_next_at_end(B, r, leg - 1))) begin_here = true;
         if (begin_here) {
             for (int f = gw; f < total_chains; f += nwarps) {
@@ -3366,9 +3368,11 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         bool any = false;  // (fast) the leg had something to repair
         auto flags = [&]() {
             for (int f = gw; f < total_chains; f += nwarps) {
-                const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, 0);
-                g_flag_chain(s, f, s.epoch0 + pass, lane);
-                g_reset_keys(s, f, lane);
+                const int r = g_find_rep(B.chain_base, R, f), c = f - B.chain_base[r];
+                if (!g_rep_on(B, r)) continue;
+                const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+                g_flag_chain(s, c, s.epoch0 + pass, lane);
+                g_reset_keys(s, c, lane);
             }
         };
         for (int w = 0; w < B.windows; ++w) {
@@ -3396,9 +3400,9 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
                     if (!fast) g_set_stamp(my_dev, leg, lane);
                     g_begin_pass(s, f - B.chain_base[r], lane);
-                    if (s.ring && !s.strict && g_leap_chain(s, f - B.chain_base[r], fast)) continue;
+                    if (s.ring && simple && g_leap_chain(s, f - B.chain_base[r])) continue;
                     g_spec_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
-                                 g_window_end(s, w), fast);
+                                 g_window_end(s, w), simple);
                 }
                 if (!barrier()) return;
                 if (gt == 0 && w == 0 && sub == 0) B.g[GG_REMAIN0 + ((leg + 1) & 1)] = 0;
@@ -3412,7 +3416,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     if (!fast) g_set_stamp(my_dev, leg, lane);
                     g_resolve_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
                                     s.epoch0 + pass, f, bl);
-                    if (!fast && sub == 0)
+                    if (!simple && sub == 0)
                         g_flag_chain(s, f - B.chain_base[r], s.epoch0 + pass, lane);
                 }
                 if (!barrier()) return;
@@ -3457,7 +3461,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 ++sub;
             }
             // the window's flag: the reads of two chains met
-            for (int r = gt; r < R && !fast; r += (int)(gridDim.x * blockDim.x))
+            for (int r = gt; r < R && !simple; r += (int)(gridDim.x * blockDim.x))
                 if (g_rep_on(B, r) && __ldcg(B.reps[r].lc + LC_WWEAK) != 0ull)
                     atomicAdd(B.reps[r].lc + LC_CWINDOWS, 1ull);
             // repair rounds
@@ -3505,7 +3509,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     if (round == 1 && ncomp <= nwarps) break;
                     z = -1;
                 }
-                if (fast && round == 1) flags();
+                if (simple && round == 1) flags();
                 if (!barrier()) return;
                 // no component met another chain: the window is repaired
                 int aborted = 0;
@@ -3513,7 +3517,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     if (g_rep_on(B, r) && __ldcg(B.reps[r].ctl + CTL_NABORT) != 0) aborted = 1;
                 if (!__syncthreads_or(aborted)) break;
             }
-            if (fast && nblk == 0) flags();
+            if (simple && nblk == 0) flags();
             any = nblk > 0;
             mark(GPH_REPAIR);
         }
@@ -3541,9 +3545,9 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
             if (!g_rep_on(B, r)) continue;
             const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
             const int c = f - B.chain_base[r];
-            g_reset_keys(s, c, lane);
+            if (!simple) g_reset_keys(s, c, lane);
             if (s.log_on) g_log_chain(s, c, (int32_t)(B.ctl[r].leg0 + B.ctl[r].legs), lane);
-            if (g_next_at_end(B, r, leg)) g_begin_state(s, c, s.ci[c], lane);
+            if (!simple && g_next_at_end(B, r, leg)) g_begin_state(s, c, s.ci[c], lane);
         }
         if (last_block())
             for (int r = threadIdx.x; r < R; r += blockDim.x)
