@@ -341,12 +341,12 @@ def measure(a, search, start, stream, flush, barrier, ws, nc, e2e=True):
     t_max, tot_lifts = aggregate(dev_ms, lifts, ws, device="cuda")
     # the hot path is one persistent kernel launch per step, timed by CUDA
     # events around the launch on the context's stream
-    kname = "k_run_graph" if graph else "k_run"
+    kname = "k_run_graph"  # (traffic.json: "k_run" is its launch on cell-scan contexts)
     kms = dev_ms / a.steps
     kl = lifts / a.steps
     peak, peak_kind = peaks()
     achieved = (kl * BYTES_PER_LIFTING) / (kms / 1000.0) / 1e9 if kms > 0 else 0.0
-    per_lift = traffic_for(kname)
+    per_lift = traffic_for("k_run_graph" if graph else "k_run")
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_source": peak_kind,
             "traffic": per_lift * kl if per_lift else None, "kernel": kname,

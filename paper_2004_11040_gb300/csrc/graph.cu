@@ -1341,8 +1341,9 @@ struct GRingDisk {
 // its ring, or out of records, is left to g_spec_chain (false).
 //
 // Bound by that chain (~100 cycles an event against ~1000 of a step) and the
-// four dependent loads before it. 1024 chains on 2^20 disks: a leg 82 us with
-// the scan of row bands this replaces, 65 with it; 16384 chains: 890 -> 605.
+// four dependent loads before it. 1024 chains on 2^20 disks: the pass 5 us, a
+// step per event 12; a leg 82 us with the scan of row bands this replaced, 65
+// with it at first, 32 now (16384 chains: 890, 605, 200).
 __device__ __noinline__ bool g_leap_chain(const GDev &s, int c) {
     const int lane = threadIdx.x & 31;
     const uint32_t i0 = s.ci[c];
@@ -2418,7 +2419,7 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
 // written since. (Claims beyond one that fails stay; the component they belong
 // to is repaired again.) A run that comes round its ring is left to the replay.
 // 1024 chains on 2^20 disks: the repair phase of a leg 33 us with a step per
-// event, 21 by stretches.
+// event, 17 by stretches.
 __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, int m, int root,
                                             uint64_t tag, uint32_t epoch, int round, int *met,
                                             uint32_t *cnt_out) {
@@ -3197,10 +3198,15 @@ constexpr int MAX_RESTARTS = 16;  // per leg, then the local repair takes over
 
 // One cooperative launch runs up to max_legs legs of every system. Per leg
 // and claim window: the parallel pass (one warp per chain), the resolve, then
-// repair rounds (conflict components by one block per system, their repairs
-// by one warp each from one queue) until no component met another chain; the
-// leg end with each system's totals. Phases are separated by grid barriers
-// whose waits are bounded (ECMC_ETIMEOUT). Restart mode takes one system.
+// repair rounds (one warp per component: in the first round the one of its
+// blocked chains, in later ones, whose components one block per system finds,
+// from a queue) until no component met another chain; the leg end with each
+// system's totals. Phases are separated by grid barriers whose waits are
+// bounded (ECMC_ETIMEOUT). Restart mode takes one system.
+//
+// Bound by latency: a leg of 1024 chains on 2^20 lattice disks takes 32 us, of
+// which the runs alone 5, the publishing 8, the continuations 8 to 17, three
+// barriers 3; DRAM and the FP64 pipes are nearly idle.
 __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBatchDev B) {
     extern __shared__ int32_t uf_sm[];  // UF_SMEM_BYTES: the union-find working set
     __shared__ int warp_tot[32];
@@ -3925,10 +3931,11 @@ static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
     // slots per cell: at most 4 centres at mutual distance >= d fit in a cell
     // with a < sqrt(2) d, at most 6 for a < 1.664 d
     g->C = a < std::sqrt(2.0) * p->d * (1.0 - 1e-9) ? 4 : 8;
-    // rings need four stretches' worth of columns and a leg that cannot come
-    // round the box; a context may go without
-    g->try_ring[0] = g->try_ring[1] = !(p->flags & ECMC_NO_ROWPASS) && nc >= 4 * (32 / g->C) &&
-                                      p->ell < p->box - 3.0 * a;
+    // a leg along rings must not come round the box; a context may go without
+    // (256 disks, 4 chains: a leg 31 us along the arrows of G(3), 23 along rings;
+    // 2^20 disks, 1024 chains: 63 and 32)
+    g->try_ring[0] = g->try_ring[1] =
+        !(p->flags & ECMC_NO_ROWPASS) && p->ell < p->box - 3.0 * a;
     // FP32 image of the scan's stop rule thr(m) = ((m a) - fx) - d > RN(cur +
     // eps): thr_f = ((m af - fxf) - df) and lim_f = trunc(cur) + epsf, with af,
     // df, epsf the FP32 roundings, fxf = trunc(fx). Each of the four FP32

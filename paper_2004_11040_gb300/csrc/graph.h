@@ -1,5 +1,5 @@
 // graph.h -- internal interface between the C ABI (ecmc.cu) and the
-// constraint-graph path (graph.cu, ECMC_GRAPH). Not part of the public ABI.
+// engine of the legs (graph.cu). Not part of the public ABI.
 #pragma once
 
 #include <cuda_runtime.h>
