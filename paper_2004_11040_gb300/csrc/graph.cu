@@ -819,7 +819,7 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_place(GBuild b, GRing r, GD
 // cell-scan context; one with graph arrows has them from k_gb_arrows). Bound
 // by the 64 bytes a record takes: a thread per disk finds its fields, then four
 // lanes write a record, so that a store covers eight whole ones. 2^20 disks:
-// 59 us with a thread per record, 22 so.
+// 59 us with a thread per record, 28 so.
 __global__ void __launch_bounds__(256) k_ring_records(GBuild b, GDev s) {
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i0 = i - lane;
