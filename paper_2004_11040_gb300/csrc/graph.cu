@@ -163,6 +163,13 @@ __device__ void gdiag(const GDev &s, int kind, double a, double b, double c, dou
     s.dbg[6] = f;
 }
 
+// A coordinate as given, -0.0 taken as 0: the build ranks coordinates by their
+// bits, where -0.0 lies above every other number. (On the integer pipe; the
+// frames' own x and y never are -0.0 again.)
+__device__ __forceinline__ double coord(double v) {
+    return dbits(v) == 0x8000000000000000ull ? 0.0 : v;
+}
+
 __device__ __forceinline__ int cell_coord(double v, double inv_a, int nc) {
     int c = __double2int_rz(__dmul_rn(v, inv_a));
     if (c >= nc) c = nc - 1;
@@ -241,7 +248,7 @@ template <int C>
 __global__ void k_gb_cells(GBuild b) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= b.n) return;
-    const double x = b.x[q], y = b.y[q];
+    const double x = coord(b.x[q]), y = coord(b.y[q]);
     if (b.bad_xy && !(x >= 0.0 && x < b.L && y >= 0.0 && y < b.L)) atomicAdd(b.bad_xy, 1ull);
     const int row = cell_coord(y, b.inv_a, b.nc), col = cell_coord(x, b.inv_a, b.nc);
     const uint32_t cell = (uint32_t)row * (uint32_t)b.nc + (uint32_t)col;
@@ -332,10 +339,10 @@ __device__ __forceinline__ bool take_best(GBest &best, float lo, float hi, uint3
 }
 
 __device__ __forceinline__ double gb_x(const GBuild &b, uint32_t loc, uint32_t id) {
-    return b.x[id];
+    return coord(b.x[id]);
 }
 __device__ __forceinline__ double gb_y(const GBuild &b, uint32_t loc, uint32_t id) {
-    return b.y[id];
+    return coord(b.y[id]);
 }
 
 // The FP32 coordinates of a cell's slots, all loads at once.
@@ -709,7 +716,7 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_count(GBuild b, GRing r) {
 #pragma unroll
         for (int z = 0; z < C; ++z) {
             if (id[z] == EMPTY) continue;
-            const unsigned long long y = dbits(b.y[id[z]]);  // y >= 0: ordered by bits
+            const unsigned long long y = dbits(coord(b.y[id[z]]));  // ordered by bits
             lo = y < lo ? y : lo;
             hi = y > hi ? y : hi;
             ++n;
@@ -797,7 +804,7 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_place(GBuild b, GRing r, GD
         for (int q = 0; q < C; ++q) id[q] = b.scid[((size_t)row * nc + col) * C + q];
 #pragma unroll
         for (int q = 0; q < C; ++q) {
-            x[q] = id[q] != EMPTY ? b.x[id[q]] : INFINITY;
+            x[q] = id[q] != EMPTY ? coord(b.x[id[q]]) : INFINITY;
             n += id[q] != EMPTY;
         }
     }
@@ -806,7 +813,7 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_place(GBuild b, GRing r, GD
 #pragma unroll
     for (int q = 0; q < C; ++q) {
         if (id[q] == EMPTY) continue;
-        int rank = 0;  // x >= 0: ordered by bits
+        int rank = 0;  // ordered by bits
 #pragma unroll
         for (int z = 0; z < C; ++z)
             rank += dbits(x[z]) < dbits(x[q]) || (z < q && dbits(x[z]) == dbits(x[q]));
@@ -827,12 +834,12 @@ __global__ void __launch_bounds__(256) k_ring_records(GBuild b, GDev s) {
     uint32_t a0 = NONE;
     if (i < s.n) {
         const uint4 at = s.pos[i];
-        const double yi = b.y[i];
-        xb = dbits(b.x[i]);
+        const double yi = coord(b.y[i]);
+        xb = dbits(coord(b.x[i]));
         s.y[i] = yi;
         if (at.z > 1u) {
             a0 = s.rid[at.x + 1u < at.y + at.z ? at.x + 1u : at.y];
-            const double ay = fabs(__dsub_rn(b.y[a0], yi));
+            const double ay = fabs(__dsub_rn(coord(b.y[a0]), yi));
             vb = dbits(__dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay))));
         }
     }
