@@ -3279,7 +3279,10 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         if (threadIdx.x < 32) (void)g_warp_dev(wdev, wrep, B.reps, r);
         __syncthreads();
         const GDev &s = wdev[0];
-        const bool need = g_rep_on(B, r) && __ldcg(s.ctl + CTL_NABORT) != 0;
+        // (a system with a chain out of records has failed its leg: no merge cures
+        // that, and every further round would fail alike)
+        const bool need = g_rep_on(B, r) && __ldcg(s.ctl + CTL_NABORT) != 0 &&
+                          __ldcg(s.lc + LC_ERR_REC) == 0ull;
         if (need && round <= 255) {
             // the chains taken over in the last round
             for (int c = threadIdx.x; c < s.k; c += blockDim.x) {
