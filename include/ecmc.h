@@ -76,7 +76,8 @@ typedef struct {
     int64_t legs;            /* breakpoints reached */
     int64_t conflict_legs;   /* legs in which two chains' scanned cells met */
     int64_t repaired_chains; /* chains in conflict components (once per repair round) */
-    int64_t horizon_asserts; /* Eq. 2 failures seen by a conflict-free chain: 0 */
+    int64_t horizon_asserts; /* Eq. 2 failures that a chain's run alone (the parallel pass)
+                                saw on a disk with a time of its own window: 0 */
     int64_t order_errors;    /* repaired events found out of time order: 0 */
     double device_ms;        /* device time spent in ecmc_run_to_breakpoint */
     int64_t continued_chains; /* of repaired_chains: in components finished by continuing

@@ -1185,6 +1185,9 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
                 // per-chain frame)
                 lap = !nsc && dbits(sum) < dbits(rt);
                 if (lap) tau = g_add(tau, L);
+                // (in the chain's own window only it has moved disks, each at
+                // its own time then: an assertion)
+                if (lap && dbits(rt) >= dbits(tw)) atomicAdd(s.lc + LC_HORIZON, 1ull);
                 hv = nsc && !(dbits(sum) > dbits(rt));
             }
         }
@@ -1393,6 +1396,13 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c) {
         const int f = fin ? __ffs(fin) - 1 : 31;  // the event that ends the run, or none
         const bool round = fin && !__shfl_sync(FULL, (int)in, f);
         const bool met = fin && !round && __shfl_sync(FULL, (int)lift, f);  // lift onto an active disk
+        // Eq. 2 on the targets with a time of this leg: before its pass there
+        // are none (an assertion)
+        const bool timed = in && lane <= f && ownn == s.stamp;
+        if (__any_sync(FULL, timed)) {
+            const double rt = shfl_f64(k.t, (lane + 1) & 31);
+            if (timed && dbits(g_add(t, tau)) < dbits(rt)) atomicAdd(s.lc + LC_HORIZON, 1ull);
+        }
         n = n0 + f + (fin && !met ? 1 : 0);
         if ((round && len > 1) || n >= s.cap) {
             if (lane == 0 && round) atomicAdd(s.lc + LC_RINGLAP, 1ull);
