@@ -217,6 +217,11 @@ struct GBuild {
     const uint32_t *scid;  // [nc*nc*C] disk per slot, EMPTY
     uint32_t *cid;         // the same, writable (null with sx)
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
+    uint32_t *far;         // [n] slots of the disks left to k_gb_far, and their number
+    unsigned *far_n;
+    int nblk;              // blocks of FAR_COLS columns in a row
+    float4 *ylim;          // [nc*nblk] least and largest y (within the cell row) per block
+                           // in the row's lower half, and in its upper one
     uint32_t *bits;        // [nb / 32 + 1]
     GDisk *g;
     double *yout;             // [n] or null: each disk's y
@@ -303,8 +308,10 @@ __device__ __forceinline__ float sqrt_f(float v) {
 }
 
 // The corridor of the disk at v (in its cell, rr rows and m columns on) seen
-// from xi, yi (-1: none; 3: FP32 cannot tell) and, for 0 .. 2, bounds of its
-// time of flight.
+// from xi, yi (-1: none; EDGE: FP32 cannot tell which, or whether none; NEXT: nor
+// whether it is ahead or a lap away) and, but for NEXT, bounds of its time of
+// flight.
+enum { EDGE = 3, NEXT = 4 };
 __device__ __forceinline__ int corridor_f(const GBuild &b, float xi, float yi, int rr, int m,
                                           float2 v, float &lo, float &hi) {
     const float dy = (float)rr * b.af + (v.y - yi);
@@ -312,7 +319,7 @@ __device__ __forceinline__ int corridor_f(const GBuild &b, float xi, float yi, i
     if (ay > b.df + b.del) return -1;
     float dx = (float)m * b.af + (v.x - xi);
     float del = b.del + (float)m * (0.25f * b.del);
-    if (ay > b.df - b.del || fabsf(ay - b.half_f) < b.del || fabsf(dx) < del) return 3;
+    if (fabsf(dx) < del) return NEXT;
     if (dx < 0.f) {  // behind in its own column: nearly a lap ahead
         dx += b.Lf;
         del += b.Lf * 0x1p-21f;
@@ -321,8 +328,36 @@ __device__ __forceinline__ int corridor_f(const GBuild &b, float xi, float yi, i
     // (2^-19 d covers the roundings of these lines)
     const float slop = b.df * 0x1p-19f + del;
     hi = dx - sqrt_f(fmaxf(d2 - af * af - d2 * 0x1p-21f, 0.f)) + slop;
-    lo = dx - sqrt_f(d2 - an * an + d2 * 0x1p-21f) - slop;
+    lo = dx - sqrt_f(fmaxf(d2 - an * an, 0.f) + d2 * 0x1p-21f) - slop;
+    if (ay > b.df - b.del || fabsf(ay - b.half_f) < b.del) return EDGE;
     return ay < b.half_f ? 0 : dy > 0.f ? 1 : 2;
+}
+
+// The corridor (-1: none) and the time of flight by their definition, in FP64.
+struct GFlight {
+    int kc;
+    double tau;
+};
+__device__ __noinline__ GFlight flight_exact(double L, double d, double d2, double xi, double yi,
+                                             double xj, double yj) {
+    GFlight f = {-1, 0.0};
+    const double dy = __dsub_rn(yj, yi);
+    double ay = fabs(dy);
+    const double la = __dsub_rn(L, ay);
+    const bool flip = dbits(la) < dbits(ay);
+    if (flip) ay = la;
+    if (dbits(ay) >= dbits(d)) return f;
+    f.kc = 0;
+    if (dbits(ay) >= dbits(__dmul_rn(0.5, d))) {
+        bool up = !dneg(dy) && dbits(dy) != 0ull;
+        if (flip) up = !up;
+        f.kc = up ? 1 : 2;
+    }
+    double dx = __dsub_rn(xj, xi);
+    if (dneg(dx)) dx = __dadd_rn(dx, L);
+    f.tau = __dsub_rn(dx, __dsqrt_rn(__dsub_rn(d2, __dmul_rn(ay, ay))));
+    if (dneg(f.tau)) f.tau = 0.0;
+    return f;
 }
 
 // The candidate of a corridor takes the place of the best or not; true where
@@ -363,107 +398,371 @@ __device__ __forceinline__ GCell<C> load_cell(const GBuild &b, uint32_t c0) {
     return r;
 }
 
-// The corridors of disk i (slot loc, FP32 place vi) by their definition, in
-// FP64: where FP32 cannot tell. The warp searches 32 columns at a time; the
-// slots of each corridor's arrow (NONE: empty) end in aj on every lane.
+// The arrow in corridor q of a disk (slot loc, FP32 place vi) by its definition,
+// where the FP32 bounds of the nearest candidates overlap: the warp looks at the
+// columns that hold disks with times of flight from lo to hi (take_best: the
+// least lower bound of those that may come first, and the least upper one), and
+// at the disk's own column, where one behind lies a lap ahead. The arrow's slot.
 template <int C>
-__device__ __noinline__ void arrows_exact(const GBuild &b, uint32_t i, uint32_t loc, float2 vi,
-                                          double xi, double yi, int cxi, int cyi, bool p1, bool p2,
-                                          uint32_t *aj) {
+__device__ __noinline__ uint32_t arrow_exact(const GBuild &b, int q, uint32_t loc, float2 vi,
+                                             double xi, double yi, int cxi, int cyi, float lo,
+                                             float hi) {
     const int nc = b.nc, lane = threadIdx.x & 31;
-    const double half = __dmul_rn(0.5, b.d);
-    unsigned long long bt[3] = {INF_BITS, INF_BITS, INF_BITS};
-    uint32_t bj[3] = {NONE, NONE, NONE}, bl[3] = {NONE, NONE, NONE};
-    for (int m0 = 0; m0 < nc; m0 += 32) {
-        const int m = m0 + lane;
+    unsigned long long bt = INF_BITS;
+    uint32_t bj = NONE, bl = NONE;
+    // (a candidate in column m lies (m - 1) a to (m + 1) a ahead, b <= d beyond tau)
+    const int m1 = min(nc - 1, (int)((hi + b.df) / b.af) + 3);
+    for (int m0 = max(0, (int)(lo / b.af) - 3); m0 <= m1; m0 += 31) {
+        const int m = lane == 31 ? 0 : m0 + lane;
         int col = cxi + m;
         if (col >= nc) col -= nc;
-        for (int rr = -1; rr <= 1; ++rr) {
-            int row = cyi + rr;
+#pragma unroll 1
+        for (int z = 0; z < 3; ++z) {
+            int row = cyi + z - 1;
             if (row < 0) row += nc;
             if (row >= nc) row -= nc;
+#pragma unroll 1
             for (int sl = 0; sl < C; ++sl) {
-                const uint32_t at = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C + sl;
-                float lo, hi;
-                bool cand = m < nc && at != loc && b.cxy[m < nc ? at : loc].x >= 0.f;
-                cand = cand && corridor_f(b, vi.x, vi.y, rr, m, b.cxy[at], lo, hi) >= 0;
-                if (!__any_sync(FULL, cand)) continue;
-                if (!cand) continue;
-                const uint32_t id = b.scid[at];
-                const double dy = __dsub_rn(gb_y(b, at, id), yi);
-                double ay = fabs(dy);
-                const double la = __dsub_rn(b.L, ay);
-                const bool flip = dbits(la) < dbits(ay);
-                if (flip) ay = la;
-                if (dbits(ay) >= dbits(b.d)) continue;
-                int kc = 0;
-                if (dbits(ay) >= dbits(half)) {
-                    bool up = !dneg(dy) && dbits(dy) != 0ull;
-                    if (flip) up = !up;
-                    kc = up ? 1 : 2;
-                }
-                double dx = __dsub_rn(gb_x(b, at, id), xi);
-                if (dneg(dx)) dx = __dadd_rn(dx, b.L);
-                double tau = __dsub_rn(dx, __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay))));
-                if (dneg(tau)) tau = 0.0;
-                const unsigned long long kt = dbits(tau);
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (q == kc && (kt < bt[q] || (kt == bt[q] && id < bj[q]))) {
-                        bt[q] = kt;
-                        bj[q] = id;
-                        bl[q] = at;
-                    }
-            }
-        }
-        float worst = -1.f;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long t2 = shfl_xor_u64(bt[q], o);
-                const uint32_t j2 = __shfl_xor_sync(FULL, bj[q], o);
-                const uint32_t l2 = __shfl_xor_sync(FULL, bl[q], o);
-                if (t2 < bt[q] || (t2 == bt[q] && j2 < bj[q])) {
-                    bt[q] = t2;
-                    bj[q] = j2;
-                    bl[q] = l2;
+                const uint32_t slot =
+                    m < nc ? ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C + sl : loc;
+                const float2 v = b.cxy[slot];
+                if (slot == loc || !(v.x >= 0.f)) continue;
+                float l, h;
+                const int kc = corridor_f(b, vi.x, vi.y, z - 1, m, v, l, h);
+                if (!(kc >= EDGE || (kc == q && l <= hi))) continue;
+                const uint32_t id = b.scid[slot];
+                const GFlight f =
+                    flight_exact(b.L, b.d, b.d2, xi, yi, gb_x(b, slot, id), gb_y(b, slot, id));
+                const unsigned long long kt = dbits(f.tau);
+                if (f.kc == q && (kt < bt || (kt == bt && id < bj))) {
+                    bt = kt;
+                    bj = id;
+                    bl = slot;
                 }
             }
-            if (q == 0 || (q == 1 ? p1 : p2))
-                worst = fmaxf(worst, d2f_trunc(__longlong_as_double((long long)bt[q])));
         }
-        const int mn = m0 + 32;
-        if ((float)mn * b.af - vi.x - b.df - (float)(mn + 4) * b.del > worst * (1.f + 0x1p-20f))
-            break;
     }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) aj[q] = bl[q];
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long t2 = shfl_xor_u64(bt, o);
+        const uint32_t j2 = __shfl_xor_sync(FULL, bj, o);
+        const uint32_t l2 = __shfl_xor_sync(FULL, bl, o);
+        if (t2 < bt || (t2 == bt && j2 < bj)) {
+            bt = t2;
+            bj = j2;
+            bl = l2;
+        }
+    }
+    return bl;
+}
+
+constexpr int FAR_COLS = 8, FAR_LANES = 8;
+static_assert(FAR_LANES >= FAR_COLS, "a lane per column of a block");
+
+// Least and largest y, relative to the corner of the cell row, of every block of
+// FAR_COLS columns in either half of the row (a lane per cell; empty: +inf,
+// -inf). Limits of a whole row would span a corridor that no disk of the row is
+// in wherever two rows of disks share a row of cells.
+template <int C>
+__global__ void k_gb_blocks(GBuild b) {
+    if (*b.far_n == 0u) return;  // nothing is searched beyond the near columns
+    static_assert(FAR_COLS == 8, "a block is a quarter of a warp's lanes");
+    const int64_t end = (int64_t)b.nc * b.nblk * FAR_COLS;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; __any_sync(FULL, q < end);
+         q += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t blk = q / FAR_COLS, row = blk / b.nblk;
+        const int col = (int)(blk - row * b.nblk) * FAR_COLS + (int)(q % FAR_COLS);
+        float lo[2] = {INFINITY, INFINITY}, hi[2] = {-INFINITY, -INFINITY};
+        if (q < end && col < b.nc) {
+            const GCell<C> cell =
+                load_cell<C>(b, ((uint32_t)row * (uint32_t)b.nc + (uint32_t)col) * C);
+#pragma unroll
+            for (int sl = 0; sl < C; ++sl) {
+                const float y = cell.v[sl].y;
+                if (!(cell.v[sl].x >= 0.f)) break;
+                const bool up = y > 0.5f * b.af;
+                lo[0] = up ? lo[0] : fminf(lo[0], y);
+                hi[0] = up ? hi[0] : fmaxf(hi[0], y);
+                lo[1] = up ? fminf(lo[1], y) : lo[1];
+                hi[1] = up ? fmaxf(hi[1], y) : hi[1];
+            }
+        }
+#pragma unroll
+        for (int o = FAR_COLS / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                lo[z] = fminf(lo[z], __shfl_xor_sync(FULL, lo[z], o));
+                hi[z] = fmaxf(hi[z], __shfl_xor_sync(FULL, hi[z], o));
+            }
+        if (q < end && q % FAR_COLS == 0) b.ylim[blk] = make_float4(lo[0], hi[0], lo[1], hi[1]);
+    }
 }
 
 // Arrows of G(3), and the whole record of every disk (static, time 0): one
 // thread per disk. A block takes BUILD_CELLS cells of consecutive numbers and
 // packs their occupied slots first, so that warps are full and neighbours read
 // the same cells. The search runs in FP32: per corridor, bounds of the time of
-// flight of the best candidate; candidates whose bounds overlap, or whose
-// corridor FP32 cannot tell, send the disk to arrows_exact (a few in 10^5). After NEAR_COLS columns the corridors that still have none -- few
-// disks, but each would hold up its warp for a search of the whole ring -- are
-// searched by the warp together, 32 columns at a time. FP64 is left with one
-// b = sqrt(d^2 - dy^2) per arrow, all lanes at once (an FP64 instruction costs
-// the same whatever its lane mask). Corridors and rows that the y bins show
-// empty are not searched. 65536 dense disks: 31 us along their dense axis, 48 to
-// 88 us along the other (few disks in some corridors), with a thread per disk
-// searching alone in FP64 100 to 550 us; 2^20 lattice disks 107 us (124 us),
-// bound by its instructions and by the scattered reads and records.
+// flight of the best candidate. FP64 is left with one b = sqrt(d^2 - dy^2) per
+// arrow, all lanes at once (an FP64 instruction costs the same whatever its lane
+// mask). Corridors and rows that the y bins show empty are not searched.
+//
+// Disks that NEAR_COLS columns do not settle, and those with candidates whose
+// bounds overlap (a few in 10^5), go on a list for k_gb_far: half of them on a
+// triangular lattice at eta 0.60, a tenth at 0.70, one in 500 along the other
+// axis. (With the far search in this kernel it took 92 registers: 129 us on 10^6
+// square-lattice disks, 108 so at 64. After 4 columns 175 + 190 us with k_gb_far
+// on 10^6 triangular disks at 0.70, after 8 198 + 75.)
 constexpr int BUILD_CELLS = 224;
 constexpr int NEAR_COLS = 8;
+
+// The search of one disk: its place, what may hold its arrows, the best so far.
+template <int C>
+struct GSearch {
+    const GBuild &b;
+    uint32_t loc, i;
+    float2 vi;
+    double xi, yi;
+    int cyi, cxi, rdn, rup;
+    bool play[3], row_up, row_dn;
+    unsigned doubt = 0u;   // corridors with candidates whose bounds overlap
+    GBest best[3];
+
+    __device__ __forceinline__ GSearch(const GBuild &build, uint32_t slot)
+        : b(build), loc(slot), i(build.scid[slot]), vi(build.cxy[slot]) {
+        const int nc = b.nc;
+        xi = gb_x(b, loc, i);
+        yi = gb_y(b, loc, i);
+        cyi = (int)((loc / C) / (uint32_t)nc);
+        cxi = (int)((loc / C) % (uint32_t)nc);
+        rdn = cyi == 0 ? nc - 1 : cyi - 1;
+        rup = cyi == nc - 1 ? 0 : cyi + 1;
+    }
+
+    // by the y bins, nothing found yet
+    __device__ __forceinline__ void begin() {
+        const float yf = d2f_trunc(yi);
+        // corridors that may hold a disk (one bin of margin on each side; the
+        // centre one holds the disk itself)
+        play[0] = true;
+        play[1] = band_any(b, yf + b.half_f - b.wf, yf + b.df + b.wf);
+        play[2] = band_any(b, yf - b.df - b.wf, yf - b.half_f + b.wf);
+        // the rows beside that hold a disk within d (by the bins): on a lattice
+        // neither does
+        const float y0 = d2f_trunc(__dmul_rn((double)cyi, b.a));
+        row_up = band_any(b, y0 + b.af - b.wf, yf + b.df + b.wf);
+        row_dn = band_any(b, yf - b.df - b.wf, y0 + b.wf);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            best[q].lo = best[q].hi = INFINITY;
+            best[q].loc = NONE;
+        }
+    }
+
+    // the corridors that column m may still improve: thr(m) within the best
+    __device__ __forceinline__ unsigned open_at(int m) const {
+        const float thr = (float)m * b.af - vi.x - b.df - (float)(m + 4) * b.del;
+        unsigned o = 0u;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (play[q] && !(thr > best[q].hi)) o |= 1u << q;
+        return o;
+    }
+
+    // the disks of a cell (its first slot c0), rr rows and m columns on
+    __device__ __forceinline__ void disks(const GCell<C> &cl, uint32_t c0, int rr, int m,
+                                          GBest (&to)[3]) {
+#pragma unroll
+        for (int sl = 0; sl < C; ++sl) {
+            const float2 v = cl.v[sl];
+            if (!(v.x >= 0.f)) break;  // (a cell's slots fill in order)
+            if (c0 + sl == loc) continue;
+            float lo, hi;
+            int kc = corridor_f(b, vi.x, vi.y, rr, m, v, lo, hi);
+            if (kc < 0) continue;
+            if (kc >= EDGE) {
+                const uint32_t id = b.scid[c0 + sl];
+                const GFlight f =
+                    flight_exact(b.L, b.d, b.d2, xi, yi, gb_x(b, c0 + sl, id), gb_y(b, c0 + sl, id));
+                if (f.kc < 0) continue;
+                kc = f.kc;
+                lo = d2f_trunc(f.tau);
+                hi = lo + lo * 0x1p-22f + 0x1p-126f;
+                lo -= lo * 0x1p-22f;
+            }
+            // (selects, not indexing, keep the corridors in registers)
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (q == kc && take_best(to[q], lo, hi, c0 + sl)) doubt |= 1u << q;
+        }
+    }
+    __device__ __forceinline__ void cell(int row, int col, int rr, int m) {
+        const uint32_t c0 = ((uint32_t)row * (uint32_t)b.nc + (uint32_t)col) * C;
+        disks(load_cell<C>(b, c0), c0, rr, m, best);
+    }
+
+    // A disk left to k_gb_far keeps what was found in its record until then.
+    __device__ __forceinline__ void keep(bool far) const {
+        uint4 *const r = reinterpret_cast<uint4 *>(b.g + i);
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            r[q] = make_uint4(__float_as_uint(best[q].lo), __float_as_uint(best[q].hi),
+                              best[q].loc,
+                              doubt | (far ? 8u : 0u) | (play[1] ? 16u : 0u) |
+                                  (play[2] ? 32u : 0u) | (row_up ? 64u : 0u) |
+                                  (row_dn ? 128u : 0u));
+    }
+    // (true: to be searched beyond the near columns)
+    __device__ __forceinline__ bool take_up() {
+        const uint4 *const r = reinterpret_cast<const uint4 *>(b.g + i);
+        unsigned f = 0u;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const uint4 u = r[q];
+            best[q].lo = __uint_as_float(u.x);
+            best[q].hi = __uint_as_float(u.y);
+            best[q].loc = u.z;
+            f = u.w;
+        }
+        doubt = f & 7u;
+        play[0] = true;
+        play[1] = (f & 16u) != 0u;
+        play[2] = (f & 32u) != 0u;
+        row_up = (f & 64u) != 0u;
+        row_dn = (f & 128u) != 0u;
+        return (f & 8u) != 0u;
+    }
+
+    // the columns up to NEAR_COLS; the number searched
+    __device__ __forceinline__ int near() {
+        int m = 0;
+        for (; m < min(NEAR_COLS, b.nc); ++m) {
+            const unsigned open = open_at(m);
+            if (!open) break;
+            int col = cxi + m;
+            if (col >= b.nc) col -= b.nc;
+            if (row_dn && (open & 5u)) cell(rdn, col, -1, m);
+            cell(cyi, col, 0, m);
+            if (row_up && (open & 3u)) cell(rup, col, 1, m);
+        }
+        return m;
+    }
+
+    // The columns beyond (FAR_LANES lanes per disk): the next FAR_LANES blocks of
+    // columns at once, and of the first one of which a row reaches a corridor
+    // that is still open a column per lane. (The first block ends with its
+    // columns before the near ones.)
+    __device__ __forceinline__ void beyond(bool far) {
+        const int lane = threadIdx.x & 31, sub = lane % FAR_LANES, base = lane - sub;
+        const int nc = b.nc, end = cxi + NEAR_COLS < nc ? cxi + NEAR_COLS : cxi + NEAR_COLS - nc;
+        const int first = end / FAR_COLS;
+        // the corridors as limits of y in the rows (e covers corridor_f's doubts
+        // and the roundings of these sums)
+        const float e = 4.f * b.del, up0 = (b.half_f - e) + vi.y, up1 = (b.df + e) + vi.y;
+        const float dn0 = vi.y - (b.df + e), dn1 = vi.y - (b.half_f - e);
+        auto in = [](const float4 &l, float lo, float hi) {
+            return (l.x < hi && l.y > lo) || (l.z < hi && l.w > lo);
+        };
+        for (int k = 0; __any_sync(FULL, far);) {
+            int blk = first + k + sub;
+            if (blk >= b.nblk) blk -= b.nblk;
+            if (blk >= b.nblk) blk -= b.nblk;
+            int c0 = k + sub == 0 ? end : blk * FAR_COLS, m = c0 - cxi;
+            if (m < 0) m += nc;
+            const unsigned open = far && k + sub <= b.nblk ? open_at(max(m, NEAR_COLS)) : 0u;
+            unsigned rows = 0u;
+            if (open) {
+                const float4 *const lim = b.ylim + blk;
+                const float4 l0 = lim[rdn * b.nblk], l1 = lim[cyi * b.nblk], l2 = lim[rup * b.nblk];
+                const bool c = (open & 1u) != 0u, u = (open & 2u) != 0u, d = (open & 4u) != 0u;
+                if (row_dn && ((d && in(l0, dn0 + b.af, dn1 + b.af)) ||
+                               (c && in(l0, dn1 + b.af, up0 + b.af))))
+                    rows |= 1u;
+                if ((u && in(l1, up0, up1)) || (d && in(l1, dn0, dn1)) || (c && in(l1, dn1, up0)))
+                    rows |= 2u;
+                if (row_up && ((u && in(l2, up0 - b.af, up1 - b.af)) ||
+                               (c && in(l2, dn1 - b.af, up0 - b.af))))
+                    rows |= 4u;
+            }
+            const unsigned hit = (__ballot_sync(FULL, rows != 0u) >> base) & ((1u << FAR_LANES) - 1u);
+            const unsigned any = (__ballot_sync(FULL, open != 0u) >> base) & ((1u << FAR_LANES) - 1u);
+            const int f = hit ? __ffs(hit) - 1 : 0, at = base + f;
+            rows = __shfl_sync(FULL, rows, at);
+            c0 = __shfl_sync(FULL, c0, at);
+            blk = __shfl_sync(FULL, blk, at);
+            const int c1 = k + f == b.nblk ? end : min(nc, blk * FAR_COLS + FAR_COLS);
+            k += hit ? f + 1 : FAR_LANES;
+            far = any != 0u;
+            if (!__any_sync(FULL, hit != 0u)) continue;
+            GBest l[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                l[q].lo = l[q].hi = INFINITY;
+                l[q].loc = NONE;
+            }
+            const int col = c0 + sub;
+            m = col - cxi;
+            if (m < 0) m += nc;
+            if (hit && col < c1 && m >= NEAR_COLS) {
+#pragma unroll 1
+                for (int z = 0; z < 3; ++z) {
+                    if (!((rows >> z) & 1u)) continue;
+                    const int row = z == 0 ? rdn : z == 1 ? cyi : rup;
+                    const uint32_t s0 = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C;
+                    disks(load_cell<C>(b, s0), s0, z - 1, m, l);
+                }
+            }
+            // the lanes' candidates, then the best so far
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                if (!__any_sync(FULL, l[q].loc != NONE)) continue;
+#pragma unroll
+                for (int o = FAR_LANES / 2; o > 0; o >>= 1) {
+                    const float lo = __shfl_xor_sync(FULL, l[q].lo, o);
+                    const float hi = __shfl_xor_sync(FULL, l[q].hi, o);
+                    const uint32_t loc2 = __shfl_xor_sync(FULL, l[q].loc, o);
+                    if (loc2 != NONE && take_best(l[q], lo, hi, loc2)) doubt |= 1u << q;
+                }
+                if (l[q].loc != NONE && take_best(best[q], l[q].lo, l[q].hi, l[q].loc))
+                    doubt |= 1u << q;
+            }
+        }
+    }
+
+    // the disk in slot l (NONE: none) and b towards it (the warp)
+    __device__ __forceinline__ uint32_t arrow(uint32_t l, double &bv) const {
+        bv = 0.0;
+        if (!__any_sync(FULL, l != NONE)) return NONE;
+        const uint32_t at = l != NONE ? l : loc, j = b.scid[at];
+        double ay = fabs(__dsub_rn(gb_y(b, at, j), yi));
+        if (__any_sync(FULL, cyi == 0 || cyi == b.nc - 1 || b.nc <= 4)) {
+            const double la = __dsub_rn(b.L, ay);
+            if (dbits(la) < dbits(ay)) ay = la;
+        }
+        const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
+        if (l != NONE) bv = v;
+        return l != NONE ? j : NONE;
+    }
+
+    // 16 bytes (part 0 .. 3) of the disk's record
+    __device__ __forceinline__ void store(int part, const uint32_t (&id)[3],
+                                          const double (&bv)[3]) const {
+        ulonglong2 u;
+        if (part == 0) u = make_ulonglong2(dbits(xi), 0ull);
+        if (part == 1)
+            u = make_ulonglong2((unsigned long long)OWN_STATIC | ((unsigned long long)id[0] << 32),
+                                (unsigned long long)id[1] | ((unsigned long long)id[2] << 32));
+        if (part == 2) u = make_ulonglong2(0ull, dbits(bv[0]));
+        if (part == 3) u = make_ulonglong2(dbits(bv[1]), dbits(bv[2]));
+        reinterpret_cast<ulonglong2 *>(b.g + i)[part] = u;
+    }
+};
 
 template <int C>
 __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
     __shared__ uint32_t list[BUILD_CELLS * C];
     __shared__ int count;
-    const int nc = b.nc, lane = threadIdx.x & 31;
-    const uint32_t ncell = (uint32_t)nc * (uint32_t)nc;
+    const int lane = threadIdx.x & 31;
+    const uint32_t ncell = (uint32_t)b.nc * (uint32_t)b.nc;
     const uint32_t cell0 = blockIdx.x * BUILD_CELLS;
     if (threadIdx.x == 0) count = 0;
     __syncthreads();
@@ -480,194 +779,84 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
     const int total = count;
     for (int e0 = 0; e0 < total; e0 += blockDim.x) {
         const int e = e0 + (int)threadIdx.x;
-        const bool has = e < total;
-        const uint32_t loc = has ? list[e] : list[0];
-        const uint32_t i = b.scid[loc];
-        const float2 vi = b.cxy[loc];
-        const double xi = gb_x(b, loc, i), yi = gb_y(b, loc, i);
-        const int cyi = (int)((loc / C) / (uint32_t)nc), cxi = (int)((loc / C) % (uint32_t)nc);
-        const float yf = d2f_trunc(yi);
-        // corridors that may hold a disk (one bin of margin on each side; the
-        // centre one holds the disk itself)
-        bool play[3];
-        play[0] = true;
-        play[1] = band_any(b, yf + b.half_f - b.wf, yf + b.df + b.wf);
-        play[2] = band_any(b, yf - b.df - b.wf, yf - b.half_f + b.wf);
-        GBest best[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            best[q].lo = best[q].hi = INFINITY;
-            best[q].loc = NONE;
-        }
-        bool doubt = false;
-        // the rows beside that hold a disk within d (by the bins): on a lattice
-        // neither does
-        const float y0 = d2f_trunc(__dmul_rn((double)cyi, b.a));
-        const bool row_up = band_any(b, y0 + b.af - b.wf, yf + b.df + b.wf);
-        const bool row_dn = band_any(b, yf - b.df - b.wf, y0 + b.wf);
-        // the corridors that column m may still improve: thr(m) within the best
-        auto open_at = [&](int m) {
-            const float thr = (float)m * b.af - vi.x - b.df - (float)(m + 4) * b.del;
-            unsigned o = 0u;
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                if (play[q] && !(thr > best[q].hi)) o |= 1u << q;
-            return o;
-        };
-        auto cell_scan = [&](int row, int col, int rr, int m) {
-            const uint32_t c0 = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C;
-            const GCell<C> cell = load_cell<C>(b, c0);
-#pragma unroll
-            for (int sl = 0; sl < C; ++sl) {
-                const float2 v = cell.v[sl];
-                if (!(v.x >= 0.f) || c0 + sl == loc) continue;
-                float lo, hi;
-                const int kc = corridor_f(b, vi.x, vi.y, rr, m, v, lo, hi);
-                if (kc < 0) continue;
-                if (kc == 3) {
-                    doubt = true;
-                    continue;
-                }
-                // (selects, not indexing, keep the corridors in registers)
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (q == kc) doubt |= take_best(best[q], lo, hi, c0 + sl);
-            }
-        };
-        const int rdn = cyi == 0 ? nc - 1 : cyi - 1, rup = cyi == nc - 1 ? 0 : cyi + 1;
-        int m = 0;
-        for (; m < min(NEAR_COLS, nc); ++m) {
-            const unsigned open = open_at(m);
-            if (!open) break;
-            int col = cxi + m;
-            if (col >= nc) col -= nc;
-            if (row_dn && (open & 5u)) cell_scan(rdn, col, -1, m);
-            cell_scan(cyi, col, 0, m);
-            if (row_up && (open & 3u)) cell_scan(rup, col, 1, m);
-        }
-        // the disks that need columns beyond, one by one by the whole warp
-        unsigned todo = __ballot_sync(FULL, has && !doubt && m == NEAR_COLS && m < nc && open_at(m));
-        while (todo) {
-            const int src = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const float sx = __shfl_sync(FULL, vi.x, src), sy = __shfl_sync(FULL, vi.y, src);
-            const int scx = __shfl_sync(FULL, cxi, src), scy = __shfl_sync(FULL, cyi, src);
-            const uint32_t sloc = __shfl_sync(FULL, loc, src);
-            GBest w[3];
-            bool sp[3], dbt = false;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                w[q].lo = __shfl_sync(FULL, best[q].lo, src);
-                w[q].hi = __shfl_sync(FULL, best[q].hi, src);
-                w[q].loc = __shfl_sync(FULL, best[q].loc, src);
-                sp[q] = __shfl_sync(FULL, (int)play[q], src) != 0;
-            }
-            for (int m0 = NEAR_COLS; m0 < nc; m0 += 32) {
-                const float thr = (float)m0 * b.af - sx - b.df - (float)(m0 + 4) * b.del;
-                unsigned open = 0u;
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (sp[q] && !(thr > w[q].hi)) open |= 1u << q;
-                if (!open) break;
-                GBest l[3];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    l[q].lo = l[q].hi = INFINITY;
-                    l[q].loc = NONE;
-                }
-                const int mm = m0 + lane;
-                if (mm < nc) {
-                    int col = scx + mm;
-                    if (col >= nc) col -= nc;
-                    for (int rr = -1; rr <= 1; ++rr) {
-                        if ((rr < 0 && !(open & 5u)) || (rr > 0 && !(open & 3u))) continue;
-                        int row = scy + rr;
-                        if (row < 0) row += nc;
-                        if (row >= nc) row -= nc;
-                        const uint32_t c0 = ((uint32_t)row * (uint32_t)nc + (uint32_t)col) * C;
-                        const GCell<C> cell = load_cell<C>(b, c0);
-#pragma unroll
-                        for (int sl = 0; sl < C; ++sl) {
-                            const float2 v = cell.v[sl];
-                            if (!(v.x >= 0.f) || c0 + sl == sloc) continue;
-                            float lo, hi;
-                            const int kc = corridor_f(b, sx, sy, rr, mm, v, lo, hi);
-                            if (kc == 3) dbt = true;
-#pragma unroll
-                            for (int q = 0; q < 3; ++q)
-                                if (q == kc) dbt |= take_best(l[q], lo, hi, c0 + sl);
-                        }
-                    }
-                }
-                // the lanes' candidates, then the best so far
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (!__any_sync(FULL, l[q].loc != NONE)) continue;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float lo = __shfl_xor_sync(FULL, l[q].lo, o);
-                        const float hi = __shfl_xor_sync(FULL, l[q].hi, o);
-                        const uint32_t lc = __shfl_xor_sync(FULL, l[q].loc, o);
-                        if (lc != NONE) dbt |= take_best(l[q], lo, hi, lc);
-                    }
-                    if (l[q].loc != NONE) dbt |= take_best(w[q], l[q].lo, l[q].hi, l[q].loc);
-                }
-            }
-            dbt = __any_sync(FULL, dbt);
-            if (lane == src) {
-                doubt = dbt;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) best[q] = w[q];
-            }
-        }
-        uint32_t aj[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) aj[q] = best[q].loc;
-        unsigned odd = __ballot_sync(FULL, has && doubt);
-        while (odd) {
-            const int src = __ffs(odd) - 1;
-            odd &= odd - 1;
-            uint32_t ex[3];
-            arrows_exact<C>(b, __shfl_sync(FULL, i, src), __shfl_sync(FULL, loc, src),
-                            make_float2(__shfl_sync(FULL, vi.x, src), __shfl_sync(FULL, vi.y, src)),
-                            __shfl_sync(FULL, xi, src), __shfl_sync(FULL, yi, src),
-                            __shfl_sync(FULL, cxi, src), __shfl_sync(FULL, cyi, src),
-                            __shfl_sync(FULL, (int)play[1], src) != 0,
-                            __shfl_sync(FULL, (int)play[2], src) != 0, ex);
-            if (lane == src) {
-#pragma unroll
-                for (int q = 0; q < 3; ++q) aj[q] = ex[q];
+        GSearch<C> r(b, list[e < total ? e : 0]);
+        r.begin();
+        const int m = r.near();
+        const bool far = m == NEAR_COLS && m < b.nc && r.open_at(m) != 0u;
+        const bool later = r.doubt != 0u || far;
+        const unsigned fm = __ballot_sync(FULL, e < total && later);
+        if (fm) {
+            unsigned at = 0u;
+            if (lane == 0) at = atomicAdd(b.far_n, (unsigned)__popc(fm));
+            at = __shfl_sync(FULL, at, 0) + __popc(fm & ((1u << lane) - 1u));
+            if (e < total && later) {
+                b.far[at] = r.loc;
+                r.keep(far);
             }
         }
         uint32_t id[3];
         double bv[3];
 #pragma unroll
+        for (int q = 0; q < 3; ++q) id[q] = r.arrow(later ? NONE : r.best[q].loc, bv[q]);
+        if (e < total && !later) {
+            if (b.yout) b.yout[r.i] = r.yi;
+#pragma unroll
+            for (int part = 0; part < 4; ++part) r.store(part, id, bv);
+        }
+    }
+}
+
+// The disks that k_gb_arrows has listed, FAR_LANES lanes each. Along rows of
+// disks little less than d apart most disks have no arrow to the rows beside or
+// one far along: the blocks of columns that hold no disk in a corridor still
+// open are passed over (k_gb_blocks).
+// Bound by its instructions at eight blocks of 64 registers a multiprocessor
+// (360000 disks, eta 0.60, half of them listed: 168 us; 217 at 92 registers).
+// One disk per lane took 284 us there and 25 for a list of 40 disks (14 so), the
+// whole warp per disk over all columns, inside k_gb_arrows and in FP64 where a
+// corridor's edge was in doubt, 1360.
+constexpr int FAR_THREADS = 128, FAR_BLOCKS = 1216;
+
+template <int C>
+__global__ void __launch_bounds__(FAR_THREADS, 8) k_gb_far(GBuild b) {
+    constexpr int PER = 32 / FAR_LANES;  // disks a warp
+    const int lane = threadIdx.x & 31, sub = lane % FAR_LANES, base = lane - sub;
+    const unsigned total = *b.far_n, step = gridDim.x * (FAR_THREADS / FAR_LANES);
+    for (unsigned e0 = (blockIdx.x * FAR_THREADS + threadIdx.x) / 32u * PER; e0 < total;
+         e0 += step) {
+        const bool has = e0 + base / FAR_LANES < total;
+        GSearch<C> r(b, b.far[has ? e0 + base / FAR_LANES : e0]);
+        const bool far = r.take_up();
+        r.beyond(has && far);
+        uint32_t aj[3];
+#pragma unroll
         for (int q = 0; q < 3; ++q) {
-            id[q] = NONE;
-            bv[q] = 0.0;
-            if (!__any_sync(FULL, aj[q] != NONE)) continue;
-            const uint32_t l = aj[q] != NONE ? aj[q] : loc;
-            const uint32_t j = b.scid[l];
-            double ay = fabs(__dsub_rn(gb_y(b, l, j), yi));
-            if (__any_sync(FULL, cyi == 0 || cyi == nc - 1 || nc <= 4)) {
-                const double la = __dsub_rn(b.L, ay);
-                if (dbits(la) < dbits(ay)) ay = la;
-            }
-            const double v = __dsqrt_rn(__dsub_rn(b.d2, __dmul_rn(ay, ay)));
-            if (aj[q] != NONE) {
-                id[q] = j;
-                bv[q] = v;
+            aj[q] = r.best[q].loc;
+            unsigned odd = __ballot_sync(FULL, has && ((r.doubt >> q) & 1u));
+            while (odd) {
+                const int src = __ffs(odd) - 1, g = src / FAR_LANES;
+                odd &= ~(((1u << FAR_LANES) - 1u) << (g * FAR_LANES));
+                const uint32_t ex = arrow_exact<C>(
+                    b, q, __shfl_sync(FULL, r.loc, src),
+                    make_float2(__shfl_sync(FULL, r.vi.x, src), __shfl_sync(FULL, r.vi.y, src)),
+                    __shfl_sync(FULL, r.xi, src), __shfl_sync(FULL, r.yi, src),
+                    __shfl_sync(FULL, r.cxi, src), __shfl_sync(FULL, r.cyi, src),
+                    __shfl_sync(FULL, r.best[q].lo, src), __shfl_sync(FULL, r.best[q].hi, src));
+                if (lane / FAR_LANES == g) aj[q] = ex;
             }
         }
-        if (has) {
-            if (b.yout) b.yout[i] = yi;
-            ulonglong2 *r = reinterpret_cast<ulonglong2 *>(b.g + i);
-            r[0] = make_ulonglong2(dbits(xi), 0ull);
-            r[1] = make_ulonglong2((unsigned long long)OWN_STATIC | ((unsigned long long)id[0] << 32),
-                                   (unsigned long long)id[1] | ((unsigned long long)id[2] << 32));
-            r[2] = make_ulonglong2(0ull, dbits(bv[0]));
-            r[3] = make_ulonglong2(dbits(bv[1]), dbits(bv[2]));
+        // a lane per arrow, then a lane per part of the record
+        double v;
+        const uint32_t j = r.arrow(sub == 0 ? aj[0] : sub == 1 ? aj[1] : sub == 2 ? aj[2] : NONE, v);
+        uint32_t id[3];
+        double bv[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            id[q] = __shfl_sync(FULL, j, base + q);
+            bv[q] = shfl_f64(v, base + q);
         }
+        if (has && sub < 4) r.store(sub, id, bv);
+        if (has && sub == 4 && b.yout) b.yout[r.i] = r.yi;
     }
 }
 
@@ -3703,21 +3892,26 @@ int gcommit(GraphCtx *g, std::string &err) {
     return 0;
 }
 
-// Bytes of a build's scratch (kept by the context for direction changes): the
-// FP32 coordinates, the y bins and the overflow count, and the ids per slot.
-static size_t build_parts(double L, double d, int nc, int C, size_t *off_bits, size_t *off_err,
-                          size_t *off_cid) {
-    const size_t nslot = (size_t)nc * nc * C;
-    const size_t nb = (size_t)((int)std::ceil(L / (d / 128.0)) + 1);
-    *off_cid = nslot * sizeof(float2);
-    *off_bits = *off_cid + ((nslot * 4 + 15) & ~(size_t)15);
-    *off_err = *off_bits + ((nb / 32 + 1) * 4 + 15) / 16 * 16;
-    return *off_err + 16;
-}
+// Parts of a build's scratch (kept by the context for direction changes): the
+// FP32 coordinates, the ids per slot, the y bins, the counts (overfull cells,
+// rows that are no rings, disks listed), the y limits of the blocks of columns
+// and the list of disks.
+struct BuildParts {
+    size_t cid, bits, err, ylim, far, total;
+    BuildParts(int64_t n, double L, double d, int nc, int C) {
+        const size_t nslot = (size_t)nc * nc * C;
+        const size_t nb = (size_t)((int)std::ceil(L / (d / 128.0)) + 1);
+        cid = nslot * sizeof(float2);
+        bits = cid + ((nslot * 4 + 15) & ~(size_t)15);
+        err = bits + ((nb / 32 + 1) * 4 + 15) / 16 * 16;
+        ylim = err + 32;
+        far = ylim + (size_t)nc * (size_t)((nc + FAR_COLS - 1) / FAR_COLS) * sizeof(float4);
+        total = far + (size_t)n * sizeof(uint32_t);
+    }
+};
 
-static int64_t graph_build_bytes(double L, double d, int nc, int C) {
-    size_t a, b, c;
-    return (int64_t)build_parts(L, d, nc, C, &a, &b, &c);
+static size_t graph_build_bytes(const GraphCtx *g) {
+    return BuildParts(g->s.n, g->s.L, g->s.d, g->nc, g->C).total;
 }
 
 static int launched(const char *what, std::string &err) {
@@ -3748,6 +3942,7 @@ static GBuild build_params(const GraphCtx *g) {
     b.df = (float)s.d;
     b.del = (float)std::ldexp(b.a, -20);
     b.nb = (int)std::ceil(s.L / w) + 1;
+    b.nblk = (g->nc + FAR_COLS - 1) / FAR_COLS;
     b.g = s.g;
     return b;
 }
@@ -3766,27 +3961,29 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned l
     b.y = y;
     b.yout = s.y;
     b.bad_xy = bad_xy;
-    size_t off_bits, off_err, off_cid;
-    const size_t total = build_parts(s.L, s.d, nc, g->C, &off_bits, &off_err, &off_cid);
+    const BuildParts at(s.n, s.L, s.d, nc, g->C);
     // scratch of the build, kept by the context for the next direction change
     if (!g->build_tmp) {
-        if (dm_alloc(&g->build_tmp, total) != 0) {
+        if (dm_alloc(&g->build_tmp, at.total) != 0) {
             g->build_tmp = nullptr;
             err = "cudaMalloc failed (graph build)";
             return ECMC_ENOMEM;
         }
-        g->bytes += (int64_t)total;
+        g->bytes += (int64_t)at.total;
     }
     char *tmp = (char *)g->build_tmp;
     b.cxy = (float2 *)tmp;
-    b.cid = (uint32_t *)(tmp + off_cid);
+    b.cid = (uint32_t *)(tmp + at.cid);
     b.scid = b.cid;
-    b.bits = (uint32_t *)(tmp + off_bits);
-    b.err = (unsigned long long *)(tmp + off_err);
+    b.bits = (uint32_t *)(tmp + at.bits);
+    b.err = (unsigned long long *)(tmp + at.err);
+    b.far_n = (unsigned *)(b.err + 2);
+    b.ylim = (float4 *)(tmp + at.ylim);
+    b.far = (uint32_t *)(tmp + at.far);
     cudaStream_t st = g->st;
     // (all ones: NaN coordinates and EMPTY ids)
-    cudaMemsetAsync(tmp, 0xFF, off_bits, st);
-    cudaMemsetAsync(tmp + off_bits, 0, total - off_bits, st);
+    cudaMemsetAsync(tmp, 0xFF, at.bits, st);
+    cudaMemsetAsync(tmp + at.bits, 0, at.ylim - at.bits, st);
     const unsigned nblk = (unsigned)((s.n + 255) / 256);
     if (g->C == 4)
         k_gb_cells<4><<<nblk, 256, 0, st>>>(b);
@@ -3823,12 +4020,21 @@ static int graph_records(GraphCtx *g, const GBuild &b, bool rings, const int32_t
             k_ring_place<8><<<grid, RING_CHUNK, 0, st>>>(b, g->ring, s);
     }
     const unsigned ablk = (unsigned)(((size_t)g->nc * g->nc + BUILD_CELLS - 1) / BUILD_CELLS);
-    if (s.ring && s.cells)
+    const unsigned bblk = (unsigned)std::min<size_t>(
+        ((size_t)g->nc * (size_t)b.nblk * FAR_COLS + 255) / 256, 1216);
+    const unsigned fblk = (unsigned)std::min<int64_t>(
+        (s.n * FAR_LANES + FAR_THREADS - 1) / FAR_THREADS, FAR_BLOCKS);
+    if (s.ring && s.cells) {
         k_ring_records<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(b, s);
-    else if (g->C == 4)
+    } else if (g->C == 4) {
         k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
-    else
+        k_gb_blocks<4><<<bblk, 256, 0, st>>>(b);
+        k_gb_far<4><<<fblk, FAR_THREADS, 0, st>>>(b);
+    } else {
         k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
+        k_gb_blocks<8><<<bblk, 256, 0, st>>>(b);
+        k_gb_far<8><<<fblk, FAR_THREADS, 0, st>>>(b);
+    }
     k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active);
     return launched("graph build", err);
 }
@@ -4434,7 +4640,7 @@ int64_t graph_plan_bytes(const ecmc_params *p, int nc) {
     if (!g) return -1;
     graph_params(g, p, nc);
     graph_plan(g);
-    int64_t total = graph_build_bytes(p->box, p->d, nc, g->C);
+    int64_t total = (int64_t)graph_build_bytes(g);
     for (auto &r : g->pending) total += (int64_t)((r.second + 255) & ~(size_t)255);
     g->pending.clear();
     delete g;
@@ -4477,7 +4683,7 @@ size_t leg_arrays(GraphCtx *g, unsigned char *base, LegArrays *out) {
     out->seen = g->s.rid;  // (written again by the build)
     take(&out->bad, 2);
     char *tmp;
-    take(&tmp, (size_t)graph_build_bytes(g->s.L, g->s.d, g->nc, g->C));
+    take(&tmp, graph_build_bytes(g));
     g->build_tmp = tmp;
     return off;
 }
