@@ -875,8 +875,8 @@ constexpr double RING_SPREAD = 0.86;
 constexpr int RING_CHUNK = 256;  // columns of a row per block of the kernels below
 
 struct GRing {
-    uint32_t *off;             // [nc * chunks + 1] disks per chunk, then first places
-    unsigned long long *band;  // [2 nc] least and largest y (bits) per row
+    uint32_t *off;                 // [nc * chunks + 1] disks per chunk, then first places
+    unsigned long long *ylo, *yhi; // [nc] least and largest y (bits) per row (all ones, 0)
 };
 
 static int ring_chunks(int nc) { return (nc + RING_CHUNK - 1) / RING_CHUNK; }
@@ -931,8 +931,8 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_count(GBuild b, GRing r) {
             n += wn[q];
         }
         if (n) {
-            atomicMin(r.band + row, lo);
-            atomicMax(r.band + nc + row, hi);
+            atomicMin(r.ylo + row, lo);
+            atomicMax(r.yhi + row, hi);
         }
         r.off[row * gridDim.x + blockIdx.x] = (uint32_t)n;
     }
@@ -948,13 +948,13 @@ __global__ void k_ring_rows(GBuild b, GRing r, int chunks, unsigned long long *b
     const int nc = b.nc;
     bool no = nc < 5;
     for (int q = threadIdx.x; q < nc; q += blockDim.x) {
-        const unsigned long long l = r.band[q];
+        const unsigned long long l = r.ylo[q];
         if (l == ~0ull) continue;
         const double yl = __longlong_as_double((long long)l),
-                     yh = __longlong_as_double((long long)r.band[nc + q]);
+                     yh = __longlong_as_double((long long)r.yhi[q]);
         no = no || !(__dsub_rn(yh, yl) < __dmul_rn(RING_SPREAD, b.d));
         const int up = q == nc - 1 ? 0 : q + 1;
-        const unsigned long long u = r.band[up];
+        const unsigned long long u = r.ylo[up];
         if (u != ~0ull) {
             const double yu = __longlong_as_double((long long)u);
             no = no || !((up ? __dsub_rn(yu, yh) : __dsub_rn(b.L, __dsub_rn(yh, yu))) >= b.d);
@@ -3892,21 +3892,25 @@ int gcommit(GraphCtx *g, std::string &err) {
     return 0;
 }
 
-// Parts of a build's scratch (kept by the context for direction changes): the
-// FP32 coordinates, the ids per slot, the y bins, the counts (overfull cells,
-// rows that are no rings, disks listed), the y limits of the blocks of columns
-// and the list of disks.
+// Parts of a build's scratch (kept by the context for direction changes). All
+// ones to start with: the FP32 coordinates, the ids per slot, the rows' least y;
+// zero: the y bins, the counts (overfull cells, rows that are no rings, disks
+// listed), the rows' largest y. Then the y limits of the blocks of columns and
+// the list of disks.
 struct BuildParts {
-    size_t cid, bits, err, ylim, far, total;
+    size_t cid, ylo, zero, err, yhi, ylim, far, total;
     BuildParts(int64_t n, double L, double d, int nc, int C) {
         const size_t nslot = (size_t)nc * nc * C;
         const size_t nb = (size_t)((int)std::ceil(L / (d / 128.0)) + 1);
-        cid = nslot * sizeof(float2);
-        bits = cid + ((nslot * 4 + 15) & ~(size_t)15);
-        err = bits + ((nb / 32 + 1) * 4 + 15) / 16 * 16;
-        ylim = err + 32;
-        far = ylim + (size_t)nc * (size_t)((nc + FAR_COLS - 1) / FAR_COLS) * sizeof(float4);
-        total = far + (size_t)n * sizeof(uint32_t);
+        auto after = [](size_t at, size_t bytes) { return (at + bytes + 15) & ~(size_t)15; };
+        cid = after(0, nslot * sizeof(float2));
+        ylo = after(cid, nslot * 4);
+        zero = after(ylo, (size_t)nc * 8);  // (the bins)
+        err = after(zero, (nb / 32 + 1) * 4);
+        yhi = after(err, 24);
+        ylim = after(yhi, (size_t)nc * 8);
+        far = after(ylim, (size_t)nc * (size_t)((nc + FAR_COLS - 1) / FAR_COLS) * sizeof(float4));
+        total = after(far, (size_t)n * sizeof(uint32_t));
     }
 };
 
@@ -3975,15 +3979,17 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned l
     b.cxy = (float2 *)tmp;
     b.cid = (uint32_t *)(tmp + at.cid);
     b.scid = b.cid;
-    b.bits = (uint32_t *)(tmp + at.bits);
+    b.bits = (uint32_t *)(tmp + at.zero);
+    g->ring.ylo = (unsigned long long *)(tmp + at.ylo);
+    g->ring.yhi = (unsigned long long *)(tmp + at.yhi);
     b.err = (unsigned long long *)(tmp + at.err);
     b.far_n = (unsigned *)(b.err + 2);
     b.ylim = (float4 *)(tmp + at.ylim);
     b.far = (uint32_t *)(tmp + at.far);
     cudaStream_t st = g->st;
     // (all ones: NaN coordinates and EMPTY ids)
-    cudaMemsetAsync(tmp, 0xFF, at.bits, st);
-    cudaMemsetAsync(tmp + at.bits, 0, at.ylim - at.bits, st);
+    cudaMemsetAsync(tmp, 0xFF, at.zero, st);
+    cudaMemsetAsync(tmp + at.zero, 0, at.ylim - at.zero, st);
     const unsigned nblk = (unsigned)((s.n + 255) / 256);
     if (g->C == 4)
         k_gb_cells<4><<<nblk, 256, 0, st>>>(b);
@@ -3991,8 +3997,6 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned l
         k_gb_cells<8><<<nblk, 256, 0, st>>>(b);
     if (g->try_ring[g->axis]) {
         const int chunks = ring_chunks(nc);
-        cudaMemsetAsync(g->ring.band, 0xFF, (size_t)nc * 8, st);
-        cudaMemsetAsync(g->ring.band + nc, 0, (size_t)nc * 8, st);
         const dim3 grid((unsigned)chunks, (unsigned)nc);
         if (g->C == 4)
             k_ring_count<4><<<grid, RING_CHUNK, 0, st>>>(b, g->ring);
@@ -4084,27 +4088,20 @@ static void graph_arrays(GraphCtx *g, Take take) {
     const size_t path = k * ((size_t)s.cap + 2);
     take(&s.g, n);
     take(&s.y, n);
-    take(&s.key, n);
-    take(&s.fl, flag_words(s));
-    take(&s.rid, n);
     take(&s.pos, n);
     take(&g->ring.off, (size_t)g->nc * ring_chunks(g->nc) + 1);
-    take(&g->ring.band, 2 * (size_t)g->nc);
     if (s.cells) {
         take(&s.pxt, path);
         take(&s.pcell, path);
     }
     take(&s.path, path);
-    take(&s.sp, k);
     take(&s.ci, k);
     take(&s.ci0, k);
     take(&s.D, k);
     take(&s.tc, k);
     take(&s.status, k);
     take(&s.partner, k);
-    take(&s.nrec, k);
     take(&s.nlift, k);
-    take(&s.memb, k);
     take(&s.tstar, 1);
     take(&s.rec, k * (size_t)s.cap);
     take(&s.ev_T, k);
@@ -4125,12 +4122,21 @@ static void graph_arrays(GraphCtx *g, Take take) {
     take(&s.comp_mem, 4 * k);  // (g_members)
     take(&s.child, k);
     take(&s.sib, k);
-    take(&s.taken, k);
     take(&s.ctl, CTL_N);
+    if (s.log_on) take(&s.log, (size_t)s.log_cap);
+    // all ones in a new context, from here on
+    take(&s.key, n);
+    take(&s.memb, k);
+    // zero, from here up to the last flag word
+    take(&s.sp, k);
+    take(&s.nrec, k);
+    take(&s.taken, k);
     take(&s.lc, 2 * LC_N);
     take(&s.dbg, 16);
     take(&s.tc_cnt, TC_N);
-    if (s.log_on) take(&s.log, (size_t)s.log_cap);
+    take(&s.fl, flag_words(s));
+    // (graph_leg has these zero too)
+    take(&s.rid, n);
 }
 
 // Requests for all of them (galloc; gcommit allocates, graph_plan_bytes adds up).
@@ -4211,19 +4217,16 @@ static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
     s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
 }
 
-// Counters, run results and touch keys of a new context.
-static void graph_clear(GraphCtx *g) {
+// Counters, run results, flag words, touch keys and member tags of a new context
+// (arrays side by side in the order of graph_arrays); zero_end: the end of the
+// zeroed part.
+static cudaError_t graph_clear(GraphCtx *g, void *zero_end) {
     const GDev &s = g->s;
-    const size_t n = (size_t)s.n, k = (size_t)s.k;
-    cudaStream_t st = g->st;
-    cudaMemsetAsync(s.nrec, 0, k * 4, st);
-    cudaMemsetAsync(s.sp, 0, k * sizeof(GSpec), st);
-    cudaMemsetAsync(s.taken, 0, k * 4, st);
-    cudaMemsetAsync(s.lc, 0, 2 * LC_N * 8, st);
-    cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
-    cudaMemsetAsync(s.tc_cnt, 0, TC_N * 8, st);
-    cudaMemsetAsync(s.key, 0xFF, n * 8, st);
-    cudaMemsetAsync(s.fl, 0, flag_words(s) * 8, st);
+    char *const ones = (char *)s.key, *const zero = (char *)s.sp;
+    const cudaError_t e = cudaMemsetAsync(ones, 0xFF, (size_t)(zero - ones), g->st);
+    return e != cudaSuccess
+               ? e
+               : cudaMemsetAsync(zero, 0, (size_t)((char *)zero_end - zero), g->st);
 }
 
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
@@ -4247,8 +4250,12 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
         graph_destroy(g);
         return rc;
     }
-    graph_clear(g);
-    rc = graph_build(g, x, y, active, bad, err);
+    if (graph_clear(g, g->s.fl + flag_words(g->s)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        err = "clearing the graph state";
+        rc = ECMC_ECUDA;
+    }
+    if (!rc) rc = graph_build(g, x, y, active, bad, err);
     if (!rc && graph_max_grid() < 1) {
         err = "cooperative launch unavailable";
         rc = ECMC_ECUDA;
@@ -4678,10 +4685,10 @@ size_t leg_arrays(GraphCtx *g, unsigned char *base, LegArrays *out) {
         off += std::max<size_t>(count, 1) * sizeof(**p);
     };
     graph_arrays(g, take);
-    take(&out->tables, 1);
-    take(&out->blocked, (size_t)g->s.k);
     out->seen = g->s.rid;  // (written again by the build)
     take(&out->bad, 2);
+    take(&out->tables, 1);
+    take(&out->blocked, (size_t)g->s.k);
     char *tmp;
     take(&tmp, graph_build_bytes(g));
     g->build_tmp = tmp;
@@ -4717,11 +4724,8 @@ int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, cons
     if (grid < 1) return ECMC_ECUDA;
     // the first half of the build reads any coordinates; ids are used after
     // the check's result
-    cu(cudaMemsetAsync(a.seen, 0, (size_t)s.n * 4, st));
-    cu(cudaMemsetAsync(a.bad, 0, 16, st));
+    cu(graph_clear(&g, a.bad + 2));
     graph_check_inputs(nullptr, nullptr, active, s.n, s.k, s.L, a.seen, a.bad, a.bad + 1, st);
-    graph_clear(&g);
-    cu(cudaMemsetAsync(s.memb, 0xFF, (size_t)s.k * 8, st));
     GBuild b;
     if (!rc) rc = graph_place(&g, x, y, a.bad, &b, err);
     unsigned long long bad[2], built[2];
