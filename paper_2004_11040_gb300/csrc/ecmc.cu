@@ -215,55 +215,40 @@ static int64_t export_layout(int64_t n, ecmc_ctx *ctx) {
     return 2 * n8;
 }
 
-// The system of a new context. With host inputs they are uploaded first; the
-// check of the inputs runs ahead of the build and is read with its result.
+// The system of a new context; host inputs are uploaded first.
 static int create_graph(ecmc_ctx *ctx, int nc, const double *x, const double *y,
                         const int32_t *active) {
     const ecmc_params *p = &ctx->p;
-    const bool dev_in = (p->flags & ECMC_INPUT_DEVICE) != 0;
-    int rc = 0;
     const size_t n = (size_t)p->n, k = (size_t)p->n_chains;
-    // one scratch allocation: the uploaded inputs, the ids seen, two counters
-    const size_t off_y = n * 8, off_a = 2 * n * 8, off_seen = (off_a + k * 4 + 15) & ~(size_t)15;
-    const size_t off_bad = (off_seen + n * 4 + 15) & ~(size_t)15;
+    int rc = 0;
     char *scratch = nullptr;
-    if (dm_alloc_t(&scratch, off_bad + 16) != 0) {
-        g_create_err = "cudaMalloc failed (inputs)";
-        return ECMC_ENOMEM;
-    }
-    double *dx = (double *)scratch, *dy = (double *)(scratch + off_y);
-    int32_t *da = (int32_t *)(scratch + off_a);
-    uint32_t *seen = (uint32_t *)(scratch + off_seen);
-    unsigned long long *bad = (unsigned long long *)(scratch + off_bad);
-    const double *sx = x, *sy = y;
-    const int32_t *sa = active;
-    cudaError_t e = cudaMemsetAsync(seen, 0, off_bad + 16 - off_seen, ctx->stream);
-    if (!dev_in) {
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(dx, x, n * 8, cudaMemcpyHostToDevice, ctx->stream);
+    if (!(p->flags & ECMC_INPUT_DEVICE)) {
+        if (dm_alloc_t(&scratch, 2 * n * 8 + k * 4) != 0) {
+            g_create_err = "cudaMalloc failed (inputs)";
+            return ECMC_ENOMEM;
+        }
+        double *dx = (double *)scratch, *dy = dx + n;
+        int32_t *da = (int32_t *)(dy + n);
+        cudaError_t e = cudaMemcpyAsync(dx, x, n * 8, cudaMemcpyHostToDevice, ctx->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(dy, y, n * 8, cudaMemcpyHostToDevice, ctx->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(da, active, k * 4, cudaMemcpyHostToDevice, ctx->stream);
-        sx = dx;
-        sy = dy;
-        sa = da;
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            g_create_err = "input upload";
+            rc = ECMC_ECUDA;
+        }
+        x = dx;
+        y = dy;
+        active = da;
     }
-    if (e == cudaSuccess) {
-        graph_check_inputs(nullptr, nullptr, sa, (int64_t)n, (int)k, p->box, seen, bad, bad + 1,
-                           ctx->stream);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        g_create_err = "input upload";
-        rc = ECMC_ECUDA;
-    } else {
+    if (!rc) {
         std::string err;
-        rc = graph_create(p, nc, sx, sy, sa, bad, ctx->stream, &ctx->graph, err);
+        rc = graph_create(p, nc, x, y, active, ctx->stream, &ctx->graph, err);
         if (rc) g_create_err = err;
     }
-    // (copies, the check or the build may still read the scratch)
+    // (copies, the check or the build may still read the inputs)
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
         (void)cudaGetLastError();
         if (!rc) {

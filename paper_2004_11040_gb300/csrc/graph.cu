@@ -201,6 +201,13 @@ __device__ __forceinline__ double shfl_f64(double v, int src) {
 
 // ------------------------------------------------------------ graph build
 
+// What a build finds: disks without a slot in their cell, rows that are no rings
+// (or none asked), disks left to k_gb_far, and of unchecked inputs coordinates
+// outside [0, L) and bad ids.
+struct BuildCounts {
+    unsigned long long full, mixed, listed, bad_xy, bad_id;
+};
+
 // Inputs and scratch of a build: a cell list of the disks (in any of a cell's
 // slots), their FP32 coordinates per slot relative to the cell's corner (an
 // error of 1e-7 d whatever the box), and one bit per y bin of width d/128 that
@@ -213,19 +220,17 @@ struct GBuild {
     float del;           // a 2^-20: bound on the FP32 error of a difference of
                          // coordinates of neighbouring cells
     const double *x, *y;
-    unsigned long long *bad_xy;  // counts coordinates outside [0, L) (or null)
-    const uint32_t *scid;  // [nc*nc*C] disk per slot, EMPTY
-    uint32_t *cid;         // the same, writable (null with sx)
+    int check;                   // count coordinates outside [0, L)
+    uint32_t *scid;        // [nc*nc*C] disk per slot, EMPTY
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
-    uint32_t *far;         // [n] slots of the disks left to k_gb_far, and their number
-    unsigned *far_n;
+    uint32_t *far;         // [n] slots of the disks left to k_gb_far
     int nblk;              // blocks of FAR_COLS columns in a row
     float4 *ylim;          // [nc*nblk] least and largest y (within the cell row) per block
                            // in the row's lower half, and in its upper one
     uint32_t *bits;        // [nb / 32 + 1]
     GDisk *g;
     double *yout;             // [n] or null: each disk's y
-    unsigned long long *err;  // cell overflow count
+    BuildCounts *count;
 };
 
 // A monotone map of y to its bin, the same wherever bins are set or asked for.
@@ -254,19 +259,20 @@ __global__ void k_gb_cells(GBuild b) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= b.n) return;
     const double x = coord(b.x[q]), y = coord(b.y[q]);
-    if (b.bad_xy && !(x >= 0.0 && x < b.L && y >= 0.0 && y < b.L)) atomicAdd(b.bad_xy, 1ull);
+    if (b.check && !(x >= 0.0 && x < b.L && y >= 0.0 && y < b.L))
+        atomicAdd(&b.count->bad_xy, 1ull);
     const int row = cell_coord(y, b.inv_a, b.nc), col = cell_coord(x, b.inv_a, b.nc);
     const uint32_t cell = (uint32_t)row * (uint32_t)b.nc + (uint32_t)col;
     const float2 v = in_cell(b, x, y, row, col);
     set_bin(b, d2f_trunc(y));
     for (int sl = 0; sl < C; ++sl) {
         const uint32_t loc = cell * C + sl;
-        if (atomicCAS(b.cid + loc, EMPTY, (uint32_t)q) == EMPTY) {
+        if (atomicCAS(b.scid + loc, EMPTY, (uint32_t)q) == EMPTY) {
             b.cxy[loc] = v;
             return;
         }
     }
-    atomicAdd(b.err, 1ull);
+    atomicAdd(&b.count->full, 1ull);
 }
 
 // Does a bin that meets [lo, hi) (periodic, hi - lo < L) hold a disk? The
@@ -465,7 +471,7 @@ static_assert(FAR_LANES >= FAR_COLS, "a lane per column of a block");
 // in wherever two rows of disks share a row of cells.
 template <int C>
 __global__ void k_gb_blocks(GBuild b) {
-    if (*b.far_n == 0u) return;  // nothing is searched beyond the near columns
+    if (b.count->listed == 0ull) return;  // nothing is searched beyond the near columns
     static_assert(FAR_COLS == 8, "a block is a quarter of a warp's lanes");
     const int64_t end = (int64_t)b.nc * b.nblk * FAR_COLS;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; __any_sync(FULL, q < end);
@@ -787,7 +793,7 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
         const unsigned fm = __ballot_sync(FULL, e < total && later);
         if (fm) {
             unsigned at = 0u;
-            if (lane == 0) at = atomicAdd(b.far_n, (unsigned)__popc(fm));
+            if (lane == 0) at = (unsigned)atomicAdd(&b.count->listed, (unsigned long long)__popc(fm));
             at = __shfl_sync(FULL, at, 0) + __popc(fm & ((1u << lane) - 1u));
             if (e < total && later) {
                 b.far[at] = r.loc;
@@ -821,7 +827,7 @@ template <int C>
 __global__ void __launch_bounds__(FAR_THREADS, 8) k_gb_far(GBuild b) {
     constexpr int PER = 32 / FAR_LANES;  // disks a warp
     const int lane = threadIdx.x & 31, sub = lane % FAR_LANES, base = lane - sub;
-    const unsigned total = *b.far_n, step = gridDim.x * (FAR_THREADS / FAR_LANES);
+    const unsigned total = (unsigned)b.count->listed, step = gridDim.x * (FAR_THREADS / FAR_LANES);
     for (unsigned e0 = (blockIdx.x * FAR_THREADS + threadIdx.x) / 32u * PER; e0 < total;
          e0 += step) {
         const bool has = e0 + base / FAR_LANES < total;
@@ -938,11 +944,11 @@ __global__ void __launch_bounds__(RING_CHUNK) k_ring_count(GBuild b, GRing r) {
     }
 }
 
-// The rows that are no rings (added to *bad), and the chunks' first places
+// Whether some row is no ring (count->mixed), and the chunks' first places
 // (one block). Two neighbour rows lie d apart when RN(ylo(above) - yhi(below))
 // >= d: rounding is monotone, so |RN(dy)| >= d for every pair; across the box
 // edge RN(L - RN(yhi(nc - 1) - ylo(0))) bounds every pair's periodic image.
-__global__ void k_ring_rows(GBuild b, GRing r, int chunks, unsigned long long *bad) {
+__global__ void k_ring_rows(GBuild b, GRing r, int chunks) {
     __shared__ int warp_tot[32];
     __shared__ int tot[2];
     const int nc = b.nc;
@@ -973,7 +979,7 @@ __global__ void k_ring_rows(GBuild b, GRing r, int chunks, unsigned long long *b
     }
     if (threadIdx.x == 0) {
         r.off[n] = (uint32_t)tot[0];
-        if (any) *bad = 1ull;
+        if (any) b.count->mixed = 1ull;
     }
 }
 
@@ -3814,17 +3820,14 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
 }
 
 // Exports positions (per disk id), local times and active disks.
-// failed: a word that is not 0 if nothing is to be written (or null).
-__global__ void k_g_export(GDev s, double *x, double *t, const int32_t *failed) {
+// (each may be null). failed: a word that is not 0 if nothing is to be written
+// (or null).
+__global__ void k_g_export(GDev s, double *x, double *t, int32_t *active, const int32_t *failed) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= s.n || (failed && *failed)) return;
     if (x) x[q] = s.g[q].x;
     if (t) t[q] = g_time(s.g[q].own, s.g[q].t, s.stamp0);
-}
-
-__global__ void k_g_export_active(GDev s, int32_t *active, const int32_t *failed) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < s.k && !(failed && *failed)) active[c] = (int32_t)s.ci[c];
+    if (active && q < s.k) active[q] = (int32_t)s.ci[q];
 }
 
 // Direction change: the disks' x and y are exchanged (x from y_old, y from
@@ -3907,7 +3910,7 @@ struct BuildParts {
         ylo = after(cid, nslot * 4);
         zero = after(ylo, (size_t)nc * 8);  // (the bins)
         err = after(zero, (nb / 32 + 1) * 4);
-        yhi = after(err, 24);
+        yhi = after(err, sizeof(BuildCounts));
         ylim = after(yhi, (size_t)nc * 8);
         far = after(ylim, (size_t)nc * (size_t)((nc + FAR_COLS - 1) / FAR_COLS) * sizeof(float4));
         total = after(far, (size_t)n * sizeof(uint32_t));
@@ -3954,17 +3957,17 @@ static GBuild build_params(const GraphCtx *g) {
 // The first half of a frame's build, queued on the context's stream: every
 // disk in a cell, and whether the rows are rings (asked again on an axis only
 // while they were: rows that motion across them has mixed stay mixed).
-// b.err[0] counts overfull cells, b.err[1] rows that are no rings, *bad_xy (if
-// not null) coordinates outside [0, L), which count as the nearest cell's.
-static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned long long *bad_xy,
-                       GBuild *out, std::string &err) {
+// check: coordinates outside [0, L), which count as the nearest cell's, are
+// counted.
+static int graph_place(GraphCtx *g, const double *x, const double *y, bool check, GBuild *out,
+                       std::string &err) {
     GDev &s = g->s;
     const int nc = g->nc;
     GBuild b = build_params(g);
     b.x = x;
     b.y = y;
     b.yout = s.y;
-    b.bad_xy = bad_xy;
+    b.check = check ? 1 : 0;
     const BuildParts at(s.n, s.L, s.d, nc, g->C);
     // scratch of the build, kept by the context for the next direction change
     if (!g->build_tmp) {
@@ -3977,13 +3980,11 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned l
     }
     char *tmp = (char *)g->build_tmp;
     b.cxy = (float2 *)tmp;
-    b.cid = (uint32_t *)(tmp + at.cid);
-    b.scid = b.cid;
+    b.scid = (uint32_t *)(tmp + at.cid);
     b.bits = (uint32_t *)(tmp + at.zero);
     g->ring.ylo = (unsigned long long *)(tmp + at.ylo);
     g->ring.yhi = (unsigned long long *)(tmp + at.yhi);
-    b.err = (unsigned long long *)(tmp + at.err);
-    b.far_n = (unsigned *)(b.err + 2);
+    b.count = (BuildCounts *)(tmp + at.err);
     b.ylim = (float4 *)(tmp + at.ylim);
     b.far = (uint32_t *)(tmp + at.far);
     cudaStream_t st = g->st;
@@ -4002,7 +4003,7 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, unsigned l
             k_ring_count<4><<<grid, RING_CHUNK, 0, st>>>(b, g->ring);
         else
             k_ring_count<8><<<grid, RING_CHUNK, 0, st>>>(b, g->ring);
-        k_ring_rows<<<1, 1024, 0, st>>>(b, g->ring, chunks, b.err + 1);
+        k_ring_rows<<<1, 1024, 0, st>>>(b, g->ring, chunks);
     }
     *out = b;
     return launched("graph build", err);
@@ -4044,33 +4045,36 @@ static int graph_records(GraphCtx *g, const GBuild &b, bool rings, const int32_t
 }
 
 // A frame from positions x, y and active disks (device): both halves, with a
-// wait for the first one's result between. bad: two counters, of coordinates
-// outside [0, L), counted here, and of bad ids, counted by a check queued before
-// (null: the inputs are known to be good).
+// wait for the first one's counts between. check: the inputs are not known to be
+// good (s.rid is zero then, for the ids seen). active: null, the disks are where
+// they were.
 static int graph_build(GraphCtx *g, const double *x, const double *y, const int32_t *active,
-                       unsigned long long *bad, std::string &err) {
+                       bool check, std::string &err) {
+    const GDev &s = g->s;
     GBuild b;
-    int rc = graph_place(g, x, y, bad, &b, err);
+    int rc = graph_place(g, x, y, check, &b, err);
     if (rc) return rc;
-    unsigned long long h[2] = {0ull, 0ull}, hb[2] = {0ull, 0ull};
-    cudaError_t e = cudaMemcpyAsync(h, b.err, sizeof h, cudaMemcpyDeviceToHost, g->st);
-    if (e == cudaSuccess && bad)
-        e = cudaMemcpyAsync(hb, bad, sizeof hb, cudaMemcpyDeviceToHost, g->st);
+    if (check)
+        graph_check_inputs(nullptr, nullptr, active, s.n, s.k, s.L, s.rid, nullptr,
+                           &b.count->bad_id, g->st);
+    BuildCounts h;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, b.count, sizeof h, cudaMemcpyDeviceToHost, g->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         err = std::string("graph build: ") + cudaGetErrorString(e);
         return ECMC_ECUDA;
     }
-    if (hb[0] || hb[1]) {
-        err = hb[0] ? "coordinate outside [0, L)" : "active ids must be distinct and in [0, n)";
+    if (h.bad_xy || h.bad_id) {
+        err = h.bad_xy ? "coordinate outside [0, L)" : "active ids must be distinct and in [0, n)";
         return ECMC_EINVAL;
     }
-    if (h[0]) {
+    if (h.full) {
         err = "more disks in a cell than it has slots (overlapping input?)";
         return ECMC_ECAPACITY;
     }
-    return graph_records(g, b, h[1] == 0ull, active, err);
+    return graph_records(g, b, h.mixed == 0ull, active, err);
 }
 
 // Flag words of a context: one per disk, or per cell.
@@ -4127,7 +4131,7 @@ static void graph_arrays(GraphCtx *g, Take take) {
     // all ones in a new context, from here on
     take(&s.key, n);
     take(&s.memb, k);
-    // zero, from here up to the last flag word
+    // zero, from here on
     take(&s.sp, k);
     take(&s.nrec, k);
     take(&s.taken, k);
@@ -4135,7 +4139,6 @@ static void graph_arrays(GraphCtx *g, Take take) {
     take(&s.dbg, 16);
     take(&s.tc_cnt, TC_N);
     take(&s.fl, flag_words(s));
-    // (graph_leg has these zero too)
     take(&s.rid, n);
 }
 
@@ -4217,21 +4220,17 @@ static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
     s.log_cap = s.log_on ? (p->log_cap > 0 ? p->log_cap : ((int64_t)1 << 22)) : 0;
 }
 
-// Counters, run results, flag words, touch keys and member tags of a new context
-// (arrays side by side in the order of graph_arrays); zero_end: the end of the
-// zeroed part.
-static cudaError_t graph_clear(GraphCtx *g, void *zero_end) {
+// Counters, run results, flag words, touch keys, member tags and the ids seen of
+// a new context (arrays side by side in the order of graph_arrays).
+static cudaError_t graph_clear(GraphCtx *g) {
     const GDev &s = g->s;
-    char *const ones = (char *)s.key, *const zero = (char *)s.sp;
+    char *const ones = (char *)s.key, *const zero = (char *)s.sp, *const end = (char *)(s.rid + s.n);
     const cudaError_t e = cudaMemsetAsync(ones, 0xFF, (size_t)(zero - ones), g->st);
-    return e != cudaSuccess
-               ? e
-               : cudaMemsetAsync(zero, 0, (size_t)((char *)zero_end - zero), g->st);
+    return e != cudaSuccess ? e : cudaMemsetAsync(zero, 0, (size_t)(end - zero), g->st);
 }
 
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
-                 const int32_t *active, unsigned long long *bad, cudaStream_t st,
-                 GraphCtx **out, std::string &err) {
+                 const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err) {
     *out = nullptr;
     if (p->n_chains > MAX_CHAINS) {
         err = "too many chains";
@@ -4250,12 +4249,12 @@ int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
         graph_destroy(g);
         return rc;
     }
-    if (graph_clear(g, g->s.fl + flag_words(g->s)) != cudaSuccess) {
+    if (graph_clear(g) != cudaSuccess) {
         (void)cudaGetLastError();
         err = "clearing the graph state";
         rc = ECMC_ECUDA;
     }
-    if (!rc) rc = graph_build(g, x, y, active, bad, err);
+    if (!rc) rc = graph_build(g, x, y, active, true, err);
     if (!rc && graph_max_grid() < 1) {
         err = "cooperative launch unavailable";
         rc = ECMC_ECUDA;
@@ -4555,7 +4554,7 @@ int graph_export(GraphCtx *g, double *x, double *t, const double **y, const int3
     *y = s.y;
     *active = (const int32_t *)s.ci;
     if (x || t)
-        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, x, t, nullptr);
+        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, x, t, nullptr, nullptr);
     return cudaGetLastError() == cudaSuccess ? 0 : ECMC_ECUDA;
 }
 
@@ -4588,7 +4587,7 @@ int graph_transpose(GraphCtx *g, std::string &err) {
     k_g_swap_xy<<<(unsigned)((s.n + 255) / 256), 256, 0, g->st>>>(s, xnew);
     // records (x, t = 0) and arrows for the new frame
     g->axis ^= 1;
-    int rc = graph_build(g, xnew, s.y, nullptr, nullptr, err);
+    int rc = graph_build(g, xnew, s.y, nullptr, false, err);
     // (the build's kernels read xnew: done before the block goes back)
     if (cudaStreamSynchronize(g->st) != cudaSuccess && rc == 0) {
         (void)cudaGetLastError();
@@ -4669,12 +4668,10 @@ struct LegTables {
 };
 
 // Places the arrays of a leg in [base, ...) on 256-byte boundaries (base null:
-// only counts). seen: the ids seen by the input check.
+// only counts).
 struct LegArrays {
     LegTables *tables;
     int32_t *blocked;
-    uint32_t *seen;
-    unsigned long long *bad;  // [2]
 };
 
 size_t leg_arrays(GraphCtx *g, unsigned char *base, LegArrays *out) {
@@ -4685,8 +4682,6 @@ size_t leg_arrays(GraphCtx *g, unsigned char *base, LegArrays *out) {
         off += std::max<size_t>(count, 1) * sizeof(**p);
     };
     graph_arrays(g, take);
-    out->seen = g->s.rid;  // (written again by the build)
-    take(&out->bad, 2);
     take(&out->tables, 1);
     take(&out->blocked, (size_t)g->s.k);
     char *tmp;
@@ -4722,22 +4717,8 @@ int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, cons
     };
     const int grid = graph_max_grid();
     if (grid < 1) return ECMC_ECUDA;
-    // the first half of the build reads any coordinates; ids are used after
-    // the check's result
-    cu(graph_clear(&g, a.bad + 2));
-    graph_check_inputs(nullptr, nullptr, active, s.n, s.k, s.L, a.seen, a.bad, a.bad + 1, st);
-    GBuild b;
-    if (!rc) rc = graph_place(&g, x, y, a.bad, &b, err);
-    unsigned long long bad[2], built[2];
-    if (!rc) {
-        cu(cudaMemcpyAsync(bad, a.bad, sizeof bad, cudaMemcpyDeviceToHost, st));
-        cu(cudaMemcpyAsync(built, b.err, sizeof built, cudaMemcpyDeviceToHost, st));
-        cu(cudaStreamSynchronize(st));
-    }
-    if (rc) return rc;
-    if (bad[0] || bad[1]) return ECMC_EINVAL;
-    if (built[0]) return ECMC_ECAPACITY;
-    rc = graph_records(&g, b, built[1] == 0ull, active, err);
+    cu(graph_clear(&g));
+    if (!rc) rc = graph_build(&g, x, y, active, true, err);
     if (rc) return rc;
     LegTables t;
     memset(&t, 0, sizeof t);
@@ -4767,8 +4748,7 @@ int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, cons
         // (a leg out of records leaves the inputs as they are; one that gave up
         // on a wait never counted itself)
         const int32_t *const failed = &a.tables->ctl.failed;
-        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t_out, failed);
-        k_g_export_active<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active, failed);
+        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t_out, active, failed);
         cu(cudaGetLastError());
     }
     cu(cudaMemcpyAsync(&t, a.tables, sizeof t, cudaMemcpyDeviceToHost, st));

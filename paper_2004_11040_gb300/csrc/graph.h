@@ -20,13 +20,12 @@ struct GraphTotals {
     double ms, pass1_ms, repair_ms, other_ms;
 };
 
-// A context on device inputs x, y (n each) and active (k), which the work it
-// queues on the stream reads; bad: two counters, the second that of
-// graph_check_inputs on active, queued before. nc cells per side. With ECMC_GRAPH the conflict flag is on the
-// disks read, otherwise on the cells scanned.
+// A context on device inputs x, y (n each) and active (k), which are checked here
+// and which the work it queues on the stream reads; nc cells per side. With
+// ECMC_GRAPH the conflict flag is on the disks read, otherwise on the cells
+// scanned.
 int graph_create(const ecmc_params *p, int nc, const double *x, const double *y,
-                 const int32_t *active, unsigned long long *bad, cudaStream_t st,
-                 GraphCtx **out, std::string &err);
+                 const int32_t *active, cudaStream_t st, GraphCtx **out, std::string &err);
 int graph_run(GraphCtx *g, int32_t n_legs, uint64_t budget, uint8_t *flags_host,
               int32_t *legs_done, GraphTotals *tot, std::string &err,
               unsigned long long wait_ns);
@@ -64,7 +63,7 @@ size_t graph_leg_bytes(const ecmc_params *p, int nc);
 int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, const double *y,
               int32_t *active, double *t_out, cudaStream_t st, uint8_t *flag, int64_t *lifts,
               std::string &err);
-// Counts coordinates outside [0, L) in *bad_xy and active ids that repeat or
+// Counts coordinates outside [0, L) in *bad_xy (not with x null) and active ids that repeat or
 // lie outside [0, n) in *bad_id (seen: n words of zero).
 void graph_check_inputs(const double *x, const double *y, const int32_t *active, int64_t n, int k,
                         double L, uint32_t *seen, unsigned long long *bad_xy,
