@@ -90,8 +90,10 @@ struct GDev {
     double *y;  // [n]
     // parallel pass: per disk the least touch key (time << 32 | chain) of the
     // chains whose run alone touches it, ~0 untouched; per chain the touched
-    // disks of its run (entry e of chain c at e * k + c)
-    unsigned long long *key;
+    // disks of its run (entry e of chain c at e * k + c). With claim windows there
+    // are two sets of keys, [2n], used in turn (keys: the first; key: the
+    // window's, in the warp's copy in shared memory)
+    unsigned long long *key, *keys;
     uint32_t *path;        // [(cap + 2) * k]
     unsigned long long *fl;  // flag words, epoch << 32 | chain + 1: per disk read, or
                              // per cell scanned
@@ -3403,10 +3405,24 @@ __device__ __forceinline__ const GDev &g_warp_dev(GDev *slot, int *rep, const GD
     return *slot;
 }
 
-// The leg's stamp in the warp's copy of the description.
-__device__ __forceinline__ void g_set_stamp(GDev *slot, int leg, int lane) {
-    if (lane == 0) slot->stamp = slot->stamp0 + (uint32_t)leg + 1u;
+// The leg's stamp and the touch keys of claim window w in the warp's copy of the
+// description.
+__device__ __forceinline__ void g_set_stamp(GDev *slot, int leg, int w, int lane) {
+    if (lane == 0) {
+        slot->stamp = slot->stamp0 + (uint32_t)leg + 1u;
+        if (slot->windows > 1) slot->key = slot->keys + ((w & 1) != 0 ? slot->n : 0);
+    }
     __syncwarp();
+}
+
+// Chain c at the start of window w > 0: its keys of the last window go (nobody
+// reads that set in this window; in a phase of its own, with a barrier, a window
+// took 16.7 us instead of 14.5).
+__device__ __noinline__ void g_drop_keys(GDev *slot, int c, int leg, int w, int lane) {
+    g_set_stamp(slot, leg, w - 1, lane);
+    g_reset_keys(*slot, c, lane);
+    __syncwarp();
+    g_set_stamp(slot, leg, w, lane);
 }
 
 constexpr int GRUN_THREADS = 256;
@@ -3626,20 +3642,6 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
             }
         };
         for (int w = 0; w < B.windows; ++w) {
-            if (w > 0) {
-                // a new claim window: the touch keys of the last one go
-                for (int f = gw; f < total_chains; f += nwarps) {
-                    const int r = g_find_rep(B.chain_base, R, f);
-                    if (!g_rep_on(B, r)) continue;
-                    g_reset_keys(g_warp_dev(my_dev, my_rep, B.reps, r), f - B.chain_base[r], lane);
-                }
-                for (int r = gt; r < R; r += (int)(gridDim.x * blockDim.x)) {
-                    if (!g_rep_on(B, r)) continue;
-                    B.reps[r].lc[LC_WBLOCKED] = 0ull;
-                    B.reps[r].lc[LC_WWEAK] = 0ull;
-                }
-                if (!barrier()) return;
-            }
             int nblk = 0;  // blocked chains of the pass, of all systems
             for (;;) {
                 ++pass;
@@ -3648,9 +3650,10 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     const int r = g_find_rep(B.chain_base, R, f);
                     if (!g_rep_on(B, r)) continue;
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
-                    if (!fast) g_set_stamp(my_dev, leg, lane);
+                    if (!fast) g_set_stamp(my_dev, leg, w, lane);
                     g_begin_pass(s, f - B.chain_base[r], lane);
                     if (s.ring && simple && g_leap_chain(s, f - B.chain_base[r])) continue;
+                    if (w > 0) g_drop_keys(my_dev, f - B.chain_base[r], leg, w, lane);
                     g_spec_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
                                  g_window_end(s, w), simple);
                 }
@@ -3663,11 +3666,18 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     const int r = g_find_rep(B.chain_base, R, f);
                     if (!g_rep_on(B, r)) continue;
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
-                    if (!fast) g_set_stamp(my_dev, leg, lane);
+                    if (!fast) g_set_stamp(my_dev, leg, w, lane);
                     g_resolve_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
                                     s.epoch0 + pass, f, bl);
-                    if (!simple && sub == 0)
-                        g_flag_chain(s, f - B.chain_base[r], s.epoch0 + pass, lane);
+                }
+                // (what a chain read its run alone left: of few chains the warps
+                // without one find the flag meanwhile)
+                for (int f = nwarps - 1 - gw; f < total_chains && !simple && sub == 0;
+                     f += nwarps) {
+                    const int r = g_find_rep(B.chain_base, R, f);
+                    if (!g_rep_on(B, r)) continue;
+                    const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
+                    g_flag_chain(s, f - B.chain_base[r], s.epoch0 + pass, lane);
                 }
                 if (!barrier()) return;
                 mark(GPH_PASS1);
@@ -3678,7 +3688,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 }
                 if (!restart) break;
                 const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, 0);
-                g_set_stamp(my_dev, leg, lane);
+                g_set_stamp(my_dev, leg, w, lane);
                 if (__ldcg(s.lc + LC_WBLOCKED) == 0ull) break;
                 if (blockIdx.x == 0) {  // T*: the earliest stop of this pass
                     double m = INFINITY;
@@ -3710,10 +3720,13 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                 tw_r = Ts;
                 ++sub;
             }
-            // the window's flag: the reads of two chains met
+            // the window's flag: the reads of two chains met (its counter is added
+            // to again behind the next pass's barrier)
             for (int r = gt; r < R && !simple; r += (int)(gridDim.x * blockDim.x))
-                if (g_rep_on(B, r) && __ldcg(B.reps[r].lc + LC_WWEAK) != 0ull)
+                if (g_rep_on(B, r) && __ldcg(B.reps[r].lc + LC_WWEAK) != 0ull) {
                     atomicAdd(B.reps[r].lc + LC_CWINDOWS, 1ull);
+                    B.reps[r].lc[LC_WWEAK] = 0ull;
+                }
             // repair rounds
             for (int round = 1; nblk > 0; ++round) {
                 int ncomp = nblk;
@@ -3738,7 +3751,7 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     const int32_t *const base = round == 1 ? B.chain_base : B.comp_base;
                     const int r = g_find_rep(base, R, f), q = f - base[r];
                     const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
-                    if (!fast) g_set_stamp(my_dev, leg, lane);
+                    if (!fast) g_set_stamp(my_dev, leg, w, lane);
                     int root, m;
                     int32_t *mem;
                     int cap = 0;
@@ -3795,7 +3808,10 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
             if (!g_rep_on(B, r)) continue;
             const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
             const int c = f - B.chain_base[r];
-            if (!simple) g_reset_keys(s, c, lane);
+            if (!simple) {
+                g_set_stamp(my_dev, leg, B.windows - 1, lane);
+                g_reset_keys(s, c, lane);
+            }
             if (s.log_on) g_log_chain(s, c, (int32_t)(B.ctl[r].leg0 + B.ctl[r].legs), lane);
             if (!simple && g_next_at_end(B, r, leg)) g_begin_state(s, c, s.ci[c], lane);
         }
@@ -4129,7 +4145,7 @@ static void graph_arrays(GraphCtx *g, Take take) {
     take(&s.ctl, CTL_N);
     if (s.log_on) take(&s.log, (size_t)s.log_cap);
     // all ones in a new context, from here on
-    take(&s.key, n);
+    take(&s.keys, s.windows > 1 ? 2 * n : n);
     take(&s.memb, k);
     // zero, from here on
     take(&s.sp, k);
@@ -4223,8 +4239,9 @@ static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
 // Counters, run results, flag words, touch keys, member tags and the ids seen of
 // a new context (arrays side by side in the order of graph_arrays).
 static cudaError_t graph_clear(GraphCtx *g) {
-    const GDev &s = g->s;
-    char *const ones = (char *)s.key, *const zero = (char *)s.sp, *const end = (char *)(s.rid + s.n);
+    GDev &s = g->s;
+    s.key = s.keys;
+    char *const ones = (char *)s.keys, *const zero = (char *)s.sp, *const end = (char *)(s.rid + s.n);
     const cudaError_t e = cudaMemsetAsync(ones, 0xFF, (size_t)(zero - ones), g->st);
     return e != cudaSuccess ? e : cudaMemsetAsync(zero, 0, (size_t)(end - zero), g->st);
 }
