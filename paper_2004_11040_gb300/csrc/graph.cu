@@ -1582,8 +1582,11 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c) {
         const bool in = lane < 31 && (uint32_t)(n0 + lane) + 1u < len && k.towards(idn, bb);
         const bool nsc = in && ownn >= OWN_ACTIVE;
         double dx = __dsub_rn(xn, x);
-        const bool neg = __double_as_longlong(dx) < 0;
-        if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
+        // (a target with a time of this leg, before whose pass there are none: an
+        // assertion on Eq. 2 below)
+        const bool neg = __double_as_longlong(dx) < 0, timed = in && ownn == s.stamp;
+        const bool any_odd = __any_sync(FULL, neg || timed);
+        if (any_odd && neg) dx = g_add(dx, L);
         double tau = __dsub_rn(dx, bb);
         if (__double_as_longlong(tau) < 0) tau = 0.0;
         const unsigned stops = __ballot_sync(FULL, lane < 31 && (nsc || !in));
@@ -1593,12 +1596,10 @@ __device__ __noinline__ bool g_leap_chain(const GDev &s, int c) {
         const int f = fin ? __ffs(fin) - 1 : 31;  // the event that ends the run, or none
         const bool round = fin && !__shfl_sync(FULL, (int)in, f);
         const bool met = fin && !round && __shfl_sync(FULL, (int)lift, f);  // lift onto an active disk
-        // Eq. 2 on the targets with a time of this leg: before its pass there
-        // are none (an assertion)
-        const bool timed = in && lane <= f && ownn == s.stamp;
-        if (__any_sync(FULL, timed)) {
+        if (any_odd) {
             const double rt = shfl_f64(k.t, (lane + 1) & 31);
-            if (timed && dbits(g_add(t, tau)) < dbits(rt)) atomicAdd(s.lc + LC_HORIZON, 1ull);
+            if (timed && lane <= f && dbits(g_add(t, tau)) < dbits(rt))
+                atomicAdd(s.lc + LC_HORIZON, 1ull);
         }
         n = n0 + f + (fin && !met ? 1 : 0);
         if ((round && len > 1) || n >= s.cap) {
