@@ -141,9 +141,9 @@ int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes);
  * the cell scan, i.e. of Alg. 2. The flag is on the disks a step reads (the
  * active disk and its arrow targets) instead of cells, so a leg's flag is 1
  * iff in some window the disks that two chains read, each run alone, overlap.
- * Limits: n_chains <= 2^20 - 2. Such contexts are batched with each other only
- * (same claim windows, no ECMC_RESTART). cells_per_side only sets the cells
- * that the graph is built from. (A context without ECMC_GRAPH finds its
+ * Limits: n_legs x windows < 2^24 in one call (EINVAL). Such contexts are
+ * batched with each other only (same claim windows, no ECMC_RESTART).
+ * cells_per_side only sets the cells that the graph is built from. (A context without ECMC_GRAPH finds its
  * liftings through G(3) too; what its flag says is what a scan of cells
  * would.)
  *
@@ -167,9 +167,10 @@ int ecmc_context_bytes(const ecmc_params *p, int64_t *bytes);
  *   leg_flags_out host, n_legs bytes or NULL: the leg's conflict flag (see
  *                 above); entries past *legs_done are untouched.
  *   legs_done     host or NULL: number of legs completed.
- * All legs run in one persistent cooperative launch (2^24 / windows of them
- * at a time); returns when they are done (the stream is synchronised).
- * Errors: EINVAL, ECUDA, ECAPACITY (undo log), ETIMEOUT (a grid barrier wait
+ * All legs run in one persistent cooperative launch (without ECMC_GRAPH: of
+ * more than 2^24 / windows legs, in several); returns when they are done (the
+ * stream is synchronised).
+ * Errors: EINVAL (with ECMC_GRAPH also n_legs x windows >= 2^24), ECUDA, ECAPACITY (undo log), ETIMEOUT (a grid barrier wait
  * passed its 60 s limit).
  */
 int ecmc_run_to_breakpoint(ecmc_ctx *ctx, int32_t n_legs, uint64_t event_budget,
@@ -281,8 +282,9 @@ int ecmc_profile(ecmc_ctx *ctx, ecmc_profile_t *out);
  *                 budget (0 = no budget); the launch ends when all stopped.
  *   liftings_out, legs_out  host, n_ctx each or NULL: per-context results.
  *   device_ms_out host or NULL: duration of the launch (CUDA events).
- *   Errors: EINVAL, ENOMEM, ECUDA, ECAPACITY, ETIMEOUT (a grid barrier wait
- *   passed its 60 s limit; the launch returned instead of waiting).
+ *   Errors: EINVAL (with ECMC_GRAPH also max_legs x windows >= 2^24), ENOMEM,
+ *   ECUDA, ECAPACITY, ETIMEOUT (a grid barrier wait passed its 60 s limit; the
+ *   launch returned instead of waiting).
  * ecmc_batch_last_error -- reason of the last failure of b.
  * ecmc_batch_destroy    -- releases the scratch to the device memory cache after
  *                         the batch's stream has finished (the contexts stay
