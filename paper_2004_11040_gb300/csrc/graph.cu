@@ -4606,6 +4606,16 @@ int graph_transpose(GraphCtx *g, std::string &err) {
     // records (x, t = 0) and arrows for the new frame
     g->axis ^= 1;
     int rc = graph_build(g, xnew, s.y, nullptr, false, err);
+    if (rc == ECMC_ECAPACITY) {
+        // (a cell overfull by overlapping disks; the records were not built) the
+        // context stays as it was
+        g->axis ^= 1;
+        if (cudaMemcpyAsync(s.y, xnew, (size_t)s.n * 8, cudaMemcpyDeviceToDevice, g->st) !=
+            cudaSuccess) {
+            (void)cudaGetLastError();
+            rc = ECMC_ECUDA;
+        }
+    }
     // (the build's kernels read xnew: done before the block goes back)
     if (cudaStreamSynchronize(g->st) != cudaSuccess && rc == 0) {
         (void)cudaGetLastError();
