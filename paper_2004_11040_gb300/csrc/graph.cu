@@ -2005,20 +2005,21 @@ __device__ __forceinline__ bool holder_ours(const GDev &s, int h, int root, uint
 // read -- i and the arrow targets -- is claimed for the pass, together with
 // the loads; what was read is used only once the claims stand. A claim of
 // another chain is a conflict unless that chain is listed in this round's
-// component (memb == tag). Candidates are the static targets (Alg. 2: j not
+// component (memb == tag). (all: every chain is, nothing to claim.) Candidates are
+// the static targets (Alg. 2: j not
 // active); a target with t_i + tau < t_j became static after chain c's disk
 // had passed it and is one lap away (lazy per-chain frame); ties go to the
 // lower disk index.
 __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, uint32_t epoch,
-                            const uint32_t a[3], const double b[3], uint32_t i, double xi,
-                            double ti, double D) {
+                            bool all, const uint32_t a[3], const double b[3], uint32_t i,
+                            double xi, double ti, double D) {
     const uint32_t mine = (uint32_t)c + 1u;
     const unsigned long long ct = ((unsigned long long)epoch << 32) | mine;
     uint32_t old[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-        if (a[q] != NONE) old[q] = g_claim(s, a[q], ct);
-    old[3] = g_claim(s, i, ct);
+        if (!all && a[q] != NONE) old[q] = g_claim(s, a[q], ct);
+    if (!all) old[3] = g_claim(s, i, ct);
     GDisk r[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q)
@@ -2283,11 +2284,11 @@ __device__ void g_resume(const GDev &s, int c) {
 
 // Pending event of member c (one thread), kept with the arrows it read.
 __device__ __noinline__ void g_compute(const GDev &s, int c, int root, uint64_t tag,
-                                       uint32_t epoch, bool &abort, int &met) {
+                                       uint32_t epoch, bool all, bool &abort, int &met) {
     const uint32_t i = s.ci[c];
     const GDisk ri = s.g[i];
     const double ti = s.tc[c], D = s.D[c];
-    const GStep o = graph_step(s, c, root, tag, epoch, ri.a, ri.b, i, ri.x, ti, D);
+    const GStep o = graph_step(s, c, root, tag, epoch, all, ri.a, ri.b, i, ri.x, ti, D);
     if (o.conflict && !abort) {
         abort = true;
         met = (int)o.partner;
@@ -3113,10 +3114,12 @@ __device__ __noinline__ bool g_replay_large(const GDev &s, const int32_t *mem, i
                                             double tend, int *met_out, double *now_out,
                                             uint32_t *seq) {
     const int lane = threadIdx.x & 31;
+    const bool all = m == s.k;
     bool abort = false;
     int met = -1;
     for (int e = lane; e < m; e += 32)
-        if (s.status[mem[e]] == ST_RUNNING) g_compute(s, mem[e], root, tag, epoch, abort, met);
+        if (s.status[mem[e]] == ST_RUNNING)
+            g_compute(s, mem[e], root, tag, epoch, all, abort, met);
     double now = Ts;
     uint32_t cnt = *seq;
     for (;;) {
@@ -3215,7 +3218,7 @@ __device__ __noinline__ bool g_replay_large(const GDev &s, const int32_t *mem, i
                 const uint32_t v = s.ev_a[3 * (size_t)c + k2];
                 redo |= v != NONE && (v == ib || v == jb);
             }
-            if (redo) g_compute(s, c, root, tag, epoch, abort, met);
+            if (redo) g_compute(s, c, root, tag, epoch, all, abort, met);
         }
         __syncwarp();
     }
