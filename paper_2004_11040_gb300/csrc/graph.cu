@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(FAR_THREADS, 8) k_gb_far(GBuild b) {
 // so the disk after the next is reached 0.02 d later at least). In a frame
 // whose rows all are rings -- a lattice start on cells aligned with it -- a
 // chain's run is a stretch of consecutive places (g_leap_chain) instead of a
-// walk from record to record. The cells' row bands decide (k_skip).
+// walk from record to record. The cells' row bands decide (k_ring_rows).
 
 constexpr double RING_SPREAD = 0.86;
 constexpr int RING_CHUNK = 256;  // columns of a row per block of the kernels below
@@ -4112,8 +4112,10 @@ static void graph_arrays(GraphCtx *g, Take take) {
     const size_t path = k * ((size_t)s.cap + 2);
     take(&s.g, n);
     take(&s.y, n);
-    take(&s.pos, n);
-    take(&g->ring.off, (size_t)g->nc * ring_chunks(g->nc) + 1);
+    // (rings are asked for on both axes or on none)
+    const bool rings = g->try_ring[0] || g->try_ring[1];
+    take(&s.pos, rings ? n : 0);
+    take(&g->ring.off, rings ? (size_t)g->nc * ring_chunks(g->nc) + 1 : 0);
     if (s.cells) {
         take(&s.pxt, path);
         take(&s.pcell, path);
