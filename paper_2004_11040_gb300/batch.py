@@ -1,6 +1,6 @@
 """Batched replicas: many independent ECMC systems of uneven size in one
 persistent launch, versus the same systems one at a time; and the autotuner
-that picks the cell size, the parallel pass and the legs per launch.
+that picks the cell size, the search and the legs per launch.
 
 Replica recipe (the batched workload): N log-uniform in [1024, 65536] with
 M = round(sqrt(N)), N := M^2; eta uniform in [0.60, 0.74]; k = M chains
@@ -52,19 +52,21 @@ def cells_for(start: synth.Start, cells) -> int:
 
 def create(reps: list[Replica], cells="lattice", undo_cap: int = 256, stream=None,
            rowpass: bool = True, graph: bool = False):
-    """The replicas' contexts: cell scan (with or without the row pass), or the
-    constraint graph (graph=True; cells then only set the graph's build)."""
+    """The replicas' contexts: with the conflict flag on scanned cells, running
+    along rings where the frame allows it (rowpass) or always along the arrows of
+    G(3); or with the flag on the disks read (graph=True)."""
     return [ecmc.System(r.start.x, r.start.y, r.start.active, r.start.box, r.ell,
                         cells_per_side=cells_for(r.start, cells), undo_cap=undo_cap,
                         stream=stream, rowpass=rowpass, graph=graph) for r in reps]
 
 
-# parallel pass of a trial: the row pass (cell scan), the general pass (cell
-# scan), or the constraint graph
+# settings of a trial: rings where the frame allows it, never rings, or a
+# constraint-graph context (its flag is on disks; without rings its legs run as
+# those of "general")
 SEARCHES = {"row": dict(rowpass=True, graph=False), "general": dict(rowpass=False, graph=False),
             "graph": dict(rowpass=False, graph=True)}
-# chains a warp advances in each search: one (the warp's lanes share a chain's
-# scan) or 32 (graph mode: a chain per thread)
+# recorded with each trial. In every setting a warp now advances one chain; the 32
+# of "graph" dates from a pass with a chain per thread, and records keep it.
 CHAINS_PER_WARP = {"row": 1, "general": 1, "graph": 32}
 
 
@@ -135,17 +137,15 @@ def _key(reps: list[Replica]) -> str:
 def autotune(reps: list[Replica], trial_budget: int = 20_000,
              cells_options=("lattice", "default"), search_options=("row", "general", "graph"),
              legs_options=(4, 16, 64), cache: str | None = CACHE, stream=None) -> dict:
-    """Tries every (cell size, parallel pass, legs per launch) on a sample of
-    the replicas and keeps the fastest by liftings per device second; every
-    trial is recorded, and the choice is cached per GPU, library build and
-    workload. The parallel pass is the row pass (a warp holds 32 slots of
-    its chain's row and runs prepared steps in batches), the general pass (a
-    warp scans 3 rows x 2 columns of cells per pass), both one chain per
-    warp, or the constraint graph (one chain per thread; its cell size only
-    sets the graph's build, so it is tried once). Fewer warps per chain (two
-    chains per warp) are not offered: every FP64 warp instruction occupies
-    the sub-partition's FP64 unit ~64 cycles whatever its lane mask, so a
-    warp's latency per step is set by its FP64 instruction count, which two
+    """Tries every (cell size, search, legs per launch) on a sample of the
+    replicas and keeps the fastest by liftings per device second; every trial is
+    recorded, and the choice is cached per GPU, library build and workload. The
+    search is one of SEARCHES: "row" runs along rings of disks where the cells
+    give them, "general" and "graph" always along the arrows of G(3); the last
+    differs in its flag, and its cell size only sets the graph's build, so it is
+    tried once. Warps per chain is not a dimension: every FP64 warp instruction
+    occupies the sub-partition's FP64 unit ~64 cycles whatever its lane mask, so
+    a warp's latency per step is set by its FP64 instruction count, which two
     chains would not share."""
     key = _key(reps)
     if cache and os.path.exists(cache):
