@@ -33,6 +33,7 @@ enum { LC_BLOCKED = 0, LC_LIFTS, LC_HORIZON, LC_ERR_CAP, LC_ERR_REC, LC_ORDER, L
        LC_P1LIFTS, LC_REPAIRED, LC_WBLOCKED, LC_CWINDOWS, LC_RESTARTS, LC_WEAK,
        LC_WWEAK,    // chains whose reads met another's, this window
        LC_RINGLAP,  // chains whose run came round its ring (a frame of rings)
+       LC_OPEN,     // steps that an open arrow left undecided (the launch is void)
        LC_N };
 enum { CTL_NCOMP = 0, CTL_NABORT, CTL_NMEMB, CTL_N };
 // cumulative counters

@@ -107,6 +107,7 @@ struct GDev {
     uint32_t *pcell;      // [(cap + 2) * k]
     // a frame of rings (ring != 0): the disks ring after ring, each in the order
     // of x; every disk's place there, its ring's first place and length, its row
+    int open;  // a launch with open arrows
     int ring;
     uint32_t *rid;  // [n]
     uint4 *pos;     // [n]
@@ -197,6 +198,16 @@ __device__ __forceinline__ double g_time(uint32_t own, double t, uint32_t stamp)
     return own >= OWN_ACTIVE || own == stamp ? t : 0.0;
 }
 
+// b of an arrow not searched to its end (a: NONE): minus the place before which
+// there is none (the sign bit also of 0).
+constexpr unsigned long long SIGN = 1ull << 63;
+__device__ __forceinline__ bool g_open(uint32_t a, double b) {
+    return a == NONE && (dbits(b) & SIGN) != 0ull;
+}
+__device__ __forceinline__ double g_unsigned(double b) {
+    return __longlong_as_double((long long)(dbits(b) & ~SIGN));
+}
+
 __device__ __forceinline__ double shfl_f64(double v, int src) {
     return __shfl_sync(FULL, v, src);
 }
@@ -208,6 +219,7 @@ __device__ __forceinline__ double shfl_f64(double v, int src) {
 // outside [0, L) and bad ids.
 struct BuildCounts {
     unsigned long long full, mixed, listed, bad_xy, bad_id;
+    unsigned long long open;  // disks whose record has an open arrow
 };
 
 // Inputs and scratch of a build: a cell list of the disks (in any of a cell's
@@ -223,9 +235,11 @@ struct GBuild {
                          // coordinates of neighbouring cells
     const double *x, *y;
     int check;                   // count coordinates outside [0, L)
+    double *start;               // [n] x of every disk, kept (arrows may stay open), or null
     uint32_t *scid;        // [nc*nc*C] disk per slot, EMPTY
     float2 *cxy;           // [nc*nc*C] FP32 coordinates within the cell, NaN in an empty slot
-    uint32_t *far;         // [n] slots of the disks left to k_gb_far
+    uint32_t *far;         // [2n] slots of the disks left to k_gb_far, and from [n] on
+                           // of those with open arrows
     int nblk;              // blocks of FAR_COLS columns in a row
     float4 *ylim;          // [nc*nblk] least and largest y (within the cell row) per block
                            // in the row's lower half, and in its upper one
@@ -472,8 +486,8 @@ static_assert(FAR_LANES >= FAR_COLS, "a lane per column of a block");
 // -inf). Limits of a whole row would span a corridor that no disk of the row is
 // in wherever two rows of disks share a row of cells.
 template <int C>
-__global__ void k_gb_blocks(GBuild b) {
-    if (b.count->listed == 0ull) return;  // nothing is searched beyond the near columns
+__global__ void k_gb_blocks(GBuild b, const unsigned long long *searched) {
+    if (*searched == 0ull) return;
     static_assert(FAR_COLS == 8, "a block is a quarter of a warp's lanes");
     const int64_t end = (int64_t)b.nc * b.nblk * FAR_COLS;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; __any_sync(FULL, q < end);
@@ -609,7 +623,7 @@ struct GSearch {
     }
 
     // A disk left to k_gb_far keeps what was found in its record until then.
-    __device__ __forceinline__ void keep(bool far) const {
+    __device__ __forceinline__ void keep(bool far, unsigned open) const {
         uint4 *const r = reinterpret_cast<uint4 *>(b.g + i);
 #pragma unroll
         for (int q = 0; q < 3; ++q)
@@ -617,10 +631,10 @@ struct GSearch {
                               best[q].loc,
                               doubt | (far ? 8u : 0u) | (play[1] ? 16u : 0u) |
                                   (play[2] ? 32u : 0u) | (row_up ? 64u : 0u) |
-                                  (row_dn ? 128u : 0u));
+                                  (row_dn ? 128u : 0u) | (open << 8));
     }
-    // (true: to be searched beyond the near columns)
-    __device__ __forceinline__ bool take_up() {
+    // (true: to be searched beyond the near columns; open: arrows that stay open)
+    __device__ __forceinline__ bool take_up(unsigned &open) {
         const uint4 *const r = reinterpret_cast<const uint4 *>(b.g + i);
         unsigned f = 0u;
 #pragma unroll
@@ -631,7 +645,8 @@ struct GSearch {
             best[q].loc = u.z;
             f = u.w;
         }
-        doubt = f & 7u;
+        open = f >> 8;
+        doubt = f & 7u & ~open;
         play[0] = true;
         play[1] = (f & 16u) != 0u;
         play[2] = (f & 32u) != 0u;
@@ -655,13 +670,13 @@ struct GSearch {
         return m;
     }
 
-    // The columns beyond (FAR_LANES lanes per disk): the next FAR_LANES blocks of
+    // The columns from `from` on (FAR_LANES lanes per disk): the next FAR_LANES blocks of
     // columns at once, and of the first one of which a row reaches a corridor
     // that is still open a column per lane. (The first block ends with its
-    // columns before the near ones.)
-    __device__ __forceinline__ void beyond(bool far) {
+    // columns before that one.)
+    __device__ __forceinline__ void beyond(bool far, int from) {
         const int lane = threadIdx.x & 31, sub = lane % FAR_LANES, base = lane - sub;
-        const int nc = b.nc, end = cxi + NEAR_COLS < nc ? cxi + NEAR_COLS : cxi + NEAR_COLS - nc;
+        const int nc = b.nc, end = cxi + from < nc ? cxi + from : cxi + from - nc;
         const int first = end / FAR_COLS;
         // the corridors as limits of y in the rows (e covers corridor_f's doubts
         // and the roundings of these sums)
@@ -676,7 +691,7 @@ struct GSearch {
             if (blk >= b.nblk) blk -= b.nblk;
             int c0 = k + sub == 0 ? end : blk * FAR_COLS, m = c0 - cxi;
             if (m < 0) m += nc;
-            const unsigned open = far && k + sub <= b.nblk ? open_at(max(m, NEAR_COLS)) : 0u;
+            const unsigned open = far && k + sub <= b.nblk ? open_at(max(m, from)) : 0u;
             unsigned rows = 0u;
             if (open) {
                 const float4 *const lim = b.ylim + blk;
@@ -710,7 +725,7 @@ struct GSearch {
             const int col = c0 + sub;
             m = col - cxi;
             if (m < 0) m += nc;
-            if (hit && col < c1 && m >= NEAR_COLS) {
+            if (hit && col < c1 && m >= from) {
 #pragma unroll 1
                 for (int z = 0; z < 3; ++z) {
                     if (!((rows >> z) & 1u)) continue;
@@ -734,6 +749,29 @@ struct GSearch {
                     doubt |= 1u << q;
             }
         }
+    }
+
+    // What an open arrow says: nothing lies in its corridor before this place.
+    __device__ __forceinline__ double open_until() const {
+        const float thr = (float)NEAR_COLS * b.af - vi.x - b.df - (float)(NEAR_COLS + 4) * b.del;
+        const double h = __dadd_rn(xi, (double)thr);
+        return __longlong_as_double((long long)(dbits(h < b.L ? h : __dsub_rn(h, b.L)) | SIGN));
+    }
+
+    // The open arrows of the disk's record, to be searched again from its own
+    // column on.
+    __device__ __forceinline__ unsigned take_open() {
+        const GDisk &r = b.g[i];
+        unsigned o = 0u;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            play[q] = r.a[q] == NONE && (dbits(r.b[q]) & SIGN) != 0ull;
+            if (play[q]) o |= 1u << q;
+            best[q].lo = best[q].hi = INFINITY;
+            best[q].loc = NONE;
+        }
+        row_up = row_dn = true;
+        return o;
     }
 
     // the disk in slot l (NONE: none) and b towards it (the warp)
@@ -766,7 +804,7 @@ struct GSearch {
 };
 
 template <int C>
-__global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
+__global__ void __launch_bounds__(256, 4) k_gb_arrows(GBuild b) {
     __shared__ uint32_t list[BUILD_CELLS * C];
     __shared__ int count;
     const int lane = threadIdx.x & 31;
@@ -790,8 +828,9 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
         GSearch<C> r(b, list[e < total ? e : 0]);
         r.begin();
         const int m = r.near();
-        const bool far = m == NEAR_COLS && m < b.nc && r.open_at(m) != 0u;
-        const bool later = r.doubt != 0u || far;
+        const unsigned open = m == NEAR_COLS && m < b.nc ? r.open_at(m) : 0u;
+        const bool far = open != 0u && !b.start;
+        const bool later = (b.start ? r.doubt & ~open : r.doubt) != 0u || far;
         const unsigned fm = __ballot_sync(FULL, e < total && later);
         if (fm) {
             unsigned at = 0u;
@@ -799,13 +838,26 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
             at = __shfl_sync(FULL, at, 0) + __popc(fm & ((1u << lane) - 1u));
             if (e < total && later) {
                 b.far[at] = r.loc;
-                r.keep(far);
+                r.keep(far, b.start ? open : 0u);
             }
         }
         uint32_t id[3];
         double bv[3];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) id[q] = r.arrow(later ? NONE : r.best[q].loc, bv[q]);
+        for (int q = 0; q < 3; ++q) {
+            const bool op = b.start && ((open >> q) & 1u);
+            id[q] = r.arrow(later || op ? NONE : r.best[q].loc, bv[q]);
+            if (op) bv[q] = r.open_until();
+        }
+        if (b.start && __any_sync(FULL, e < total && open != 0u)) {
+            const unsigned om = __ballot_sync(FULL, e < total && open != 0u);
+            unsigned at = 0u;
+            if (lane == 0)
+                at = (unsigned)atomicAdd(&b.count->open, (unsigned long long)__popc(om));
+            at = __shfl_sync(FULL, at, 0) + __popc(om & ((1u << lane) - 1u));
+            if (e < total && open != 0u) b.far[b.n + at] = r.loc;
+        }
+        if (e < total && b.start) b.start[r.i] = r.xi;
         if (e < total && !later) {
             if (b.yout) b.yout[r.i] = r.yi;
 #pragma unroll
@@ -825,21 +877,31 @@ __global__ void __launch_bounds__(256) k_gb_arrows(GBuild b) {
 // corridor's edge was in doubt, 1360.
 constexpr int FAR_THREADS = 128, FAR_BLOCKS = 1216;
 
-template <int C>
+//
+// OPEN: the disks with open arrows instead, which are completed; nothing else of
+// their records changes.
+template <int C, bool OPEN>
 __global__ void __launch_bounds__(FAR_THREADS, 8) k_gb_far(GBuild b) {
     constexpr int PER = 32 / FAR_LANES;  // disks a warp
     const int lane = threadIdx.x & 31, sub = lane % FAR_LANES, base = lane - sub;
-    const unsigned total = (unsigned)b.count->listed, step = gridDim.x * (FAR_THREADS / FAR_LANES);
+    const unsigned total = (unsigned)(OPEN ? b.count->open : b.count->listed),
+                   step = gridDim.x * (FAR_THREADS / FAR_LANES);
     for (unsigned e0 = (blockIdx.x * FAR_THREADS + threadIdx.x) / 32u * PER; e0 < total;
          e0 += step) {
         const bool has = e0 + base / FAR_LANES < total;
-        GSearch<C> r(b, b.far[has ? e0 + base / FAR_LANES : e0]);
-        const bool far = r.take_up();
-        r.beyond(has && far);
+        const unsigned e = has ? e0 + base / FAR_LANES : e0;
+        GSearch<C> r(b, b.far[OPEN ? b.n + e : e]);
+        unsigned open = 0u;  // arrows: that stay open; OPEN: that are completed
+        bool far = true;
+        if (OPEN)
+            open = r.take_open();
+        else
+            far = r.take_up(open);
+        r.beyond(has && far, OPEN ? 0 : NEAR_COLS);
         uint32_t aj[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            aj[q] = r.best[q].loc;
+            aj[q] = !OPEN && ((open >> q) & 1u) ? NONE : r.best[q].loc;
             unsigned odd = __ballot_sync(FULL, has && ((r.doubt >> q) & 1u));
             while (odd) {
                 const int src = __ffs(odd) - 1, g = src / FAR_LANES;
@@ -856,6 +918,14 @@ __global__ void __launch_bounds__(FAR_THREADS, 8) k_gb_far(GBuild b) {
         // a lane per arrow, then a lane per part of the record
         double v;
         const uint32_t j = r.arrow(sub == 0 ? aj[0] : sub == 1 ? aj[1] : sub == 2 ? aj[2] : NONE, v);
+        if (OPEN) {
+            if (has && sub < 3 && ((open >> sub) & 1u)) {
+                b.g[r.i].b[sub] = v;
+                b.g[r.i].a[sub] = j;
+            }
+            continue;
+        }
+        if (sub < 3 && ((open >> sub) & 1u)) v = r.open_until();
         uint32_t id[3];
         double bv[3];
 #pragma unroll
@@ -1055,11 +1125,12 @@ __global__ void __launch_bounds__(256) k_ring_records(GBuild b, GDev s) {
     }
 }
 
-// The chains' start disks active (after a build).
-__global__ void k_g_init_chains(GDev s, const int32_t *active) {
+// The chains' start disks active (after a build); copied to kept (or null).
+__global__ void k_g_init_chains(GDev s, const int32_t *active, int32_t *kept) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= s.k) return;
     const uint32_t a = active ? (uint32_t)active[c] : s.ci[c];
+    if (kept) kept[c] = (int32_t)a;
     s.ci[c] = a;
     s.ci0[c] = a;
     s.g[a].own = OWN_ACTIVE | (uint32_t)c;
@@ -1126,6 +1197,26 @@ __device__ __forceinline__ void g_fetch_first(const GDisk *g, uint32_t i, GDisk 
 // The targets (tid on lanes 0 .. 2) that are no disk, bit p.
 __device__ __forceinline__ unsigned g_none(uint32_t tid) {
     return __ballot_sync(FULL, tid == NONE) & 7u;
+}
+
+// A step whose target an open arrow may hide: nothing of the launch will stand
+// (the error word ends it after the leg; the host looks for LC_OPEN first).
+__device__ __noinline__ void g_undecided(const GDev &s) {
+    atomicAdd(s.lc + LC_OPEN, 1ull);
+    atomicAdd(s.lc + LC_ERR_REC, 1ull);
+}
+
+// Open arrows among the targets (first: the record of target 0) become targets at
+// their place, static and never moved; b, on the lanes of such a target (0 .. 2,
+// repeated), is 0 from then on.
+__device__ __noinline__ void g_open_targets(uint32_t tid, double tb, GDisk *first) {
+    const int lane = threadIdx.x & 31;
+    if (lane < 3 && g_open(tid, tb)) {
+        first[lane].x = g_unsigned(tb);
+        first[lane].t = 0.0;
+        first[lane].own = OWN_STATIC;
+    }
+    __syncwarp();
 }
 
 // FP64 fix-ups of the uncommon case, out of line: the compiler then never
@@ -1250,6 +1341,9 @@ __device__ __forceinline__ void g_begin_state(const GDev &s, int c, uint32_t i, 
 // A step is bound by its instructions (one warp runs alone on its
 // sub-partition, ~10 cycles an instruction), so the loop holds what every
 // step needs; everything else waits for the flush or stands behind any_odd.
+//
+// OPEN: in a launch with open arrows (a few instructions more a step: 0.13 us).
+template <bool OPEN>
 __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, double tend,
                                           bool begin) {
     const int lane = threadIdx.x & 31;
@@ -1284,6 +1378,12 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
     double tb = g[i].b[l3];
     unsigned none = g_none(tid);
     g_copy_wait();
+    // (an arrow not searched to its end: the step that would need it is no step)
+    bool op = OPEN && g_open(tid, tb);
+    if (OPEN && none) {
+        g_open_targets(tid, tb, lv.r[0]);
+        if (op) tb = 0.0;
+    }
     if (lane == 0 && (g_static(own0) || (own0 & OWN_CHAIN) != (uint32_t)c))
         gdiag(s, 6, tw, c, i, own0, 0, 0);
     if (lane == 31) {
@@ -1332,7 +1432,7 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         const GDisk *const R = &lv.r[cb][sl];
         // the records beyond the targets
         g_fetch(g, R, none, lv.r[cb ^ 1]);
-        const bool ev = lane < 3 && tid != NONE;
+        const bool ev = lane < 3 && (tid != NONE || (OPEN && op));
         double rx = R[l3].x, rt = R[l3].t;
         uint32_t own = R[l3].own;
         if (n >= n_stop) {
@@ -1418,7 +1518,11 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
             const double tj = shfl_f64(rt, wl);
             if (lane == (n & 31)) E.tj = bt < dbits(D) ? tj : 0.0;
         }
-        const bool lift = bt < dbits(D);
+        bool lift = bt < dbits(D);
+        if (OPEN && lift && bj == NONE) {
+            if (lane == 0) g_undecided(s);
+            lift = false;
+        }
         const double ts = lift ? __longlong_as_double((long long)bt) : D;
         const double T = __dadd_rn(ti, ts);
         if (n >= room) {  // out of records: the repair goes on from here, or reports it
@@ -1453,6 +1557,11 @@ __device__ __noinline__ void g_spec_chain(const GDev &s, int c, double tw, doubl
         g_copy_wait();
         cb ^= 1;
         sl = 3 * wl;
+        if (OPEN) {
+            op = g_open(tid, tb);
+            if (none) g_open_targets(tid, tb, &lv.r[cb][sl]);
+            if (op) tb = 0.0;
+        }
     }
     g_copy_wait();
     // (the reads of a step that was evaluated but not taken)
@@ -2034,6 +2143,16 @@ __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, uint32
     uint32_t bjid = NONE;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
+        if (g_open(a[q], b[q])) {  // (as a target at its place)
+            double dx = __dsub_rn(g_unsigned(b[q]), xi);
+            if (dneg(dx)) dx = __dadd_rn(dx, s.L);
+            if (bq < 0 || dbits(dx) < bt) {
+                bt = dbits(dx);
+                bq = q;
+                bjid = NONE;
+            }
+            continue;
+        }
         if (a[q] == NONE || !g_static(r[q].own)) continue;
         const double rt = g_time(r[q].own, r[q].t, s.stamp);
         double dx = __dsub_rn(r[q].x, xi);
@@ -2060,7 +2179,8 @@ __device__ GStep graph_step(const GDev &s, int c, int root, uint64_t tag, uint32
             o.partner = (uint32_t)h;
         }
     }
-    if (bq >= 0 && bt < dbits(D)) {
+    if (bq >= 0 && bt < dbits(D) && bjid == NONE) g_undecided(s);
+    if (bq >= 0 && bt < dbits(D) && bjid != NONE) {
         o.lift = 1;
         o.tau = __longlong_as_double((long long)bt);
         o.j = bjid;
@@ -2368,6 +2488,7 @@ __device__ void g_finish(const GDev &s, const int32_t *mem, int m, int root, boo
 // another component.
 enum { CONT_DONE = 0, CONT_FAIL = 1, CONT_FOREIGN = 2 };
 
+template <bool OPEN>
 __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m, int root,
                                        uint64_t tag, uint32_t epoch, int round, double tw,
                                        double tend, int *met, uint32_t *cnt_out) {
@@ -2434,6 +2555,11 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
             return true;
         };
         g_copy_wait();
+        bool op = OPEN && g_open(tid, tb);
+        if (OPEN && none) {
+            g_open_targets(tid, tb, lv.r[0]);
+            if (op) tb = 0.0;
+        }
         GEvs E;
         E.i = NONE;
         E.x = E.t = E.D = E.tau = E.tj = 0.0;
@@ -2462,6 +2588,7 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
             const GDisk *const R = &lv.r[cb][sl];
             g_fetch(g, R, none, lv.r[cb ^ 1]);
             const bool ev = lane < 3 && tid != NONE;
+            const bool evo = lane < 3 && (tid != NONE || (OPEN && op));
             const double rx = R[l3].x, rt = R[l3].t;
             const uint32_t own = R[l3].own;
             const unsigned long long cw = R[l3].claim;
@@ -2489,7 +2616,7 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
             // reach or where it fails Eq. 2
             double sum = __dadd_rn(ti, __double_as_longlong(tau) < 0 ? 0.0 : tau);
             const bool nsc = ev && own >= OWN_ACTIVE;
-            const bool neg = ev && __double_as_longlong(dx) < 0;
+            const bool neg = evo && __double_as_longlong(dx) < 0;
             bool bad = ev && own == stamp && dbits(rt) != 0ull && !(dbits(sum) > dbits(rt));
             bool viol = false;
             uint32_t ns_owner = NONE;
@@ -2507,13 +2634,17 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
                 if (sb) ns_owner = __shfl_sync(FULL, own, __ffs(sb) - 1) & OWN_CHAIN;
             }
             if (__double_as_longlong(tau) < 0) tau = 0.0;
-            const unsigned long long tk = ev && !nsc ? dbits(tau) : INF_BITS;
+            const unsigned long long tk = evo && !nsc ? dbits(tau) : INF_BITS;
             const int wl = g_winner(tk, tid);
             const unsigned long long bt = shfl_u64(tk, wl);
-            const bool lift = bt < dbits(D);
+            bool lift = bt < dbits(D);
+            const uint32_t bj = __shfl_sync(FULL, tid, wl);
+            if (OPEN && lift && bj == NONE) {
+                if (lane == 0) g_undecided(s);
+                lift = false;
+            }
             const double ts = lift ? __longlong_as_double((long long)bt) : D;
             const double T = lift ? shfl_f64(sum, wl) : g_add(ti, D);
-            const uint32_t bj = __shfl_sync(FULL, tid, wl);
             const double xj = shfl_f64(rx, wl);
             const double tj = shfl_f64(own == stamp ? rt : 0.0, wl);
             if (!strict && ev && held == 0u)
@@ -2571,6 +2702,11 @@ __device__ __noinline__ int g_continue(const GDev &s, const int32_t *mem, int m,
             g_copy_wait();
             cb ^= 1;
             sl = 3 * wl;
+            if (OPEN) {
+                op = g_open(tid, tb);
+                if (none) g_open_targets(tid, tb, &lv.r[cb][sl]);
+                if (op) tb = 0.0;
+            }
             if (n - nf == 32 || n > n_lap) {
                 if (!claims_stand()) {
                     how = CONT_FOREIGN;
@@ -2799,6 +2935,7 @@ __device__ __noinline__ int g_continue_ring(const GDev &s, const int32_t *mem, i
 // one event later.
 constexpr int SMALL_REPLAY = 10;
 
+template <bool OPEN>
 __device__ __noinline__ bool g_replay_small(const GDev &s, const int32_t *mem, int m,
                                             uint32_t epoch, int round, double Ts, double tend,
                                             int *met_out, double *now_out, uint32_t *seq) {
@@ -2830,6 +2967,7 @@ __device__ __noinline__ bool g_replay_small(const GDev &s, const int32_t *mem, i
     // this lane's target: place, time, owner and its own arrows
     double rx = 0.0, rt = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0;
     uint32_t own = 0u, a0 = NONE, a1 = NONE, a2 = NONE;
+    bool op = false;
     int met = -1;
     // The claims asked for and not checked yet: the holder that a record's word
     // of this pass names, or what the exchange for a free disk found.
@@ -2838,6 +2976,12 @@ __device__ __noinline__ bool g_replay_small(const GDev &s, const int32_t *mem, i
     auto take = [&](bool mine) {
         held = 0u;
         cas = 0ull;
+        if (OPEN && mine) op = g_open(tid, tb);
+        if (OPEN && mine && op) {  // (an open arrow: a target at its place)
+            rx = g_unsigned(tb);
+            rt = tb = 0.0;
+            own = OWN_STATIC;
+        }
         if (mine && tid != NONE) {
             const ulonglong2 *r = reinterpret_cast<const ulonglong2 *>(g + tid);
             const ulonglong2 u0 = __ldcg(r), u1 = __ldcg(r + 1), u2 = __ldcg(r + 2),
@@ -2883,7 +3027,7 @@ __device__ __noinline__ bool g_replay_small(const GDev &s, const int32_t *mem, i
     while (!abort) {
         // every member's next event (Sec. 2.2): the least (tau, j) of its
         // static targets, one lap on where the target came after it had passed
-        const bool stc = run && tid != NONE && g_static(own);
+        const bool stc = run && (tid != NONE || (OPEN && op)) && g_static(own);
         double dx = __dsub_rn(rx, xi);
         const bool neg = stc && __double_as_longlong(dx) < 0;
         if (__any_sync(FULL, neg) && neg) dx = g_add(dx, L);
@@ -2912,7 +3056,11 @@ __device__ __noinline__ bool g_replay_small(const GDev &s, const int32_t *mem, i
             bj = j2;
             w = 2;
         }
-        const bool lift = bt < dbits(D);
+        bool lift = bt < dbits(D);
+        if (OPEN && lift && bj == NONE) {
+            if (p == 0) g_undecided(s);
+            lift = false;
+        }
         const double ts = lift ? __longlong_as_double((long long)bt) : D;
         const double T = __dadd_rn(ti, ts);
         // the earliest (T, chain)
@@ -3270,8 +3418,11 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int32_t *mem, int
         int met = -1;
         const int how = s.ring && !s.strict
                             ? g_continue_ring(s, mem, m, root, tag, epoch, round, &met, &seq)
-                            : g_continue(s, mem, m, root, tag, epoch, round, tw, tend, &met,
-                                         &seq);
+                        : s.open
+                            ? g_continue<true>(s, mem, m, root, tag, epoch, round, tw, tend, &met,
+                                               &seq)
+                            : g_continue<false>(s, mem, m, root, tag, epoch, round, tw, tend, &met,
+                                                &seq);
         if (how == CONT_DONE) {
             if (lane == 0) atomicAdd(s.lc + LC_CONTINUED, (unsigned long long)m);
             g_finish(s, mem, m, root, false, -1, Ts, true);
@@ -3302,7 +3453,9 @@ __device__ __noinline__ void g_repair_component(const GDev &s, int32_t *mem, int
         double now = Ts;
         const bool abort =
             m <= SMALL_REPLAY
-                ? g_replay_small(s, mem, m, epoch, round, Ts, tend, &met, &now, &seq)
+                ? (s.open ? g_replay_small<true>(s, mem, m, epoch, round, Ts, tend, &met, &now, &seq)
+                          : g_replay_small<false>(s, mem, m, epoch, round, Ts, tend, &met, &now,
+                                                  &seq))
                 : g_replay_large(s, mem, m, root, tag, epoch, round, Ts, tend, &met, &now,
                                  &seq);
         int more = 0;
@@ -3341,6 +3494,7 @@ struct GCtl {
     int32_t err;     // LC_ERR_* seen, or too many repair rounds
     int32_t failed;  // 1 until a leg is done without one
     int32_t dbg;     // an internal check recorded in GDev::dbg (set at the end)
+    int32_t open;    // an open arrow left a step undecided: nothing of the launch stands
 };
 
 enum { GG_WORK = 0, GG_ANY, GG_ERR, GG_REMAIN0, GG_REMAIN1, GG_COUNT, GG_PASSES,
@@ -3592,8 +3746,9 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
         c.horizon += (int64_t)lc[LC_HORIZON];
         c.order_err += (int64_t)lc[LC_ORDER];
         if (lc[LC_ERR_REC] != 0ull || lc[LC_ERR_CAP] != 0ull) c.err = 1;
-        c.failed = c.err;
-        if (c.err || (c.budget > 0 && c.lifts >= c.budget)) c.done = 1;
+        if (lc[LC_OPEN] != 0ull) c.open = 1;
+        c.failed = c.err || c.open;
+        if (c.failed || (c.budget > 0 && c.lifts >= c.budget)) c.done = 1;
         *cp = c;
 #pragma unroll
         for (int q = 0; q < LC_N; ++q) lcp[q] = 0ull;
@@ -3658,8 +3813,11 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     g_begin_pass(s, f - B.chain_base[r], lane);
                     if (s.ring && simple && g_leap_chain(s, f - B.chain_base[r])) continue;
                     if (w > 0) g_drop_keys(my_dev, f - B.chain_base[r], leg, w, lane);
-                    g_spec_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
-                                 g_window_end(s, w), simple);
+                    const double t0 = restart ? tw_r : g_window_start(s, w);
+                    if (s.open)
+                        g_spec_chain<true>(s, f - B.chain_base[r], t0, g_window_end(s, w), simple);
+                    else
+                        g_spec_chain<false>(s, f - B.chain_base[r], t0, g_window_end(s, w), simple);
                 }
                 if (!barrier()) return;
                 if (gt == 0 && w == 0 && sub == 0) B.g[GG_REMAIN0 + ((leg + 1) & 1)] = 0;
@@ -3801,7 +3959,9 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
             const GCtl *const cp = B.ctl;
             const int64_t lifts = (int64_t)__ldcg((const unsigned long long *)&cp->lifts) +
                                   (int64_t)(__ldcg(s.lc + LC_P1LIFTS) + __ldcg(s.lc + LC_LIFTS));
-            const bool err = __ldcg(s.lc + LC_ERR_REC) != 0ull || __ldcg(s.lc + LC_ERR_CAP) != 0ull;
+            // (one round of loads)
+            const bool err =
+                (__ldcg(s.lc + LC_ERR_REC) | __ldcg(s.lc + LC_ERR_CAP)) != 0ull;
             if (err || (cp->budget > 0 && lifts >= cp->budget)) break;
             continue;
         }
@@ -3850,6 +4010,16 @@ __global__ void k_g_export(GDev s, double *x, double *t, int32_t *active, const 
     if (active && q < s.k) active[q] = (int32_t)s.ci[q];
 }
 
+// Every disk back where it was when its frame was built (start).
+__global__ void k_g_restore(GDev s, const double *start) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= s.n) return;
+    GDisk &r = s.g[q];
+    *reinterpret_cast<ulonglong2 *>(&r.x) = make_ulonglong2(dbits(start[q]), 0ull);
+    r.own = OWN_STATIC;
+    r.claim = 0ull;
+}
+
 // Direction change: the disks' x and y are exchanged (x from y_old, y from
 // x_old); the graph is then rebuilt for the new frame.
 __global__ void k_g_swap_xy(GDev s, double *xnew) {
@@ -3879,6 +4049,12 @@ struct GraphCtx {
     int C = 4;                          // slots per cell of a build
     bool try_ring[2] = {false, false};  // per axis: its last frame was of rings, or none was
     int axis = 0;
+    // Arrows may be open (the frame is new, and few legs may be all it runs): the
+    // build that would complete them, and whether a launch has run since.
+    bool places = false;  // s.pos is there; without rings it keeps the frame's start
+    bool open = false, fresh = false;
+    bool one_leg = false;  // one leg is all it runs
+    GBuild build;
     std::vector<std::pair<void **, size_t>> pending;
     int64_t bytes = 0;  // device memory held
 };
@@ -3933,7 +4109,7 @@ struct BuildParts {
         yhi = after(err, sizeof(BuildCounts));
         ylim = after(yhi, (size_t)nc * 8);
         far = after(ylim, (size_t)nc * (size_t)((nc + FAR_COLS - 1) / FAR_COLS) * sizeof(float4));
-        total = after(far, (size_t)n * sizeof(uint32_t));
+        total = after(far, 2 * (size_t)n * sizeof(uint32_t));
     }
 };
 
@@ -4029,6 +4205,44 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, bool check
     return launched("graph build", err);
 }
 
+// Legs that a frame's first launch may run with open arrows. An open arrow tells
+// of a place at least (NEAR_COLS - 1) a - d ahead of the disk when the frame was
+// built; a chain moves a disk by ell a leg at most, and on boxes at all dense by
+// the gaps. Calls of few legs do not earn the search for these arrows back (with
+// it 10^6 triangular disks at eta 0.60 took 1080 us to create, FIG so); before
+// longer ones it is done first.
+//
+// On small boxes the search is cheap, and doing it apart costs as much again (two
+// turns of 65536 disks and 16 legs: 923 us with it at the turn, 957 before the
+// legs): only boxes of OPEN_DISKS or more, or a single leg, go without.
+constexpr int64_t OPEN_DISKS = (int64_t)1 << 17;
+
+static int open_legs(const GraphCtx *g) {
+    return (int)std::min(8.0, NEAR_COLS * (g->box / g->nc) / g->s.ell);
+}
+
+// What a frame with open arrows keeps behind the disks' places (s.pos has 16 bytes
+// a disk): the chains' disks, and the length of the log before the first launch.
+static int32_t *graph_kept(const GraphCtx *g) { return (int32_t *)((double *)g->s.pos + g->s.n); }
+static unsigned long long *graph_log_kept(const GraphCtx *g) {
+    return (unsigned long long *)g->s.pos + g->s.n + (g->s.k + 1) / 2;
+}
+
+// The disks that k_gb_arrows listed, or (OPEN) those with open arrows.
+template <int C, bool OPEN>
+static void graph_far(const GraphCtx *g, cudaStream_t st) {
+    const GBuild &b = g->build;
+    // (with open arrows left open nothing listed needs the columns beyond)
+    if (OPEN || !b.start) {
+        const unsigned nb = (unsigned)std::min<size_t>(
+            ((size_t)g->nc * (size_t)b.nblk * FAR_COLS + 255) / 256, 1216);
+        k_gb_blocks<C><<<nb, 256, 0, st>>>(b, OPEN ? &b.count->open : &b.count->listed);
+    }
+    const unsigned nf = (unsigned)std::min<int64_t>(
+        (b.n * FAR_LANES + FAR_THREADS - 1) / FAR_THREADS, FAR_BLOCKS);
+    k_gb_far<C, OPEN><<<nf, FAR_THREADS, 0, st>>>(b);
+}
+
 // The second half: the records, along the rings (rings) or with the arrows of
 // G(3), and the chains on their start disks (null: where they are).
 static int graph_records(GraphCtx *g, const GBuild &b, bool rings, const int32_t *active,
@@ -4044,24 +4258,47 @@ static int graph_records(GraphCtx *g, const GBuild &b, bool rings, const int32_t
         else
             k_ring_place<8><<<grid, RING_CHUNK, 0, st>>>(b, g->ring, s);
     }
+    g->fresh = true;
+    g->open = !s.ring && s.cells && !s.strict && g->places && open_legs(g) >= 1 &&
+              (g->one_leg || s.n >= OPEN_DISKS);
+    g->build = b;
+    g->build.start = g->open ? (double *)s.pos : nullptr;
     const unsigned ablk = (unsigned)(((size_t)g->nc * g->nc + BUILD_CELLS - 1) / BUILD_CELLS);
-    const unsigned bblk = (unsigned)std::min<size_t>(
-        ((size_t)g->nc * (size_t)b.nblk * FAR_COLS + 255) / 256, 1216);
-    const unsigned fblk = (unsigned)std::min<int64_t>(
-        (s.n * FAR_LANES + FAR_THREADS - 1) / FAR_THREADS, FAR_BLOCKS);
     if (s.ring && s.cells) {
         k_ring_records<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(b, s);
     } else if (g->C == 4) {
-        k_gb_arrows<4><<<ablk, 256, 0, st>>>(b);
-        k_gb_blocks<4><<<bblk, 256, 0, st>>>(b);
-        k_gb_far<4><<<fblk, FAR_THREADS, 0, st>>>(b);
+        k_gb_arrows<4><<<ablk, 256, 0, st>>>(g->build);
+        graph_far<4, false>(g, st);
     } else {
-        k_gb_arrows<8><<<ablk, 256, 0, st>>>(b);
-        k_gb_blocks<8><<<bblk, 256, 0, st>>>(b);
-        k_gb_far<8><<<fblk, FAR_THREADS, 0, st>>>(b);
+        k_gb_arrows<8><<<ablk, 256, 0, st>>>(g->build);
+        graph_far<8, false>(g, st);
     }
-    k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, active);
+    k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(
+        s, active, g->open ? graph_kept(g) : nullptr);
     return launched("graph build", err);
+}
+
+// Open arrows completed, on stream st.
+static void graph_complete(GraphCtx *g, cudaStream_t st) {
+    g->build.x = g->build.start;
+    g->build.y = g->s.y;
+    g->build.start = nullptr;
+    if (g->C == 4)
+        graph_far<4, true>(g, st);
+    else
+        graph_far<8, true>(g, st);
+    g->open = false;
+}
+
+// A launch that an open arrow left undecided is undone: disks, chains and the
+// length of the log as they were when the frame was built; the arrows completed.
+static void graph_undo(GraphCtx *g, cudaStream_t st) {
+    const GDev &s = g->s;
+    k_g_restore<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, g->build.start);
+    k_g_init_chains<<<(unsigned)((s.k + 127) / 128), 128, 0, st>>>(s, graph_kept(g), nullptr);
+    cudaMemsetAsync(s.dbg, 0, 16 * 8, st);
+    if (s.log_on) cudaMemcpyAsync(s.tc_cnt, graph_log_kept(g), 8, cudaMemcpyDeviceToDevice, st);
+    graph_complete(g, st);
 }
 
 // A frame from positions x, y and active disks (device): both halves, with a
@@ -4112,10 +4349,8 @@ static void graph_arrays(GraphCtx *g, Take take) {
     const size_t path = k * ((size_t)s.cap + 2);
     take(&s.g, n);
     take(&s.y, n);
-    // (rings are asked for on both axes or on none)
-    const bool rings = g->try_ring[0] || g->try_ring[1];
-    take(&s.pos, rings ? n : 0);
-    take(&g->ring.off, rings ? (size_t)g->nc * ring_chunks(g->nc) + 1 : 0);
+    take(&s.pos, g->places ? n : 0);
+    take(&g->ring.off, g->places ? (size_t)g->nc * ring_chunks(g->nc) + 1 : 0);
     if (s.cells) {
         take(&s.pxt, path);
         take(&s.pcell, path);
@@ -4222,6 +4457,7 @@ static void graph_params(GraphCtx *g, const ecmc_params *p, int nc) {
     // 2^20 disks, 1024 chains: 63 and 32)
     g->try_ring[0] = g->try_ring[1] =
         !(p->flags & ECMC_NO_ROWPASS) && p->ell < p->box - 3.0 * a;
+    g->places = g->try_ring[0];
     // FP32 image of the scan's stop rule thr(m) = ((m a) - fx) - d > RN(cur +
     // eps): thr_f = ((m af - fxf) - df) and lim_f = trunc(cur) + epsf, with af,
     // df, epsf the FP32 roundings, fxf = trunc(fx). Each of the four FP32
@@ -4432,6 +4668,12 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
             }
             g->flags_cap = max_legs;
         }
+        // (open arrows are for one system and few legs from the frame's start)
+        if (g->open && !(n == 1 && g->fresh && max_legs <= open_legs(g))) graph_complete(g, st);
+        if (g->open && g->s.log_on)
+            cu(cudaMemcpyAsync(graph_log_kept(g), g->s.tc_cnt, 8, cudaMemcpyDeviceToDevice, st),
+               "log");
+        g->fresh = false;
         if (g->s.epoch0 > 0xC0000000u || g->s.stamp0 > 0x3E000000u) {
             k_g_clear_epochs<<<(unsigned)((g->s.n + 255) / 256), 256, 0, st>>>(g->s);
             cu(cudaGetLastError(), "epochs");
@@ -4441,6 +4683,7 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
             g->s.stamp0 = 1;  // (the last leg's times, for ecmc_positions)
         }
         S[r] = g->s;
+        S[r].open = g->open ? 1 : 0;
         ctl[r].budget = budgets ? (int64_t)budgets[r] : 0;
         // (only a run of one system reports its flags)
         ctl[r].flags = n > 1                    ? nullptr
@@ -4498,6 +4741,15 @@ int graph_batch_run(GBatchScratch **scratch, GraphCtx *const *gs, int32_t n, int
         timed_out ? (uint32_t)max_legs * (uint32_t)W * (MAX_RESTARTS + 2u) : (uint32_t)gg[GG_PASSES];
     for (int r = 0; r < n; ++r) {
         const GCtl &c = ctl[r];
+        if (c.open && !timed_out) {  // (n == 1)
+            gs[r]->s.epoch0 += passes;
+            gs[r]->s.stamp0 += (uint32_t)c.legs;
+            graph_undo(gs[r], st);
+            cu(cudaGetLastError(), "open arrows");
+            return rc ? rc
+                      : graph_batch_run(scratch, gs, n, max_legs, budgets, st, tots, legs_out,
+                                        ms_out, err, wait_ns);
+        }
         gs[r]->log_legs += c.legs;
         gs[r]->s.epoch0 += passes;
         gs[r]->s.stamp0 += timed_out ? (uint32_t)max_legs : (uint32_t)c.legs;
@@ -4750,43 +5002,55 @@ int graph_leg(const ecmc_params *p, int nc, unsigned char *base, double *x, cons
     };
     const int grid = graph_max_grid();
     if (grid < 1) return ECMC_ECUDA;
+    g.one_leg = true;
     cu(graph_clear(&g));
     if (!rc) rc = graph_build(&g, x, y, active, true, err);
     if (rc) return rc;
     LegTables t;
-    memset(&t, 0, sizeof t);
-    t.dev = s;
-    t.chain_base[1] = s.k;
-    t.ctl.failed = 1;
-    GBatchDev B;
-    B.reps = &a.tables->dev;
-    B.ctl = &a.tables->ctl;
-    B.chain_base = a.tables->chain_base;
-    B.comp_base = a.tables->comp_base;
-    B.bar = &a.tables->bar;
-    B.g = a.tables->g;
-    B.blocked = a.blocked;
-    B.phase_ns = a.tables->phase;
-    B.R = 1;
-    B.max_legs = 1;
-    B.windows = 1;
-    B.pad = 0;
-    B.wait_ns = BARRIER_TIMEOUT_NS;
-    cu(cudaMemcpyAsync(a.tables, &t, sizeof t, cudaMemcpyHostToDevice, st));
-    void *args[] = {&B};
-    cu(cudaLaunchCooperativeKernel((void *)k_run_graph, grid, GRUN_THREADS, args, UF_SMEM_BYTES,
-                                   st));
-    s.stamp0 = 1;  // (the leg's times)
-    if (!rc) {
-        // (a leg out of records leaves the inputs as they are; one that gave up
-        // on a wait never counted itself)
-        const int32_t *const failed = &a.tables->ctl.failed;
-        k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(s, x, t_out, active, failed);
+    for (;;) {
+        memset(&t, 0, sizeof t);
+        t.dev = s;
+        t.dev.open = g.open ? 1 : 0;
+        t.chain_base[1] = s.k;
+        t.ctl.failed = 1;
+        GBatchDev B;
+        B.reps = &a.tables->dev;
+        B.ctl = &a.tables->ctl;
+        B.chain_base = a.tables->chain_base;
+        B.comp_base = a.tables->comp_base;
+        B.bar = &a.tables->bar;
+        B.g = a.tables->g;
+        B.blocked = a.blocked;
+        B.phase_ns = a.tables->phase;
+        B.R = 1;
+        B.max_legs = 1;
+        B.windows = 1;
+        B.pad = 0;
+        B.wait_ns = BARRIER_TIMEOUT_NS;
+        cu(cudaMemcpyAsync(a.tables, &t, sizeof t, cudaMemcpyHostToDevice, st));
+        void *args[] = {&B};
+        cu(cudaLaunchCooperativeKernel((void *)k_run_graph, grid, GRUN_THREADS, args,
+                                       UF_SMEM_BYTES, st));
+        if (!rc) {
+            // (a leg out of records leaves the inputs as they are; one that gave up
+            // on a wait never counted itself)
+            const int32_t *const failed = &a.tables->ctl.failed;
+            GDev done = s;
+            done.stamp0 = s.stamp0 + 1;  // (the leg's times)
+            k_g_export<<<(unsigned)((s.n + 255) / 256), 256, 0, st>>>(done, x, t_out, active,
+                                                                      failed);
+            cu(cudaGetLastError());
+        }
+        cu(cudaMemcpyAsync(&t, a.tables, sizeof t, cudaMemcpyDeviceToHost, st));
+        cu(cudaStreamSynchronize(st));
+        if (rc) return rc;
+        if (!t.ctl.open || t.g[GG_ERR]) break;
+        s.epoch0 += (uint32_t)t.g[GG_PASSES];
+        s.stamp0 += 1;
+        graph_undo(&g, st);
+        cu(cudaMemsetAsync(s.memb, 0xFF, (size_t)s.k * 8, st));
         cu(cudaGetLastError());
     }
-    cu(cudaMemcpyAsync(&t, a.tables, sizeof t, cudaMemcpyDeviceToHost, st));
-    cu(cudaStreamSynchronize(st));
-    if (rc) return rc;
     if (t.ctl.err) return ECMC_ECAPACITY;
     if (t.g[GG_ERR] || t.ctl.dbg) return ECMC_ECUDA;
     if (flag) *flag = t.ctl.conflict_legs != 0;
