@@ -4207,10 +4207,11 @@ static int graph_place(GraphCtx *g, const double *x, const double *y, bool check
 
 // Legs that a frame's first launch may run with open arrows. An open arrow tells
 // of a place at least (NEAR_COLS - 1) a - d ahead of the disk when the frame was
-// built; a chain moves a disk by ell a leg at most, and on boxes at all dense by
-// the gaps. Calls of few legs do not earn the search for these arrows back (with
-// it 10^6 triangular disks at eta 0.60 took 1080 us to create, FIG so); before
-// longer ones it is done first.
+// built; a chain moves a disk by ell a leg at most, and on dense boxes by the
+// gaps. Calls of few legs do not earn the search for these arrows back (with it
+// 10^6 triangular disks at eta 0.60 took 1080 us to create, 460 so); before longer
+// ones, and before a launch with other systems, it is done first. A launch in
+// which a step comes to such a place is undone and run again with all arrows.
 //
 // On small boxes the search is cheap, and doing it apart costs as much again (two
 // turns of 65536 disks and 16 legs: 923 us with it at the turn, 957 before the
