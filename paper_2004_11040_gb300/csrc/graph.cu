@@ -101,6 +101,7 @@ struct GDev {
     // the scan, and per entry of path what its step's scan needs -- the active
     // disk's x and the least of D and its best time of flight, and its cell
     int cells;
+    uint32_t epoch0;       // epoch of the launch's first pass, less one
     double inv_a;
     StopK sk;
     double2 *pxt;         // [(cap + 2) * k]
@@ -111,7 +112,6 @@ struct GDev {
     int ring;
     uint32_t *rid;  // [n]
     uint4 *pos;     // [n]
-    uint32_t epoch0;       // epoch of the launch's first pass, less one
     GSpec *sp;             // [k] the run alone of each chain, for the resolve
     uint32_t stamp0;       // stamp of the launch's first leg, less one
     uint32_t stamp;        // stamp of the leg (the warp's copy in shared memory)
@@ -141,6 +141,9 @@ struct GDev {
     int log_on;
     double *dbg;  // [16] first failed internal check
 };
+// (a warp copies its system's description in rounds of 128 bytes, one after another;
+// a fifth cost batches 2%)
+static_assert(sizeof(GDev) <= 512, "four rounds");
 
 // Record e of chain c, stored by event index, then chain (the first events of
 // a leg of all chains lie in one dense block).
@@ -3612,6 +3615,22 @@ __device__ __noinline__ void g_drop_keys(GDev *slot, int c, int leg, int w, int 
     g_set_stamp(slot, leg, w, lane);
 }
 
+// The flags of a pass with claim windows or restarts, while chains resolve: what a
+// chain read its run alone left, so of few chains the warps without one find it (a
+// call of its own: the loop inside the kernel cost batches without claim windows
+// 0.8%).
+__device__ __noinline__ void g_flag_strict(const GDev *reps, const GCtl *ctl, const int32_t *base,
+                                           int R, GDev *slot, int *rep, int f, int nwarps,
+                                           uint32_t pass) {
+    const int total = base[R], lane = threadIdx.x & 31;
+    for (; f < total; f += nwarps) {
+        const int r = g_find_rep(base, R, f);
+        if (ctl[r].done) continue;
+        const GDev &s = g_warp_dev(slot, rep, reps, r);
+        g_flag_chain(s, f - base[r], s.epoch0 + pass, lane);
+    }
+}
+
 constexpr int GRUN_THREADS = 256;
 constexpr int GRUN_MIN_BLOCKS = 2;
 constexpr int MAX_RESTARTS = 16;  // per leg, then the local repair takes over
@@ -3861,15 +3880,9 @@ __global__ void __launch_bounds__(GRUN_THREADS, GRUN_MIN_BLOCKS) k_run_graph(GBa
                     g_resolve_chain(s, f - B.chain_base[r], restart ? tw_r : g_window_start(s, w),
                                     s.epoch0 + pass, f, bl);
                 }
-                // (what a chain read its run alone left: of few chains the warps
-                // without one find the flag meanwhile)
-                for (int f = nwarps - 1 - gw; f < total_chains && !simple && sub == 0;
-                     f += nwarps) {
-                    const int r = g_find_rep(B.chain_base, R, f);
-                    if (!g_rep_on(B, r)) continue;
-                    const GDev &s = g_warp_dev(my_dev, my_rep, B.reps, r);
-                    g_flag_chain(s, f - B.chain_base[r], s.epoch0 + pass, lane);
-                }
+                if (!simple && sub == 0)
+                    g_flag_strict(B.reps, B.ctl, B.chain_base, R, my_dev, my_rep,
+                                  nwarps - 1 - gw, nwarps, pass);
                 if (!barrier()) return;
                 mark(GPH_PASS1);
                 {
